@@ -628,7 +628,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     mbar_init(cx.bar(kQEmpty), 2);
     for (int s = 0; s < 2; ++s) {
       mbar_init(cx.bar(kRawFull + s), 1);     // the TMA thread's expect-tx; the copies complete the bytes
-      mbar_init(cx.bar(kRawEmpty + s), 128);  // the dequant threads have the stage's contents in registers
+      mbar_init(cx.bar(kRawEmpty + s), 128);  // the dequant threads have expanded the stage's contents
     }
     mbar_init(cx.bar(kOFree + 0), 128 * kC);
     mbar_init(cx.bar(kOFree + 1), 128 * kC);
@@ -1146,13 +1146,18 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (PAIR && ct >= 0) {
           load_raw_staged<BITS, G, kNW>(rv, raw_codes + kRawVCodes, raw_meta + kRawVScale, raw_meta + kRawVZero, dt,
                                         ct * kBlockN + dt < p.n_cached, v_word0);
-          mbar_arrive(cx.bar(kRawEmpty + (n_raw & 1)));      // the stage's contents are in registers
-          ++n_raw;
         }
         if (ct >= 0) {
           dequant_values<BITS, GROUP, kNW>(rv, smem + kOffV + s * kTileBytes, dt, v_word0, v_piece0);
           fence_proxy_async_smem();
           if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v1), v1 < p.n_cached, v_word0);
+          if constexpr (PAIR) {
+            // The staging ring's stage goes back to the TMA thread only here, where everything read from it has been used
+            // and the proxy fence above has been passed: an arrival right behind the loads let the next bulk copy, when
+            // the TMA thread was already waiting for it (a range that starts in the cache), overtake them.
+            mbar_arrive(cx.bar(kRawEmpty + (n_raw & 1)));
+            ++n_raw;
+          }
         }
         arrive_lead(kVFull + s);
         KVQ_STAMP(21);

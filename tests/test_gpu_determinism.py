@@ -53,3 +53,24 @@ def test_repeated_launches_give_identical_bytes(name, heads, tokens, chunks, lau
     assert int(status.item()) == 0
     for a, b in zip(cache.buffers, first_bytes):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("bits,group", [(2, 32), (2, 128), (4, 32)])
+def test_pair_ranges_that_start_in_the_cache_give_identical_bytes(bits, group):
+    """More units than SM pairs, so that the last round is cut into ranges: most of them start in the cache, where the
+    TMA thread waits for the dequantizing warps to give back a stage of packed tiles and refills it at once."""
+    from paper_2605_26266_b200 import binding as B
+    b, h, m, n, d = 2, 32, 2048, 8192, 128
+    g = torch.Generator(device="cuda").manual_seed(7)
+    draw = lambda t: torch.randn(b, h, t, d, device="cuda", generator=g)
+    cache = B.Cache(b, h, d, bits, group, n)
+    heavy = draw(n) / (sum(draw(n).square() for _ in range(3)) / 3).sqrt()           # Student-t(3) keys
+    heavy[..., :8] *= 10.0                                                           # a few keys carry a row: one wrong value row shows
+    B.kvq_quantize_append(cache, heavy.to(torch.bfloat16), draw(n).to(torch.bfloat16))
+    del heavy
+    q, k, v = (draw(m).to(torch.bfloat16) for _ in range(3))
+    first = None
+    for i in range(60):
+        out = B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_TCGEN05_PAIR)
+        first = out if first is None else first
+        assert torch.equal(out.view(torch.int16), first.view(torch.int16)), f"launch {i}"
