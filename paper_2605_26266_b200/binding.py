@@ -91,6 +91,8 @@ def _load():
 
 
 lib = _load()
+_quantize_append, _attn_workspace_bytes, _attn_corrected = lib.kvq_quantize_append, lib.kvq_attn_workspace_bytes, lib.kvq_attn_corrected
+_BF16 = torch.bfloat16
 
 
 class KvqError(RuntimeError):
@@ -107,13 +109,22 @@ def _check(status: int, where: str):
         raise KvqError(status, where)
 
 
+def _strides_of(st) -> kvq_strides:
+    assert len(st) == 4 and st[3] == 1, "tensor must be [batch, heads, tokens, head_dim] with unit inner stride"
+    return kvq_strides(st[0], st[1], st[2])
+
+
 def _strides(t: torch.Tensor) -> kvq_strides:
-    assert t.dim() == 4 and t.stride(3) == 1, "tensor must be [batch, heads, tokens, head_dim] with unit inner stride"
-    return kvq_strides(t.stride(0), t.stride(1), t.stride(2))
+    return _strides_of(t.stride())
+
+
+# The current stream's handle without the Stream object around it: a small append is a few microseconds of Python around a
+# kernel of two, and the object alone was two of them.
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def _ptr(t):
@@ -171,12 +182,14 @@ def kvq_cache_bytes(desc: kvq_cache_desc):
 def kvq_quantize_append(cache: Cache, k: torch.Tensor, v: torch.Tensor, cache_len: int | None = None) -> int:
     """Appends the chunk k, v ([batch, heads, n, head_dim] BF16, CUDA) at token `cache_len`
     (default: the cache's running length) and returns the new length."""
-    assert k.dtype == torch.bfloat16 and v.dtype == torch.bfloat16 and k.is_cuda and v.is_cuda
-    assert k.shape == v.shape and k.stride() == v.stride()
+    assert k.dtype is _BF16 and v.dtype is _BF16 and k.is_cuda and v.is_cuda
+    shape, st = k.shape, k.stride()
+    assert shape == v.shape and st == v.stride()
     pos = cache.length if cache_len is None else cache_len
-    n = k.shape[2]
-    _check(lib.kvq_quantize_append(C.byref(cache.desc), pos, k.data_ptr(), v.data_ptr(), _strides(k), n, _stream()),
-           "kvq_quantize_append")
+    n = shape[2]
+    status = _quantize_append(C.byref(cache.desc), pos, k.data_ptr(), v.data_ptr(), _strides_of(st), n, _stream())
+    if status:
+        _check(status, "kvq_quantize_append")
     cache.length = pos + n
     return cache.length
 
@@ -201,21 +214,27 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
     """out = corrected attention of q over [cache window ; current chunk].  Tensors are
     [batch, heads, tokens, head_dim] BF16 CUDA; returns `out` (allocated if not given)."""
     for t in (q, k_cur, v_cur):
-        assert t.dtype == torch.bfloat16 and t.is_cuda
-    assert k_cur.shape == v_cur.shape and k_cur.stride() == v_cur.stride()
+        assert t.dtype is _BF16 and t.is_cuda
+    kv_shape, kv_st = k_cur.shape, k_cur.stride()
+    assert kv_shape == v_cur.shape and kv_st == v_cur.stride()
     n_cache = cache.length - cache_begin if cache_len is None else cache_len
     if out is None:
         out = torch.empty_like(q, memory_format=torch.contiguous_format)
-    m, n_cur = q.shape[2], k_cur.shape[2]
-    need = kvq_attn_workspace_bytes(cache, n_cache, m, n_cur, flags)
-    if need and (cache.workspace is None or cache.workspace.numel() < need):
-        cache.workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
-    ws = cache.workspace if need else None
-    _check(lib.kvq_attn_corrected(
-        C.byref(cache.desc), cache_begin, n_cache, q.data_ptr(), _strides(q), k_cur.data_ptr(), v_cur.data_ptr(),
-        _strides(k_cur), m, n_cur, out.data_ptr(), _strides(out), float(softmax_scale), flags,
-        _ptr(lse), _ptr(cached_mass), _ptr(ws), ws.numel() if ws is not None else 0, _ptr(status_word), _stream()),
-        "kvq_attn_corrected")
+    m, n_cur, desc, size = q.shape[2], kv_shape[2], C.byref(cache.desc), C.c_size_t(0)
+    status = _attn_workspace_bytes(desc, n_cache, m, n_cur, flags, C.byref(size))
+    if status:
+        _check(status, "kvq_attn_workspace_bytes")
+    need, ws = size.value, None
+    if need:
+        ws = cache.workspace
+        if ws is None or ws.numel() < need:
+            ws = cache.workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+    status = _attn_corrected(
+        desc, cache_begin, n_cache, q.data_ptr(), _strides_of(q.stride()), k_cur.data_ptr(), v_cur.data_ptr(),
+        _strides_of(kv_st), m, n_cur, out.data_ptr(), _strides_of(out.stride()), float(softmax_scale), flags, _ptr(lse),
+        _ptr(cached_mass), _ptr(ws), ws.numel() if need else 0, _ptr(status_word), _stream())
+    if status:
+        _check(status, "kvq_attn_corrected")
     return out
 
 
