@@ -1,26 +1,32 @@
 // Quantize-append kernel: Hadamard rotation (keys), group-wise asymmetric round-to-nearest
 // quantization (Eq. (1)), bit packing and coalesced append of one finished chunk's K and V.
 //
-// Eight lanes own one token-head vector (lane l8 holds channels [l8*EPL, (l8+1)*EPL), EPL = head_dim/8), so a
-// warp works on four vectors at a time.  The Walsh-Hadamard butterfly runs its first log2(EPL) stages inside a
-// lane and the remaining three across lanes with shuffles; group minimum/maximum are shuffle reductions over
-// the lanes of a group, and a lane's codes fill whole 32-bit words.  Every add, subtract, multiply and divide
-// is a single IEEE binary32 operation (no contraction), so the stored codes, steps and zero-points are
-// reproducible bit for bit.  A CTA stages the packed bytes of 32 consecutive tokens in shared memory and
-// writes them out with 128-bit stores (tokens of one (batch, head) are contiguous in the cache).  CTAs are
-// persistent (a few per SM) and keep the next tile's loads in flight while they work on the current one.
-// By its bytes the kernel would be HBM-bound on its BF16 input; in fact it is bound by instruction issue: the
-// bit-exact contract fixes one IEEE operation per butterfly, division, rounding and clamp, about 230 warp
-// instructions per token-head, against 576 bytes.
+// Four lanes own one token-head vector (lane lv holds channels [lv*EPL, (lv+1)*EPL), EPL = head_dim/4), so a warp
+// works on eight consecutive tokens, each warp by itself: a lane's codes fill a whole store (16 to 128 bits), the stores
+// of a warp are contiguous, and nothing is staged in shared memory.  The Walsh-Hadamard butterfly runs its first
+// log2(EPL) stages inside a lane and the remaining two across lanes with shuffles; group minimum/maximum are shuffle
+// reductions over the lanes of a group.  Every add, subtract, multiply and divide is a single IEEE binary32 operation
+// (no contraction), so the stored codes, steps and zero-points are reproducible bit for bit.
+//
+// By its bytes the kernel would be HBM-bound on its BF16 input; in fact it is bound by instruction issue, because the
+// bit-exact contract fixes the operations.  A lane therefore keeps its values as pairs (channel i, channel i + EPL/2) in
+// the two halves of 64-bit registers and does everything but the last in-lane butterfly stage and the minimum/maximum
+// with the packed instructions (add/mul/fma.rn.f32x2: two IEEE operations each), and adds the zero-point, clamps and packs
+// the codes two at a time as 16-bit integers.  Measured at 24 heads x 4680 tokens, 128 channels, 2 bits, group 64
+// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 22.5 us as here with
+// eight lanes per vector (shorter lanes repeat the per-group work more often), 21.8 us with four (3.0 TB/s); two
+// tokens in flight per lane and persistent warps with a prefetch: 26.6 us (fewer warps fit).
+#include <math_constants.h>
+
 #include "kvq_common.cuh"
 
 namespace kvq {
 namespace {
 
-constexpr int kTileTokens = 32;
-constexpr int kWarps = 8;
-constexpr int kTokPerWarp = kTileTokens / kWarps;
-constexpr int kCtasPerSm = 4;      // persistent grid: SMs x this (a multiple of the SM count)
+constexpr int kWarps = 4;
+constexpr int kLanes = 4;          // lanes per token-head vector
+constexpr int kTokPerWarp = 32 / kLanes;
+constexpr int kCtasPerSm = 5;      // register budget: up to 96 a thread, nothing spilled
 
 struct QParams {
   const uint16_t* k; const uint16_t* v;
@@ -30,68 +36,87 @@ struct QParams {
   int skip_k;                  // per-channel keys: the keys are written by quantize_k_per_channel_kernel instead
   const int8_t* signs;
   uint8_t* codes[2]; uint8_t* scale[2]; uint16_t* zero[2];
-  int tiles_per_bh;
-  int64_t total_tiles;
 };
 
-// y = c_d * H_d * x for a vector spread over 8 lanes (lane l8 holds channels [l8*EPL, (l8+1)*EPL)):
-// stages h = 1, 2, 4, ... in that order, one rounding per operation.  The first log2(EPL) stages stay in
-// registers, the last three exchange with lanes l8^1, l8^2, l8^4.
+// The EPL values of a lane as pairs: v[i] = (x[i], x[i + EPL/2]).
 template <int EPL>
-__device__ __forceinline__ void hadamard(float (&x)[EPL], int l8, float c_d) {
+struct Pairs { float2 v[EPL / 2]; };
+
+// y = c_d * H_d * x for a vector spread over four lanes (lane lv holds channels [lv*EPL, (lv+1)*EPL)):
+// stages h = 1, 2, 4, ... in that order, one rounding per operation.  The first log2(EPL) stages stay in
+// registers (the last of them, h = EPL/2, inside the pairs), the last two exchange with lanes lv^1 and lv^2.
+template <int EPL>
+__device__ __forceinline__ void hadamard(Pairs<EPL>& x, int lv, float c_d) {
+  constexpr int HP = EPL / 2;
+  const float2 minus = make_float2(-1.0f, -1.0f);
 #pragma unroll
-  for (int h = 1; h < EPL; h *= 2) {
+  for (int h = 1; h < HP; h *= 2) {
 #pragma unroll
-    for (int i = 0; i < EPL; ++i) {
+    for (int i = 0; i < HP; ++i) {
       if ((i & h) == 0) {
-        const float a = x[i], b = x[i + h];
-        x[i] = __fadd_rn(a, b);
-        x[i + h] = __fsub_rn(a, b);
+        const float2 a = x.v[i], b = x.v[i + h];
+        x.v[i] = __fadd2_rn(a, b);
+        x.v[i + h] = __ffma2_rn(b, minus, a);          // a - b, rounded once
       }
     }
   }
 #pragma unroll
-  for (int lm = 1; lm < 8; lm *= 2) {
-    const float sg = (l8 & lm) ? -1.0f : 1.0f;       // upper partner: other - own; fma(+-1, own, other) rounds once
+  for (int i = 0; i < HP; ++i) {
+    const float a = x.v[i].x, b = x.v[i].y;
+    x.v[i] = make_float2(__fadd_rn(a, b), __fsub_rn(a, b));
+  }
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-      const float o = __shfl_xor_sync(0xFFFFFFFFu, x[e], lm);
-      x[e] = __fmaf_rn(sg, x[e], o);
+  for (int lm = 1; lm < kLanes; lm *= 2) {
+    const float sg = (lv & lm) ? -1.0f : 1.0f;       // upper partner: other - own; fma(+-1, own, other) rounds once
+    const float2 sg2 = make_float2(sg, sg);
+#pragma unroll
+    for (int i = 0; i < HP; ++i) {
+      const float2 o = make_float2(__shfl_xor_sync(0xFFFFFFFFu, x.v[i].x, lm), __shfl_xor_sync(0xFFFFFFFFu, x.v[i].y, lm));
+      x.v[i] = __ffma2_rn(sg2, x.v[i], o);
     }
   }
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) x[e] = __fmul_rn(x[e], c_d);
+  for (int i = 0; i < HP; ++i) x.v[i] = __fmul2_rn(x.v[i], make_float2(c_d, c_d));
 }
 
-// Quantizes the vector held by 8 lanes and stages codes / step / zero-point of token slot `tok` in shared
-// memory.  The per-group work (range, step, zero-point) is shared by the GROUP/EPL lanes of a group.
-template <int EPL, int BITS, int GROUP>
-__device__ __forceinline__ void quantize_stage(const float (&x)[EPL], int l8, int tok,
-                                               uint32_t* s_codes, uint8_t* s_scale, uint16_t* s_zero) {
-  constexpr float L = (float)((1 << BITS) - 1);
-  constexpr int kBitsPerLane = EPL * BITS;             // 16, 32 or 64
-  constexpr int kWordsPerTok = 8 * kBitsPerLane / 32;
-  constexpr int lanes_per_group = GROUP / EPL;
-  constexpr int G = (8 * EPL) / GROUP;
+// What a lane stores for its vector: its codes (32 to 128 bits, 16 at the least) and its group's step and zero-point.
+template <int EPL, int BITS>
+struct Quantized { uint32_t w[EPL * BITS > 32 ? EPL * BITS / 32 : 1]; uint32_t sbyte, zbits; };
 
-  float mn = fminf(x[0], x[1]), mx = fmaxf(x[0], x[1]);
+// Quantizes the vector held by kLanes lanes.  The per-group work (range, step, zero-point) is shared by the GROUP/EPL
+// lanes of a group.
+template <int EPL, int BITS, int GROUP>
+__device__ __forceinline__ Quantized<EPL, BITS> quantize(const Pairs<EPL>& x) {
+  constexpr float L = (float)((1 << BITS) - 1);
+  constexpr int HP = EPL / 2;
+  constexpr int lanes_per_group = GROUP / EPL;
+
+  float mn = fminf(x.v[0].x, x.v[0].y), mx = fmaxf(x.v[0].x, x.v[0].y);
+  float seen = mx;                                    // NaN if any value is (a maximum that propagates it)
 #pragma unroll
-  for (int e = 2; e < EPL; e += 2) {                  // three-input minimum and maximum: one instruction per two elements
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(mn) : "f"(mn), "f"(x[e]), "f"(x[e + 1]));
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(mx) : "f"(mx), "f"(x[e]), "f"(x[e + 1]));
+  for (int i = 1; i < HP; ++i) {                      // three-input minimum and maximum: one instruction per two elements
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(mn) : "f"(mn), "f"(x.v[i].x), "f"(x.v[i].y));
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(seen) : "f"(seen), "f"(x.v[i].x), "f"(x.v[i].y));
+  }
+  if (!__any_sync(0xFFFFFFFFu, !(seen == seen) || !(x.v[0].x == x.v[0].x) || !(x.v[0].y == x.v[0].y))) {
+    mx = seen;
+  } else {                                            // some value of the warp is NaN: the maximum of the others
+    seen = CUDART_NAN_F;
+#pragma unroll
+    for (int i = 1; i < HP; ++i) mx = fmaxf(mx, fmaxf(x.v[i].x, x.v[i].y));
   }
 #pragma unroll
   for (int off = 1; off < lanes_per_group; off *= 2) {
     mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, off));
     mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
   }
-  // Divisions.  x / b as q0 = x*r, rem = fma(-q0, b, x), q = fma(rem, r, q0) with r = RN(1/b) is the correctly
-  // rounded quotient for every divisor used here (3, 15 and the 126 positive E4M3 values: checked against
-  // IEEE division for all 2^23 significands of x) as long as nothing overflows.  A quotient too small to be
-  // computed exactly needs no care: it is below 2^-40 and rounds to the integer 0, or to the step floor 2^-9,
-  // either way.  Rounding to an integer is q + 1.5*2^23 - 1.5*2^23 (the FMA pipe instead of the quarter-rate
-  // conversion unit), which is rint(q) while |q| < 2^22.  Vectors with magnitudes or quotients beyond those
-  // bounds take IEEE division and rintf instead, the whole warp together.
+  // Divisions.  x / b as q0 = x*r, rem = fma(-q0, b, x), q = fma(rem, r, q0) with r = RN(1/b) (Markstein's correction
+  // of an approximate quotient by its exact remainder) is the correctly rounded quotient for every divisor used here
+  // (3, 15 and the 126 positive E4M3 values: checked against IEEE division for all 2^23 significands of x) as long
+  // as nothing overflows.  A quotient too small to be computed exactly needs no care: it is below 2^-40 and rounds to
+  // the integer 0, or to the step floor 2^-9, either way.  Rounding to an integer is q + 1.5*2^23 (the FMA pipe instead
+  // of the quarter-rate conversion unit), whose low mantissa bits are rint(q) while |q| < 2^22.  Vectors with magnitudes
+  // or quotients beyond those bounds take IEEE division and rintf instead, the whole warp together.
   const float range = __fsub_rn(mx, mn);
   const float amax = fmaxf(fabsf(range), fmaxf(fabsf(mn), fabsf(mx)));
   auto fast_div = [](float a, float b, float r) {
@@ -105,190 +130,149 @@ __device__ __forceinline__ void quantize_stage(const float (&x)[EPL], int l8, in
   if (sbyte == 0) sbyte = 1;                       // floor at the smallest subnormal 2^-9
   const float ds = e4m3_byte_to_f32(sbyte);
   const float rds = __frcp_rn(ds);
-  const bool slow = __any_sync(0xFFFFFFFFu, big || !(__fmul_rn(amax, rds) < 0x1p21f));
+  const float reach = __fmul_rn(amax, rds);        // bound of |x / step|
   constexpr float kRound = 12582912.f;             // 1.5 * 2^23
-  const float z = __fsub_rn(0.0f, slow ? rintf(__fdiv_rn(mn, ds)) : __fsub_rn(__fadd_rn(fast_div(mn, ds, rds), kRound), kRound));
-  const uint32_t zbits = f32_to_bf16_bits(z);
-  const float zs = bf16_bits_to_f32(zbits);
-
-  // Codes are packed 16 bits at a time as exact float sums c_e * 2^(bit position), then read out of the low
-  // mantissa bits of sum + 2^23.
-  constexpr int kChunks = kBitsPerLane / 16;
-  float acc[kChunks];
+  Quantized<EPL, BITS> out;
+  out.sbyte = sbyte;
+  constexpr int F = HP < 16 / BITS ? HP : 16 / BITS;   // codes in a 16-bit field
+  constexpr int kAcc = HP / F;                         // words of two such fields
+  uint32_t acc[kAcc];
+  if (!__any_sync(0xFFFFFFFFu, big || !(reach < 0x1p13f) || !(seen == seen))) {
+    // rint(x / step) is the low half of the bits of x / step + 1.5*2^23, a 16-bit integer here, as is the zero-point:
+    // two values at a time, one byte permutation gathers the halves, one instruction adds the zero-point and clamps to
+    // [0, L], one integer multiply-add puts the codes into the 16-bit fields of channels [.., EPL/2) and [EPL/2, ..).
+    const float z = __fsub_rn(0.0f, __fsub_rn(__fadd_rn(fast_div(mn, ds, rds), kRound), kRound));
+    out.zbits = f32_to_bf16_bits(z);
+    const uint32_t zi = __float_as_uint(__fadd_rn(bf16_bits_to_f32(out.zbits), kRound));
+    const uint32_t z2 = __byte_perm(zi, zi, 0x1010);
+    const float2 r2 = make_float2(rds, rds), nds2 = make_float2(-ds, -ds), round2 = make_float2(kRound, kRound);
 #pragma unroll
-  for (int k = 0; k < kChunks; ++k) acc[k] = 8388608.f;
-  if (!slow) {
-    // q + 1.5*2^23 is 1.5*2^23 + rint(q); taking off 1.5*2^23 - zero (an integer below 2^24, so exact) leaves
-    // rint(q) + zero, the sum Eq. (1) clamps.  While the zero-point is exact in BF16 (|zero| <= 256) the sum cannot
-    // be negative (x >= min and both roundings are monotonic), so the lower clamp is only taken when some group of
-    // the warp has a rounded zero-point.
+    for (int i = 0; i < HP; ++i) {
+      const float2 q0 = __fmul2_rn(x.v[i], r2);
+      const float2 q = __ffma2_rn(__ffma2_rn(q0, nds2, x.v[i]), r2, q0);
+      const float2 n = __fadd2_rn(q, round2);
+      const uint32_t n2 = __byte_perm(__float_as_uint(n.x), __float_as_uint(n.y), 0x5410);
+      const uint32_t c2 = __viaddmin_s16x2_relu(n2, z2, BITS == 2 ? 0x00030003u : 0x000F000Fu);
+      const int k = i / F, pos = (i % F) * BITS;
+      acc[k] = pos == 0 ? c2 : c2 * (1u << pos) + acc[k];
+    }
+  } else {
+    const bool slow = __any_sync(0xFFFFFFFFu, big || !(reach < 0x1p21f));
+    const float z = __fsub_rn(0.0f, slow ? rintf(__fdiv_rn(mn, ds)) : __fsub_rn(__fadd_rn(fast_div(mn, ds, rds), kRound), kRound));
+    out.zbits = f32_to_bf16_bits(z);
+    const float zs = bf16_bits_to_f32(out.zbits);
     const float kz = __fsub_rn(kRound, zs);
-    if (__any_sync(0xFFFFFFFFu, zs != z)) {
+    const bool low = __any_sync(0xFFFFFFFFu, zs != z);
+    // the lower clamp first where it is needed: fminf / fmaxf return the other operand for a NaN
+    auto code = [&](float v) {
+      float c;
+      if (slow) c = fmaxf(__fadd_rn(rintf(__fdiv_rn(v, ds)), zs), 0.0f);
+      else { c = __fsub_rn(__fadd_rn(fast_div(v, ds, rds), kRound), kz); if (low) c = fmaxf(c, 0.0f); }
+      return (uint32_t)fminf(c, L);
+    };
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) {
-        const float c = fminf(fmaxf(__fsub_rn(__fadd_rn(fast_div(x[e], ds, rds), kRound), kz), 0.0f), L);
-        acc[(e * BITS) / 16] = __fmaf_rn(c, (float)(1u << ((e * BITS) % 16)), acc[(e * BITS) / 16]);
-      }
-    } else {
+    for (int k = 0; k < kAcc; ++k) acc[k] = 0;
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) {
-        const float c = fminf(__fsub_rn(__fadd_rn(fast_div(x[e], ds, rds), kRound), kz), L);
-        acc[(e * BITS) / 16] = __fmaf_rn(c, (float)(1u << ((e * BITS) % 16)), acc[(e * BITS) / 16]);
-      }
-    }
-  } else {
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-      const float c = fminf(fmaxf(__fadd_rn(rintf(__fdiv_rn(x[e], ds)), zs), 0.0f), L);
-      acc[(e * BITS) / 16] = __fmaf_rn(c, (float)(1u << ((e * BITS) % 16)), acc[(e * BITS) / 16]);
+    for (int i = 0; i < HP; ++i) {
+      const int k = i / F, pos = (i % F) * BITS;
+      acc[k] |= (code(x.v[i].x) | (code(x.v[i].y) << 16)) << pos;
     }
   }
-  uint32_t piece[(kBitsPerLane + 31) / 32];
-  if constexpr (kChunks == 1) {
-    piece[0] = __float_as_uint(acc[0]) & 0xFFFFu;
-  } else {
+  if constexpr (F * BITS == 8) out.w[0] = (acc[0] | (acc[0] >> 8)) & 0xFFFFu;
+  else if constexpr (kAcc == 1) out.w[0] = acc[0];
+  else {
 #pragma unroll
-    for (int k = 0; k < kChunks; k += 2)
-      piece[k / 2] = __byte_perm(__float_as_uint(acc[k]), __float_as_uint(acc[k + 1]), 0x5410);
+    for (int k = 0; k < kAcc; k += 2) {            // low fields: the first half of the lane's channels
+      out.w[k / 2] = __byte_perm(acc[k], acc[k + 1], 0x5410);
+      out.w[(kAcc + k) / 2] = __byte_perm(acc[k], acc[k + 1], 0x7632);
+    }
   }
-  if constexpr (kBitsPerLane == 16) {                  // two lanes share a word
-    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, piece[0], 1);
-    if ((l8 & 1) == 0) s_codes[tok * kWordsPerTok + (l8 >> 1)] = piece[0] | (other << 16);
-  } else if constexpr (kBitsPerLane == 32) {
-    s_codes[tok * kWordsPerTok + l8] = piece[0];
-  } else {
-    *reinterpret_cast<uint2*>(&s_codes[tok * kWordsPerTok + 2 * l8]) = make_uint2(piece[0], piece[1]);
-  }
-  if ((l8 % lanes_per_group) == 0) {
-    s_scale[tok * G + l8 / lanes_per_group] = (uint8_t)sbyte;
-    s_zero[tok * G + l8 / lanes_per_group] = (uint16_t)zbits;
-  }
-}
-
-// Cooperative shared->global copy with the widest store both sides allow.
-__device__ __forceinline__ void copy_out(uint8_t* dst, const uint8_t* src, int nbytes, int tid, int nthreads) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src) | (uintptr_t)nbytes;
-  if ((a & 15) == 0) {
-    for (int i = tid; i < nbytes / 16; i += nthreads)
-      reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
-  } else if ((a & 3) == 0) {
-    for (int i = tid; i < nbytes / 4; i += nthreads)
-      reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
-  } else if ((a & 1) == 0) {
-    for (int i = tid; i < nbytes / 2; i += nthreads)
-      reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
-  } else {
-    for (int i = tid; i < nbytes; i += nthreads) dst[i] = src[i];
-  }
+  return out;
 }
 
 template <int EPL>
 struct RawVec { uint4 r[EPL / 8]; };      // EPL BF16 values of one lane
 
 template <int EPL>
-__device__ __forceinline__ void load_raw_vec(RawVec<EPL>& v, const uint16_t* p, int l8) {
+__device__ __forceinline__ void load_raw_vec(RawVec<EPL>& v, const uint16_t* p, int lv) {
 #pragma unroll
-  for (int i = 0; i < EPL / 8; ++i) v.r[i] = __ldg(reinterpret_cast<const uint4*>(p) + l8 * (EPL / 8) + i);
+  for (int i = 0; i < EPL / 8; ++i) v.r[i] = __ldg(reinterpret_cast<const uint4*>(p) + lv * (EPL / 8) + i);
 }
 template <int EPL>
-__device__ __forceinline__ void decode_vec(const RawVec<EPL>& v, float (&x)[EPL]) {
+__device__ __forceinline__ void decode_vec(const RawVec<EPL>& v, Pairs<EPL>& x) {
 #pragma unroll
   for (int i = 0; i < EPL / 8; ++i) {
     const uint32_t w[4] = {v.r[i].x, v.r[i].y, v.r[i].z, v.r[i].w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      x[8 * i + 2 * e] = bf16_bits_to_f32(w[e] & 0xFFFFu);
-      x[8 * i + 2 * e + 1] = bf16_bits_to_f32(w[e] >> 16);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int c = 8 * i + 2 * e + j;                      // channel of the lane
+        const float f = j ? __uint_as_float(w[e] & 0xFFFF0000u) : __uint_as_float(w[e] << 16);
+        if (c < EPL / 2) x.v[c].x = f; else x.v[c - EPL / 2].y = f;
+      }
     }
   }
 }
+template <int EPL>
+__device__ __forceinline__ void apply_signs(Pairs<EPL>& x, const int8_t* signs) {
+#pragma unroll
+  for (int i = 0; i < EPL / 2; ++i)
+    x.v[i] = __fmul2_rn(x.v[i], make_float2((float)signs[i], (float)signs[i + EPL / 2]));
+}
 
-// Persistent CTAs: each walks tiles of 32 consecutive tokens of one (batch, head) with a stride of gridDim.x
-// and has the next tile's loads in flight while it rotates, quantizes and packs the current one.  A warp
-// works on four token-head vectors at a time, eight lanes per vector.
+// A warp takes eight consecutive tokens of one (batch, head), four lanes per token.  Blocks are not persistent: enough
+// warps are resident to hide the loads, and the hardware deals the blocks out evenly.
 template <int D, int BITS, int GROUP>
-__global__ void __launch_bounds__(kWarps * 32) quantize_append_kernel(QParams p) {
-  constexpr int EPL = D / 8;
+__global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) quantize_append_kernel(QParams p) {
+  constexpr int EPL = D / kLanes;
   constexpr int CB = D * BITS / 8;
-  __shared__ __align__(16) uint32_t s_codes[2][kTileTokens * CB / 4];
-  __shared__ __align__(16) uint8_t s_scale[2][kTileTokens * 4];
-  __shared__ __align__(16) uint16_t s_zero[2][kTileTokens * 4];
-
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int l8 = lane & 7;
-  const int tok = warp * kTokPerWarp + (lane >> 3);          // token slot inside the tile
   constexpr int G = D / GROUP;
+  constexpr int lanes_per_group = GROUP / EPL;
+  const int lane = threadIdx.x & 31, lv = lane & (kLanes - 1);
   const float c_d = (D == 64) ? 0.125f : __uint_as_float(0x3DB504F3u);
-
-  RawVec<EPL> rk, rv;
-  auto fetch = [&](int tile_g) {
-    const int bh = tile_g / p.tiles_per_bh;
-    const int tile = tile_g - bh * p.tiles_per_bh;
-    const int b = bh / p.heads, h = bh - b * p.heads;
-    const int64_t t = (int64_t)tile * kTileTokens + tok;
-    if (t < p.n_tokens) {
-      const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + t * p.st;
-      load_raw_vec<EPL>(rk, p.k + off, l8);
-      load_raw_vec<EPL>(rv, p.v + off, l8);
-    } else {                                                  // slots past the end quantize zeros, never stored
+  const int bh = blockIdx.y, b = bh / p.heads, h = bh - b * p.heads;
+  const int64_t t0 = ((int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5)) * kTokPerWarp;
+  if (t0 >= p.n_tokens) return;                               // the whole warp
+  const int64_t t = t0 + lane / kLanes;
+  const bool valid = t < p.n_tokens;
+  RawVec<EPL> raw[2];
+  if (valid) {
+    const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + t * p.st;
+    if (!p.skip_k) load_raw_vec<EPL>(raw[0], p.k + off, lv);
+    load_raw_vec<EPL>(raw[1], p.v + off, lv);
+  } else {                                                    // tokens past the end quantize zeros, never stored
 #pragma unroll
-      for (int i = 0; i < EPL / 8; ++i) { rk.r[i] = make_uint4(0, 0, 0, 0); rv.r[i] = make_uint4(0, 0, 0, 0); }
+    for (int w = 0; w < 2; ++w)
+#pragma unroll
+      for (int i = 0; i < EPL / 8; ++i) raw[w].r[i] = make_uint4(0, 0, 0, 0);
+  }
+  // slot of this token, modulo the capacity (p.cache_len is already reduced, and an append brings at most
+  // `capacity` tokens, so one subtraction does)
+  int64_t slot = p.cache_len + t;
+  if (slot >= p.capacity) slot -= p.capacity;
+  const int64_t at = (int64_t)bh * p.capacity + slot;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    if (w == 0 && p.skip_k) continue;
+    Pairs<EPL> x;
+    decode_vec<EPL>(raw[w], x);
+    if (w == 0 ? p.rotate : p.rotate_v) {                     // values are stored rotated with KVQ_ROTATE_V only
+      if (p.signs) apply_signs<EPL>(x, p.signs + lv * EPL);
+      hadamard<EPL>(x, lv, c_d);
     }
-  };
-
-  int tile_g = blockIdx.x;
-  const int total_tiles = (int)p.total_tiles;
-  if (tile_g < total_tiles) fetch(tile_g);
-  for (; tile_g < total_tiles; tile_g += gridDim.x) {
-    const int bh = tile_g / p.tiles_per_bh;
-    const int tile = tile_g - bh * p.tiles_per_bh;
-    const int64_t t0 = (int64_t)tile * kTileTokens;
-    const int nt = (int)min((int64_t)kTileTokens, p.n_tokens - t0);
-    float x[EPL];
-    decode_vec<EPL>(rk, x);
-    const RawVec<EPL> rv_cur = rv;
-    if (tile_g + (int)gridDim.x < total_tiles) fetch(tile_g + (int)gridDim.x);
-    if (!p.skip_k) {
-      if (p.rotate) {
-        if (p.signs) {
-#pragma unroll
-          for (int e = 0; e < EPL; ++e) x[e] = __fmul_rn(x[e], (float)p.signs[l8 * EPL + e]);
-        }
-        hadamard<EPL>(x, l8, c_d);
-      }
-      quantize_stage<EPL, BITS, GROUP>(x, l8, tok, s_codes[0], s_scale[0], s_zero[0]);
-    }
-    decode_vec<EPL>(rv_cur, x);
-    if (p.rotate_v) {                                       // values stored rotated too (KVQ_ROTATE_V)
-      if (p.signs) {
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) x[e] = __fmul_rn(x[e], (float)p.signs[l8 * EPL + e]);
-      }
-      hadamard<EPL>(x, l8, c_d);
-    }
-    quantize_stage<EPL, BITS, GROUP>(x, l8, tok, s_codes[1], s_scale[1], s_zero[1]);
-    __syncthreads();
-    // The tile goes to slots slot0 .. slot0 + nt - 1, modulo the capacity: one piece, or two when a ring
-    // cache wraps inside the tile (p.cache_len is already reduced modulo the capacity, so one subtraction does).
-    int64_t slot0 = p.cache_len + t0;
-    if (slot0 >= p.capacity) slot0 -= p.capacity;
-    const int n_first = (int)min((int64_t)nt, p.capacity - slot0);
-#pragma unroll 1
-    for (int piece = 0; piece < 2; ++piece) {
-      const int ntok = piece ? nt - n_first : n_first;
-      if (ntok <= 0) break;
-      const int skip = piece ? n_first : 0;                    // tokens of the tile stored by the first piece
-      const int64_t tok_index = (int64_t)bh * p.capacity + (piece ? 0 : slot0);
-#pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        if (w == 0 && p.skip_k) continue;
-        copy_out(p.codes[w] + tok_index * CB, reinterpret_cast<const uint8_t*>(s_codes[w]) + skip * CB, ntok * CB, threadIdx.x, kWarps * 32);
-        copy_out(p.scale[w] + tok_index * G, s_scale[w] + skip * G, ntok * G, threadIdx.x, kWarps * 32);
-        copy_out(reinterpret_cast<uint8_t*>(p.zero[w] + tok_index * G), reinterpret_cast<const uint8_t*>(s_zero[w] + skip * G),
-                 ntok * G * 2, threadIdx.x, kWarps * 32);
+    const Quantized<EPL, BITS> q = quantize<EPL, BITS, GROUP>(x);
+    if (valid) {
+      uint8_t* dst = p.codes[w] + at * CB + lv * (EPL * BITS / 8);
+      if constexpr (EPL * BITS == 16) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)q.w[0];
+      else if constexpr (EPL * BITS == 32) *reinterpret_cast<uint32_t*>(dst) = q.w[0];
+      else if constexpr (EPL * BITS == 64) *reinterpret_cast<uint2*>(dst) = make_uint2(q.w[0], q.w[1]);
+      else *reinterpret_cast<uint4*>(dst) = make_uint4(q.w[0], q.w[1], q.w[2], q.w[3]);
+      if ((lv % lanes_per_group) == 0) {
+        p.scale[w][at * G + lv / lanes_per_group] = (uint8_t)q.sbyte;
+        p.zero[w][at * G + lv / lanes_per_group] = (uint16_t)q.zbits;
       }
     }
-    __syncthreads();
   }
 }
 
@@ -300,7 +284,7 @@ __global__ void __launch_bounds__(kWarps * 32) quantize_append_kernel(QParams p)
 // the layout every other kernel reads.  An analysis option: nothing here is tuned.
 template <int D, int BITS>
 __global__ void __launch_bounds__(256) quantize_k_per_channel_kernel(QParams p) {
-  constexpr int EPL = D / 8;
+  constexpr int EPL = D / kLanes;
   constexpr int CB = D * BITS / 8;
   constexpr int LDY = D + 1;
   extern __shared__ __align__(16) uint8_t pc_smem[];
@@ -309,22 +293,22 @@ __global__ void __launch_bounds__(256) quantize_k_per_channel_kernel(QParams p) 
   uint8_t* codes = pc_smem + (size_t)g * LDY * sizeof(float);          // [g][D]
   const int bh = blockIdx.y, b = bh / p.heads, h = bh - b * p.heads;
   const int64_t t0 = (int64_t)blockIdx.x * g;                          // first token of the block within the chunk
-  const int lane = threadIdx.x & 31, l8 = lane & 7;
+  const int lane = threadIdx.x & 31, lv = lane & (kLanes - 1);
   const float c_d = (D == 64) ? 0.125f : __uint_as_float(0x3DB504F3u);
-  for (int r = threadIdx.x >> 3; r < g; r += 32) {                     // 8 lanes per token, 32 tokens per pass
+  for (int r = threadIdx.x / kLanes; r < g; r += 256 / kLanes) {       // kLanes lanes per token
     RawVec<EPL> raw;
-    load_raw_vec<EPL>(raw, p.k + (int64_t)b * p.sb + (int64_t)h * p.sh + (t0 + r) * p.st, l8);
-    float x[EPL];
+    load_raw_vec<EPL>(raw, p.k + (int64_t)b * p.sb + (int64_t)h * p.sh + (t0 + r) * p.st, lv);
+    Pairs<EPL> x;
     decode_vec<EPL>(raw, x);
     if (p.rotate) {
-      if (p.signs) {
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) x[e] = __fmul_rn(x[e], (float)p.signs[l8 * EPL + e]);
-      }
-      hadamard<EPL>(x, l8, c_d);
+      if (p.signs) apply_signs<EPL>(x, p.signs + lv * EPL);
+      hadamard<EPL>(x, lv, c_d);
     }
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) y[r * LDY + l8 * EPL + e] = x[e];
+    for (int i = 0; i < EPL / 2; ++i) {
+      y[r * LDY + lv * EPL + i] = x.v[i].x;
+      y[r * LDY + lv * EPL + i + EPL / 2] = x.v[i].y;
+    }
   }
   __syncthreads();
   int64_t slot0 = p.cache_len + t0;                                    // whole blocks never straddle the end of a ring
@@ -392,13 +376,9 @@ int launch_quantize_append(const kvq_cache_desc* d, int64_t cache_len, const voi
   p.codes[0] = static_cast<uint8_t*>(d->k_codes); p.codes[1] = static_cast<uint8_t*>(d->v_codes);
   p.scale[0] = static_cast<uint8_t*>(d->k_scale); p.scale[1] = static_cast<uint8_t*>(d->v_scale);
   p.zero[0] = static_cast<uint16_t*>(d->k_zero); p.zero[1] = static_cast<uint16_t*>(d->v_zero);
-  p.tiles_per_bh = (int)((n_tokens + kTileTokens - 1) / kTileTokens);
-  p.total_tiles = (int64_t)d->batch * d->heads * p.tiles_per_bh;
-  int sms = 0;
-  { const int r = device_sm_count(&sms); if (r != KVQ_OK) return r; }
-  const int64_t blocks = p.total_tiles < (int64_t)sms * kCtasPerSm ? p.total_tiles : (int64_t)sms * kCtasPerSm;
-  dim3 grid((unsigned)blocks), block(kWarps * 32);
-  if (p.total_tiles > 0x7FFFFFFFLL - 65536) return KVQ_ERR_UNSUPPORTED;
+  const int64_t blocks = (n_tokens + kWarps * kTokPerWarp - 1) / (kWarps * kTokPerWarp);
+  if (blocks > 0x7FFFFFFFLL) return KVQ_ERR_UNSUPPORTED;
+  const dim3 grid((unsigned)blocks, (unsigned)(d->batch * d->heads)), block(kWarps * 32);
 #define KVQ_QA(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) { quantize_append_kernel<D_, B_, G_><<<grid, block, 0, st>>>(p); launched = true; }
   bool launched = false;
   KVQ_QA(128, 2, 32) KVQ_QA(128, 2, 64) KVQ_QA(128, 2, 128) KVQ_QA(128, 4, 32) KVQ_QA(128, 4, 64) KVQ_QA(128, 4, 128)

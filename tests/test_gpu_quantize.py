@@ -112,6 +112,25 @@ def test_degenerate_groups_and_strided_input(B):
         T.assert_cache_equal(T.gpu_cache_arrays(g, 40), o, 40)
 
 
+@pytest.mark.parametrize("d,bits,group", [(64, 2, 32), (128, 2, 128), (128, 4, 32)])
+def test_quotients_around_the_16_bit_path_bit_exact(B, d, bits, group):
+    """Constant groups get the smallest step (2^-9), so a value c has the quotient 512 c: on both sides of the bounds
+    2^13 and 2^21 where the kernel changes between its 16-bit, 32-bit and IEEE-division forms, with either sign, alone in
+    a warp's tokens or beside ordinary ones; 19 tokens leave a ragged last warp."""
+    c = np.array([0.5, 1.0, 15.9, 16.0, 16.125, 17.0, 31.0, 63.75, 64.0, 64.5, 255.0, 256.0, 4080.0, 4096.0, 4112.0, 5000.0,
+                  2.0 ** -20, 1e30, 7.0], np.float32)
+    x = np.random.default_rng(3).standard_normal((1, 2, c.size, d)).astype(np.float32)
+    x[0, 0] = c[:, None]
+    x[0, 1, ::2, :group] = -c[::2, None]
+    kb, vb = inputs.f32_to_bf16_bits(x), inputs.f32_to_bf16_bits(x[:, ::-1].copy())
+    for rotate in (False, True):
+        g = B.Cache(1, 2, d, bits, group, 128, rotate_k=rotate)
+        o = O.Cache(1, 2, d, bits, group, 128, rotate_k=rotate)
+        B.kvq_quantize_append(g, T.to_dev(kb), T.to_dev(vb))
+        O.quantize_append(o, 0, kb, vb)
+        T.assert_cache_equal(T.gpu_cache_arrays(g, c.size), o, c.size)
+
+
 def test_append_errors(B):
     g = B.Cache(1, 1, 128, 2, 128, 128)
     k = torch.zeros(1, 1, 100, 128, dtype=torch.bfloat16, device="cuda")
