@@ -83,10 +83,11 @@ extern "C" {
                                       KVQ_ERR_UNSUPPORTED): an analysis option, several times slower. */
 #define KVQ_KERNEL_AUTO       0u         /* head_dim 128 with TMA-addressable strides: the pair kernel unless its units of 512
                                             query rows pad m_tokens too far beyond a multiple of 256 (by more than 1/0.88
-                                            at 2 bits, 1/0.86 at 4), then the one-CTA tcgen05 kernel; everything else: the
-                                            warp-level kernel */
+                                            at 2 bits, 1/0.86 at 4), then the one-CTA tcgen05 kernel; head_dim 64 with such
+                                            strides and the workspace that kvq_attn_workspace_bytes asks for: the one-CTA
+                                            tcgen05 kernel; everything else: the warp-level kernel */
 #define KVQ_KERNEL_MMA_SYNC   (1u << 8)  /* force the warp-level mma.sync kernel (cross-check / fallback shapes) */
-#define KVQ_KERNEL_TCGEN05    (2u << 8)  /* force the tcgen05/TMEM kernel; KVQ_ERR_UNSUPPORTED if the shape is not covered */
+#define KVQ_KERNEL_TCGEN05    (2u << 8)  /* force the tcgen05/TMEM kernel; KVQ_ERR_UNSUPPORTED unless head_dim is 128 */
 #define KVQ_KERNEL_TCGEN05_PAIR (3u << 8) /* the tcgen05 kernel on pairs of SMs (thread-block clusters of two CTAs that share
                                             one tcgen05.mma of 256 rows): each CTA of a pair expands only half of every
                                             cached key and value tile.  Same shapes as KVQ_KERNEL_TCGEN05; results equal to

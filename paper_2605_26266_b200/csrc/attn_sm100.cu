@@ -44,12 +44,16 @@
 // caller's workspace and a small kernel merges them.
 //
 // The same source also gives the pair kernel (template parameter PAIR): a cluster of two CTAs on 512 query rows
-// whose tensor cores work as one (tcgen05 cta_group::2), described at the kernel.
+// whose tensor cores work as one (tcgen05 cta_group::2), described at the kernel; and the kernel for heads of 64
+// channels (D = 64, one CTA per unit): operand tiles one 64-column block wide at the same places, half the MMA steps of a
+// score, 16 heads x 1560 queries over 7 700 keys in 141 us against 650 us in the warp-level kernel.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA records a diagnostic in the caller's status
 // word, all roles leave their loops, in-flight work is drained with a bounded wait, TMEM is freed and the
 // kernel returns.
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "kvq_common.cuh"
 #include "sm100_ptx.cuh"
@@ -58,7 +62,7 @@ namespace kvq {
 namespace {
 using namespace ptx;
 
-constexpr int kD = 128;
+constexpr int kD = 128;                            // the widest head: strides of the operand tiles in shared memory
 constexpr int kBlockM = 128;
 constexpr int kBlockN = 128;
 constexpr int kThreads = 512;
@@ -123,7 +127,8 @@ struct TParams {
   const uint16_t* ax_rows; // workspace: bias operand rows written by rotate_query_kernel, [batch*heads][m_tokens][8]
 };
 
-// One partial result: the segment's own normalised output O / l as BF16, then FP32 m[256], l_cur[256],
+// One partial result: the segment's own normalised output O / l as BF16 (heads of 128 channels; heads of 64 have
+// room for FP32 in the same slot, pieces of 4 columns), then FP32 m[256], l_cur[256],
 // l_cached[256] (running maximum in log2 units and the row sums over current and cached keys).  The output is
 // stored by 16-byte pieces of 8 columns, piece (column group g, row r) at (g * 256 + r) * 16: the softmax
 // threads hold one row each, so the 32 lanes of a store instruction write 512 contiguous bytes (row-major, they
@@ -276,9 +281,9 @@ __device__ __forceinline__ uint32_t xtile_offset(int row, int kc) {
   return (uint32_t)((row >> 3) * 256 + kc * 128 + (row & 7) * 16);
 }
 
-template <int BITS>
+template <int BITS, int D = kD>
 struct Raw {   // packed codes and metadata of one cached token (keys or values)
-  static constexpr int kWords = kD * BITS / 32;
+  static constexpr int kWords = D * BITS / 32;
   uint32_t w[kWords];
   uint32_t sbytes;       // scale bytes of up to 4 groups
   uint32_t z01, z23;     // zero-points (BF16 bits) of up to 4 groups
@@ -286,8 +291,8 @@ struct Raw {   // packed codes and metadata of one cached token (keys or values)
 
 // Loads NW code words of the token, starting at word `word0` (a multiple of 4), into r.w[0 .. NW), and the token's
 // metadata.  NW is the whole row, or half of it for a CTA of a pair.
-template <int BITS, int G, int NW = Raw<BITS>::kWords>
-__device__ __forceinline__ void load_raw(Raw<BITS>& r, const uint8_t* codes, const uint8_t* scale, const uint16_t* zero,
+template <int BITS, int G, int D, int NW = Raw<BITS, D>::kWords>
+__device__ __forceinline__ void load_raw(Raw<BITS, D>& r, const uint8_t* codes, const uint8_t* scale, const uint16_t* zero,
                                          int64_t tok, bool valid, int word0 = 0) {
   if (!valid) {   // rows past the end of the cache dequantize to exact zeros
 #pragma unroll
@@ -295,7 +300,7 @@ __device__ __forceinline__ void load_raw(Raw<BITS>& r, const uint8_t* codes, con
     r.sbytes = 0; r.z01 = 0; r.z23 = 0;
     return;
   }
-  const uint4* cw = reinterpret_cast<const uint4*>(codes + tok * (kD * BITS / 8)) + (word0 >> 2);
+  const uint4* cw = reinterpret_cast<const uint4*>(codes + tok * (D * BITS / 8)) + (word0 >> 2);
 #pragma unroll
   for (int i = 0; i < NW / 4; ++i) {
     const uint4 v = __ldg(cw + i);
@@ -314,8 +319,8 @@ __device__ __forceinline__ void load_raw(Raw<BITS>& r, const uint8_t* codes, con
 }
 
 // The same from the staging ring in shared memory (pair kernel): `key` is the token's place in its tile.
-template <int BITS, int G, int NW>
-__device__ __forceinline__ void load_raw_staged(Raw<BITS>& r, const uint8_t* codes, const uint8_t* scale, const uint8_t* zero,
+template <int BITS, int G, int D, int NW>
+__device__ __forceinline__ void load_raw_staged(Raw<BITS, D>& r, const uint8_t* codes, const uint8_t* scale, const uint8_t* zero,
                                                 int key, bool valid, int word0) {
   if (!valid) {
 #pragma unroll
@@ -323,7 +328,7 @@ __device__ __forceinline__ void load_raw_staged(Raw<BITS>& r, const uint8_t* cod
     r.sbytes = 0; r.z01 = 0; r.z23 = 0;
     return;
   }
-  const uint4* cw = reinterpret_cast<const uint4*>(codes + key * (kD * BITS / 8)) + (word0 >> 2);
+  const uint4* cw = reinterpret_cast<const uint4*>(codes + key * (D * BITS / 8)) + (word0 >> 2);
 #pragma unroll
   for (int i = 0; i < NW / 4; ++i) {
     const uint4 v = cw[i];
@@ -341,10 +346,10 @@ __device__ __forceinline__ void load_raw_staged(Raw<BITS>& r, const uint8_t* cod
   }
 }
 
-template <int BITS>
-__device__ __forceinline__ float raw_step(const Raw<BITS>& r, int j) { return e4m3_byte_to_f32((r.sbytes >> (8 * j)) & 0xFFu); }
-template <int BITS>
-__device__ __forceinline__ float raw_zero(const Raw<BITS>& r, int j) {
+template <int BITS, int D>
+__device__ __forceinline__ float raw_step(const Raw<BITS, D>& r, int j) { return e4m3_byte_to_f32((r.sbytes >> (8 * j)) & 0xFFu); }
+template <int BITS, int D>
+__device__ __forceinline__ float raw_zero(const Raw<BITS, D>& r, int j) {
   const uint32_t z = (j < 2) ? r.z01 : r.z23;
   return bf16_bits_to_f32((z >> (16 * (j & 1))) & 0xFFFFu);
 }
@@ -363,14 +368,14 @@ __device__ __forceinline__ uint32_t pick_group(const uint32_t* a, int j) {
 // Pairs are (i, i + 8) of each 16-code word (2-bit) or (i, i + 4) of each 8-code word (4-bit): the
 // contraction dimension is stored permuted, and the rotated query is stored with the same permutation.
 // Expands the NW words r.w[0 .. NW), which are words word0 .. word0 + NW - 1 of the token, into row `row` of the tile.
-template <int BITS, int GROUP, int NW = Raw<BITS>::kWords>
-__device__ __forceinline__ void dequant_keys(const Raw<BITS>& r, uint8_t* tile, int row, int word0 = 0) {
-  constexpr int G = kD / GROUP;
+template <int BITS, int GROUP, int D, int NW = Raw<BITS, D>::kWords>
+__device__ __forceinline__ void dequant_keys(const Raw<BITS, D>& r, uint8_t* tile, int row, int word0 = 0) {
+  constexpr int G = D / GROUP;
   constexpr float kOff = (BITS == 2) ? 4.f : 16.f;
   uint32_t step2[4], c2[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float ds = raw_step<BITS>(r, j), zs = raw_zero<BITS>(r, j);
+    const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
     step2[j] = pack_f16x2_sat(ds, ds);
     const float c = -(kOff + zs) * ds;
     c2[j] = pack_f16x2_sat(c, c);
@@ -414,13 +419,13 @@ __device__ __forceinline__ void dequant_keys(const Raw<BITS>& r, uint8_t* tile, 
 // multiply (the 16 + zero offset times the step is not always representable in BF16).  Words as for the keys;
 // the 16-byte pieces land at piece index (token's piece index - piece0), so that a CTA of a pair keeps its 64
 // channels in one 64-column block.
-template <int BITS, int GROUP, int NW = Raw<BITS>::kWords>
-__device__ __forceinline__ void dequant_values(const Raw<BITS>& r, uint8_t* tile, int row, int word0 = 0, int piece0 = 0) {
-  constexpr int G = kD / GROUP;
+template <int BITS, int GROUP, int D, int NW = Raw<BITS, D>::kWords>
+__device__ __forceinline__ void dequant_values(const Raw<BITS, D>& r, uint8_t* tile, int row, int word0 = 0, int piece0 = 0) {
+  constexpr int G = D / GROUP;
   uint32_t step2[4], c2[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float ds = raw_step<BITS>(r, j), zs = raw_zero<BITS>(r, j);
+    const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
     step2[j] = pack_bf16x2(ds, ds);
     const float c = (BITS == 2) ? -(4.f + zs) * ds : (16.f + zs);
     c2[j] = pack_bf16x2(c, c);
@@ -472,31 +477,32 @@ __device__ __forceinline__ void dequant_values(const Raw<BITS>& r, uint8_t* tile
 // and -(sigma/24) nu_{m,j} (per-group squared norms of q~) as a BF16 high part plus a BF16 low part.  The
 // attention kernel swaps the rotated tile in by TMA once the current chunk's score MMAs are done, so units
 // split over several CTAs rotate their rows once instead of once per CTA.
-// 16 lanes per row, 8 channels per lane; a warp handles two rows, a block of 8 warps 16 rows (many small
+// D / 8 lanes per row, 8 channels per lane; with 128 channels a warp handles two rows, a block of 8 warps 16 (many small
 // blocks: the kernel is a chain of dependent shuffles per row, so it wants every row in flight at once).
 struct RotParams {
   const uint16_t* q; int64_t q_sb, q_sh, q_st;
-  uint16_t* qr;            // [batch * heads][m_tokens][128] FP16
+  uint16_t* qr;            // [batch * heads][m_tokens][D] FP16
   uint16_t* ax;            // [batch * heads][m_tokens][8] BF16: high parts of groups 0..3, then low parts
   const int8_t* signs;
   int heads, m_tokens, rotate;
   float ax_coef;           // -sigma / 24
 };
 
-template <int BITS, int GROUP>
+template <int BITS, int GROUP, int D>
 __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
+  constexpr int kLanes = D / 8;                      // per row
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int l16 = lane & 15, rsub = lane >> 4;
+  const int ln = lane & (kLanes - 1), rsub = lane / kLanes;
   constexpr int lanes_per_group = GROUP / 8;
   const int bh = blockIdx.y, b = bh / p.heads, h = bh - b * p.heads;
   float sgn[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) sgn[e] = (p.rotate && p.signs) ? (float)p.signs[l16 * 8 + e] : 1.0f;
+  for (int e = 0; e < 8; ++e) sgn[e] = (p.rotate && p.signs) ? (float)p.signs[ln * 8 + e] : 1.0f;
   {
-    const int row = blockIdx.x * 16 + warp * 2 + rsub;
+    const int row = (blockIdx.x * 8 + warp) * (32 / kLanes) + rsub;
     const bool valid = row < p.m_tokens;             // no early exit: the shuffles below need every lane
     uint4 raw = make_uint4(0, 0, 0, 0);
-    if (valid) raw = __ldg(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + l16);
+    if (valid) raw = __ldg(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
     float x[8];
     x[0] = bf16_bits_to_f32(raw.x & 0xFFFFu); x[1] = bf16_bits_to_f32(raw.x >> 16);
     x[2] = bf16_bits_to_f32(raw.y & 0xFFFFu); x[3] = bf16_bits_to_f32(raw.y >> 16);
@@ -511,14 +517,14 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
         for (int i = 0; i < 8; ++i)
           if ((i & hh) == 0) { const float a = x[i], c = x[i + hh]; x[i] = a + c; x[i + hh] = a - c; }
 #pragma unroll
-      for (int lm = 1; lm < 16; lm *= 2)
+      for (int lm = 1; lm < kLanes; lm *= 2)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float o = __shfl_xor_sync(0xFFFFFFFFu, x[e], lm);
-          x[e] = (l16 & lm) ? (o - x[e]) : (x[e] + o);
+          x[e] = (ln & lm) ? (o - x[e]) : (x[e] + o);
         }
 #pragma unroll
-      for (int e = 0; e < 8; ++e) x[e] *= 0.08838834764831845f;
+      for (int e = 0; e < 8; ++e) x[e] *= D == 64 ? 0.125f : 0.08838834764831845f;
     }
     float nu = 0.f;
 #pragma unroll
@@ -533,12 +539,12 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
       uint32_t h4[4], l4[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int src = (lane & 16) + ((j * lanes_per_group) & 15);
+        const int src = (lane & ~(kLanes - 1)) + ((j * lanes_per_group) & (kLanes - 1));
         const uint32_t hj = __shfl_sync(0xFFFFFFFFu, hi, src), lj = __shfl_sync(0xFFFFFFFFu, lo, src);
-        const bool have = j * GROUP < kD;
+        const bool have = j * GROUP < D;
         h4[j] = have ? hj : 0u; l4[j] = have ? lj : 0u;
       }
-      if (valid && l16 == 0)
+      if (valid && ln == 0)
         *reinterpret_cast<uint4*>(p.ax + ((int64_t)bh * p.m_tokens + row) * 8) =
             make_uint4(h4[0] | (h4[1] << 16), h4[2] | (h4[3] << 16), l4[0] | (l4[1] << 16), l4[2] | (l4[3] << 16));
     }
@@ -546,7 +552,7 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
     if constexpr (BITS == 2) {
       // physical column 16w + 2i + hsel <- channel 16w + i + 8*hsel: even lanes own the low half
       // of a 16-channel word, odd lanes the high half; swap four values with the neighbour
-      const bool odd = l16 & 1;
+      const bool odd = ln & 1;
       float rcv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) rcv[i] = __shfl_xor_sync(0xFFFFFFFFu, odd ? x[i] : x[4 + i], 1);
@@ -561,7 +567,7 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
       for (int i = 0; i < 4; ++i) { y[2 * i] = x[i]; y[2 * i + 1] = x[4 + i]; }
     }
     if (valid)
-      *(reinterpret_cast<uint4*>(p.qr + ((int64_t)bh * p.m_tokens + row) * kD) + l16) =
+      *(reinterpret_cast<uint4*>(p.qr + ((int64_t)bh * p.m_tokens + row) * D) + ln) =
         make_uint4(pack_f16x2_sat(y[0], y[1]), pack_f16x2_sat(y[2], y[3]), pack_f16x2_sat(y[4], y[5]), pack_f16x2_sat(y[6], y[7]));
   }
 }
@@ -577,7 +583,7 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
 // ring for the PACKED tiles: the TMA thread brings the codes and metadata of the next cached tile in with bulk
 // copies, and the dequant warps expand them from shared memory (the one-CTA kernel has no room for that and
 // reads them from global memory into registers a tile ahead).
-template <int BITS, int GROUP, bool PAIR>
+template <int BITS, int GROUP, bool PAIR, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qr,
                     const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const TParams p) {
@@ -604,7 +610,19 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const int n_rt = (p.n_cur + kBlockN - 1) / kBlockN;
   const int n_ct = (p.n_cached + kBlockN - 1) / kBlockN;
   const int T = n_rt + n_ct;
-  constexpr int G = kD / GROUP;
+  constexpr int G = D / GROUP;
+  constexpr int kBlocks = D / 64;                                 // 64-column blocks of an operand tile
+  constexpr uint32_t kLoadBytes = kBlocks * kHalfTile;            // bytes of a tile
+  // Heads of 64 channels: the products are 80 columns wide.  Column 64 of every value tile is one (the second 64-column
+  // block of the stages, otherwise unused, holds it for good), so that O carries the row sum of the weights as they were
+  // rounded to BF16, and the output is normalised by it: the rounding of the largest weights then cancels.
+  constexpr bool kOnes = D == 64;
+  constexpr int kNV = kOnes ? 80 : D;                             // columns of O
+  // They also follow the running maximum exactly (the largest weight of a row is then 1, without a rounding): the
+  // warp-level kernel, which served these heads before, does, and with the lazy maximum the outputs were up to 18 %
+  // further from 64-bit results than its.  16 x 1560 queries over 6 144 tokens: 120 us lazy, 141 us exact, 650 us there.
+  constexpr float kGrowth = D == 64 ? 0.f : kRescaleThreshold;
+  static_assert(D == 128 || !PAIR, "a pair's CTAs take one 64-channel block of the values each");
 
   if (tid == 0) {
     misc[1] = 0;
@@ -638,6 +656,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // bias operand tiles start as zeros (columns beyond the group count stay zero for good)
   for (int i = tid; i < 4 * kXBytes / 16; i += kThreads)
     reinterpret_cast<uint4*>(smem + kOffAx)[i] = make_uint4(0, 0, 0, 0);
+  if constexpr (kOnes) {                         // two 16-byte pieces per row: 1, 0 ... 0
+    const int row = (tid >> 1) & 127, piece = tid & 1;            // 512 threads: two stages x 128 rows x two pieces
+    *reinterpret_cast<uint4*>(smem + kOffV + (tid >> 8) * kTileBytes + sw128_offset(row, 8 + piece)) = make_uint4(piece ? 0u : 0x3F80u, 0, 0, 0);
+  }
   if (warp == 0) {
     if constexpr (PAIR) { tmem_alloc_pair(sbase + kOffMisc, 512); tmem_relinquish_pair(); }
     else { tmem_alloc(sbase + kOffMisc, 512); tmem_relinquish(); }
@@ -665,7 +687,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // multiple of 128), so every source address and size below is a multiple of 16 bytes.
       int n_raw = 0;
       auto stage_packed = [&](int ct, int bh) -> bool {
-        constexpr int kCB = kD * BITS / 8;
+        constexpr int kCB = D * BITS / 8;
         const int rs = n_raw & 1;
         if (!cx.wait(kRawEmpty + rs, ((n_raw >> 1) & 1) ^ 1, 104)) return false;
         const uint32_t bar = cx.bar(kRawFull + rs);
@@ -705,9 +727,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (!(ok = cx.wait(kQEmpty, (nseg & 1) ^ 1, 100))) break;
         // a segment that starts in the cache never needs the unrotated query: load the rotated one right away
         const bool cached0 = sg.tb >= n_rt;
-        expect_tx_lead(kQFull, 2 * kTileBytes);
+        expect_tx_lead(kQFull, 2 * kLoadBytes);
         for (int qt = 0; qt < 2; ++qt)
-          for (int kb = 0; kb < 2; ++kb)
+          for (int kb = 0; kb < kBlocks; ++kb)
             load_q(sbase + kOffQ + qt * kTileBytes + kb * kHalfTile, cached0 ? &tm_qr : &tm_q, lead(kQFull), kb * 64, row0 + qt * kBlockM, h, b);
         if (cached0 || sg.te <= n_rt) arrive_lead(kQRotFull);   // this thread's share of the phase
         for (int t = sg.tb; t < sg.te; ++t, ++it) {
@@ -716,15 +738,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if (t == n_rt && !cached0) {
             // first cached tile: once no MMA reads the unrotated query any more, the rotated tile replaces it
             if (!(ok = cx.wait(kQCurDone, nseg & 1, 103))) break;
-            expect_tx_lead(kQRotFull, 2 * kTileBytes);
+            expect_tx_lead(kQRotFull, 2 * kLoadBytes);
             for (int qt = 0; qt < 2; ++qt)
-              for (int kb = 0; kb < 2; ++kb)
+              for (int kb = 0; kb < kBlocks; ++kb)
                 load_q(sbase + kOffQ + qt * kTileBytes + kb * kHalfTile, &tm_qr, lead(kQRotFull), kb * 64, row0 + qt * kBlockM, h, b);
             rot_seg = nseg;
           }
           if (!(ok = cx.wait(kKEmpty + s, ph ^ 1, 101))) break;
           if (t < n_rt) {
-            expect_tx_lead(kKFull + s, kTileBytes / kC);
+            expect_tx_lead(kKFull + s, kLoadBytes / kC);
             if constexpr (PAIR) {
               // this CTA's 32 keys of each half of the tile (local rows 32 hf .. 32 hf + 31): boxes of 32 rows
               for (int hf = 0; hf < 2; ++hf)
@@ -732,7 +754,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                   tma_load_4d_pair(sbase + kOffK + s * kTileBytes + kb * kHalfTile + hf * 32 * 128, &tm_k, lead(kKFull + s), kb * 64,
                               t * kBlockN + 64 * hf + 32 * (int)rank, h, b);
             } else {
-              for (int kb = 0; kb < 2; ++kb)
+              for (int kb = 0; kb < kBlocks; ++kb)
                 tma_load_4d(sbase + kOffK + s * kTileBytes + kb * kHalfTile, &tm_k, cx.bar(kKFull + s), kb * 64, t * kBlockN, h, b);
             }
           } else {
@@ -740,11 +762,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           }
           if (!(ok = cx.wait(kVEmpty + s, ph ^ 1, 102))) break;
           if (t < n_rt) {
-            expect_tx_lead(kVFull + s, kTileBytes / kC);
+            expect_tx_lead(kVFull + s, kLoadBytes / kC);
             if constexpr (PAIR) {   // this CTA's 64 value channels of all 128 keys: one 64-column block
               tma_load_4d_pair(sbase + kOffV + s * kTileBytes, &tm_v, lead(kVFull + s), 64 * (int)rank, t * kBlockN, h, b);
             } else {
-              for (int kb = 0; kb < 2; ++kb)
+              for (int kb = 0; kb < kBlocks; ++kb)
                 tma_load_4d(sbase + kOffV + s * kTileBytes + kb * kHalfTile, &tm_v, cx.bar(kVFull + s), kb * 64, t * kBlockN, h, b);
             }
             issued_it = it;
@@ -786,7 +808,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       constexpr int kM = PAIR ? 256 : 128;
       const uint32_t idesc_bf16 = make_idesc_bf16(kM, 64, 0, 0);
       const uint32_t idesc_f16 = idesc_bf16 & ~((7u << 7) | (7u << 10));     // A, B format 0 = FP16
-      const uint32_t idesc_pv = make_idesc_bf16(kM, 128, 0, 1);               // B (values) is MN-major
+      const uint32_t idesc_pv = make_idesc_bf16(kM, kNV, 0, 1);               // B (values) is MN-major
       // commit: one arrival when every MMA issued so far has completed; of a pair, on the barrier of both CTAs
       auto commit = [&](int i) { if constexpr (PAIR) tc_commit_pair(cx.bar(i), (uint16_t)3); else tc_commit(cx.bar(i)); };
       // Descriptors are built once; stepping along K only adds a constant to the 14-bit address field
@@ -823,10 +845,12 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           mma_ss_off<2>(d_tmem, qd, kd, idesc, 1);
           mma_ss_off<4>(d_tmem, qd, kd, idesc, 1);
           mma_ss_off<6>(d_tmem, qd, kd, idesc, 1);
-          mma_ss_off<kBlk>(d_tmem, qd, kd, idesc, 1);
-          mma_ss_off<kBlk + 2>(d_tmem, qd, kd, idesc, 1);
-          mma_ss_off<kBlk + 4>(d_tmem, qd, kd, idesc, 1);
-          mma_ss_off<kBlk + 6>(d_tmem, qd, kd, idesc, 1);
+          if constexpr (D == 128) {
+            mma_ss_off<kBlk>(d_tmem, qd, kd, idesc, 1);
+            mma_ss_off<kBlk + 2>(d_tmem, qd, kd, idesc, 1);
+            mma_ss_off<kBlk + 4>(d_tmem, qd, kd, idesc, 1);
+            mma_ss_off<kBlk + 6>(d_tmem, qd, kd, idesc, 1);
+          }
           if (cached && p.correction) mma_ss(d_tmem, axd, bxd, idesc_bf16, 1);
         }
         commit(kSFull + 2 * hf + qt);
@@ -965,7 +989,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             for (int c = 0; c < 4; ++c) mx[c] = max3(mx[c], __uint_as_float(sr[i + 2 * c]), __uint_as_float(sr[i + 2 * c + 1]));
           }
           const float m_new = fmaxf(m_run, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c_row);
-          if (__any_sync(0xFFFFFFFFu, m_new - m_run > kRescaleThreshold)) {
+          if (__any_sync(0xFFFFFFFFu, m_new - m_run > kGrowth)) {
             if (!fresh) {
               // the product of the previous half (the last one issued on this O) must have retired
               ok = __all_sync(0xFFFFFFFFu, cx.wait(kODone + 2 * (hf ^ 1) + qt, (it - (hf ^ 1)) & 1, 302));
@@ -973,7 +997,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
               tc_fence_after();
               const float f = ex2(m_run - m_new);
 #pragma unroll 1
-              for (int c = 0; c < 8; ++c) {
+              for (int c = 0; c < kNV / 16; ++c) {
                 uint32_t r[16];
                 tmem_ld16(o_addr + 16 * c, r);
                 tmem_wait_ld();
@@ -1016,23 +1040,35 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // a whole unit writes its rows of the output; a partial segment writes the same normalised rows into its
       // slot, with the statistics the merge kernel weighs them by
       const float l = lcur + lcac;
-      const float inv = 1.0f / l;
+      float norm = l;
+      if constexpr (kOnes) {
+        uint32_t r[16];
+        tmem_ld16(o_addr + 64, r);
+        tmem_wait_ld();
+        norm = __uint_as_float(r[0]);
+      }
+      const float inv = 1.0f / norm;
       const bool store = !whole || row < p.m_tokens;
       // consecutive 8-column pieces: 16 bytes apart in a row of the output, 4096 bytes apart in a slot
       uint8_t* dst = whole ? reinterpret_cast<uint8_t*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st)
                            : slot + r256 * 16;
       const int piece = whole ? 16 : 4096;
 #pragma unroll 1
-      for (int hf = 0; hf < 2; ++hf) {               // 64 columns at a time
+      for (int hf = 0; hf < kBlocks; ++hf) {         // 64 columns at a time
         uint32_t sr[64];
         tmem_ld32(o_addr + 64 * hf, sr);
         tmem_ld32(o_addr + 64 * hf + 32, sr + 32);
         tmem_wait_ld();
-        if (hf == 1) {                               // the whole row is in registers: O can be overwritten
+        if (hf == kBlocks - 1) {                     // the whole row is in registers: O can be overwritten
           tc_fence_before();
           arrive_lead(kOFree + qt);
         }
-        if (store) {
+        if (D == 64 && !whole) {                     // partial rows of 64 channels stay FP32, pieces of 4 columns
+#pragma unroll
+          for (int i = 0; i < 64; i += 4)
+            *reinterpret_cast<float4*>(dst + (i >> 2) * piece) =
+                make_float4(__uint_as_float(sr[i]) * inv, __uint_as_float(sr[i + 1]) * inv, __uint_as_float(sr[i + 2]) * inv, __uint_as_float(sr[i + 3]) * inv);
+        } else if (store) {
 #pragma unroll
           for (int i = 0; i < 64; i += 8) {
             uint4 v;
@@ -1048,7 +1084,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (whole) {
           const int64_t idx = (int64_t)bh * p.m_tokens + row;
           if (p.lse) p.lse[idx] = (m_run + log2f(l)) * 0.6931471805599453f;
-          if (p.cached_mass) p.cached_mass[idx] = lcac * inv;
+          if (p.cached_mass) p.cached_mass[idx] = lcac / l;
         } else {
           float* st = reinterpret_cast<float*>(slot + kSlotStats);
           st[r256] = m_run; st[256 + r256] = lcur; st[512 + r256] = lcac;
@@ -1064,7 +1100,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // One CTA: thread dt expands key dt of the tile, keys and values.  A CTA of a pair expands half of each
     // tile: of the keys, its 32 keys of either half tile (local row dt / 2 = 32 hf + j is key 64 hf + 32 rank + j),
     // two threads per key with 64 channels each; of the values, channels [64 rank, 64 rank + 64) of key dt.
-    constexpr int kNW = Raw<BITS>::kWords / kC;                    // code words per thread and tile (keys or values)
+    constexpr int kNW = Raw<BITS, D>::kWords / kC;                    // code words per thread and tile (keys or values)
     const int k_row = PAIR ? (dt >> 1) : dt;                       // row of the key stage this thread writes
     const int k_key = PAIR ? 64 * (k_row >> 5) + 32 * (int)rank + (k_row & 31) : dt;   // its key within the tile
     const int k_word0 = PAIR ? (dt & 1) * kNW : 0;                 // first code word of the key it expands
@@ -1075,7 +1111,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     int it = 0, nseg = 0;
     int n_raw = 0;                         // cached tiles taken from the staging ring so far (pair kernel)
     bool ok = true;
-    Raw<BITS> rk, rv;
+    Raw<BITS, D> rk, rv;
     while (ok && sch.next(sg)) {
       const int bh = sg.unit / p.q_blocks;
       // key k of the window lives in slot cache_begin + k, taken modulo the capacity (ring caches wrap; for
@@ -1088,8 +1124,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const int t_rot = max(sg.tb, n_rt);          // first cached tile of the segment: the query is rotated there
       if (!PAIR && sg.te > n_rt) {                 // one CTA: packed data comes one tile ahead into registers
         const int k0 = (t_rot - n_rt) * kBlockN + k_key, v0 = (t_rot - n_rt) * kBlockN + dt;
-        load_raw<BITS, G, kNW>(rk, p.k_codes, p.k_scale, p.k_zero, tok_of(k0), k0 < p.n_cached, k_word0);
-        load_raw<BITS, G, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v0), v0 < p.n_cached, v_word0);
+        load_raw<BITS, G, D, kNW>(rk, p.k_codes, p.k_scale, p.k_zero, tok_of(k0), k0 < p.n_cached, k_word0);
+        load_raw<BITS, G, D, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v0), v0 < p.n_cached, v_word0);
       }
       for (int t = sg.tb; t < sg.te; ++t, ++it) {
         const int s = it & 1;
@@ -1105,19 +1141,19 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (PAIR && ct >= 0) {
           ok = __all_sync(0xFFFFFFFFu, cx.wait(kRawFull + (n_raw & 1), (n_raw >> 1) & 1, 406));
           if (!ok) break;
-          load_raw_staged<BITS, G, kNW>(rk, raw_codes, raw_meta, raw_meta + kRawKZero, k_key,
+          load_raw_staged<BITS, G, D, kNW>(rk, raw_codes, raw_meta, raw_meta + kRawKZero, k_key,
                                         ct * kBlockN + k_key < p.n_cached, k_word0);
         }
         if (ct >= 0) {
-          dequant_keys<BITS, GROUP, kNW>(rk, smem + kOffK + s * kTileBytes, k_row, k_word0);
+          dequant_keys<BITS, GROUP, D, kNW>(rk, smem + kOffK + s * kTileBytes, k_row, k_word0);
           if (p.correction && k_word0 == 0) {   // B_extra row: step_j^2, exact in BF16
-            const float d0 = raw_step<BITS>(rk, 0), d1 = raw_step<BITS>(rk, 1), d2 = raw_step<BITS>(rk, 2), d3 = raw_step<BITS>(rk, 3);
+            const float d0 = raw_step<BITS, D>(rk, 0), d1 = raw_step<BITS, D>(rk, 1), d2 = raw_step<BITS, D>(rk, 2), d3 = raw_step<BITS, D>(rk, 3);
             const uint32_t b01 = pack_bf16x2(d0 * d0, G > 1 ? d1 * d1 : 0.f), b23 = pack_bf16x2(G > 2 ? d2 * d2 : 0.f, G > 3 ? d3 * d3 : 0.f);
             // columns 0..3 meet the high parts of A_extra, columns 4..7 the low parts
             *reinterpret_cast<uint4*>(smem + kOffBx + s * kXBytes + xtile_offset(k_row, 0)) = make_uint4(b01, b23, b01, b23);
           }
           fence_proxy_async_smem();
-          if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, kNW>(rk, p.k_codes, p.k_scale, p.k_zero, tok_of(k1), k1 < p.n_cached, k_word0);
+          if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, D, kNW>(rk, p.k_codes, p.k_scale, p.k_zero, tok_of(k1), k1 < p.n_cached, k_word0);
         }
         arrive_lead(kKFull + s);
         KVQ_STAMP(20);
@@ -1144,13 +1180,13 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (!ok) break;
         KVQ_STAMP(23);
         if (PAIR && ct >= 0) {
-          load_raw_staged<BITS, G, kNW>(rv, raw_codes + kRawVCodes, raw_meta + kRawVScale, raw_meta + kRawVZero, dt,
+          load_raw_staged<BITS, G, D, kNW>(rv, raw_codes + kRawVCodes, raw_meta + kRawVScale, raw_meta + kRawVZero, dt,
                                         ct * kBlockN + dt < p.n_cached, v_word0);
         }
         if (ct >= 0) {
-          dequant_values<BITS, GROUP, kNW>(rv, smem + kOffV + s * kTileBytes, dt, v_word0, v_piece0);
+          dequant_values<BITS, GROUP, D, kNW>(rv, smem + kOffV + s * kTileBytes, dt, v_word0, v_piece0);
           fence_proxy_async_smem();
-          if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v1), v1 < p.n_cached, v_word0);
+          if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, D, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v1), v1 < p.n_cached, v_word0);
           if constexpr (PAIR) {
             // The staging ring's stage goes back to the TMA thread only here, where everything read from it has been used
             // and the proxy fence above has been passed: an arrival right behind the loads let the next bulk copy, when
@@ -1181,10 +1217,12 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 }
 
 // Combines the partial results of every unit whose key tiles were split over several CTAs.
-// grid (n_units - n_whole, 16): a block handles 16 rows x 128 columns; thread = (8-column piece, row).
+// grid (n_units - n_whole, 16): a block handles 16 rows x D columns; thread = (piece, row).
 // pair = 1: the schedule's units are 512 rows worked on by CTA pairs (n_ctas counts pairs); the grid has two blocks
 // per unit in x, one for each 256-row half, whose partial results are those of the CTAs of that rank.
+template <int D>
 __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_ctas, int pair) {
+  constexpr int kCols = D / 16;                        // columns of a 16-byte piece: 8 in BF16, 4 in FP32 (64 channels)
   const int su = pair ? blockIdx.x >> 1 : blockIdx.x, rank = pair ? blockIdx.x & 1 : 0, kc = pair ? 2 : 1;
   const int unit = p.n_whole + su;
   const int T = p.tiles;
@@ -1211,10 +1249,11 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   __syncthreads();
   const int c_first = s_first, c_last = s_last, first_slot = s_first_slot;
   if (c_first == c_last) return;                       // the unit was computed whole by one CTA
-  // A thread combines the 8-column piece (cg, row): consecutive lanes take consecutive rows, which are 16 bytes
+  // A thread combines the piece (cg, row): consecutive lanes take consecutive rows, which are 16 bytes
   // apart in a slot.  The finished pieces change places through shared memory so that the output rows are
   // written 256 contiguous bytes at a time.
-  __shared__ uint4 s_tile[16 * 16];
+  using Out = typename std::conditional<D == 64, uint2, uint4>::type;
+  __shared__ Out s_tile[16 * 16];
   const int cg = threadIdx.x >> 4, rr = threadIdx.x & 15;
   const int bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
   const int r256 = blockIdx.y * 16 + rr;
@@ -1233,7 +1272,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
     m = fmaxf(fmaxf(m, fmaxf(mm[0], mm[1])), fmaxf(mm[2], mm[3]));
   }
   // out = sum_i w_i O_i / sum_i w_i with w_i = l_i 2^(m_i - m): every partial row is already normalised by its l_i
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float acc[kCols] = {};
   float l_cur = 0.f, l_cac = 0.f;
   for (int c0 = c_first; c0 <= c_last; c0 += 4) {
     float sm[4], sc[4], sa[4];
@@ -1253,23 +1292,29 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
       const float lc = f * sc[j], la = f * sa[j];
       l_cur += lc; l_cac += la;
       const float w = lc + la;
-      acc[0] += w * bf16_bits_to_f32(a[j].x & 0xFFFFu); acc[1] += w * bf16_bits_to_f32(a[j].x >> 16);
-      acc[2] += w * bf16_bits_to_f32(a[j].y & 0xFFFFu); acc[3] += w * bf16_bits_to_f32(a[j].y >> 16);
-      acc[4] += w * bf16_bits_to_f32(a[j].z & 0xFFFFu); acc[5] += w * bf16_bits_to_f32(a[j].z >> 16);
-      acc[6] += w * bf16_bits_to_f32(a[j].w & 0xFFFFu); acc[7] += w * bf16_bits_to_f32(a[j].w >> 16);
+      const uint32_t pw[4] = {a[j].x, a[j].y, a[j].z, a[j].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if constexpr (D == 64) {
+          acc[e] += w * __uint_as_float(pw[e]);
+        } else {
+          acc[2 * e] += w * bf16_bits_to_f32(pw[e] & 0xFFFFu);
+          acc[2 * e + 1] += w * bf16_bits_to_f32(pw[e] >> 16);
+        }
+      }
     }
   }
   const float l = l_cur + l_cac, inv = 1.0f / l;
-  uint4 v;
+  Out v;
   v.x = cvt_bf16x2(acc[0] * inv, acc[1] * inv); v.y = cvt_bf16x2(acc[2] * inv, acc[3] * inv);
-  v.z = cvt_bf16x2(acc[4] * inv, acc[5] * inv); v.w = cvt_bf16x2(acc[6] * inv, acc[7] * inv);
+  if constexpr (D == 128) { v.z = cvt_bf16x2(acc[4] * inv, acc[5] * inv); v.w = cvt_bf16x2(acc[6] * inv, acc[7] * inv); }
   s_tile[rr * 16 + (cg ^ rr)] = v;
   __syncthreads();
   {
     const int orr = threadIdx.x >> 4, ocg = threadIdx.x & 15;          // output side: a row per 16 lanes
     const int orow = row - rr + orr;
     if (orow < p.m_tokens)
-      *reinterpret_cast<uint4*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)orow * p.o_st + ocg * 8) = s_tile[orr * 16 + (ocg ^ orr)];
+      *reinterpret_cast<Out*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)orow * p.o_st + ocg * kCols) = s_tile[orr * 16 + (ocg ^ orr)];
   }
   if (cg == 0 && row < p.m_tokens) {
     const int64_t idx = (int64_t)bh * p.m_tokens + row;
@@ -1299,11 +1344,11 @@ int get_encode_fn(EncodeTiledFn* fn) {
   return KVQ_OK;
 }
 
-// Byte strides of a [batch, heads, tokens, 128] BF16 tensor as a tensor map wants them: non-zero multiples of 16
+// Byte strides of a [batch, heads, tokens, dim] BF16 tensor as a tensor map wants them: non-zero multiples of 16
 // below 2^40.  A size-1 dimension may come with any stride and gets a harmless valid one.  False if a real
 // dimension's stride cannot be encoded (0, as in a tensor expanded over heads, or too large).
-bool map_strides(kvq_strides s, int64_t tokens, int heads, int batch, cuuint64_t out[3]) {
-  const cuuint64_t st = tokens > 1 ? (cuuint64_t)s.t * 2 : (cuuint64_t)kD * 2;
+bool map_strides(kvq_strides s, int64_t tokens, int heads, int batch, int dim, cuuint64_t out[3]) {
+  const cuuint64_t st = tokens > 1 ? (cuuint64_t)s.t * 2 : (cuuint64_t)dim * 2;
   const cuuint64_t sh = heads > 1 ? (cuuint64_t)s.h * 2 : st * (cuuint64_t)tokens;
   const cuuint64_t sb = batch > 1 ? (cuuint64_t)s.b * 2 : sh * (cuuint64_t)heads;
   out[0] = st; out[1] = sh; out[2] = sb;
@@ -1313,12 +1358,12 @@ bool map_strides(kvq_strides s, int64_t tokens, int heads, int batch, cuuint64_t
   return true;
 }
 
-// [batch, heads, tokens, 128] BF16 tensor -> 4-D map with a 64-column x 128-row box, 128-byte swizzle.
+// [batch, heads, tokens, dim] BF16 tensor -> 4-D map with a 64-column x 128-row box, 128-byte swizzle.
 int make_map(EncodeTiledFn enc, CUtensorMap* map, const void* ptr, kvq_strides s, int64_t tokens, int heads, int batch,
-             int box_rows = kBlockN) {
-  cuuint64_t dims[4] = {(cuuint64_t)kD, (cuuint64_t)tokens, (cuuint64_t)heads, (cuuint64_t)batch};
+             int dim, int box_rows = kBlockN) {
+  cuuint64_t dims[4] = {(cuuint64_t)dim, (cuuint64_t)tokens, (cuuint64_t)heads, (cuuint64_t)batch};
   cuuint64_t strides[3];
-  if (!map_strides(s, tokens, heads, batch, strides)) return KVQ_ERR_UNSUPPORTED;
+  if (!map_strides(s, tokens, heads, batch, dim, strides)) return KVQ_ERR_UNSUPPORTED;
   cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
@@ -1353,7 +1398,7 @@ int max_resident_pairs() {
   if (current_device(&dev) != KVQ_OK) return num_sms() / 2;
   int n = cache[dev].load(std::memory_order_relaxed);
   if (n == 0) {
-    auto kern = attn_tcgen05_kernel<2, 128, true>;     // every instantiation has the same footprint
+    auto kern = attn_tcgen05_kernel<2, 128, true, 128>;     // every instantiation has the same footprint
     n = num_sms() / 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)n); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes;
@@ -1387,18 +1432,19 @@ Plan plan_grid(int64_t n_units, int64_t tiles, bool pair = false) {
   return {(int)(c < 1 ? 1 : c), 0};
 }
 
-template <int BITS, int GROUP, bool PAIR>
+template <int BITS, int GROUP, bool PAIR, int D = 128>
 int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk, const CUtensorMap& mv, const TParams& p,
            const RotParams& rp, dim3 grid, cudaStream_t st) {
   static PerDevice configured;                       // the attribute is per device
   int dev = 0;
   { const int r = current_device(&dev); if (r != KVQ_OK) return r; }
   if (configured.first(dev)) {
-    KVQ_CUDA_TRY(cudaFuncSetAttribute(attn_tcgen05_kernel<BITS, GROUP, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+    KVQ_CUDA_TRY(cudaFuncSetAttribute(attn_tcgen05_kernel<BITS, GROUP, PAIR, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     configured.done(dev);
   }
   if (rp.qr) {                      // there are cached keys: rotate the query chunk first
-    rotate_query_kernel<BITS, GROUP><<<dim3((unsigned)((rp.m_tokens + 15) / 16), (unsigned)(p.n_units / p.q_blocks)), 256, 0, st>>>(rp);
+    constexpr int kRows = 2048 / D;  // of a block
+    rotate_query_kernel<BITS, GROUP, D><<<dim3((unsigned)((rp.m_tokens + kRows - 1) / kRows), (unsigned)(p.n_units / p.q_blocks)), 256, 0, st>>>(rp);
     KVQ_CUDA_TRY(cudaGetLastError());
   }
   if constexpr (PAIR) {             // grid.x counts pairs: two CTAs each, launched as clusters of two
@@ -1408,13 +1454,13 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk,
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    KVQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tcgen05_kernel<BITS, GROUP, true>, mq, mqr, mk, mv, p));
+    KVQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tcgen05_kernel<BITS, GROUP, true, D>, mq, mqr, mk, mv, p));
   } else {
-    attn_tcgen05_kernel<BITS, GROUP, false><<<grid, kThreads, kSmemBytes, st>>>(mq, mqr, mk, mv, p);
+    attn_tcgen05_kernel<BITS, GROUP, false, D><<<grid, kThreads, kSmemBytes, st>>>(mq, mqr, mk, mv, p);
   }
   KVQ_CUDA_TRY(cudaGetLastError());
   if (p.n_whole != p.n_units) {   // units were split over CTAs: combine their partial results
-    attn_merge_kernel<<<dim3((unsigned)((p.n_units - p.n_whole) * (PAIR ? 2 : 1)), 16), 256, 0, st>>>(p, (int)grid.x, PAIR ? 1 : 0);
+    attn_merge_kernel<D><<<dim3((unsigned)((p.n_units - p.n_whole) * (PAIR ? 2 : 1)), 16), 256, 0, st>>>(p, (int)grid.x, PAIR ? 1 : 0);
     KVQ_CUDA_TRY(cudaGetLastError());
   }
   return KVQ_OK;
@@ -1423,14 +1469,14 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk,
 }  // namespace
 
 bool attn_tcgen05_supports(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur) {
-  return d->head_dim == kD && m_tokens >= 1 && n_cur >= 1;
+  return (d->head_dim == 64 || d->head_dim == 128) && m_tokens >= 1 && n_cur >= 1;
 }
 
 bool attn_tcgen05_addressable(const AttnArgs& a) {
   cuuint64_t st[3];
-  return map_strides(a.qs, a.m_tokens, a.desc->heads, a.desc->batch, st) &&
-         map_strides(a.kvs, a.n_cur, a.desc->heads, a.desc->batch, st) &&
-         map_strides(a.vs, a.n_cur, a.desc->heads, a.desc->batch, st);
+  const int heads = a.desc->heads, batch = a.desc->batch, dim = a.desc->head_dim;
+  return map_strides(a.qs, a.m_tokens, heads, batch, dim, st) && map_strides(a.kvs, a.n_cur, heads, batch, dim, st) &&
+         map_strides(a.vs, a.n_cur, heads, batch, dim, st);
 }
 
 static void schedule_shape(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur,
@@ -1441,12 +1487,12 @@ static void schedule_shape(const kvq_cache_desc* d, int64_t cache_len, int64_t m
   *tiles = (n_cur + kBlockN - 1) / kBlockN + (cache_len + kBlockN - 1) / kBlockN;
 }
 
-// Bytes of the rotated-query area of the workspace: q~ rows (256 bytes each), then bias rows (16 bytes each),
+// Bytes of the rotated-query area of the workspace: q~ rows (2 * head_dim bytes each), then bias rows (16 bytes each),
 // rounded up to a multiple of 256.  Nothing when there are no cached keys.
 static size_t rot_area_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens) {
   if (cache_len <= 0) return 0;
   const size_t rows = (size_t)d->batch * d->heads * (size_t)m_tokens;
-  return (rows * (2 * kD + 16) + 255) / 256 * 256;
+  return (rows * (2 * (size_t)d->head_dim + 16) + 255) / 256 * 256;
 }
 
 size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair) {
@@ -1478,10 +1524,10 @@ static int launch_planned(const AttnArgs& a, const Plan& pl, int64_t qb, int64_t
   int r = get_encode_fn(&enc);
   if (r != KVQ_OK) return r;
   CUtensorMap mq, mqr, mk, mv;
-  if ((r = make_map(enc, &mq, a.q, a.qs, a.m_tokens, d->heads, d->batch)) != KVQ_OK) return r;
+  if ((r = make_map(enc, &mq, a.q, a.qs, a.m_tokens, d->heads, d->batch, d->head_dim)) != KVQ_OK) return r;
   // a CTA of a pair loads its 32 keys of each half tile: boxes of 32 rows
-  if ((r = make_map(enc, &mk, a.k_cur, a.kvs, a.n_cur, d->heads, d->batch, pair ? 32 : kBlockN)) != KVQ_OK) return r;
-  if ((r = make_map(enc, &mv, a.v_cur, a.vs, a.n_cur, d->heads, d->batch)) != KVQ_OK) return r;
+  if ((r = make_map(enc, &mk, a.k_cur, a.kvs, a.n_cur, d->heads, d->batch, d->head_dim, pair ? 32 : kBlockN)) != KVQ_OK) return r;
+  if ((r = make_map(enc, &mv, a.v_cur, a.vs, a.n_cur, d->heads, d->batch, d->head_dim)) != KVQ_OK) return r;
   if ((int64_t)d->batch * d->heads > 65535) return KVQ_ERR_UNSUPPORTED;   // second grid dimension of the pre-pass
   RotParams rp{};
   mqr = mq;                                                  // never read when there are no cached keys
@@ -1489,12 +1535,13 @@ static int launch_planned(const AttnArgs& a, const Plan& pl, int64_t qb, int64_t
     const int64_t rows = (int64_t)d->batch * d->heads * a.m_tokens;
     rp.q = static_cast<const uint16_t*>(a.q); rp.q_sb = a.qs.b; rp.q_sh = a.qs.h; rp.q_st = a.qs.t;
     rp.qr = reinterpret_cast<uint16_t*>(rot_area);
-    rp.ax = reinterpret_cast<uint16_t*>(rot_area + (size_t)rows * 2 * kD);
+    rp.ax = reinterpret_cast<uint16_t*>(rot_area + (size_t)rows * 2 * d->head_dim);
     rp.signs = d->signs;
     rp.heads = d->heads; rp.m_tokens = (int)a.m_tokens; rp.rotate = (d->flags & KVQ_ROTATE_K) ? 1 : 0;
     rp.ax_coef = -a.softmax_scale / 24.0f;
-    const kvq_strides dense{(int64_t)d->heads * a.m_tokens * kD, a.m_tokens * (int64_t)kD, (int64_t)kD};
-    if ((r = make_map(enc, &mqr, rp.qr, dense, a.m_tokens, d->heads, d->batch)) != KVQ_OK) return r;
+    const int64_t dim = d->head_dim;
+    const kvq_strides dense{d->heads * a.m_tokens * dim, a.m_tokens * dim, dim};
+    if ((r = make_map(enc, &mqr, rp.qr, dense, a.m_tokens, d->heads, d->batch, d->head_dim)) != KVQ_OK) return r;
   }
   TParams p;
   p.out = static_cast<uint16_t*>(a.out); p.o_sb = a.os.b; p.o_sh = a.os.h; p.o_st = a.os.t;
@@ -1517,6 +1564,12 @@ static int launch_planned(const AttnArgs& a, const Plan& pl, int64_t qb, int64_t
   dim3 grid((unsigned)pl.ctas);
 #define KVQ_LAUNCH(B_, G_) (pair ? launch<B_, G_, true>(mq, mqr, mk, mv, p, rp, grid, a.stream) \
                                  : launch<B_, G_, false>(mq, mqr, mk, mv, p, rp, grid, a.stream))
+  if (d->head_dim == 64) {                                   // one CTA per unit only
+#define KVQ_LAUNCH64(B_, G_) launch<B_, G_, false, 64>(mq, mqr, mk, mv, p, rp, grid, a.stream)
+    if (d->bits == 2) return d->group == 32 ? KVQ_LAUNCH64(2, 32) : KVQ_LAUNCH64(2, 64);
+    return d->group == 32 ? KVQ_LAUNCH64(4, 32) : KVQ_LAUNCH64(4, 64);
+#undef KVQ_LAUNCH64
+  }
   if (d->bits == 2) {
     if (d->group == 32) return KVQ_LAUNCH(2, 32);
     if (d->group == 64) return KVQ_LAUNCH(2, 64);

@@ -97,7 +97,8 @@ static bool use_tcgen05(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur
   if (kern == KVQ_KERNEL_MMA_SYNC) return false;
   // the exact correction (a table look-up per score and group) exists in the warp-level kernel only
   const bool ok = attn_tcgen05_supports(d, m_tokens, n_cur) && !(flags & KVQ_CORRECTION_EXACT) && !(d->flags & KVQ_K_PER_CHANNEL);
-  if ((kern == KVQ_KERNEL_TCGEN05 || kern == KVQ_KERNEL_TCGEN05_PAIR) && !ok) *err = KVQ_ERR_UNSUPPORTED;
+  // heads of 64 channels: chosen by KVQ_KERNEL_AUTO only
+  if ((kern == KVQ_KERNEL_TCGEN05 || kern == KVQ_KERNEL_TCGEN05_PAIR) && !(ok && d->head_dim == 128)) *err = KVQ_ERR_UNSUPPORTED;
   return ok;
 }
 // Which tcgen05 kernel: the one asked for, else (KVQ_KERNEL_AUTO) the pair kernel unless its units of 512 query
@@ -107,6 +108,7 @@ static bool use_tcgen05(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur
 static bool is_pair(const kvq_cache_desc* d, uint32_t flags, int64_t m_tokens) {
   const uint32_t kern = flags & KVQ_KERNEL_MASK;
   if (kern != KVQ_KERNEL_AUTO) return kern == KVQ_KERNEL_TCGEN05_PAIR;
+  if (d->head_dim != 128) return false;                // a pair splits the value channels into blocks of 64
   const int64_t rows_pair = (m_tokens + 511) / 512 * 512, rows_single = (m_tokens + 255) / 256 * 256;
   return rows_pair * (d->bits == 4 ? 86 : 88) <= rows_single * 100;
 }
@@ -246,6 +248,12 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
     tc = false;
   }
   const size_t rotv = rotv_bytes(desc, cache_len, m_tokens, n_cur);
+  // The warp-level kernel, the only one for heads of 64 channels before the tcgen05 kernel took them, needs no workspace
+  // of its own: a call that brings none, or too little, keeps it.
+  if (tc && desc->head_dim == 64) {
+    const size_t need = rotv + attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, false);
+    if (need > 0 && (!workspace || workspace_bytes < need || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)) tc = false;
+  }
   {
     const size_t need = rotv + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : 0);
     if (need > 0) {
@@ -277,7 +285,7 @@ int kvq_attn_corrected_static_scratch(const kvq_cache_desc* desc, int64_t cache_
   int r = check_attn_call(desc, cache_begin, cache_len, q, q_strides, k_cur, v_cur, kv_strides, m_tokens, n_cur,
                           out_bf16, o_strides, softmax_scale, flags);
   if (r != KVQ_OK) return r;
-  if (!attn_tcgen05_supports(desc, m_tokens, n_cur) || (flags & KVQ_CORRECTION_EXACT) ||
+  if (desc->head_dim != 128 || !attn_tcgen05_supports(desc, m_tokens, n_cur) || (flags & KVQ_CORRECTION_EXACT) ||
       (desc->flags & (KVQ_ROTATE_V | KVQ_K_PER_CHANNEL)))
     return KVQ_ERR_UNSUPPORTED;
   if (m_tokens == 0) return KVQ_OK;
