@@ -1,0 +1,602 @@
+// Corrected chunk attention for a few query rows over a long cache (small steps of a decoding reply, short chunks).
+//
+// The tcgen05 kernel works on 256 query rows at a time; with 16 of them it spends its time on padding (scores,
+// exponentials, and a dequantization into shared memory that 16 rows cannot pay for).  Here a CTA takes 16 rows of one
+// (batch, head) and a range of the keys, each of its four warps takes every fourth step of 32 keys, and the packed codes
+// go from global memory through registers straight into the B operands of mma.sync: the contraction over channels
+// may run in any order, so a lane takes the D/4 consecutive channels whose codes it can load at once, and the output
+// channels may be numbered in any order, so a lane takes D/8 consecutive ones of the values of its four keys.  A lane's
+// channels then lie in one group: one step and one zero-point per key and lane.  Nothing is staged in shared memory but the
+// query rows.
+//
+// Algorithm 1 as in the other kernels: rotated query and dequantized keys in FP16, weights and values in BF16, FP32
+// sums, exact running maximum; the bias -(sigma/24) sum_j nu_j step_j^2 is one more MMA step (nu as a BF16 high and low
+// part, step^2 is exact in BF16).  Ranges of one (batch, head) leave FP32 partial rows that a second kernel merges in a
+// fixed order.
+//
+// What bounds it: instruction issue and latency (37 warp instructions per key and 16 rows at 4 bits, half of them the
+// expansion of the codes; two CTAs of four warps an SM, the ALU pipe half busy), then HBM.  16 rows over 16 384 tokens
+// of 32 heads at 4 bits, group 128: 42 us with the merge, against 87 us in the tcgen05 kernel; three CTAs with spilled
+// registers 47 us, four 76 us; the four score tiles of a step one after the other instead of in turn 45 us.
+#include <cuda_fp16.h>
+
+#include "kvq_common.cuh"
+
+namespace kvq {
+namespace {
+
+constexpr int kRows = 16;
+constexpr int kWarps = 4;
+constexpr int kStep = 32;            // keys a warp takes at a time
+constexpr int kCtasPerSm = 2;      // up to 255 registers a thread, nothing spilled
+constexpr float kLog2e = 1.4426950408889634f;
+
+struct SParams {
+  const uint16_t* q; const uint16_t* kc; const uint16_t* vc; uint16_t* out;
+  int64_t q_sb, q_sh, q_st, kv_sb, kv_sh, kv_st, v_sb, v_sh, v_st, o_sb, o_sh, o_st;
+  const uint8_t* codes[2]; const uint8_t* scale[2]; const uint16_t* zero[2];    // keys, values
+  const int8_t* signs;
+  int64_t capacity, cache_begin;
+  int heads, rotate, correction;
+  int m_tokens, n_cached, n_cur;
+  int q_blocks, splits;
+  float scale_log2, ax_coef;           // sigma * log2(e), -sigma / 24
+  float* lse; float* cached_mass;
+  float* partial;                      // splits > 1: one slot per CTA, see slot_floats
+};
+
+// Partial rows of a CTA: O[16][D] (not normalised), then m[16] (log2 units), l_cur[16], l_cached[16].
+__host__ __device__ constexpr int slot_floats(int D) { return kRows * D + 64; }
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+__device__ __forceinline__ uint32_t pack_f16_sat(float lo, float hi) {
+  lo = fminf(fmaxf(lo, -65504.f), 65504.f);
+  hi = fminf(fmaxf(hi, -65504.f), 65504.f);
+  return (uint32_t)__half_as_ushort(__float2half_rn(lo)) | ((uint32_t)__half_as_ushort(__float2half_rn(hi)) << 16);
+}
+__device__ __forceinline__ uint32_t fma_f16x2(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+__device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+__device__ __forceinline__ uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// x shifted so that bit `from` lands on bit `to` (both known at compile time once unrolled)
+__device__ __forceinline__ uint32_t move_bits(uint32_t x, int from, int to) { return from <= to ? x << (to - from) : x >> (from - to); }
+
+// What a lane expands in one step: of the keys 8 t + lane / 4 (t = 0 .. 3) the codes of its D/4 channels, of the values
+// 2 (lane % 4) + {0, 1} + 8 t those of its D/8 channels; and of each the step and zero-point of the lane's group.
+template <int D, int BITS>
+struct Keys {
+  static constexpr int W = D / 4 * BITS / 32;
+  uint32_t w[4][W], meta[4];                                       // zero-point (BF16 bits) << 16 | step byte
+};
+template <int D, int BITS>
+struct Values {
+  static constexpr int B = D / 8 * BITS / 8;                       // bytes: 2, 4 or 8
+  static constexpr int W = B < 4 ? 1 : B / 4;
+  uint32_t w[8][W], meta[8];
+};
+// First tokens of the two halves of a step (16 slots each never straddle the end of the slab, 32 may).
+struct Step { int64_t tok[2]; int n_valid; };
+
+template <int D, int BITS, int GROUP>
+__device__ __forceinline__ void load_keys(Keys<D, BITS>& r, const SParams& p, const Step& st, int g, int c) {
+  constexpr int CB = D * BITS / 8, G = D / GROUP, W = Keys<D, BITS>::W;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int64_t tok = st.tok[t >> 1] + g + 8 * (t & 1);
+    const uint8_t* src = p.codes[0] + tok * CB + c * (W * 4);
+    if constexpr (W == 1) r.w[t][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+    else if constexpr (W == 2) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; }
+    else { const uint4 v = __ldg(reinterpret_cast<const uint4*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; r.w[t][2] = v.z; r.w[t][3] = v.w; }
+    const int64_t at = tok * G + c * (D / 4) / GROUP;
+    r.meta[t] = __ldg(p.scale[0] + at) | ((uint32_t)__ldg(p.zero[0] + at) << 16);
+  }
+  if (st.n_valid < kStep) {                                        // tokens past the window: finite scores, masked later
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (8 * t + g >= st.n_valid) r.meta[t] = 0u;
+  }
+}
+template <int D, int BITS, int GROUP>
+__device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p, const Step& st, int g, int c) {
+  constexpr int CB = D * BITS / 8, G = D / GROUP, B = Values<D, BITS>::B;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int64_t tok = st.tok[i >> 2] + 2 * c + (i & 1) + 8 * ((i >> 1) & 1);
+    const uint8_t* src = p.codes[1] + tok * CB + g * B;
+    if constexpr (B == 2) r.w[i][0] = __ldg(reinterpret_cast<const uint16_t*>(src));
+    else if constexpr (B == 4) r.w[i][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+    else { const uint2 v = __ldg(reinterpret_cast<const uint2*>(src)); r.w[i][0] = v.x; r.w[i][1] = v.y; }
+    const int64_t at = tok * G + g * (D / 8) / GROUP;
+    r.meta[i] = __ldg(p.scale[1] + at) | ((uint32_t)__ldg(p.zero[1] + at) << 16);
+  }
+  if (st.n_valid < kStep) {                                        // step and zero-point 0: exact zeros whatever the codes are
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (2 * c + (i & 1) + 8 * (i >> 1) >= st.n_valid) r.meta[i] = 0u;
+  }
+}
+
+template <int D, int BITS, int GROUP>
+__global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(const SParams p) {
+  constexpr int LD = D + 8;                                        // padded rows of the query tiles
+  constexpr int KS = D / 16;                                       // MMA steps over the channels
+  constexpr int NT = D / 8;                                        // output tiles of 8 channels
+  constexpr int G = D / GROUP;
+  constexpr int KW = Keys<D, BITS>::W;
+  constexpr int kOStride = D + 4;
+  // the query tiles are done with when the warps' outputs are exchanged
+  __shared__ __align__(16) union {
+    struct { uint16_t q[kRows * LD], qr[kRows * LD]; float nu[kRows * 4]; } in;
+    struct { float o[kWarps][kRows * kOStride]; } x;
+  } sm;
+  __shared__ float s_stat[kWarps][3][kRows];                       // m, l_cur, l_cached
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  const int unit = blockIdx.x / p.splits, split = blockIdx.x - unit * p.splits;
+  const int bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
+  const int row0 = (unit - bh * p.q_blocks) * kRows;
+
+  // ---- query rows: as they are, and rotated (FP16, in the order the expanded codes come in), per-group norms ----
+  {
+    constexpr int LPR = D / 8;                                     // lanes per row, 8 channels each
+    const int ln = lane % LPR;
+    for (int r = warp * (32 / LPR) + lane / LPR; r < kRows; r += kWarps * 32 / LPR) {
+      const int row = row0 + r;
+      uint4 raw = make_uint4(0, 0, 0, 0);
+      if (row < p.m_tokens) raw = __ldg(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
+      *reinterpret_cast<uint4*>(sm.in.q + r * LD + ln * 8) = raw;
+      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+      float x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = bf16_bits_to_f32(e & 1 ? w[e >> 1] >> 16 : w[e >> 1] & 0xFFFFu);
+      if (p.rotate) {
+        if (p.signs) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] *= (float)p.signs[ln * 8 + e];
+        }
+#pragma unroll
+        for (int hh = 1; hh < 8; hh *= 2)
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if ((i & hh) == 0) { const float u = x[i], v = x[i + hh]; x[i] = u + v; x[i + hh] = u - v; }
+#pragma unroll
+        for (int lm = 1; lm < LPR; lm *= 2)
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const float o = __shfl_xor_sync(0xFFFFFFFFu, x[e], lm);
+            x[e] = (ln & lm) ? (o - x[e]) : (x[e] + o);
+          }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] *= D == 64 ? 0.125f : 0.08838834764831845f;
+      }
+      float nu = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) nu += x[e] * x[e];
+#pragma unroll
+      for (int off = 1; off < GROUP / 8; off *= 2) nu += __shfl_xor_sync(0xFFFFFFFFu, nu, off);
+      if (ln % (GROUP / 8) == 0) sm.in.nu[r * 4 + ln / (GROUP / 8)] = nu;
+      // a word of 32 / BITS codes expands to the pairs (i, i + 16 / BITS): that order, pair by pair
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        constexpr int N = 32 / BITS;
+        const int ch = ln * 8 + e, i = ch % N;
+        const float v = fminf(fmaxf(x[e], -65504.f), 65504.f);
+        sm.in.qr[r * LD + ch / N * N + 2 * (i % (N / 2)) + i / (N / 2)] = __half_as_ushort(__float2half_rn(v));
+      }
+    }
+  }
+  __syncthreads();
+  uint32_t qf[KS][4];
+  constexpr int KPW = 8 / BITS;                                    // MMA steps per word of codes
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) {
+    const int col = (c * KW + ks / KPW) * (32 / BITS) + 4 * (ks % KPW);
+    const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.qr + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.qr + (g + 8) * LD + col);
+    qf[ks][0] = lo.x; qf[ks][1] = hi.x; qf[ks][2] = lo.y; qf[ks][3] = hi.y;
+  }
+  // bias operand: columns 2 c, 2 c + 1 are the high and low part of lane c's group; one lane per group counts it
+  uint32_t ax[2] = {0u, 0u};
+  if (p.correction && c % (4 / G) == 0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float a = p.ax_coef * sm.in.nu[(g + 8 * i) * 4 + c / (4 / G)];
+      const uint32_t hi = f32_to_bf16_bits(a);
+      ax[i] = hi | (f32_to_bf16_bits(a - bf16_bits_to_f32(hi)) << 16);
+    }
+  }
+
+  float acc[NT][4];
+#pragma unroll
+  for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+  float m_run[2] = {-INFINITY, -INFINITY}, l_cur[2] = {0.f, 0.f}, l_cac[2] = {0.f, 0.f};
+  uint32_t pf[8];
+  // online softmax over the 32 scores of a step (this lane: rows g, g + 8, keys 8 t + 2 c + {0, 1}); leaves the weights in pf
+  auto softmax_step = [&](float (&s)[4][4], int n_valid, float (&l)[2]) {
+    if (n_valid < kStep) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (8 * t + 2 * c + (e & 1) >= n_valid) s[t][e] = -INFINITY;
+    }
+    float m_new[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      float mx = -INFINITY;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) mx = fmaxf(mx, fmaxf(s[t][2 * r], s[t][2 * r + 1]));
+      mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
+      m_new[r] = fmaxf(m_run[r], mx * p.scale_log2);
+    }
+    if (__any_sync(0xFFFFFFFFu, m_new[0] > m_run[0] || m_new[1] > m_run[1])) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float f = ex2(m_run[r] - m_new[r]);
+        l_cur[r] *= f; l_cac[r] *= f;
+        m_run[r] = m_new[r];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+          const float2 o = __fmul2_rn(make_float2(acc[j][2 * r], acc[j][2 * r + 1]), make_float2(f, f));
+          acc[j][2 * r] = o.x; acc[j][2 * r + 1] = o.y;
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float w0 = ex2(fmaf(s[t][2 * r], p.scale_log2, -m_run[r])), w1 = ex2(fmaf(s[t][2 * r + 1], p.scale_log2, -m_run[r]));
+        l[r] += w0 + w1;
+        pf[2 * t + r] = pack_bf16(w0, w1);
+      }
+  };
+
+  // ---- this CTA's share of the steps: cached keys first, then the current chunk's; warp w takes every fourth ----
+  const int n_cs = (p.n_cached + kStep - 1) / kStep, n_steps = n_cs + (p.n_cur + kStep - 1) / kStep;
+  const int first = (int)((int64_t)n_steps * split / p.splits), last = (int)((int64_t)n_steps * (split + 1) / p.splits);
+  int st = first + warp;
+  const int last_c = min(last, n_cs);
+  auto step_of = [&](int i) {
+    Step x;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      int64_t slot = p.cache_begin + (int64_t)i * kStep + 16 * u;
+      if (slot >= p.capacity) slot -= p.capacity;
+      x.tok[u] = (int64_t)bh * p.capacity + slot;
+    }
+    x.n_valid = p.n_cached - i * kStep;
+    return x;
+  };
+  Keys<D, BITS> keys;
+  if (st < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st), g, c);
+#pragma unroll 1
+  for (; st < last_c; st += kWarps) {
+    Values<D, BITS> vals;                                          // on their way while the scores are computed
+    load_values<D, BITS, GROUP>(vals, p, step_of(st), g, c);
+    float s[4][4];
+    // (OFF + code) * step - (OFF + zero) * step with OFF from the exponent bits OR-ed over the code, one FMA per pair
+    constexpr float kOff = BITS == 2 ? 4.f : 16.f;
+    uint32_t step2[4], off2[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
+      step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(-(kOff + zs) * ds, -(kOff + zs) * ds);
+      s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
+      if (p.correction) mma_bf16(s[t], ax[0], ax[1], 0u, 0u, pack_bf16(ds * ds, ds * ds), 0u);
+    }
+    // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
+#pragma unroll
+    for (int wi = 0; wi < KW; ++wi)
+#pragma unroll
+      for (int j = 0; j < KPW; ++j)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          uint32_t bf[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t x = move_bits(keys.w[t][wi], (2 * j + i) * BITS, BITS == 2 ? 8 : 6);
+            bf[i] = fma_f16x2(BITS == 2 ? (x & 0x03000300u) | 0x44004400u : (x & 0x03C003C0u) | 0x4C004C00u, step2[t], off2[t]);
+          }
+          const uint32_t (&a)[4] = qf[wi * KPW + j];
+          mma_f16(s[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
+        }
+    if (st + kWarps < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st + kWarps), g, c);
+    softmax_step(s, p.n_cached - st * kStep, l_cac);
+    // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+      uint32_t step2[2], off2[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float ds[2], zs[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const uint32_t meta = vals.meta[4 * kk + 2 * u + i];
+          ds[i] = e4m3_byte_to_f32(meta & 0xFFu);
+          zs[i] = __uint_as_float(meta & 0xFFFF0000u);
+        }
+        step2[u] = pack_bf16(ds[0], ds[1]);
+        off2[u] = BITS == 2 ? pack_bf16(-(4.f + zs[0]) * ds[0], -(4.f + zs[1]) * ds[1]) : pack_bf16(16.f + zs[0], 16.f + zs[1]);
+      }
+      constexpr int kPer = 16 / BITS;                              // codes in half a word
+#pragma unroll
+      for (int hw = 0; hw < NT / kPer; ++hw) {
+        uint32_t z[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          z[u] = __byte_perm(vals.w[4 * kk + 2 * u][hw / 2], vals.w[4 * kk + 2 * u + 1][hw / 2], hw & 1 ? 0x7632 : 0x5410);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          uint32_t bf[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const uint32_t x = move_bits(z[u], i * BITS, BITS == 2 ? 5 : 3);
+            if constexpr (BITS == 2) bf[u] = fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u]);
+            else bf[u] = mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
+          }
+          mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], bf[0], bf[1]);
+        }
+      }
+    }
+  }
+  // ---- current chunk: unrotated query, BF16 keys and values, no bias ----
+#pragma unroll 1
+  for (; st < last; st += kWarps) {
+    const int k0 = (st - n_cs) * kStep, nv = p.n_cur - k0;
+    float s[4][4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
+      const uint4* src = reinterpret_cast<const uint4*>(p.kc + (int64_t)b * p.kv_sb + (int64_t)h * p.kv_sh + (int64_t)min(k0 + 8 * t + g, p.n_cur - 1) * p.kv_st + c * (D / 4));
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) {
+        const uint4 v = __ldg(src + i);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int col = c * (D / 4) + 8 * i + 4 * j;
+          const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.q + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.q + (g + 8) * LD + col);
+          mma_bf16(s[t], lo.x, hi.x, lo.y, hi.y, j ? v.z : v.x, j ? v.w : v.y);
+        }
+      }
+    }
+    softmax_step(s, nv, l_cur);
+    const uint16_t* vbase = p.vc + (int64_t)b * p.v_sb + (int64_t)h * p.v_sh + g * (D / 8);
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+      for (int i = 0; i < D / 64; ++i) {                           // 8 of the lane's channels at a time
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int key = 16 * kk + 2 * c + (u & 1) + 8 * (u >> 1);
+          v[u] = key < nv ? __ldg(reinterpret_cast<const uint4*>(vbase + (int64_t)(k0 + key) * p.v_st) + i) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t sel = e & 1 ? 0x7632 : 0x5410;
+          auto word = [&](const uint4& x) { return (e >> 1) == 0 ? x.x : (e >> 1) == 1 ? x.y : (e >> 1) == 2 ? x.z : x.w; };
+          mma_bf16(acc[8 * i + e], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3],
+                   __byte_perm(word(v[0]), word(v[1]), sel), __byte_perm(word(v[2]), word(v[3]), sel));
+        }
+      }
+  }
+
+  // ---- the four warps' partial rows ----
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    l_cur[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cur[r], 1);
+    l_cur[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cur[r], 2);
+    l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 1);
+    l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 2);
+    if (c == 0) { s_stat[warp][0][g + 8 * r] = m_run[r]; s_stat[warp][1][g + 8 * r] = l_cur[r]; s_stat[warp][2][g + 8 * r] = l_cac[r]; }
+  }
+  __syncthreads();                                                 // also: the query tiles are free
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      sm.x.o[warp][(g + 8 * (e >> 1)) * kOStride + (2 * c + (e & 1)) * (D / 8) + j] = acc[j][e];
+  __syncthreads();
+  constexpr int kPerRow = kWarps * 32 / kRows;                     // threads per row
+  const int r = threadIdx.x / kPerRow, t8 = threadIdx.x % kPerRow, row = row0 + r;
+  if (row >= p.m_tokens) return;
+  float m = -INFINITY, f[kWarps], lc = 0.f, la = 0.f;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) m = fmaxf(m, s_stat[w][0][r]);
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {                               // a warp without keys has m = -inf: weight 0
+    f[w] = ex2(s_stat[w][0][r] - m);
+    lc += f[w] * s_stat[w][1][r]; la += f[w] * s_stat[w][2][r];
+  }
+  const float l = lc + la, inv = 1.0f / l;
+  float* slot = p.partial + (size_t)blockIdx.x * slot_floats(D);
+  uint16_t* dst = p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st;
+#pragma unroll
+  for (int i = 0; i < D / 4; i += kPerRow) {
+    const int ch = (i + t8) * 4;
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const float4 v = *reinterpret_cast<const float4*>(&sm.x.o[w][r * kOStride + ch]);
+      o[0] += f[w] * v.x; o[1] += f[w] * v.y; o[2] += f[w] * v.z; o[3] += f[w] * v.w;
+    }
+    if (p.splits > 1) *reinterpret_cast<float4*>(slot + r * D + ch) = make_float4(o[0], o[1], o[2], o[3]);
+    else *reinterpret_cast<uint2*>(dst + ch) = make_uint2(pack_bf16(o[0] * inv, o[1] * inv), pack_bf16(o[2] * inv, o[3] * inv));
+  }
+  if (t8 == 0) {
+    if (p.splits > 1) {
+      float* stat = slot + kRows * D;
+      stat[r] = m; stat[16 + r] = lc; stat[32 + r] = la;
+    } else {
+      const int64_t idx = (int64_t)bh * p.m_tokens + row;
+      if (p.lse) p.lse[idx] = (m + log2f(l)) * 0.6931471805599453f;
+      if (p.cached_mass) p.cached_mass[idx] = la * inv;
+    }
+  }
+}
+
+// Combines the partial rows of a unit's splits in a fixed order: a block per row, warp w taking every fourth split, its
+// lanes the channels, so that the loads of a row are all in flight together.
+template <int D>
+__global__ void __launch_bounds__(kWarps * 32) attn_short_merge_kernel(const SParams p) {
+  constexpr int E = D / 32;                                        // channels of a lane
+  const int unit = blockIdx.x / kRows, r = blockIdx.x % kRows, bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
+  const int row = (unit - bh * p.q_blocks) * kRows + r;
+  if (row >= p.m_tokens) return;                                   // the whole block
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ float s_o[kWarps][D], s_l[kWarps][2];
+  const float* slots = p.partial + (size_t)unit * p.splits * slot_floats(D);
+  float m = -INFINITY;
+  for (int s = lane; s < p.splits; s += 32) m = fmaxf(m, slots[(size_t)s * slot_floats(D) + kRows * D + r]);
+#pragma unroll
+  for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
+  float o[E] = {}, lc = 0.f, la = 0.f;
+#pragma unroll 4
+  for (int s = warp; s < p.splits; s += kWarps) {
+    const float* sl = slots + (size_t)s * slot_floats(D);
+    const float f = ex2(sl[kRows * D + r] - m);
+    lc += f * sl[kRows * D + 16 + r]; la += f * sl[kRows * D + 32 + r];
+    float v[E];
+    if constexpr (E == 4) { const float4 u = *reinterpret_cast<const float4*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w; }
+    else { const float2 u = *reinterpret_cast<const float2*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; }
+#pragma unroll
+    for (int e = 0; e < E; ++e) o[e] += f * v[e];
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) s_o[warp][lane * E + e] = o[e];
+  if (lane == 0) { s_l[warp][0] = lc; s_l[warp][1] = la; }
+  __syncthreads();
+  lc = la = 0.f;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) { lc += s_l[w][0]; la += s_l[w][1]; }
+  const float l = lc + la, inv = 1.0f / l;
+  if (threadIdx.x < D) {
+    float x = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) x += s_o[w][threadIdx.x];
+    p.out[(int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st + threadIdx.x] = (uint16_t)f32_to_bf16_bits(x * inv);
+  }
+  if (threadIdx.x == 0) {
+    const int64_t idx = (int64_t)bh * p.m_tokens + row;
+    if (p.lse) p.lse[idx] = (m + log2f(l)) * 0.6931471805599453f;
+    if (p.cached_mass) p.cached_mass[idx] = la * inv;
+  }
+}
+
+// Units (batch*head, 16 rows) and into how many ranges the keys of each are cut: as many as let every CTA be resident at
+// once, but no range below 2 steps a warp, nor more than the merge can have in flight.
+struct Plan { int64_t q_blocks, units; int splits; };
+Plan plan(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {
+  int sms = 0;
+  if (device_sm_count(&sms) != KVQ_OK) sms = 148;                  // sizes only: the launch itself fails loudly
+  Plan pl;
+  pl.q_blocks = (m_tokens + kRows - 1) / kRows;
+  pl.units = (int64_t)d->batch * d->heads * pl.q_blocks;
+  const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
+  int64_t s = (int64_t)sms * kCtasPerSm / pl.units;
+  if (s > steps / (2 * kWarps)) s = steps / (2 * kWarps);
+  if (s > 128) s = 128;
+  pl.splits = (int)(s < 1 ? 1 : s);
+  return pl;
+}
+
+template <int D, int BITS, int GROUP>
+int launch(const SParams& p, const Plan& pl, cudaStream_t st) {
+  attn_short_kernel<D, BITS, GROUP><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
+  KVQ_CUDA_TRY(cudaGetLastError());
+  if (pl.splits > 1) {
+    attn_short_merge_kernel<D><<<(unsigned)(pl.units * kRows), kWarps * 32, 0, st>>>(p);
+    KVQ_CUDA_TRY(cudaGetLastError());
+  }
+  return KVQ_OK;
+}
+
+}  // namespace
+
+bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, uint32_t flags) {
+  if ((flags & KVQ_KERNEL_MASK) != KVQ_KERNEL_AUTO || (flags & KVQ_CORRECTION_EXACT) || (d->flags & KVQ_K_PER_CHANNEL) || m_tokens < 1)
+    return false;
+  // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
+  // prologue and a larger merge.  Measured (2 and 4 bits, 4 to 64 heads): one block of rows is 1.4 to 2 times as fast
+  // here; two are up to about 16 000 (head, 128-key tile) pairs (102 against 115 us at 6 464, 262 against 297 at 15 456, 485
+  // against 467 at 29 056); three and four only where those fixed costs weigh (33 against 47 us for three blocks at 892 pairs,
+  // 35 against 33 for four at 704, 117 against 78 at 3 520).
+  const int64_t blocks = (m_tokens + kRows - 1) / kRows;
+  const int64_t pairs = (int64_t)d->batch * d->heads * ((cache_len + 127) / 128 + (n_cur + 127) / 128);
+  return blocks == 1 || (blocks == 2 && pairs <= 16384) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 600);
+}
+
+size_t attn_short_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {
+  const Plan pl = plan(d, cache_len, m_tokens, n_cur);
+  return pl.splits > 1 ? ((size_t)pl.units * pl.splits * slot_floats(d->head_dim) * sizeof(float) + 255) / 256 * 256 : 0;
+}
+
+int attn_short_kernel_launches(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {
+  return plan(d, cache_len, m_tokens, n_cur).splits > 1 ? 2 : 1;
+}
+
+int launch_attn_short(const AttnArgs& a) {
+  const kvq_cache_desc* d = a.desc;
+  const Plan pl = plan(d, a.cache_len, a.m_tokens, a.n_cur);
+  SParams p;
+  p.q = static_cast<const uint16_t*>(a.q); p.kc = static_cast<const uint16_t*>(a.k_cur);
+  p.vc = static_cast<const uint16_t*>(a.v_cur); p.out = static_cast<uint16_t*>(a.out);
+  p.q_sb = a.qs.b; p.q_sh = a.qs.h; p.q_st = a.qs.t;
+  p.kv_sb = a.kvs.b; p.kv_sh = a.kvs.h; p.kv_st = a.kvs.t;
+  p.v_sb = a.vs.b; p.v_sh = a.vs.h; p.v_st = a.vs.t;
+  p.o_sb = a.os.b; p.o_sh = a.os.h; p.o_st = a.os.t;
+  p.codes[0] = static_cast<const uint8_t*>(d->k_codes); p.codes[1] = static_cast<const uint8_t*>(d->v_codes);
+  p.scale[0] = static_cast<const uint8_t*>(d->k_scale); p.scale[1] = static_cast<const uint8_t*>(d->v_scale);
+  p.zero[0] = static_cast<const uint16_t*>(d->k_zero); p.zero[1] = static_cast<const uint16_t*>(d->v_zero);
+  p.signs = d->signs;
+  p.capacity = d->capacity; p.cache_begin = a.cache_begin % d->capacity;
+  p.heads = d->heads; p.rotate = (d->flags & KVQ_ROTATE_K) ? 1 : 0;
+  p.correction = (a.flags & KVQ_CORRECTION_ON) ? 1 : 0;
+  p.m_tokens = (int)a.m_tokens; p.n_cached = (int)a.cache_len; p.n_cur = (int)a.n_cur;
+  p.q_blocks = (int)pl.q_blocks; p.splits = pl.splits;
+  p.scale_log2 = a.softmax_scale * kLog2e;
+  p.ax_coef = -a.softmax_scale / 24.0f;
+  p.lse = a.lse; p.cached_mass = a.cached_mass;
+  p.partial = static_cast<float*>(a.workspace);
+#define KVQ_SHORT(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) return launch<D_, B_, G_>(p, pl, a.stream);
+  KVQ_SHORT(128, 2, 32) KVQ_SHORT(128, 2, 64) KVQ_SHORT(128, 2, 128) KVQ_SHORT(128, 4, 32) KVQ_SHORT(128, 4, 64) KVQ_SHORT(128, 4, 128)
+  KVQ_SHORT(64, 2, 32) KVQ_SHORT(64, 2, 64) KVQ_SHORT(64, 4, 32) KVQ_SHORT(64, 4, 64)
+#undef KVQ_SHORT
+  return KVQ_ERR_UNSUPPORTED;
+}
+
+}  // namespace kvq

@@ -209,6 +209,10 @@ int kvq_attn_workspace_bytes(const kvq_cache_desc* desc, int64_t cache_len, int6
   int err;
   const bool tc = use_tcgen05(desc, m_tokens, n_cur, flags, &err);
   if (err != KVQ_OK) return err;
+  if (attn_short_supports(desc, cache_len, m_tokens, n_cur, flags)) {
+    *out_bytes = rotv_bytes(desc, cache_len, m_tokens, n_cur) + attn_short_workspace_bytes(desc, cache_len, m_tokens, n_cur);
+    return KVQ_OK;
+  }
   *out_bytes = rotv_bytes(desc, cache_len, m_tokens, n_cur) + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : 0);
   return KVQ_OK;
 }
@@ -221,7 +225,8 @@ int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len, int6
   int err;
   const bool tc = use_tcgen05(desc, m_tokens, n_cur, flags, &err);
   if (err != KVQ_OK) return err;
-  *out_count = (tc ? attn_tcgen05_kernel_launches(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : (m_tokens > 0 ? 1 : 0)) +
+  const bool few = attn_short_supports(desc, cache_len, m_tokens, n_cur, flags);
+  *out_count = (few ? attn_short_kernel_launches(desc, cache_len, m_tokens, n_cur) : tc ? attn_tcgen05_kernel_launches(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : (m_tokens > 0 ? 1 : 0)) +
                (rotv_bytes(desc, cache_len, m_tokens, n_cur) ? 2 : 0);      // value pre-pass and output post-pass
   return KVQ_OK;
 }
@@ -248,13 +253,17 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
     tc = false;
   }
   const size_t rotv = rotv_bytes(desc, cache_len, m_tokens, n_cur);
+  auto holds = [&](size_t need) {          // the call's workspace has room for `need` bytes
+    return need == 0 || (workspace && workspace_bytes >= need && reinterpret_cast<uintptr_t>(workspace) % 256 == 0);
+  };
+  // A few query rows have a kernel of their own; a call whose workspace suits only the kernel that served it before that
+  // one existed keeps it.
+  const bool few = attn_short_supports(desc, cache_len, m_tokens, n_cur, flags) &&
+                   holds(rotv + attn_short_workspace_bytes(desc, cache_len, m_tokens, n_cur));
   // The warp-level kernel, the only one for heads of 64 channels before the tcgen05 kernel took them, needs no workspace
   // of its own: a call that brings none, or too little, keeps it.
-  if (tc && desc->head_dim == 64) {
-    const size_t need = rotv + attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, false);
-    if (need > 0 && (!workspace || workspace_bytes < need || reinterpret_cast<uintptr_t>(workspace) % 256 != 0)) tc = false;
-  }
-  {
+  if (tc && desc->head_dim == 64 && !holds(rotv + attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, false))) tc = false;
+  if (!few) {
     const size_t need = rotv + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : 0);
     if (need > 0) {
       if (!workspace || workspace_bytes < need) return KVQ_ERR_WORKSPACE;
@@ -262,7 +271,7 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
     }
   }
   if (m_tokens == 0) return KVQ_OK;
-  if (tc)     // the launcher takes the choice between the two tcgen05 kernels from the flags
+  if (tc && !few)     // the launcher takes the choice between the two tcgen05 kernels from the flags
     a.flags = (a.flags & ~KVQ_KERNEL_MASK) | (is_pair(desc, flags, m_tokens) ? KVQ_KERNEL_TCGEN05_PAIR : KVQ_KERNEL_TCGEN05);
   if (rotv) {
     // values are cached rotated: bring the current chunk's values into the same space, attend, rotate the output back
@@ -271,7 +280,7 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
     a.v_cur = workspace; a.vs = dense;
     a.workspace = static_cast<uint8_t*>(workspace) + rotv; a.workspace_bytes = workspace_bytes - rotv;
   }
-  r = tc ? launch_attn_tcgen05(a) : launch_attn_mma_sync(a);
+  r = few ? launch_attn_short(a) : tc ? launch_attn_tcgen05(a) : launch_attn_mma_sync(a);
   if (r == KVQ_OK && rotv) r = launch_rotate_rows(desc, out_bf16, o_strides, out_bf16, o_strides, m_tokens, true, a.stream);
   return r;
 }

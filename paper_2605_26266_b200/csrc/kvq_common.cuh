@@ -66,6 +66,11 @@ struct AttnArgs {
   cudaStream_t stream;
 };
 int launch_attn_mma_sync(const AttnArgs& a);
+// Kernel for a few query rows (attn_short.cu), chosen by KVQ_KERNEL_AUTO only.
+bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, uint32_t flags);
+size_t attn_short_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur);
+int attn_short_kernel_launches(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur);
+int launch_attn_short(const AttnArgs& a);
 // Per-row Jensen-Shannon divergence of the attention weights against those of the BF16 keys k_ref (analysis kernel).
 int launch_attn_jsd(const AttnArgs& a, const void* k_ref, kvq_strides ref_strides, float* jsd_out);
 // y = (1/sqrt d) H (signs . x) per row (inverse: x = signs . ((1/sqrt d) H y)), BF16 [batch, heads, tokens, head_dim]
