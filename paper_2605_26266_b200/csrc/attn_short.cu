@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(con
   } sm;
   __shared__ float s_stat[kWarps][3][kRows];                       // m, l_cur, l_cached
 
+  allow_next_grid();                                               // the merge kernel
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
   const int unit = blockIdx.x / p.splits, split = blockIdx.x - unit * p.splits;
   const int bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
@@ -474,6 +475,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(con
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32) attn_short_merge_kernel(const SParams p) {
   constexpr int E = D / 32;                                        // channels of a lane
+  wait_for_previous_grid();                                        // the partial rows
   const int unit = blockIdx.x / kRows, r = blockIdx.x % kRows, bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
   const int row = (unit - bh * p.q_blocks) * kRows + r;
   if (row >= p.m_tokens) return;                                   // the whole block
@@ -538,10 +540,8 @@ template <int D, int BITS, int GROUP>
 int launch(const SParams& p, const Plan& pl, cudaStream_t st) {
   attn_short_kernel<D, BITS, GROUP><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
   KVQ_CUDA_TRY(cudaGetLastError());
-  if (pl.splits > 1) {
-    attn_short_merge_kernel<D><<<(unsigned)(pl.units * kRows), kWarps * 32, 0, st>>>(p);
-    KVQ_CUDA_TRY(cudaGetLastError());
-  }
+  if (pl.splits > 1)
+    return launch_after(true, 1, dim3((unsigned)(pl.units * kRows)), dim3(kWarps * 32), 0, st, attn_short_merge_kernel<D>, p);
   return KVQ_OK;
 }
 

@@ -492,6 +492,7 @@ struct RotParams {
 template <int BITS, int GROUP, int D>
 __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
   constexpr int kLanes = D / 8;                      // per row
+  allow_next_grid();                                 // the attention kernel: its prologue and first tiles need nothing from here
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ln = lane & (kLanes - 1), rsub = lane / kLanes;
   constexpr int lanes_per_group = GROUP / 8;
@@ -673,6 +674,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
   // TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512); P_q aliases the first 64 columns of S_q.
 
+  allow_next_grid();                             // the merge kernel
   if (warp < 4) {
     setmaxnreg_dec<kRegsIssue>();
   if (warp == 0) {
@@ -728,6 +730,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (!(ok = cx.wait(kQEmpty, (nseg & 1) ^ 1, 100))) break;
         // a segment that starts in the cache never needs the unrotated query: load the rotated one right away
         const bool cached0 = sg.tb >= n_rt;
+        if (cached0) wait_for_previous_grid();          // the pre-pass: rotated queries
         expect_tx_lead(kQFull, p.n_qt * kLoadBytes);
         for (int qt = 0; qt < p.n_qt; ++qt)
           for (int kb = 0; kb < kBlocks; ++kb)
@@ -739,6 +742,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if (t == n_rt && !cached0) {
             // first cached tile: once no MMA reads the unrotated query any more, the rotated tile replaces it
             if (!(ok = cx.wait(kQCurDone, nseg & 1, 103))) break;
+            wait_for_previous_grid();
             expect_tx_lead(kQRotFull, p.n_qt * kLoadBytes);
             for (int qt = 0; qt < p.n_qt; ++qt)
               for (int kb = 0; kb < kBlocks; ++kb)
@@ -1173,6 +1177,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if constexpr (PAIR) ok = __all_sync(0xFFFFFFFFu, cx.wait(kQEmpty, (nseg & 1) ^ 1, 402));
           else ok = __all_sync(0xFFFFFFFFu, cx.wait(kQFull, nseg & 1, 402));
           if (!ok) break;
+          wait_for_previous_grid();                     // the pre-pass wrote them
           const int row0 = unit_row0(sg.unit, bh);
 #pragma unroll
           for (int qt = 0; qt < 2; ++qt) {
@@ -1216,6 +1221,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // A pair leaves together: neither CTA's shared memory or TMEM may go while the other still arrives on its
   // barriers or the leader's MMAs still read its operands (every role above has come out through bounded waits).
   if constexpr (PAIR) cluster_sync_all();
+  wait_for_previous_grid();                      // also in a CTA that had no cached tile
   if (warp == 0) {
     tc_fence_after();
     if constexpr (PAIR) tmem_dealloc_pair(tmem, 512); else tmem_dealloc(tmem, 512);
@@ -1231,6 +1237,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 template <int D>
 __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_ctas, int pair) {
   constexpr int kCols = D / 16;                        // columns of a 16-byte piece: 8 in BF16, 4 in FP32 (64 channels)
+  wait_for_previous_grid();                            // the attention kernel's partial rows
   const int su = pair ? blockIdx.x >> 1 : blockIdx.x, rank = pair ? blockIdx.x & 1 : 0, kc = pair ? 2 : 1;
   const int unit = p.n_whole + su;
   const int T = p.tiles;
@@ -1455,23 +1462,14 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk,
     rotate_query_kernel<BITS, GROUP, D><<<dim3((unsigned)((rp.m_tokens + kRows - 1) / kRows), (unsigned)(p.n_units / p.q_blocks)), 256, 0, st>>>(rp);
     KVQ_CUDA_TRY(cudaGetLastError());
   }
-  if constexpr (PAIR) {             // grid.x counts pairs: two CTAs each, launched as clusters of two
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * grid.x); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    KVQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, attn_tcgen05_kernel<BITS, GROUP, true, D>, mq, mqr, mk, mv, p));
-  } else {
-    attn_tcgen05_kernel<BITS, GROUP, false, D><<<grid, kThreads, kSmemBytes, st>>>(mq, mqr, mk, mv, p);
-  }
-  KVQ_CUDA_TRY(cudaGetLastError());
-  if (p.n_whole != p.n_units) {   // units were split over CTAs: combine their partial results
-    attn_merge_kernel<D><<<dim3((unsigned)((p.n_units - p.n_whole) * (PAIR ? 2 : 1)), 16), 256, 0, st>>>(p, (int)grid.x, PAIR ? 1 : 0);
-    KVQ_CUDA_TRY(cudaGetLastError());
-  }
-  return KVQ_OK;
+  // grid.x counts pairs in the pair kernel: two CTAs each, launched as clusters of two.  Behind the pre-pass the kernel may
+  // start early: it has the current chunk's tiles to work on first.
+  constexpr int kC = PAIR ? 2 : 1;
+  int r = launch_after(rp.qr != nullptr, kC, dim3(kC * grid.x), dim3(kThreads), kSmemBytes, st, attn_tcgen05_kernel<BITS, GROUP, PAIR, D>, mq, mqr, mk, mv, p);
+  if (r != KVQ_OK) return r;
+  if (p.n_whole != p.n_units)     // units were split over CTAs: combine their partial results
+    r = launch_after(true, 1, dim3((unsigned)((p.n_units - p.n_whole) * kC), 16), dim3(256), 0, st, attn_merge_kernel<D>, p, (int)grid.x, PAIR ? 1 : 0);
+  return r;
 }
 
 }  // namespace

@@ -90,6 +90,35 @@ void set_attn_wait_budget(uint32_t cycles);
 int launch_attn_tcgen05_static(const AttnArgs& a);
 
 #ifdef __CUDACC__
+// Launches `kern` so that its blocks may start before the previous kernel in the stream has finished (it waits by itself,
+// see wait_for_previous_grid), in clusters of `cluster` blocks; overlap = false: an ordinary launch.
+template <typename... Params, typename... Args>
+int launch_after(bool overlap, int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, void (*kern)(Params...), const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
+  KVQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+  return KVQ_OK;
+}
+
+// Kernels of one call overlap where the second does not need the first at once (launch_after): the first allows the next
+// grid's blocks to start when its own have all started, the second waits before it touches what the first writes.  Every
+// block of the second waits, so that work ordered behind it is ordered behind the first too.
+__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- device-side number-format helpers -------------------------------------------------
 
 // FP32 -> E4M3 byte, round-to-nearest-even, saturating to +-448 (hardware conversion).
