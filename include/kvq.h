@@ -151,7 +151,7 @@ int kvq_quantize_append(const kvq_cache_desc* desc, int64_t cache_len,
 /*
  * Bytes of device workspace kvq_attn_corrected needs for this problem (may be 0).  With the tcgen05 kernel
  * and a non-empty cache window it holds the rotated query chunk (Section 3.1: q~ = H q in FP16, plus the
- * per-group squared norms nu of Eq. 15, 272 bytes per query row, written by a pre-pass kernel of the same
+ * per-group squared norms nu of Eq. 15, 2 * head_dim + 16 bytes per query row, written by a pre-pass kernel of the same
  * call) and, when the key tiles of a unit are split over several CTAs, their partial results.
  * out_bytes is host memory.  Same errors as kvq_attn_corrected's argument checks.
  */
