@@ -1183,7 +1183,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           for (int qt = 0; qt < 2; ++qt) {
             const int row = row0 + qt * kBlockM + dt;
             uint4 a = make_uint4(0, 0, 0, 0);
-            if (row < p.m_tokens) a = __ldg(reinterpret_cast<const uint4*>(p.ax_rows + ((int64_t)bh * p.m_tokens + row) * 8));
+            // an ordinary load: the pre-pass may still write these rows while this kernel runs (it starts early), and the
+            // read-only path is defined for memory that nothing writes meanwhile
+            if (row < p.m_tokens) a = *reinterpret_cast<const uint4*>(p.ax_rows + ((int64_t)bh * p.m_tokens + row) * 8);
             *reinterpret_cast<uint4*>(smem + kOffAx + qt * kXBytes + xtile_offset(dt, 0)) = a;
           }
           fence_proxy_async_smem();

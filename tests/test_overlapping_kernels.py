@@ -1,0 +1,29 @@
+"""Kernels of one call overlap (programmatic dependent launch): what an earlier kernel of the call writes into the workspace
+may still be written while a later one runs.  Such memory must not be read through the read-only path (`__ldg`,
+ld.global.nc), which is defined only for memory that nothing writes during the kernel.  Checked in the sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_26266_b200", "csrc")
+
+
+def ldg_arguments(text):
+    """The argument of every __ldg( ... ), parentheses matched."""
+    for m in re.finditer(r"__ldg\(", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        yield text[m.end():i - 1]
+
+
+# workspace memory written and read inside one call: bias rows and rotated queries of the pre-pass, partial rows for the merge
+@pytest.mark.parametrize("name,pointers", [("attn_sm100.cu", ("ax_rows", "partial", "slot_of", "sl")), ("attn_short.cu", ("partial", "slots", "sl"))])
+def test_workspace_is_not_read_through_the_read_only_path(name, pointers):
+    with open(os.path.join(CSRC, name)) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    assert "wait_for_previous_grid()" in text and all(p in text for p in pointers[:1])
+    bad = [a for a in ldg_arguments(text) if any(re.search(rf"\b{p}\b", a) for p in pointers)]
+    assert not bad, bad
