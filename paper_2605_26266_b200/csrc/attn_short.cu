@@ -149,7 +149,11 @@ __device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p
   }
 }
 
-template <int D, int BITS, int GROUP>
+// ANY_ZERO: groups whose constants are not exact (key_constant_exact, value_constant_exact) are expanded in FP32, as in the
+// warp-level kernel, which served the calls this is set for before: heads of 64 channels, and chunks TMA cannot address.  The
+// tests of the constants and the registers of the second form cost 128 channels 45 -> 51 us (16 rows over 16 384 tokens of
+// 32 heads at 4 bits); without it they are expanded as in the tcgen05 kernel.
+template <int D, int BITS, int GROUP, bool ANY_ZERO>
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(const SParams p) {
   constexpr int LD = D + 8;                                        // padded rows of the query tiles
   constexpr int KS = D / 16;                                       // MMA steps over the channels
@@ -311,66 +315,88 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(con
     float s[4][4];
     // (OFF + code) * step - (OFF + zero) * step with OFF from the exponent bits OR-ed over the code, one FMA per pair
     constexpr float kOff = BITS == 2 ? 4.f : 16.f;
+    constexpr uint32_t kMask = (1u << BITS) - 1;
     uint32_t step2[4], off2[4];
+    bool exact = true;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
-      step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(-(kOff + zs) * ds, -(kOff + zs) * ds);
+      const float off = -(kOff + zs) * ds;
+      step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(off, off);
+      if (ANY_ZERO) exact &= key_constant_exact<BITS>(off, zs, ds);
       s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
       if (p.correction) mma_bf16(s[t], ax[0], ax[1], 0u, 0u, pack_bf16(ds * ds, ds * ds), 0u);
     }
     // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
+    auto scores = [&](auto expand) {
 #pragma unroll
-    for (int wi = 0; wi < KW; ++wi)
+      for (int wi = 0; wi < KW; ++wi)
 #pragma unroll
-      for (int j = 0; j < KPW; ++j)
+        for (int j = 0; j < KPW; ++j)
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          uint32_t bf[2];
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const uint32_t x = move_bits(keys.w[t][wi], (2 * j + i) * BITS, BITS == 2 ? 8 : 6);
-            bf[i] = fma_f16x2(BITS == 2 ? (x & 0x03000300u) | 0x44004400u : (x & 0x03C003C0u) | 0x4C004C00u, step2[t], off2[t]);
+          for (int t = 0; t < 4; ++t) {
+            const uint32_t (&a)[4] = qf[wi * KPW + j];
+            mma_f16(s[t], a[0], a[1], a[2], a[3], expand(t, wi, 2 * j), expand(t, wi, 2 * j + 1));
           }
-          const uint32_t (&a)[4] = qf[wi * KPW + j];
-          mma_f16(s[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
-        }
+    };
+    if (!ANY_ZERO || __all_sync(0xFFFFFFFFu, exact)) {
+      scores([&](int t, int wi, int i) {
+        const uint32_t x = move_bits(keys.w[t][wi], i * BITS, BITS == 2 ? 8 : 6);
+        return fma_f16x2(BITS == 2 ? (x & 0x03000300u) | 0x44004400u : (x & 0x03C003C0u) | 0x4C004C00u, step2[t], off2[t]);
+      });
+    } else {                                                       // (code - zero) * step in FP32, rounded once
+      scores([&](int t, int wi, int i) {
+        const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
+        const uint32_t x = keys.w[t][wi] >> (i * BITS);
+        return pack_f16_sat(((float)(x & kMask) - zs) * ds, ((float)((x >> 16) & kMask) - zs) * ds);
+      });
+    }
     if (st + kWarps < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st + kWarps), g, c);
     softmax_step(s, p.n_cached - st * kStep, l_cac);
     // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
       uint32_t step2[2], off2[2];
+      bool exact = true;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        float ds[2], zs[2];
+        float ds[2], off[2];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const uint32_t meta = vals.meta[4 * kk + 2 * u + i];
+          const float zs = __uint_as_float(meta & 0xFFFF0000u);
           ds[i] = e4m3_byte_to_f32(meta & 0xFFu);
-          zs[i] = __uint_as_float(meta & 0xFFFF0000u);
+          off[i] = BITS == 2 ? -(4.f + zs) * ds[i] : 16.f + zs;
+          if (ANY_ZERO) exact &= value_constant_exact<BITS>(off[i], zs);
         }
         step2[u] = pack_bf16(ds[0], ds[1]);
-        off2[u] = BITS == 2 ? pack_bf16(-(4.f + zs[0]) * ds[0], -(4.f + zs[1]) * ds[1]) : pack_bf16(16.f + zs[0], 16.f + zs[1]);
+        off2[u] = pack_bf16(off[0], off[1]);
       }
       constexpr int kPer = 16 / BITS;                              // codes in half a word
+      auto products = [&](auto expand) {
 #pragma unroll
-      for (int hw = 0; hw < NT / kPer; ++hw) {
-        uint32_t z[2];
+        for (int hw = 0; hw < NT / kPer; ++hw) {
+          uint32_t z[2];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
-          z[u] = __byte_perm(vals.w[4 * kk + 2 * u][hw / 2], vals.w[4 * kk + 2 * u + 1][hw / 2], hw & 1 ? 0x7632 : 0x5410);
+          for (int u = 0; u < 2; ++u)
+            z[u] = __byte_perm(vals.w[4 * kk + 2 * u][hw / 2], vals.w[4 * kk + 2 * u + 1][hw / 2], hw & 1 ? 0x7632 : 0x5410);
 #pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          uint32_t bf[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const uint32_t x = move_bits(z[u], i * BITS, BITS == 2 ? 5 : 3);
-            if constexpr (BITS == 2) bf[u] = fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u]);
-            else bf[u] = mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
-          }
-          mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], bf[0], bf[1]);
+          for (int i = 0; i < kPer; ++i)
+            mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], expand(z[0], 0, i), expand(z[1], 1, i));
         }
+      };
+      if (!ANY_ZERO || __all_sync(0xFFFFFFFFu, exact)) {
+        products([&](uint32_t z, int u, int i) {
+          const uint32_t x = move_bits(z, i * BITS, BITS == 2 ? 5 : 3);
+          return BITS == 2 ? fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u])
+                           : mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
+        });
+      } else {
+        products([&](uint32_t z, int u, int i) {
+          const uint32_t x = z >> (i * BITS), m0 = vals.meta[4 * kk + 2 * u], m1 = vals.meta[4 * kk + 2 * u + 1];
+          return pack_bf16(((float)(x & kMask) - __uint_as_float(m0 & 0xFFFF0000u)) * e4m3_byte_to_f32(m0 & 0xFFu),
+                           ((float)((x >> 16) & kMask) - __uint_as_float(m1 & 0xFFFF0000u)) * e4m3_byte_to_f32(m1 & 0xFFu));
+        });
       }
     }
   }
@@ -537,8 +563,9 @@ Plan plan(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t 
 }
 
 template <int D, int BITS, int GROUP>
-int launch(const SParams& p, const Plan& pl, cudaStream_t st) {
-  attn_short_kernel<D, BITS, GROUP><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
+int launch(const SParams& p, const Plan& pl, bool any_zero, cudaStream_t st) {
+  if (D == 64 || any_zero) attn_short_kernel<D, BITS, GROUP, true><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
+  else attn_short_kernel<D, BITS, GROUP, D == 64><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
   KVQ_CUDA_TRY(cudaGetLastError());
   if (pl.splits > 1)
     return launch_after(true, 1, dim3((unsigned)(pl.units * kRows)), dim3(kWarps * 32), 0, st, attn_short_merge_kernel<D>, p);
@@ -592,7 +619,8 @@ int launch_attn_short(const AttnArgs& a) {
   p.ax_coef = -a.softmax_scale / 24.0f;
   p.lse = a.lse; p.cached_mass = a.cached_mass;
   p.partial = static_cast<float*>(a.workspace);
-#define KVQ_SHORT(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) return launch<D_, B_, G_>(p, pl, a.stream);
+  const bool any_zero = !attn_tcgen05_addressable(a);
+#define KVQ_SHORT(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) return launch<D_, B_, G_>(p, pl, any_zero, a.stream);
   KVQ_SHORT(128, 2, 32) KVQ_SHORT(128, 2, 64) KVQ_SHORT(128, 2, 128) KVQ_SHORT(128, 4, 32) KVQ_SHORT(128, 4, 64) KVQ_SHORT(128, 4, 128)
   KVQ_SHORT(64, 2, 32) KVQ_SHORT(64, 2, 64) KVQ_SHORT(64, 4, 32) KVQ_SHORT(64, 4, 64)
 #undef KVQ_SHORT

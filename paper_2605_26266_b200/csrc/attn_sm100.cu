@@ -374,12 +374,31 @@ __device__ __forceinline__ void dequant_keys(const Raw<BITS, D>& r, uint8_t* til
   constexpr int G = D / GROUP;
   constexpr float kOff = (BITS == 2) ? 4.f : 16.f;
   uint32_t step2[4], c2[4];
+  bool exact = true;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
     step2[j] = pack_f16x2_sat(ds, ds);
     const float c = -(kOff + zs) * ds;
     c2[j] = pack_f16x2_sat(c, c);
+    if (D == 64 && j < G) exact &= key_constant_exact<BITS>(c, zs, ds);
+  }
+  if (D == 64 && __any_sync(0xFFFFFFFFu, !exact)) {      // the warp together: (code - zero) * step in FP32, rounded once
+    constexpr int kPer = 32 / BITS;
+#pragma unroll
+    for (int wi = 0; wi < NW; ++wi) {
+      const int gw = word0 + wi, j = (gw * kPer) / GROUP;
+      const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
+      auto x = [&](int i) { return ((float)((r.w[wi] >> (BITS * i)) & ((1u << BITS) - 1)) - zs) * ds; };
+#pragma unroll
+      for (int q = 0; q < kPer / 8; ++q) {
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = pack_f16x2_sat(x(4 * q + i), x(4 * q + i + kPer / 2));
+        *reinterpret_cast<uint4*>(tile + sw128_offset(row, gw * (kPer / 8) + q)) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+    return;
   }
   if constexpr (BITS == 2) {
 #pragma unroll
@@ -424,12 +443,31 @@ template <int BITS, int GROUP, int D, int NW = Raw<BITS, D>::kWords>
 __device__ __forceinline__ void dequant_values(const Raw<BITS, D>& r, uint8_t* tile, int row, int word0 = 0, int piece0 = 0) {
   constexpr int G = D / GROUP;
   uint32_t step2[4], c2[4];
+  bool exact = true;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
     step2[j] = pack_bf16x2(ds, ds);
     const float c = (BITS == 2) ? -(4.f + zs) * ds : (16.f + zs);
     c2[j] = pack_bf16x2(c, c);
+    if (D == 64 && j < G) exact &= value_constant_exact<BITS>(c, zs);
+  }
+  if (D == 64 && __any_sync(0xFFFFFFFFu, !exact)) {      // as for the keys
+    constexpr int kPer = 32 / BITS;
+#pragma unroll
+    for (int wi = 0; wi < NW; ++wi) {
+      const int gw = word0 + wi, j = (gw * kPer) / GROUP;
+      const float ds = raw_step<BITS, D>(r, j), zs = raw_zero<BITS, D>(r, j);
+      auto x = [&](int i) { return ((float)((r.w[wi] >> (BITS * i)) & ((1u << BITS) - 1)) - zs) * ds; };
+#pragma unroll
+      for (int q = 0; q < kPer / 8; ++q) {
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = cvt_bf16x2(x(8 * q + 2 * i), x(8 * q + 2 * i + 1));
+        *reinterpret_cast<uint4*>(tile + sw128_offset(row, gw * (kPer / 8) + q - piece0)) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+    return;
   }
   if constexpr (BITS == 2) {
 #pragma unroll

@@ -1,0 +1,53 @@
+"""Dequantized keys and values are (code - zero) * step rounded once (FP16 keys, saturated there; BF16 values), also for
+groups far from zero, whose zero-points lie far outside the code range.  One cached token carries the whole weight of every
+row: the output is then its dequantized value, and the log-sum-exp of a row whose query is a unit vector one channel of its
+dequantized key.  The kernels for heads of 64 channels, and the one for few rows where it takes a chunk shared by all heads."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import kvq_oracle as O
+from paper_2605_26266_b200 import inputs
+from tests import kvq_testlib as T
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("mean", [0.0, 12.0, -30.0, 80.0, 3000.0, 65300.0])
+@pytest.mark.parametrize("d,bits,group,m", [(64, 2, 32, 129), (64, 4, 32, 300), (64, 4, 64, 129), (64, 2, 64, 16), (64, 4, 32, 16),
+                                            (128, 2, 32, 16), (128, 4, 64, 16), (128, 2, 128, 16)])
+def test_one_rounding(d, bits, group, m, mean):
+    from paper_2605_26266_b200 import binding as B
+    batch, heads = 2, 24
+    r = np.random.default_rng(int(abs(mean)) + d + bits + group)
+    shape = (batch, heads, 1, d)
+    # every other group of a token sits at the mean, so that exact and inexact ones meet in a warp
+    shift = np.where((np.arange(d) // 32 + np.arange(heads)[:, None]) % 2, np.float32(mean), np.float32(0))[None, :, None, :]
+    k, v = (inputs.f32_to_bf16_bits(r.standard_normal(shape, dtype=np.float32) + shift) for _ in range(2))
+    g, o = B.Cache(batch, heads, d, bits, group, 128, rotate_k=False), O.Cache(batch, heads, d, bits, group, 128, rotate_k=False)
+    B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(v))
+    O.quantize_append(o, 0, k, v)
+
+    def hat(which):
+        code, byte, zero = (getattr(o, which + s)[:, :, 0] for s in ("_codes", "_scale", "_zero"))
+        x = O.unpack_codes(code, bits).reshape(batch, heads, d // group, group).astype(np.float64)
+        return ((x - O.bf16_bits_to_f64(zero)[..., None]) * O.e4m3_decode(byte)[..., None]).reshape(batch, heads, d)
+
+    want_k = np.clip(hat("k"), -65504.0, 65504.0).astype(np.float16).astype(np.float64)
+    want_v = inputs.f32_to_bf16_bits(hat("v").astype(np.float32))        # up to 24 significant bits: exact in float32
+    kc = torch.full((batch, heads, 1, d), -1000.0, dtype=torch.bfloat16, device="cuda")      # weight 2^-1300
+    vc = torch.ones_like(kc)
+    if d == 128:
+        kc, vc = (t[:, :1].expand(-1, heads, -1, -1) for t in (kc, vc))                       # no tensor map can address it
+    for first in range(0, d, m):
+        channels = (first + np.arange(m)) % d
+        q = np.zeros((batch, heads, m, d), dtype=np.float32)
+        q[:, :, np.arange(m), channels] = 1.0
+        lse = torch.empty(batch, heads, m, dtype=torch.float32, device="cuda")
+        out = B.kvq_attn_corrected(g, T.to_dev(inputs.f32_to_bf16_bits(q)), kc, vc, 1.0, B.KVQ_CORRECTION_OFF, cache_len=1, lse=lse)
+        got_v = out.view(torch.int16).cpu().numpy().view(np.uint16)
+        bad = (got_v != want_v[:, :, None]) & ((got_v | want_v[:, :, None]) != 0x8000)       # either sign of zero
+        assert not bad.any(), f"{bad.sum()} of {bad.size} values"
+        s, got_s = want_k[:, :, channels], lse.cpu().numpy().astype(np.float64)
+        # scale_log2, its product with the score and the one with ln 2: three roundings of 2^-24
+        assert (np.abs(got_s - s) <= 4 * 2.0 ** -24 * np.abs(s) + 1e-30).all(), np.abs(got_s / np.where(s == 0, 1, s) - 1).max()
