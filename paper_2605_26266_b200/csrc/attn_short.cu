@@ -20,6 +20,8 @@
 // registers 47 us, four 76 us; the four score tiles of a step one after the other instead of in turn 45 us.
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "kvq_common.cuh"
 
 namespace kvq {
@@ -150,11 +152,13 @@ __device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p
 }
 
 // ANY_ZERO: groups whose constants are not exact (key_constant_exact, value_constant_exact) are expanded in FP32, as in the
-// warp-level kernel, which served the calls this is set for before: heads of 64 channels, and chunks TMA cannot address.  The
-// tests of the constants and the registers of the second form cost 128 channels 45 -> 51 us (16 rows over 16 384 tokens of
-// 32 heads at 4 bits); without it they are expanded as in the tcgen05 kernel.
+// warp-level kernel, which served the calls this is set for before: heads of 64 channels, and chunks TMA cannot address.  A
+// warp works in 16 bits, notes whether it met such a group, and then takes its steps once more in FP32.  Any branch inside a
+// step costs every call: 16 rows over 8 192 tokens of 160 heads of 64 channels take 109 us without the second form, 115 us as
+// here, 140 us with a branch at each step or an early exit.  Three CTAs an SM for 64 channels (two with the registers of the
+// second form: 237 against 140 us for 32 such rows).
 template <int D, int BITS, int GROUP, bool ANY_ZERO>
-__global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(const SParams p) {
+__global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_short_kernel(const SParams p) {
   constexpr int LD = D + 8;                                        // padded rows of the query tiles
   constexpr int KS = D / 16;                                       // MMA steps over the channels
   constexpr int NT = D / 8;                                        // output tiles of 8 channels
@@ -306,74 +310,73 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(con
     x.n_valid = p.n_cached - i * kStep;
     return x;
   };
-  Keys<D, BITS> keys;
-  if (st < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st), g, c);
-#pragma unroll 1
-  for (; st < last_c; st += kWarps) {
-    Values<D, BITS> vals;                                          // on their way while the scores are computed
-    load_values<D, BITS, GROUP>(vals, p, step_of(st), g, c);
-    float s[4][4];
-    // (OFF + code) * step - (OFF + zero) * step with OFF from the exponent bits OR-ed over the code, one FMA per pair
+  // kFp32: (code - zero) * step in FP32, rounded once.  Otherwise in 16 bits; with ANY_ZERO false if some constants were not
+  // exact (such steps are in the sums by then).
+  auto cached_steps = [&](auto fp32) {
+    constexpr bool kFp32 = decltype(fp32)::value;
     constexpr float kOff = BITS == 2 ? 4.f : 16.f;
     constexpr uint32_t kMask = (1u << BITS) - 1;
-    uint32_t step2[4], off2[4];
+    Keys<D, BITS> keys;
     bool exact = true;
+    if (st < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st), g, c);
+#pragma unroll 1
+    for (; st < last_c; st += kWarps) {
+      Values<D, BITS> vals;                                        // on their way while the scores are computed
+      load_values<D, BITS, GROUP>(vals, p, step_of(st), g, c);
+      float s[4][4];
+      // (OFF + code) * step - (OFF + zero) * step with OFF from the exponent bits OR-ed over the code, one FMA per pair
+      uint32_t step2[4], off2[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
-      const float off = -(kOff + zs) * ds;
-      step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(off, off);
-      if (ANY_ZERO) exact &= key_constant_exact<BITS>(off, zs, ds);
-      s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
-      if (p.correction) mma_bf16(s[t], ax[0], ax[1], 0u, 0u, pack_bf16(ds * ds, ds * ds), 0u);
-    }
-    // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
-    auto scores = [&](auto expand) {
+      for (int t = 0; t < 4; ++t) {
+        const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
+        const float off = -(kOff + zs) * ds;
+        step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(off, off);
+        if (ANY_ZERO && !kFp32) exact &= key_constant_exact<BITS>(zs);
+        s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
+        if (p.correction) mma_bf16(s[t], ax[0], ax[1], 0u, 0u, pack_bf16(ds * ds, ds * ds), 0u);
+      }
+      // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
 #pragma unroll
       for (int wi = 0; wi < KW; ++wi)
 #pragma unroll
         for (int j = 0; j < KPW; ++j)
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
+            uint32_t bf[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              if constexpr (kFp32) {
+                const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
+                const uint32_t x = keys.w[t][wi] >> ((2 * j + i) * BITS);
+                bf[i] = pack_f16_sat(((float)(x & kMask) - zs) * ds, ((float)((x >> 16) & kMask) - zs) * ds);
+              } else {
+                const uint32_t x = move_bits(keys.w[t][wi], (2 * j + i) * BITS, BITS == 2 ? 8 : 6);
+                bf[i] = fma_f16x2(BITS == 2 ? (x & 0x03000300u) | 0x44004400u : (x & 0x03C003C0u) | 0x4C004C00u, step2[t], off2[t]);
+              }
+            }
             const uint32_t (&a)[4] = qf[wi * KPW + j];
-            mma_f16(s[t], a[0], a[1], a[2], a[3], expand(t, wi, 2 * j), expand(t, wi, 2 * j + 1));
+            mma_f16(s[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
           }
-    };
-    if (!ANY_ZERO || __all_sync(0xFFFFFFFFu, exact)) {
-      scores([&](int t, int wi, int i) {
-        const uint32_t x = move_bits(keys.w[t][wi], i * BITS, BITS == 2 ? 8 : 6);
-        return fma_f16x2(BITS == 2 ? (x & 0x03000300u) | 0x44004400u : (x & 0x03C003C0u) | 0x4C004C00u, step2[t], off2[t]);
-      });
-    } else {                                                       // (code - zero) * step in FP32, rounded once
-      scores([&](int t, int wi, int i) {
-        const float ds = e4m3_byte_to_f32(keys.meta[t] & 0xFFu), zs = __uint_as_float(keys.meta[t] & 0xFFFF0000u);
-        const uint32_t x = keys.w[t][wi] >> (i * BITS);
-        return pack_f16_sat(((float)(x & kMask) - zs) * ds, ((float)((x >> 16) & kMask) - zs) * ds);
-      });
-    }
-    if (st + kWarps < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st + kWarps), g, c);
-    softmax_step(s, p.n_cached - st * kStep, l_cac);
-    // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
+      if (st + kWarps < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st + kWarps), g, c);
+      softmax_step(s, p.n_cached - st * kStep, l_cac);
+      // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
 #pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-      uint32_t step2[2], off2[2];
-      bool exact = true;
+      for (int kk = 0; kk < 2; ++kk) {
+        uint32_t step2[2], off2[2];
+        float ds[2][2], zs[2][2];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        float ds[2], off[2];
+        for (int u = 0; u < 2; ++u) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const uint32_t meta = vals.meta[4 * kk + 2 * u + i];
-          const float zs = __uint_as_float(meta & 0xFFFF0000u);
-          ds[i] = e4m3_byte_to_f32(meta & 0xFFu);
-          off[i] = BITS == 2 ? -(4.f + zs) * ds[i] : 16.f + zs;
-          if (ANY_ZERO) exact &= value_constant_exact<BITS>(off[i], zs);
+          for (int i = 0; i < 2; ++i) {
+            const uint32_t meta = vals.meta[4 * kk + 2 * u + i];
+            ds[u][i] = e4m3_byte_to_f32(meta & 0xFFu);
+            zs[u][i] = __uint_as_float(meta & 0xFFFF0000u);
+            if (ANY_ZERO && !kFp32) exact &= value_constant_exact<BITS>(zs[u][i]);
+          }
+          step2[u] = pack_bf16(ds[u][0], ds[u][1]);
+          off2[u] = BITS == 2 ? pack_bf16(-(4.f + zs[u][0]) * ds[u][0], -(4.f + zs[u][1]) * ds[u][1]) : pack_bf16(16.f + zs[u][0], 16.f + zs[u][1]);
         }
-        step2[u] = pack_bf16(ds[0], ds[1]);
-        off2[u] = pack_bf16(off[0], off[1]);
-      }
-      constexpr int kPer = 16 / BITS;                              // codes in half a word
-      auto products = [&](auto expand) {
+        constexpr int kPer = 16 / BITS;                            // codes in half a word
 #pragma unroll
         for (int hw = 0; hw < NT / kPer; ++hw) {
           uint32_t z[2];
@@ -381,24 +384,33 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) attn_short_kernel(con
           for (int u = 0; u < 2; ++u)
             z[u] = __byte_perm(vals.w[4 * kk + 2 * u][hw / 2], vals.w[4 * kk + 2 * u + 1][hw / 2], hw & 1 ? 0x7632 : 0x5410);
 #pragma unroll
-          for (int i = 0; i < kPer; ++i)
-            mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], expand(z[0], 0, i), expand(z[1], 1, i));
+          for (int i = 0; i < kPer; ++i) {
+            uint32_t bf[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              if constexpr (kFp32) {
+                const uint32_t x = z[u] >> (i * BITS);
+                bf[u] = pack_bf16(((float)(x & kMask) - zs[u][0]) * ds[u][0], ((float)((x >> 16) & kMask) - zs[u][1]) * ds[u][1]);
+              } else {
+                const uint32_t x = move_bits(z[u], i * BITS, BITS == 2 ? 5 : 3);
+                if constexpr (BITS == 2) bf[u] = fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u]);
+                else bf[u] = mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
+              }
+            }
+            mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], bf[0], bf[1]);
+          }
         }
-      };
-      if (!ANY_ZERO || __all_sync(0xFFFFFFFFu, exact)) {
-        products([&](uint32_t z, int u, int i) {
-          const uint32_t x = move_bits(z, i * BITS, BITS == 2 ? 5 : 3);
-          return BITS == 2 ? fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u])
-                           : mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
-        });
-      } else {
-        products([&](uint32_t z, int u, int i) {
-          const uint32_t x = z >> (i * BITS), m0 = vals.meta[4 * kk + 2 * u], m1 = vals.meta[4 * kk + 2 * u + 1];
-          return pack_bf16(((float)(x & kMask) - __uint_as_float(m0 & 0xFFFF0000u)) * e4m3_byte_to_f32(m0 & 0xFFu),
-                           ((float)((x >> 16) & kMask) - __uint_as_float(m1 & 0xFFFF0000u)) * e4m3_byte_to_f32(m1 & 0xFFu));
-        });
       }
     }
+    return !ANY_ZERO || kFp32 || __all_sync(0xFFFFFFFFu, exact);
+  };
+  if (!cached_steps(std::false_type{})) {                          // the warp's steps once more
+    st = first + warp;
+    m_run[0] = m_run[1] = -INFINITY;
+    l_cur[0] = l_cur[1] = l_cac[0] = l_cac[1] = 0.f;
+#pragma unroll
+    for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+    cached_steps(std::true_type{});
   }
   // ---- current chunk: unrotated query, BF16 keys and values, no bias ----
 #pragma unroll 1

@@ -381,7 +381,7 @@ __device__ __forceinline__ void dequant_keys(const Raw<BITS, D>& r, uint8_t* til
     step2[j] = pack_f16x2_sat(ds, ds);
     const float c = -(kOff + zs) * ds;
     c2[j] = pack_f16x2_sat(c, c);
-    if (D == 64 && j < G) exact &= key_constant_exact<BITS>(c, zs, ds);
+    if (D == 64 && j < G) exact &= key_constant_exact<BITS>(zs);
   }
   if (D == 64 && __any_sync(0xFFFFFFFFu, !exact)) {      // the warp together: (code - zero) * step in FP32, rounded once
     constexpr int kPer = 32 / BITS;
@@ -450,7 +450,7 @@ __device__ __forceinline__ void dequant_values(const Raw<BITS, D>& r, uint8_t* t
     step2[j] = pack_bf16x2(ds, ds);
     const float c = (BITS == 2) ? -(4.f + zs) * ds : (16.f + zs);
     c2[j] = pack_bf16x2(c, c);
-    if (D == 64 && j < G) exact &= value_constant_exact<BITS>(c, zs);
+    if (D == 64 && j < G) exact &= value_constant_exact<BITS>(zs);
   }
   if (D == 64 && __any_sync(0xFFFFFFFFu, !exact)) {      // as for the keys
     constexpr int kPer = 32 / BITS;

@@ -143,18 +143,16 @@ __device__ __forceinline__ uint32_t f32_to_bf16_bits(float x) {
   return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
-// The 16-bit forms of x^ = (code - zero) * step round once, as the FP32 form followed by one conversion does, if their
-// constants are exact: for keys (FP16, OFF = 4 or 16) and 2-bit values (BF16) that is (OFF + zero) * step, subtracted by an
-// FMA; for 4-bit values 16 + zero, subtracted before the multiplication.  So it is for zero-points up to a few times the
-// code range (keys: up to 100; 2-bit values: -20 .. 12; 4-bit values: -241 .. 240).  The keys must also stay below the largest FP16
-// value, where the FP32 form saturates.  NaN and infinities are not exact.
+// The 16-bit forms of x^ = (code - zero) * step round once, as the FP32 form followed by one conversion does, while their
+// constants are exact.  Keys (FP16) and 2-bit values (BF16) subtract (OFF + zero) * step, OFF = 4 or 16, with an FMA: an
+// integer of 7 (4) bits times a step of 4 is exact in 11 (8), and with |OFF + zero| up to 112 no key reaches the largest
+// FP16 value, where the FP32 form saturates.  4-bit values subtract 16 + zero before the multiplication: exact while code -
+// zero and 16 + zero have 8 bits.  False for NaN and infinities.
 template <int BITS>
-__device__ __forceinline__ bool key_constant_exact(float c, float zero, float step) {
-  return __half2float(__float2half_rn(c)) == c && (fabsf(zero) + 32.f) * step <= 65504.f;
-}
+__device__ __forceinline__ bool key_constant_exact(float zero) { return fabsf((BITS == 2 ? 4.f : 16.f) + zero) <= 112.f; }
 template <int BITS>
-__device__ __forceinline__ bool value_constant_exact(float c, float zero) {
-  return bf16_bits_to_f32(f32_to_bf16_bits(c)) == c && zero >= -241.f && zero <= 240.f;
+__device__ __forceinline__ bool value_constant_exact(float zero) {
+  return BITS == 2 ? fabsf(4.f + zero) <= 16.f : fabsf(16.f + zero - 15.5f) <= 240.5f;
 }
 #endif
 

@@ -51,3 +51,32 @@ def test_one_rounding(d, bits, group, m, mean):
         s, got_s = want_k[:, :, channels], lse.cpu().numpy().astype(np.float64)
         # scale_log2, its product with the score and the one with ln 2: three roundings of 2^-24
         assert (np.abs(got_s - s) <= 4 * 2.0 ** -24 * np.abs(s) + 1e-30).all(), np.abs(got_s / np.where(s == 0, 1, s) - 1).max()
+
+
+@pytest.mark.parametrize("d,bits,group,m", [(64, 2, 32, 16), (64, 4, 32, 30), (64, 4, 64, 200), (64, 2, 64, 300), (128, 4, 32, 16), (128, 2, 64, 16)])
+def test_groups_far_from_zero_among_others(d, bits, group, m):
+    """Only tokens from 40 on lie far from zero: a warp of the few-row kernel meets them after steps it has already summed."""
+    from paper_2605_26266_b200 import binding as B
+    heads, n, n_cur = 6, 700, 33
+    r = np.random.default_rng(d + bits + group)
+    far = (40.0 * (np.arange(n) >= 40)[:, None] * np.where(np.arange(heads) % 2, 1.0, -1.0)[:, None, None])[None].astype(np.float32)
+    draw = lambda t, x=0: inputs.f32_to_bf16_bits((r.standard_normal((1, heads, t, d)) + x).astype(np.float32))
+    g, o = (X.Cache(1, heads, d, bits, group, 768, rotate_k=False) for X in (B, O))
+    k, v = draw(n, far), draw(n, far)
+    B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(v))
+    O.quantize_append(o, 0, k, v)
+    q, kc, vc = draw(m), draw(n_cur), draw(n_cur)
+    dq, dk, dv = (T.to_dev(x) for x in (q, kc, vc))
+    if d == 128:
+        kc, vc = (np.repeat(x[:, :1], heads, 1) for x in (kc, vc))
+        dk, dv = (x[:, :1].expand(-1, heads, -1, -1) for x in (dk, dv))
+    lse = torch.empty(1, heads, m, dtype=torch.float32, device="cuda")
+    mass = torch.empty_like(lse)
+    sigma = 0.25 * T.sigma_of(d)
+    out = B.kvq_attn_corrected(g, dq, dk, dv, sigma, B.KVQ_CORRECTION_ON, cache_len=n, lse=lse, cached_mass=mass)
+    want = O.attn_corrected(o, 0, n, q, kc, vc, sigma, correction=True)
+    rel, _ = T.attn_errors(T.from_dev_bf16(out).reshape(want["out"].shape), want["out"])
+    assert rel <= T.REL_L2_TOL, rel
+    # FP16 keys of magnitude 40: sigma |q| 40 2^-12 / sqrt(3) = 1.4e-3 a score
+    assert np.abs(lse.cpu().numpy().reshape(want["lse"].shape) - want["lse"]).max() < 2e-2
+    assert np.abs(mass.cpu().numpy().reshape(want["cached_mass"].shape) - want["cached_mass"]).max() < 1e-2
