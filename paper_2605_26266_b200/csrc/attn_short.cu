@@ -236,14 +236,18 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
     const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.qr + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.qr + (g + 8) * LD + col);
     qf[ks][0] = lo.x; qf[ks][1] = hi.x; qf[ks][2] = lo.y; qf[ks][3] = hi.y;
   }
-  // bias operand: columns 2 c, 2 c + 1 are the high and low part of lane c's group; one lane per group counts it
-  uint32_t ax[2] = {0u, 0u};
+  // bias operand: columns 2 c, 2 c + 1 are the high and low part of lane c's group, with ANY_ZERO column 2 c + 8 is the rest
+  // (the warp-level kernel applies the bias in FP32); one lane per group counts it
+  uint32_t ax[4] = {0u, 0u, 0u, 0u};
   if (p.correction && c % (4 / G) == 0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const float a = p.ax_coef * sm.in.nu[(g + 8 * i) * 4 + c / (4 / G)];
       const uint32_t hi = f32_to_bf16_bits(a);
-      ax[i] = hi | (f32_to_bf16_bits(a - bf16_bits_to_f32(hi)) << 16);
+      const float rest = a - bf16_bits_to_f32(hi);
+      const uint32_t lo = f32_to_bf16_bits(rest);
+      ax[i] = hi | (lo << 16);
+      if (ANY_ZERO) ax[2 + i] = f32_to_bf16_bits(rest - bf16_bits_to_f32(lo));
     }
   }
 
@@ -333,7 +337,10 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
         step2[t] = pack_f16_sat(ds, ds); off2[t] = pack_f16_sat(off, off);
         if (ANY_ZERO && !kFp32) exact &= key_constant_exact<BITS>(zs);
         s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
-        if (p.correction) mma_bf16(s[t], ax[0], ax[1], 0u, 0u, pack_bf16(ds * ds, ds * ds), 0u);
+        if (p.correction) {
+          const uint32_t b = pack_bf16(ds * ds, ds * ds);
+          mma_bf16(s[t], ax[0], ax[1], ax[2], ax[3], b, ANY_ZERO ? b : 0u);
+        }
       }
       // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
 #pragma unroll

@@ -10,7 +10,7 @@
 //
 // Score of a cached key (Eq. (15) / Eq. (25)):  s = sigma*q~.k^ - (sigma^2/24) sum_j step_j^2 nu_j.
 // The bias is folded into the score contraction as one extra K=16 MMA step per half tile:
-// A_extra[m, j] = -(sigma/24) nu_{m,j} (split into a BF16 high and low part, two columns) and
+// A_extra[m, j] = -(sigma/24) nu_{m,j} (split into a BF16 high and low part, two columns; three for 64 channels) and
 // B_extra[i, j] = step_{i,j}^2 (exact in BF16), so the softmax warps spend no instruction on
 // it; correction off simply skips that step.
 //
@@ -521,7 +521,7 @@ __device__ __forceinline__ void dequant_values(const Raw<BITS, D>& r, uint8_t* t
 struct RotParams {
   const uint16_t* q; int64_t q_sb, q_sh, q_st;
   uint16_t* qr;            // [batch * heads][m_tokens][D] FP16
-  uint16_t* ax;            // [batch * heads][m_tokens][8] BF16: high parts of groups 0..3, then low parts
+  uint16_t* ax;            // [batch * heads][m_tokens][8] BF16: high parts of groups 0..3 (64 channels: of 0 and 1, then the rests), then low parts
   const int8_t* signs;
   int heads, m_tokens, rotate;
   float ax_coef;           // -sigma / 24
@@ -575,7 +575,8 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
       // zeros for groups the format does not have; gathered from the group leaders and written by lane 0 of the row
       const float a = p.ax_coef * nu;
       const uint32_t hi = f32_to_bf16_bits(a);
-      const uint32_t lo = f32_to_bf16_bits(a - bf16_bits_to_f32(hi));
+      const float rest = a - bf16_bits_to_f32(hi);
+      const uint32_t lo = f32_to_bf16_bits(rest);
       uint32_t h4[4], l4[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -583,6 +584,14 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
         const uint32_t hj = __shfl_sync(0xFFFFFFFFu, hi, src), lj = __shfl_sync(0xFFFFFFFFu, lo, src);
         const bool have = j * GROUP < D;
         h4[j] = have ? hj : 0u; l4[j] = have ? lj : 0u;
+      }
+      if constexpr (D == 64) {                         // at most two groups: the free columns take the rest, and a is whole
+        const uint32_t third = f32_to_bf16_bits(rest - bf16_bits_to_f32(lo));
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t tj = __shfl_sync(0xFFFFFFFFu, third, (lane & ~(kLanes - 1)) + ((j * lanes_per_group) & (kLanes - 1)));
+          h4[2 + j] = j * GROUP < D ? tj : 0u;
+        }
       }
       if (valid && ln == 0)
         *reinterpret_cast<uint4*>(p.ax + ((int64_t)bh * p.m_tokens + row) * 8) =
@@ -1198,8 +1207,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           dequant_keys<BITS, GROUP, D, kNW>(rk, smem + kOffK + s * kTileBytes, k_row, k_word0);
           if (p.correction && k_word0 == 0) {   // B_extra row: step_j^2, exact in BF16
             const float d0 = raw_step<BITS, D>(rk, 0), d1 = raw_step<BITS, D>(rk, 1), d2 = raw_step<BITS, D>(rk, 2), d3 = raw_step<BITS, D>(rk, 3);
-            const uint32_t b01 = pack_bf16x2(d0 * d0, G > 1 ? d1 * d1 : 0.f), b23 = pack_bf16x2(G > 2 ? d2 * d2 : 0.f, G > 3 ? d3 * d3 : 0.f);
-            // columns 0..3 meet the high parts of A_extra, columns 4..7 the low parts
+            const uint32_t b01 = pack_bf16x2(d0 * d0, G > 1 ? d1 * d1 : 0.f);
+            const uint32_t b23 = D == 64 ? b01 : pack_bf16x2(G > 2 ? d2 * d2 : 0.f, G > 3 ? d3 * d3 : 0.f);
+            // columns 0..3 meet the high parts of A_extra (64 channels: high parts and rests), columns 4..7 the low parts
             *reinterpret_cast<uint4*>(smem + kOffBx + s * kXBytes + xtile_offset(k_row, 0)) = make_uint4(b01, b23, b01, b23);
           }
           fence_proxy_async_smem();

@@ -80,3 +80,32 @@ def test_groups_far_from_zero_among_others(d, bits, group, m):
     # FP16 keys of magnitude 40: sigma |q| 40 2^-12 / sqrt(3) = 1.4e-3 a score
     assert np.abs(lse.cpu().numpy().reshape(want["lse"].shape) - want["lse"]).max() < 2e-2
     assert np.abs(mass.cpu().numpy().reshape(want["cached_mass"].shape) - want["cached_mass"]).max() < 1e-2
+
+
+@pytest.mark.parametrize("d,bits,group,m", [(64, 2, 32, 300), (64, 4, 64, 129), (64, 2, 64, 16), (64, 4, 32, 16), (128, 4, 32, 16), (128, 2, 128, 16)])
+def test_bias_keeps_32_bits(d, bits, group, m):
+    """One cached key that is zero wherever the query is not, with a large step: a row's score is its bias alone."""
+    from paper_2605_26266_b200 import binding as B
+    heads = 24
+    r = np.random.default_rng(d + bits + group + m)
+    k = np.zeros((1, heads, 1, d), dtype=np.float32)
+    top = 20.0 * (1 + np.arange(heads))[None, :, None, None]
+    k[..., 0::group], k[..., 1::group] = top, -top
+    q = r.uniform(1.0, 2.0, (1, heads, m, d)).astype(np.float32)
+    q[..., 0::group] = q[..., 1::group] = 0.0
+    k, q = inputs.f32_to_bf16_bits(k), inputs.f32_to_bf16_bits(q)
+    g, o = (X.Cache(1, heads, d, bits, group, 128, rotate_k=False) for X in (B, O))
+    B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(k))
+    O.quantize_append(o, 0, k, k)
+    kc = np.full((1, 1 if d == 128 else heads, 1, d), 0xC900, dtype=np.uint16)                # -2^19: no weight on the current key
+    dk = T.to_dev(kc).expand(-1, heads, -1, -1)
+    lse = torch.empty(1, heads, m, dtype=torch.float32, device="cuda")
+    sigma = T.sigma_of(d)
+    B.kvq_attn_corrected(g, T.to_dev(q), dk, dk, sigma, B.KVQ_CORRECTION_ON, cache_len=1, lse=lse)
+    nu = (O.bf16_bits_to_f64(q) ** 2).reshape(1, heads, m, d // group, group).sum(-1)
+    step = O.e4m3_decode(o.k_scale[:, :, 0])
+    want = -(np.float64(np.float32(sigma)) ** 2 / 24.0) * (nu * step[:, :, None] ** 2).sum(-1)
+    # about ten roundings of 2^-24 (the sum of squares, the coefficient, the products, the change of base); a bias of 16
+    # significant bits is off by up to 2^-17
+    err = np.abs(lse.cpu().numpy() / want - 1).max()
+    assert err <= 2.0 ** -20, err
