@@ -257,6 +257,8 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
   float m_run[2] = {-INFINITY, -INFINITY}, l_cur[2] = {0.f, 0.f}, l_cac[2] = {0.f, 0.f};
   uint32_t pf[8];
   // online softmax over the 32 scores of a step (this lane: rows g, g + 8, keys 8 t + 2 c + {0, 1}); leaves the weights in pf
+  // The maximum is kept as a raw score and subtracted before the scale: exact for the largest score however large it is (a key
+  // masked with the lowest number), where the exact product of an FMA and a rounded maximum would differ.
   auto softmax_step = [&](float (&s)[4][4], int n_valid, float (&l)[2]) {
     if (n_valid < kStep) {
 #pragma unroll
@@ -273,12 +275,12 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
       for (int t = 0; t < 4; ++t) mx = fmaxf(mx, fmaxf(s[t][2 * r], s[t][2 * r + 1]));
       mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
       mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2));
-      m_new[r] = fmaxf(m_run[r], mx * p.scale_log2);
+      m_new[r] = fmaxf(m_run[r], mx);
     }
     if (__any_sync(0xFFFFFFFFu, m_new[0] > m_run[0] || m_new[1] > m_run[1])) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const float f = ex2(m_run[r] - m_new[r]);
+        const float f = ex2((m_run[r] - no_key_yet(m_new[r])) * p.scale_log2);
         l_cur[r] *= f; l_cac[r] *= f;
         m_run[r] = m_new[r];
 #pragma unroll
@@ -289,13 +291,16 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
       }
     }
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < 2; ++r) {
+      const float m = no_key_yet(m_run[r]);
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const float w0 = ex2(fmaf(s[t][2 * r], p.scale_log2, -m_run[r])), w1 = ex2(fmaf(s[t][2 * r + 1], p.scale_log2, -m_run[r]));
+        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(s[t][2 * r], s[t][2 * r + 1]), make_float2(-m, -m)), make_float2(p.scale_log2, p.scale_log2));
+        const float w0 = ex2(x.x), w1 = ex2(x.y);
         l[r] += w0 + w1;
         pf[2 * t + r] = pack_bf16(w0, w1);
       }
+    }
   };
 
   // ---- this CTA's share of the steps: cached keys first, then the current chunk's; warp w takes every fourth ----
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
     l_cur[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cur[r], 2);
     l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 1);
     l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 2);
-    if (c == 0) { s_stat[warp][0][g + 8 * r] = m_run[r]; s_stat[warp][1][g + 8 * r] = l_cur[r]; s_stat[warp][2][g + 8 * r] = l_cac[r]; }
+    if (c == 0) { s_stat[warp][0][g + 8 * r] = m_run[r] * p.scale_log2; s_stat[warp][1][g + 8 * r] = l_cur[r]; s_stat[warp][2][g + 8 * r] = l_cac[r]; }
   }
   __syncthreads();                                                 // also: the query tiles are free
 #pragma unroll
@@ -485,7 +490,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_sh
   for (int w = 0; w < kWarps; ++w) m = fmaxf(m, s_stat[w][0][r]);
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) {                               // a warp without keys has m = -inf: weight 0
-    f[w] = ex2(s_stat[w][0][r] - m);
+    f[w] = ex2(s_stat[w][0][r] - no_key_yet(m));
     lc += f[w] * s_stat[w][1][r]; la += f[w] * s_stat[w][2][r];
   }
   const float l = lc + la, inv = 1.0f / l;

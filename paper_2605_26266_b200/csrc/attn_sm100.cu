@@ -1020,6 +1020,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     while (ok && sch.next(sg)) {
       float m_run = -INFINITY, lcur = 0.f, lcac = 0.f;   // running max (log2 units), row sums over current / cached keys
       bool fresh = true;                                 // no product has been added to O in this segment yet
+      bool odd_max = true;                               // 64 channels: a maximum of the warp is -inf (no key yet) or very large
       for (int t = sg.tb; ok && t < sg.te; ++t, ++it) {
         const bool cached = t >= n_rt;
         const int n_valid = cached ? min(kBlockN, p.n_cached - (t - n_rt) * kBlockN) : min(kBlockN, p.n_cur - t * kBlockN);
@@ -1049,12 +1050,13 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           }
           const float m_new = fmaxf(m_run, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c_row);
           if (__any_sync(0xFFFFFFFFu, m_new - m_run > kGrowth)) {
+            if (D == 64) odd_max = __any_sync(0xFFFFFFFFu, !(fabsf(m_new) < 0x1p24f));
             if (!fresh) {
               // the product of the previous half (the last one issued on this O) must have retired
               ok = __all_sync(0xFFFFFFFFu, cx.wait(kODone + 2 * (hf ^ 1) + qt, (it - (hf ^ 1)) & 1, 302));
               if (!ok) break;
               tc_fence_after();
-              const float f = ex2(m_run - m_new);
+              const float f = ex2(m_run - (D == 64 ? no_key_yet(m_new) : m_new));
 #pragma unroll 1
               for (int c = 0; c < kNV / 16; ++c) {
                 uint32_t r[16];
@@ -1068,17 +1070,40 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
             m_run = m_new;
           }
-          const float2 c2 = make_float2(c_row, c_row), nm2 = make_float2(-m_run, -m_run);
           float2 sum2 = make_float2(0.f, 0.f);
           KVQ_STAMP(3);
+          if (D == 64 && odd_max) {
+            // Rows whose scores so far are -inf, or so large that an FMA's exact product and the rounded maximum differ by more
+            // than an exponential can take (a key masked with the lowest number): product and difference one by one, as in
+            // the warp-level kernel, which served heads of 64 channels before.  The scores are fetched once more, so that
+            // the loop below keeps its registers (16 heads x 1560 rows over 7 700 keys: 137 us without this, 141 as here, 146 with
+            // the scores changed in place).
+            const float m = no_key_yet(m_run);
+#pragma unroll 1
+            for (int c = 0; c < 64; c += 32) {
+              uint32_t r[32];
+              tmem_ld32(s_addr + 64 * hf + c, r);
+              tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 64; i += 2) {
-            const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2);
-            const float2 pr = ((i >> 1) & 3) < (PAIR ? kPolyPairs : 0) ? ex2_poly2(x) : make_float2(ex2(x.x), ex2(x.y));
-            sum2 = __fadd2_rn(sum2, pr);
-            sr[i >> 1] = cvt_bf16x2(pr.x, pr.y);
+              for (int i = 0; i < 32; i += 2) {
+                const float x0 = c + i < nv ? __uint_as_float(r[i]) : -INFINITY, x1 = c + i + 1 < nv ? __uint_as_float(r[i + 1]) : -INFINITY;
+                const float p0 = ex2(__fsub_rn(__fmul_rn(x0, c_row), m)), p1 = ex2(__fsub_rn(__fmul_rn(x1, c_row), m));
+                sum2.x += p0; sum2.y += p1;
+                r[i >> 1] = cvt_bf16x2(p0, p1);
+              }
+              tmem_st16(s_addr + 64 * hf + c / 2, r);
+            }
+          } else {
+            const float2 c2 = make_float2(c_row, c_row), nm2 = make_float2(-m_run, -m_run);
+#pragma unroll
+            for (int i = 0; i < 64; i += 2) {
+              const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2);
+              const float2 pr = ((i >> 1) & 3) < (PAIR ? kPolyPairs : 0) ? ex2_poly2(x) : make_float2(ex2(x.x), ex2(x.y));
+              sum2 = __fadd2_rn(sum2, pr);
+              sr[i >> 1] = cvt_bf16x2(pr.x, pr.y);
+            }
+            tmem_st32(s_addr + 64 * hf, sr);
           }
-          tmem_st32(s_addr + 64 * hf, sr);
           if (cached) lcac += sum2.x + sum2.y; else lcur += sum2.x + sum2.y;
           tmem_wait_st();
           tc_fence_before();
@@ -1106,7 +1131,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         tmem_wait_ld();
         norm = __uint_as_float(r[0]);
       }
-      const float inv = 1.0f / norm;
+      const float inv = D == 64 && !whole && norm == 0.f ? 0.f : 1.0f / norm;      // a range without a weight adds nothing
       const bool store = !whole || row < p.m_tokens;
       // consecutive 8-column pieces: 16 bytes apart in a row of the output, 4096 bytes apart in a slot
       uint8_t* dst = whole ? reinterpret_cast<uint8_t*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st)

@@ -143,6 +143,9 @@ __device__ __forceinline__ uint32_t f32_to_bf16_bits(float x) {
   return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
+// A running maximum as the subtrahend of the scores: 0 while all of them were -inf, whose weights are then 0 and not NaN.
+__device__ __forceinline__ float no_key_yet(float m) { return m == __int_as_float(0xFF800000) ? 0.f : m; }
+
 // The 16-bit forms of x^ = (code - zero) * step round once, as the FP32 form followed by one conversion does, while their
 // constants are exact.  Keys (FP16) and 2-bit values (BF16) subtract (OFF + zero) * step, OFF = 4 or 16, with an FMA: an
 // integer of 7 (4) bits times a step of 4 is exact in 11 (8), and with |OFF + zero| up to 112 no key reaches the largest
