@@ -569,17 +569,21 @@ __global__ void __launch_bounds__(kWarps * 32) attn_short_merge_kernel(const SPa
   }
 }
 
+int64_t resident_ctas() {
+  int sms = 0;
+  if (device_sm_count(&sms) != KVQ_OK) sms = 148;                  // sizes only: the launch itself fails loudly
+  return (int64_t)sms * kCtasPerSm;
+}
+
 // Units (batch*head, 16 rows) and into how many ranges the keys of each are cut: as many as let every CTA be resident at
 // once, but no range below 2 steps a warp, nor more than the merge can have in flight.
 struct Plan { int64_t q_blocks, units; int splits; };
 Plan plan(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {
-  int sms = 0;
-  if (device_sm_count(&sms) != KVQ_OK) sms = 148;                  // sizes only: the launch itself fails loudly
   Plan pl;
   pl.q_blocks = (m_tokens + kRows - 1) / kRows;
   pl.units = (int64_t)d->batch * d->heads * pl.q_blocks;
   const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
-  int64_t s = (int64_t)sms * kCtasPerSm / pl.units;
+  int64_t s = resident_ctas() / pl.units;
   if (s > steps / (2 * kWarps)) s = steps / (2 * kWarps);
   if (s > 128) s = 128;
   pl.splits = (int)(s < 1 ? 1 : s);
@@ -602,13 +606,17 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   if ((flags & KVQ_KERNEL_MASK) != KVQ_KERNEL_AUTO || (flags & KVQ_CORRECTION_EXACT) || (d->flags & KVQ_K_PER_CHANNEL) || m_tokens < 1)
     return false;
   // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
-  // prologue and a larger merge.  Measured (2 and 4 bits, 4 to 64 heads): one block of rows is 1.4 to 2 times as fast
-  // here; two are up to about 16 000 (head, 128-key tile) pairs (102 against 115 us at 6 464, 262 against 297 at 15 456, 485
-  // against 467 at 29 056); three and four only where those fixed costs weigh (33 against 47 us for three blocks at 892 pairs,
-  // 35 against 33 for four at 704, 117 against 78 at 3 520).
+  // prologue and a larger merge.  Measured with both kernels as they are, 2 to 1024 heads (us here against there, 128 channels, 2
+  // bits): one block of rows is 1 to 2 times as fast here.  Two are up to about 4 200 (head, 128-key tile) pairs (48 against 50
+  // at 2 080 of 32 heads, 4 bits 87 against 93 at 4 160 of 64; 149 against 142 at 8 224), three up to 1 200 (47 against 48 at 1 088),
+  // four up to 400 (22 against 28 at 130, 22 against 22 at 320, 34 against 28 at 544), as long as all CTAs run at once: 32 rows
+  // of 160 heads take 18 against 15 at 160 pairs, 242 against 179 at 10 400.  64 channels, where the other kernel has more fixed
+  // cost to each tile, stay ahead further: two blocks 69 against 73 at 4 160, 141 against 157 at 10 400 of 160 heads.
   const int64_t blocks = (m_tokens + kRows - 1) / kRows;
-  const int64_t pairs = (int64_t)d->batch * d->heads * ((cache_len + 127) / 128 + (n_cur + 127) / 128);
-  return blocks == 1 || (blocks == 2 && pairs <= 16384) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 600);
+  if (blocks == 1) return true;
+  const int64_t bh = (int64_t)d->batch * d->heads, pairs = bh * ((cache_len + 127) / 128 + (n_cur + 127) / 128);
+  if (d->head_dim == 64) return (blocks == 2 && pairs <= 16384) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 600);
+  return bh * blocks <= resident_ctas() && ((blocks == 2 && pairs <= 4200) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 400));
 }
 
 size_t attn_short_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {

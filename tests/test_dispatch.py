@@ -1,0 +1,36 @@
+"""Which kernel KVQ_KERNEL_AUTO plans for chunks of a few rows, read from the host-side size and launch-count queries (no GPU
+needed; on a machine without one they plan for 148 SMs)."""
+import ctypes as C
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2605_26266_b200 import build
+    build.build_library()
+    from paper_2605_26266_b200 import binding
+    return binding
+
+
+def plan(B, d, batch, heads, m, n_cur, n, flags):
+    desc = B.kvq_cache_desc(batch, heads, d, 2, 64, B.KVQ_ROTATE_K, 65536)
+    size, count = C.c_size_t(0), C.c_int(0)
+    assert B.lib.kvq_attn_workspace_bytes(C.byref(desc), n, m, n_cur, flags, C.byref(size)) == B.KVQ_OK
+    assert B.lib.kvq_attn_kernel_launches(C.byref(desc), n, m, n_cur, flags, C.byref(count)) == B.KVQ_OK
+    return size.value, count.value
+
+
+@pytest.mark.parametrize("batch,heads,m,n,few", [
+    (1, 32, 1, 16384, True), (1, 160, 16, 8192, True), (8, 128, 16, 2048, True),         # one block of rows: always
+    (1, 32, 32, 8000, True), (1, 64, 17, 2048, True), (1, 64, 48, 2048, True), (1, 8, 64, 2048, True), (1, 64, 64, 512, True),
+    # several blocks of many heads: more CTAs than run at once
+    (1, 160, 17, 0, False), (1, 160, 32, 8192, False), (4, 128, 32, 128, False), (4, 80, 48, 0, False), (8, 128, 64, 128, False),
+    # several blocks over long caches
+    (1, 32, 32, 32768, False), (1, 32, 48, 8192, False), (1, 32, 64, 2048, False), (1, 8, 65, 0, False),
+])
+def test_few_rows_take_their_kernel_where_it_is_faster(B, batch, heads, m, n, few):
+    auto = plan(B, 128, batch, heads, m, m, n, B.KVQ_CORRECTION_ON)
+    # the tcgen05 kernel that serves them otherwise: with a cache it has a pre-pass and room for the rotated queries
+    tcgen05 = plan(B, 128, batch, heads, m, m, n, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_TCGEN05)
+    assert (auto != tcgen05) if few else (auto == tcgen05)
