@@ -194,7 +194,11 @@ int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len,
  * cached_mass_out  optional device float [batch,heads,m_tokens]: P_S of Eq. (4), the softmax mass on
  *                  cached keys; NULL to skip.
  * workspace        device scratch of at least kvq_attn_workspace_bytes() bytes, 256-byte aligned;
- *                  may be NULL when that size is 0.  Contents need not be initialised.
+ *                  may be NULL when that size is 0.  Contents need not be initialised.  KVQ_KERNEL_AUTO has a
+ *                  slower kernel for a call whose workspace is missing, too small or not aligned where that kernel
+ *                  served such calls without one (heads of 64 channels, tensors TMA cannot address; unless KVQ_ROTATE_V),
+ *                  and for a few query rows the tcgen05 kernel if the workspace suits only that; otherwise it is refused
+ *                  (KVQ_ERR_WORKSPACE, KVQ_ERR_ALIGNMENT).
  * status_word      optional device int32, must be zero on entry: set to a non-zero diagnostic if a
  *                  bounded device-side wait expires (the output is then undefined); NULL to skip.
  * Errors: KVQ_ERR_INVALID_ARG, KVQ_ERR_UNSUPPORTED, KVQ_ERR_ALIGNMENT, KVQ_ERR_CAPACITY,

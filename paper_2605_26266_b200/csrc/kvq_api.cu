@@ -253,21 +253,23 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
     tc = false;
   }
   const size_t rotv = rotv_bytes(desc, cache_len, m_tokens, n_cur);
-  auto holds = [&](size_t need) {          // the call's workspace has room for `need` bytes
-    return need == 0 || (workspace && workspace_bytes >= need && reinterpret_cast<uintptr_t>(workspace) % 256 == 0);
-  };
+  const bool aligned = reinterpret_cast<uintptr_t>(workspace) % 256 == 0;
+  auto holds = [&](size_t need) { return need == 0 || (workspace && workspace_bytes >= need && aligned); };   // room for `need` bytes
   // A few query rows have a kernel of their own; a call whose workspace suits only the kernel that served it before that
   // one existed keeps it.
-  const bool few = attn_short_supports(desc, cache_len, m_tokens, n_cur, flags) &&
-                   holds(rotv + attn_short_workspace_bytes(desc, cache_len, m_tokens, n_cur));
+  const bool few_rows = attn_short_supports(desc, cache_len, m_tokens, n_cur, flags);
+  const size_t few_need = few_rows ? rotv + attn_short_workspace_bytes(desc, cache_len, m_tokens, n_cur) : 0;
+  const bool few = few_rows && holds(few_need);
   // The warp-level kernel, the only one for heads of 64 channels before the tcgen05 kernel took them, needs no workspace
-  // of its own: a call that brings none, or too little, keeps it.
+  // of its own: a call that brings none, too little, or one that is not aligned, keeps it.
   if (tc && desc->head_dim == 64 && !holds(rotv + attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, false))) tc = false;
   if (!few) {
     const size_t need = rotv + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : 0);
     if (need > 0) {
-      if (!workspace || workspace_bytes < need) return KVQ_ERR_WORKSPACE;
-      if (reinterpret_cast<uintptr_t>(workspace) % 256 != 0) return KVQ_ERR_ALIGNMENT;
+      if (!workspace) return KVQ_ERR_WORKSPACE;
+      // large enough for the kernel kvq_attn_workspace_bytes plans with, which only its alignment keeps from it
+      if (workspace_bytes < need) return few_rows && workspace_bytes >= few_need && !aligned ? KVQ_ERR_ALIGNMENT : KVQ_ERR_WORKSPACE;
+      if (!aligned) return KVQ_ERR_ALIGNMENT;
     }
   }
   if (m_tokens == 0) return KVQ_OK;

@@ -34,3 +34,20 @@ def test_few_rows_take_their_kernel_where_it_is_faster(B, batch, heads, m, n, fe
     # the tcgen05 kernel that serves them otherwise: with a cache it has a pre-pass and room for the rotated queries
     tcgen05 = plan(B, 128, batch, heads, m, m, n, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_TCGEN05)
     assert (auto != tcgen05) if few else (auto == tcgen05)
+
+
+@pytest.mark.parametrize("d,flags,offset,size,status", [
+    (128, 0, 16, 0, "KVQ_ERR_ALIGNMENT"), (128, 0, 128, 4096, "KVQ_ERR_ALIGNMENT"), (128, 0, 0, -1, "KVQ_ERR_WORKSPACE"),
+    (128, 0, 16, -1, "KVQ_ERR_WORKSPACE"), (128, 4, 16, 0, "KVQ_ERR_ALIGNMENT"), (64, 4, 16, 0, "KVQ_ERR_ALIGNMENT"),
+])
+def test_workspace_errors_of_a_few_rows(B, d, flags, offset, size, status):
+    """A workspace of the size asked for that is not 256-byte aligned is an alignment error, a smaller one a size error (`size`:
+    bytes beyond what kvq_attn_workspace_bytes asks for).  Refused on the host: the pointers are never used."""
+    m = n_cur = 16
+    desc = B.kvq_cache_desc(1, 2, d, 2, 64, B.KVQ_ROTATE_K | flags, 4096, *([1 << 20] * 6))
+    need = C.c_size_t(0)
+    assert B.lib.kvq_attn_workspace_bytes(C.byref(desc), 2000, m, n_cur, B.KVQ_CORRECTION_ON, C.byref(need)) == B.KVQ_OK
+    st = B.kvq_strides(2 * m * d, m * d, d)
+    r = B.lib.kvq_attn_corrected(C.byref(desc), 0, 2000, 1 << 20, st, 1 << 20, 1 << 20, st, m, n_cur, 1 << 20, st, 0.1,
+                                 B.KVQ_CORRECTION_ON, None, None, (1 << 20) + offset, need.value + size, None, None)
+    assert r == getattr(B, status)
