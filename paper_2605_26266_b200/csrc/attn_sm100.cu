@@ -1572,6 +1572,12 @@ static void schedule_shape(const kvq_cache_desc* d, int64_t cache_len, int64_t m
   *tiles = (n_cur + kBlockN - 1) / kBlockN + (cache_len + kBlockN - 1) / kBlockN;
 }
 
+bool attn_tcgen05_counts(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur) {
+  int64_t qb, nu, tiles;
+  schedule_shape(d, cache_len, m_tokens, n_cur, &qb, &nu, &tiles, false);
+  return nu * tiles <= 0x7FFFFFFFLL;
+}
+
 // Bytes of the rotated-query area of the workspace: q~ rows (2 * head_dim bytes each), then bias rows (16 bytes each),
 // rounded up to a multiple of 256.  Nothing when there are no cached keys.
 static size_t rot_area_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens) {

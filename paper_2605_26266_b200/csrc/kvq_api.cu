@@ -91,7 +91,7 @@ static size_t rotv_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   return ((size_t)d->batch * d->heads * (size_t)n_cur * d->head_dim * 2 + 255) / 256 * 256;
 }
 
-static bool use_tcgen05(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur, uint32_t flags, int* err) {
+static bool use_tcgen05(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, uint32_t flags, int* err) {
   const uint32_t kern = flags & KVQ_KERNEL_MASK;
   *err = KVQ_OK;
   if (kern == KVQ_KERNEL_MMA_SYNC) return false;
@@ -99,6 +99,9 @@ static bool use_tcgen05(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur
   const bool ok = attn_tcgen05_supports(d, m_tokens, n_cur) && !(flags & KVQ_CORRECTION_EXACT) && !(d->flags & KVQ_K_PER_CHANNEL);
   // heads of 64 channels: chosen by KVQ_KERNEL_AUTO only
   if ((kern == KVQ_KERNEL_TCGEN05 || kern == KVQ_KERNEL_TCGEN05_PAIR) && !(ok && d->head_dim == 128)) *err = KVQ_ERR_UNSUPPORTED;
+  // ... and not beyond the kernel's 2^31 tile steps, which for 128 channels is an error at the launch: the warp-level
+  // kernel, which served 64 channels before, has no such limit
+  if (d->head_dim == 64 && !attn_tcgen05_counts(d, cache_len, m_tokens, n_cur)) return false;
   return ok;
 }
 // Which tcgen05 kernel: the one asked for, else (KVQ_KERNEL_AUTO) the pair kernel unless its units of 512 query
@@ -207,7 +210,7 @@ int kvq_attn_workspace_bytes(const kvq_cache_desc* desc, int64_t cache_len, int6
   int r = check_attn_args(desc, 0, cache_len, m_tokens, n_cur, flags);
   if (r != KVQ_OK) return r;
   int err;
-  const bool tc = use_tcgen05(desc, m_tokens, n_cur, flags, &err);
+  const bool tc = use_tcgen05(desc, cache_len, m_tokens, n_cur, flags, &err);
   if (err != KVQ_OK) return err;
   if (attn_short_supports(desc, cache_len, m_tokens, n_cur, flags)) {
     *out_bytes = rotv_bytes(desc, cache_len, m_tokens, n_cur) + attn_short_workspace_bytes(desc, cache_len, m_tokens, n_cur);
@@ -223,7 +226,7 @@ int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len, int6
   int r = check_attn_args(desc, 0, cache_len, m_tokens, n_cur, flags);
   if (r != KVQ_OK) return r;
   int err;
-  const bool tc = use_tcgen05(desc, m_tokens, n_cur, flags, &err);
+  const bool tc = use_tcgen05(desc, cache_len, m_tokens, n_cur, flags, &err);
   if (err != KVQ_OK) return err;
   const bool few = attn_short_supports(desc, cache_len, m_tokens, n_cur, flags);
   *out_count = (few ? attn_short_kernel_launches(desc, cache_len, m_tokens, n_cur) : tc ? attn_tcgen05_kernel_launches(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : (m_tokens > 0 ? 1 : 0)) +
@@ -241,7 +244,7 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
                           out_bf16, o_strides, softmax_scale, flags);
   if (r != KVQ_OK) return r;
   int err;
-  bool tc = use_tcgen05(desc, m_tokens, n_cur, flags, &err);
+  bool tc = use_tcgen05(desc, cache_len, m_tokens, n_cur, flags, &err);
   if (err != KVQ_OK) return err;
   AttnArgs a = make_attn_args(desc, cache_begin, cache_len, q, q_strides, k_cur, v_cur, kv_strides, m_tokens, n_cur,
                               out_bf16, o_strides, softmax_scale, flags, lse_out, cached_mass_out, workspace,

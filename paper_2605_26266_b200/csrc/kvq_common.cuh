@@ -78,6 +78,8 @@ int launch_rotate_rows(const kvq_cache_desc* d, const void* src, kvq_strides ss,
                        int64_t tokens, bool inverse, cudaStream_t st);
 // tcgen05 kernel: returns KVQ_ERR_UNSUPPORTED for shapes it does not cover.
 bool attn_tcgen05_supports(const kvq_cache_desc* d, int64_t m_tokens, int64_t n_cur);
+// Do the problem's tile steps (one-CTA kernel) fit the kernel's 32-bit counts?
+bool attn_tcgen05_counts(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur);
 // Can TMA address the call's Q, K_cur, V_cur (no zero stride in a real dimension, byte strides below 2^40)?
 bool attn_tcgen05_addressable(const AttnArgs& a);
 // pair: the CTA-pair form of the kernel (KVQ_KERNEL_TCGEN05_PAIR), which plans 512-row units over SM pairs

@@ -51,3 +51,12 @@ def test_workspace_errors_of_a_few_rows(B, d, flags, offset, size, status):
     r = B.lib.kvq_attn_corrected(C.byref(desc), 0, 2000, 1 << 20, st, 1 << 20, 1 << 20, st, m, n_cur, 1 << 20, st, 0.1,
                                  B.KVQ_CORRECTION_ON, None, None, (1 << 20) + offset, need.value + size, None, None)
     assert r == getattr(B, status)
+
+
+def test_64_channels_beyond_the_counts_of_the_tcgen05_kernel(B):
+    """More than 2^31 tile steps: the warp-level kernel, without a workspace, as before 64 channels had another kernel."""
+    assert plan(B, 64, 1, 64, 1 << 20, 1 << 20, 65536, B.KVQ_CORRECTION_ON) == (0, 1)
+    assert plan(B, 64, 1, 64, 1 << 18, 1 << 18, 65536, B.KVQ_CORRECTION_ON)[0] > 0
+    desc, size = B.kvq_cache_desc(1, 64, 64, 2, 64, B.KVQ_ROTATE_K, 65536), C.c_size_t(0)
+    for m in (1 << 18, 1 << 20):
+        assert B.lib.kvq_attn_workspace_bytes(C.byref(desc), 65536, m, m, B.KVQ_KERNEL_TCGEN05, C.byref(size)) == B.KVQ_ERR_UNSUPPORTED
