@@ -119,11 +119,13 @@ def _strides(t: torch.Tensor) -> kvq_strides:
 
 
 # The current stream's handle without the Stream object around it: a small append is a few microseconds of Python around a
-# kernel of two, and the object alone was two of them.
-_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# kernel of two, and the object alone was two of them.  A torch that lacks the two functions gets the object.
+_raw_stream, _current_device = (getattr(torch._C, f, None) for f in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
 
 
 def _stream() -> int:
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_current_device())
 
 

@@ -115,3 +115,18 @@ def test_wait_budget_argument_and_status_word_mapping(binding):
     assert b.kvq_status_word_result(0) == b.KVQ_OK
     for word in (100, 204, 301, 404, -1):
         assert b.kvq_status_word_result(word) == b.KVQ_ERR_TIMEOUT
+
+
+def test_binding_imports_where_torch_lacks_the_raw_stream_functions(binding):
+    """A torch without CUDA has neither; the binding then asks the public Stream object."""
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "for f in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, f): delattr(torch._C, f)\n"
+            "from paper_2605_26266_b200 import binding\n"
+            "class S: cuda_stream = 7\n"
+            "torch.cuda.current_stream = lambda: S\n"
+            "assert binding._stream() == 7 and binding.kvq_version() == 1\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
