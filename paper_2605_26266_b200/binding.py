@@ -230,7 +230,11 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
     if need:
         ws = cache.workspace
         if ws is None or ws.numel() < need:
-            ws = cache.workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+            ws = torch.empty(need, dtype=torch.uint8, device=q.device)
+            # Heads of 64 channels had no workspace once, so that calls on one cache could run on several streams and threads:
+            # each call has its own, which the allocator hands out in stream order.
+            if cache.desc.head_dim != 64:
+                cache.workspace = ws
     status = _attn_corrected(
         desc, cache_begin, n_cache, q.data_ptr(), _strides_of(q.stride()), k_cur.data_ptr(), v_cur.data_ptr(),
         _strides_of(kv_st), m, n_cur, out.data_ptr(), _strides_of(out.stride()), float(softmax_scale), flags, _ptr(lse),

@@ -83,3 +83,26 @@ def test_head64_without_workspace_runs_the_warp_level_kernel():
         with pytest.raises(B.KvqError) as e:
             B.kvq_attn_corrected(g, q, kc, vc, sigma, forced, cache_begin=begin, cache_len=n)
         assert e.value.status == B.KVQ_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("m", [16, 256])
+def test_head64_calls_on_several_streams_share_nothing(m):
+    """Attention calls that only read one cache, on two streams at once: no workspace is kept on the cache, results are those of
+    calls one after the other."""
+    from paper_2605_26266_b200 import binding as B
+    w = inputs.Workload("streams", 760 + m, 1, 8, 64, 32, 0, 2, 64, 1)
+    g = B.Cache(1, 8, 64, 2, 64, 4096)
+    _, k, v = inputs.make_chunk(w, 0, tokens=4000)
+    B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(v))
+    chunks = [[T.to_dev(x) for x in inputs.make_chunk(w, 1 + i, tokens=m)] for i in range(2)]
+    want = [B.kvq_attn_corrected(g, *c, T.sigma_of(64)) for c in chunks]
+    assert g.workspace is None
+    torch.cuda.synchronize()
+    streams, got = [torch.cuda.Stream() for _ in chunks], [[], []]
+    for _ in range(50):
+        for i, c in enumerate(chunks):
+            with torch.cuda.stream(streams[i]):
+                got[i].append(B.kvq_attn_corrected(g, *c, T.sigma_of(64)))
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert all(torch.equal(o.view(torch.int16), want[i].view(torch.int16)) for o in got[i])
