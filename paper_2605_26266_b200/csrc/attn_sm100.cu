@@ -1353,12 +1353,18 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   // 16 bytes per partial, so the kernel lives on loads in flight.
   // CTA c of the schedule is CTA kc * c + rank of the grid; every CTA of the grid has two slots
   auto slot_of = [&](int c) { return p.partial + (size_t)(2 * (kc * c + rank) + (c == c_first ? first_slot : 0)) * kSlotBytes; };
+  // With fewer tile steps than CTAs (a last round of few units of few tiles) some ranges between the first and the last are
+  // empty: their CTAs left nothing, and whatever their slots hold is not this call's.
+  const long long split_steps = (long long)(p.n_units - p.n_whole) * T;
+  auto has_part = [&](int c) {
+    return c <= c_last && (split_steps >= n_ctas || split_steps * (c + 1) / n_ctas != split_steps * c / n_ctas);
+  };
   float m = -INFINITY;
   for (int c0 = c_first; c0 <= c_last; c0 += 4) {
     float mm[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      mm[j] = (c0 + j <= c_last) ? reinterpret_cast<const float*>(slot_of(c0 + j) + kSlotStats)[r256] : -INFINITY;
+      mm[j] = has_part(c0 + j) ? reinterpret_cast<const float*>(slot_of(c0 + j) + kSlotStats)[r256] : -INFINITY;
     m = fmaxf(fmaxf(m, fmaxf(mm[0], mm[1])), fmaxf(mm[2], mm[3]));
   }
   // out = sum_i w_i O_i / sum_i w_i with w_i = l_i 2^(m_i - m): every partial row is already normalised by its l_i
@@ -1369,7 +1375,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
     uint4 a[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const bool have = c0 + j <= c_last;
+      const bool have = has_part(c0 + j);
       const uint8_t* sl = slot_of(have ? c0 + j : c_last);
       const float* st = reinterpret_cast<const float*>(sl + kSlotStats);
       sm[j] = have ? st[r256] : -INFINITY;                  // weight 2^(-inf) = 0 for the slots that are not there
