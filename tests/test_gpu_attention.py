@@ -171,7 +171,7 @@ def test_rotation_off_window_scale_and_strides(B):
 
 
 def test_auto_dispatch_and_forced_kernel_errors(B):
-    # head_dim 128 -> tcgen05 kernel, head_dim 64 -> warp-level kernel; forcing tcgen05 on 64 is refused
+    # both head widths run through AUTO (140 rows: a tcgen05 kernel); forcing tcgen05 on 64 is refused
     for d in (64, 128):
         w = inputs.Workload("auto", 310 + d, 1, 2, d, 140, 0, 2, 64, 0)
         g, o, n, sel = _build(B, w, 2, tokens=90, cap=256)

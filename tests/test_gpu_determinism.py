@@ -74,3 +74,37 @@ def test_pair_ranges_that_start_in_the_cache_give_identical_bytes(bits, group):
         out = B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_TCGEN05_PAIR)
         first = out if first is None else first
         assert torch.equal(out.view(torch.int16), first.view(torch.int16)), f"launch {i}"
+
+
+@pytest.mark.parametrize("d,heads,rows,n,bits,kernel", [
+    (64, 2, 256, 1024, 2, "KVQ_KERNEL_AUTO"), (64, 16, 300, 3000, 4, "KVQ_KERNEL_AUTO"),      # tcgen05, every unit split
+    (64, 80, 300, 700, 2, "KVQ_KERNEL_AUTO"),                                                 # whole units
+    (64, 8, 16, 3000, 2, "KVQ_KERNEL_AUTO"), (128, 8, 16, 3000, 4, "KVQ_KERNEL_AUTO"), (128, 3, 30, 2000, 2, "KVQ_KERNEL_AUTO"),   # a few rows, split
+    (128, 8, 48, 3000, 2, "KVQ_KERNEL_TCGEN05"), (128, 8, 128, 3000, 4, "KVQ_KERNEL_TCGEN05"),   # one query tile
+])
+def test_overlapping_kernels_on_a_poisoned_workspace(d, heads, rows, n, bits, kernel):
+    """The kernels of a call overlap: one that read what the one before it has not written yet would find NaN (the workspace is
+    filled with it before each call) or the other problem's data (two problems in turn, back to back on one workspace)."""
+    from paper_2605_26266_b200 import binding as B
+    w = inputs.Workload("overlap", 880 + d + rows, 1, heads, d, 32, 0, bits, 32, 1, k_outliers=2, k_outlier_scale=4.0)
+    cache = B.Cache(1, heads, d, bits, 32, 4096)
+    _, k, v = inputs.make_chunk(w, 0, tokens=n)
+    B.kvq_quantize_append(cache, T.to_dev(k), T.to_dev(v))
+    flags, sigma = B.KVQ_CORRECTION_ON | getattr(B, kernel), 1.0 / math.sqrt(d)
+    chunks = [[T.to_dev(x) for x in inputs.make_chunk(w, 1 + i, tokens=rows)] for i in range(2)]
+    cache.workspace = torch.empty(B.kvq_attn_workspace_bytes(cache, n, rows, rows, flags), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def call(i):
+        lse = torch.empty(1, heads, rows, dtype=torch.float32, device="cuda")
+        return B.kvq_attn_corrected(cache, *chunks[i], sigma, flags, lse=lse, status_word=status), lse
+
+    first, got = [call(0), call(1)], []
+    for _ in range(40):
+        cache.workspace.fill_(0xFF)
+        got.append((0, call(0)))
+        got.append((1, call(1)))                             # straight behind, on the other's leftovers
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.isfinite(first[0][0].float()).all()
+    for i, (out, lse) in got:
+        assert torch.equal(out.view(torch.int16), first[i][0].view(torch.int16)) and torch.equal(lse, first[i][1])

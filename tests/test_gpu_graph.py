@@ -60,3 +60,33 @@ def test_step_replayed_from_a_graph_equals_the_eager_step(heads, tokens, kernel)
     assert torch.equal(out_g.view(torch.int16), out_e.view(torch.int16))
     for a, b in zip(cache.buffers, eager.buffers):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+
+
+@pytest.mark.parametrize("d,heads,tokens", [(64, 4, 300), (64, 8, 16), (128, 8, 16)])
+def test_auto_kernels_replayed_from_a_graph(d, heads, tokens):
+    """The kernels KVQ_KERNEL_AUTO takes for 64 channels and for a few rows; their kernels of one call overlap in the graph too."""
+    from paper_2605_26266_b200 import binding as B
+    w = inputs.Workload("graph", 870 + d + tokens, 1, heads, d, 32, 0, 2, 64, 1)
+    cache = B.Cache(1, heads, d, 2, 64, 4096)
+    _, k, v = inputs.make_chunk(w, 0, tokens=3000)
+    B.kvq_quantize_append(cache, T.to_dev(k), T.to_dev(v))
+    q, k, v = (T.to_dev(x) for x in inputs.make_chunk(w, 1, tokens=tokens))
+    flags, sigma = B.KVQ_CORRECTION_ON, 1.0 / math.sqrt(d)
+    assert B.kvq_attn_kernel_launches(cache, 3000, tokens, tokens, flags) >= 2
+    cache.workspace = torch.empty(B.kvq_attn_workspace_bytes(cache, 3000, tokens, tokens, flags), dtype=torch.uint8, device="cuda")
+    want = B.kvq_attn_corrected(cache, q, k, v, sigma, flags)
+    out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            B.kvq_attn_corrected(cache, q, k, v, sigma, flags, out=out)
+            B.kvq_attn_corrected(cache, out, k, v, sigma, flags, out=out)      # the next call of the step, in place
+    torch.cuda.synchronize()
+    again = B.kvq_attn_corrected(cache, want, k, v, sigma, flags)
+    for _ in range(3):
+        out.zero_()
+        cache.workspace.fill_(0xFF)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16))

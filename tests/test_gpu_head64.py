@@ -106,3 +106,22 @@ def test_head64_calls_on_several_streams_share_nothing(m):
     torch.cuda.synchronize()
     for i in range(2):
         assert all(torch.equal(o.view(torch.int16), want[i].view(torch.int16)) for o in got[i])
+
+
+@pytest.mark.parametrize("m", [16, 200])
+def test_head64_token_interleaved(m):
+    """[batch, tokens, heads, head_dim] storage of inputs and output."""
+    from paper_2605_26266_b200 import binding as B
+    w = inputs.Workload("inter", 770 + m, 2, 3, 64, 32, 0, 2, 32, 1)
+    g, o = (X.Cache(2, 3, 64, 2, 32, 1024) for X in (B, O))
+    _, k, v = inputs.make_chunk(w, 0, tokens=900)
+    B.kvq_quantize_append(g, *(T.to_dev(x).permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for x in (k, v)))
+    O.quantize_append(o, 0, k, v)
+    T.assert_cache_equal(T.gpu_cache_arrays(g, 900), o, 900)
+    q, k, v = inputs.make_chunk(w, 1, tokens=m)
+    qd, kd, vd = (T.to_dev(x).permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for x in (q, k, v))
+    out = torch.empty_like(qd)
+    assert not out.is_contiguous()
+    B.kvq_attn_corrected(g, qd, kd, vd, T.sigma_of(64), out=out)
+    want = O.attn_corrected(o, 0, 900, q, k, v, T.sigma_of(64), correction=True)["out"]
+    T.assert_attn_close(T.from_dev_bf16(out).reshape(want.shape), want)

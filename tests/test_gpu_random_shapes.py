@@ -1,6 +1,6 @@
 """Seeded random shapes: small problems with lengths that hit every tile boundary case (1 row, 1 key, exact
-multiples, one past a multiple), random formats, windows, rotation flags and ring wrap, both kernels against
-the oracle.  Sizes stay small so that the oracle runs all rows."""
+multiples, one past a multiple), random formats, windows, rotation flags and ring wrap, the forced kernels and the one
+KVQ_KERNEL_AUTO takes (64 channels: the tcgen05 kernel, a few rows: theirs) against the oracle.  Sizes stay small so that the oracle runs all rows."""
 import numpy as np
 import pytest
 import torch
@@ -54,7 +54,7 @@ def test_random_shape(c):
     begin = start + c["begin"]
     want = O.attn_corrected(o, begin, c["n_cached"], q, kc, vc, sigma, correction=c["corr"])
     flag = B.KVQ_CORRECTION_ON if c["corr"] else B.KVQ_CORRECTION_OFF
-    for kname, kflag in [("mma_sync", B.KVQ_KERNEL_MMA_SYNC)] + ([("tcgen05", B.KVQ_KERNEL_TCGEN05), ("tcgen05_pair", B.KVQ_KERNEL_TCGEN05_PAIR)] if d == 128 else []):
+    for kname, kflag in [("mma_sync", B.KVQ_KERNEL_MMA_SYNC), ("auto", B.KVQ_KERNEL_AUTO)] + ([("tcgen05", B.KVQ_KERNEL_TCGEN05), ("tcgen05_pair", B.KVQ_KERNEL_TCGEN05_PAIR)] if d == 128 else []):
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
         lse = torch.zeros(q.shape[:3], dtype=torch.float32, device="cuda")
         mass = torch.zeros_like(lse)

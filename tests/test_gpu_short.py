@@ -1,6 +1,7 @@
 """Chunks of a few query rows (the kernel KVQ_KERNEL_AUTO takes for them): edges of its row blocks and key steps, splits that
 leave a single step or end in the current chunk, every format, ring windows that wrap inside a step, rotated values, shared
-(stride 0) chunks, against the oracle; and the kernels that served such calls before where the workspace is sized for them."""
+(stride 0) and token-interleaved chunks, against the oracle; and the kernels that served such calls before where the
+workspace is sized for them, or missing."""
 import ctypes as C
 
 import numpy as np
@@ -96,3 +97,51 @@ def test_short_chunk_with_a_smaller_workspace_or_shared_heads():
     want = O.attn_corrected(o, begin, n, q, np.repeat(kc[:, :1], 2, 1), np.repeat(vc[:, :1], 2, 1), sigma)["out"]
     got = B.kvq_attn_corrected(g, dq, shared_k, shared_v, sigma, cache_begin=begin, cache_len=n)
     T.assert_attn_close(T.from_dev_bf16(got).reshape(want.shape), want)
+
+
+@pytest.mark.parametrize("heads,n,opt", [(2, 1000, {}), (140, 2000, {}), (2, 1000, dict(rotate_v=True))])
+def test_workspace_that_suits_only_the_former_kernel(heads, n, opt):
+    """Few keys or many heads: the tcgen05 kernel needs less room than the splits of the few-row kernel.  A call that brings just
+    that gets that kernel's bytes, and nothing behind the workspace is touched."""
+    from paper_2605_26266_b200 import binding as B
+    g, o, begin, n, q, kc, vc = problem(B, (128, 2, 64, 1, heads, 16, 16, n, opt), 21)
+    sigma, flags = T.sigma_of(128), B.KVQ_CORRECTION_ON
+    need, former = (B.kvq_attn_workspace_bytes(g, n, 16, 16, f) for f in (flags, flags | B.KVQ_KERNEL_TCGEN05))
+    assert 0 < former < need
+    dq, dk, dv = T.to_dev(q), T.to_dev(kc), T.to_dev(vc)
+    want = B.kvq_attn_corrected(g, dq, dk, dv, sigma, flags | B.KVQ_KERNEL_TCGEN05, cache_begin=begin, cache_len=n)
+    ws, out, st = torch.full((need,), 0xA5, dtype=torch.uint8, device="cuda"), torch.empty_like(dq), B._strides
+    r = B.lib.kvq_attn_corrected(C.byref(g.desc), begin, n, dq.data_ptr(), st(dq), dk.data_ptr(), dv.data_ptr(), st(dk), 16, 16,
+                                 out.data_ptr(), st(out), sigma, flags, None, None, ws.data_ptr(), former, None, B._stream())
+    torch.cuda.synchronize()
+    assert r == B.KVQ_OK and torch.equal(out.view(torch.int16), want.view(torch.int16)) and bool((ws[former:] == 0xA5).all())
+    few = B.kvq_attn_corrected(g, dq, dk, dv, sigma, flags, cache_begin=begin, cache_len=n)
+    assert not torch.equal(few.view(torch.int16), want.view(torch.int16))                  # another kernel, with the room it asks for
+    if heads == 2:
+        T.assert_attn_close(T.from_dev_bf16(few).reshape(1, 2, 16, 128), O.attn_corrected(o, begin, n, q, kc, vc, sigma)["out"].reshape(1, 2, 16, 128))
+
+
+def test_64_channels_without_workspace_keep_the_warp_level_kernel():
+    from paper_2605_26266_b200 import binding as B
+    g, _, begin, n, q, kc, vc = problem(B, (64, 2, 64, 1, 2, 16, 16, 2000, {}), 22)
+    dq, dk, dv = T.to_dev(q), T.to_dev(kc), T.to_dev(vc)
+    sigma, st, out = T.sigma_of(64), B._strides, torch.empty_like(dq)
+    want = B.kvq_attn_corrected(g, dq, dk, dv, sigma, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_MMA_SYNC, cache_begin=begin, cache_len=n)
+    ws = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    for ptr, size in ((None, 0), (ws.data_ptr(), 256), (ws.data_ptr() + 16, 1 << 19)):       # none, too small, not aligned
+        out.zero_()
+        r = B.lib.kvq_attn_corrected(C.byref(g.desc), begin, n, dq.data_ptr(), st(dq), dk.data_ptr(), dv.data_ptr(), st(dk), 16, 16,
+                                     out.data_ptr(), st(out), sigma, B.KVQ_CORRECTION_ON, None, None, ptr, size, None, B._stream())
+        torch.cuda.synchronize()
+        assert r == B.KVQ_OK and torch.equal(out.view(torch.int16), want.view(torch.int16))
+
+
+def test_short_chunk_token_interleaved():
+    from paper_2605_26266_b200 import binding as B
+    g, o, begin, n, q, kc, vc = problem(B, (128, 4, 32, 2, 3, 20, 20, 700, dict(signs=True)), 23)
+    qd, kd, vd = (T.to_dev(x).permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for x in (q, kc, vc))
+    out = torch.empty_like(qd)
+    assert not out.is_contiguous()
+    B.kvq_attn_corrected(g, qd, kd, vd, T.sigma_of(128), cache_begin=begin, cache_len=n, out=out)
+    want = O.attn_corrected(o, begin, n, q, kc, vc, T.sigma_of(128))["out"]
+    T.assert_attn_close(T.from_dev_bf16(out).reshape(want.shape), want)

@@ -49,3 +49,37 @@ def test_expired_wait_sets_the_status_word_and_the_kernel_returns(kernel):
     want = O.attn_corrected(o, 0, n, q, k, v, sigma, correction=True)
     T.assert_attn_close(T.from_dev_bf16(out), want["out"], "after a timed-out call")
 
+
+
+@pytest.mark.parametrize("d,rows,kernel", [(64, 256, "KVQ_KERNEL_AUTO"), (64, 100, "KVQ_KERNEL_AUTO"), (128, 100, "KVQ_KERNEL_TCGEN05")])
+def test_expired_wait_of_the_64_channel_and_one_tile_forms(d, rows, kernel):
+    """The same for heads of 64 channels (chosen by AUTO only) and for one query tile in use (up to 128 rows).  Units of 10 tiles
+    dealt out whole; a first poll can be long enough for every wait of a launch, so the call is repeated until one expires."""
+    from paper_2605_26266_b200 import binding as B
+    heads, picked = 148, [0, 71, 147]
+    w = inputs.Workload("timeout", 92, 1, heads, d, 512, 2, 2, 64, 3)
+    g, o = B.Cache(1, heads, d, 2, 64, w.capacity), O.Cache(1, len(picked), d, 2, 64, w.capacity)
+    n = 0
+    for c in range(2):
+        _, k, v = inputs.make_chunk(w, c)
+        B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(v))
+        n = O.quantize_append(o, n, k[:, picked], v[:, picked])
+    q, k, v = inputs.make_chunk(w, 2, tokens=rows)
+    args = (g, T.to_dev(q), T.to_dev(k), T.to_dev(v), T.sigma_of(d), B.KVQ_CORRECTION_ON | getattr(B, kernel))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    try:
+        B.kvq_set_wait_budget_cycles(2)
+        for _ in range(50):
+            B.kvq_attn_corrected(*args, cache_len=n, status_word=status)
+            torch.cuda.synchronize()
+            if int(status.item()):
+                break
+    finally:
+        B.kvq_set_wait_budget_cycles(0)
+    assert int(status.item()) in SITE_CODES
+    status.zero_()
+    out = B.kvq_attn_corrected(*args, cache_len=n, status_word=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    want = O.attn_corrected(o, 0, n, q[:, picked], k[:, picked], v[:, picked], T.sigma_of(d), correction=True)["out"]
+    T.assert_attn_close(T.from_dev_bf16(out)[0][picked], want)
