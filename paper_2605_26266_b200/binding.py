@@ -152,6 +152,21 @@ class Cache:
             self.desc.signs = self.signs.data_ptr()
         self.length = 0
         self.workspace = None
+        self._stream_workspaces = {}
+
+    def _stream_workspace(self, need, stream, device):
+        """Heads of 64 channels had no workspace once, so that calls which only read one cache could run on several streams
+        and threads: a buffer for each stream (at most eight are kept), a fresh one for a call that is being captured."""
+        capturing = torch.cuda.is_current_stream_capturing()
+        kept = self._stream_workspaces
+        ws = None if capturing else kept.get(stream)
+        if ws is None or ws.numel() < need:
+            ws = torch.empty(need, dtype=torch.uint8, device=device)
+            if not capturing:
+                if stream not in kept and len(kept) >= 8:
+                    kept.pop(list(kept)[0], None)
+                kept[stream] = ws
+        return ws
 
     @property
     def groups(self):
@@ -226,19 +241,18 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
     status = _attn_workspace_bytes(desc, n_cache, m, n_cur, flags, C.byref(size))
     if status:
         _check(status, "kvq_attn_workspace_bytes")
-    need, ws = size.value, None
+    need, ws, stream = size.value, None, _stream()
     if need:
         ws = cache.workspace
         if ws is None or ws.numel() < need:
-            ws = torch.empty(need, dtype=torch.uint8, device=q.device)
-            # Heads of 64 channels had no workspace once, so that calls on one cache could run on several streams and threads:
-            # each call has its own, which the allocator hands out in stream order.
-            if cache.desc.head_dim != 64:
-                cache.workspace = ws
+            if cache.desc.head_dim == 64:
+                ws = cache._stream_workspace(need, stream, q.device)
+            else:
+                ws = cache.workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
     status = _attn_corrected(
         desc, cache_begin, n_cache, q.data_ptr(), _strides_of(q.stride()), k_cur.data_ptr(), v_cur.data_ptr(),
         _strides_of(kv_st), m, n_cur, out.data_ptr(), _strides_of(out.stride()), float(softmax_scale), flags, _ptr(lse),
-        _ptr(cached_mass), _ptr(ws), ws.numel() if need else 0, _ptr(status_word), _stream())
+        _ptr(cached_mass), _ptr(ws), ws.numel() if need else 0, _ptr(status_word), stream)
     if status:
         _check(status, "kvq_attn_corrected")
     return out

@@ -87,8 +87,8 @@ def test_head64_without_workspace_runs_the_warp_level_kernel():
 
 @pytest.mark.parametrize("m", [16, 256])
 def test_head64_calls_on_several_streams_share_nothing(m):
-    """Attention calls that only read one cache, on two streams at once: no workspace is kept on the cache, results are those of
-    calls one after the other."""
+    """Attention calls that only read one cache, on two streams at once: each stream has its workspace, results are those of
+    calls one after the other.  More streams than buffers are kept; a captured call keeps none."""
     from paper_2605_26266_b200 import binding as B
     w = inputs.Workload("streams", 760 + m, 1, 8, 64, 32, 0, 2, 64, 1)
     g = B.Cache(1, 8, 64, 2, 64, 4096)
@@ -106,6 +106,21 @@ def test_head64_calls_on_several_streams_share_nothing(m):
     torch.cuda.synchronize()
     for i in range(2):
         assert all(torch.equal(o.view(torch.int16), want[i].view(torch.int16)) for o in got[i])
+    kept = g._stream_workspaces
+    assert len({w.data_ptr() for w in kept.values()}) == len(kept) == 3
+    more = [torch.cuda.Stream() for _ in range(12)]
+    for st in more:
+        with torch.cuda.stream(st):
+            got[0].append(B.kvq_attn_corrected(g, *chunks[0], T.sigma_of(64)))
+    before = list(kept)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=more[-1]):
+        got[1].append(B.kvq_attn_corrected(g, *chunks[1], T.sigma_of(64)))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert len(kept) == 8 and list(kept) == before
+    for i in range(2):
+        assert torch.equal(got[i][-1].view(torch.int16), want[i].view(torch.int16))
 
 
 @pytest.mark.parametrize("m", [16, 200])
