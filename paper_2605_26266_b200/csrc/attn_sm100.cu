@@ -1295,7 +1295,12 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   __syncthreads();
   // A pair leaves together: neither CTA's shared memory or TMEM may go while the other still arrives on its
   // barriers or the leader's MMAs still read its operands (every role above has come out through bounded waits).
-  if constexpr (PAIR) cluster_sync_all();
+  // The leader's commits arrive on the peer's barriers too, asynchronously: the peer waits for its copy of the last ones, or they
+  // could land in the shared memory of a CTA that has left.
+  if constexpr (PAIR) {
+    if (rank != 0 && (warp == 1 || warp == 2)) cx.drain(kDrain + warp - 1, 0);
+    cluster_sync_all();
+  }
   wait_for_previous_grid();                      // also in a CTA that had no cached tile
   if (warp == 0) {
     tc_fence_after();

@@ -27,3 +27,13 @@ def test_workspace_is_not_read_through_the_read_only_path(name, pointers):
     assert "wait_for_previous_grid()" in text and all(p in text for p in pointers[:1])
     bad = [a for a in ldg_arguments(text) if any(re.search(rf"\b{p}\b", a) for p in pointers)]
     assert not bad, bad
+
+
+def test_both_ctas_of_a_pair_wait_for_the_last_commits():
+    """Commits of a pair (tc_commit_pair) arrive on the barriers of both CTAs at times of their own.  The leader drains its copy of
+    the last ones; the peer has to drain its own before the cluster barrier that lets it leave."""
+    with open(os.path.join(CSRC, "attn_sm100.cu")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    end = text[text.rindex("++nseg;"):text.index("tmem_dealloc_pair(tmem")]
+    assert re.search(r"rank != 0 && [^;]*cx\.drain\(kDrain \+ warp - 1, 0\);\s*cluster_sync_all\(\);", end)
+    assert re.search(r"commit\(kDrain \+ qt\);\s*cx\.drain\(kDrain \+ qt, 0\);", text)
