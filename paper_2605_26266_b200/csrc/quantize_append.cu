@@ -2,19 +2,20 @@
 // quantization (Eq. (1)), bit packing and coalesced append of one finished chunk's K and V.
 //
 // Four lanes own one token-head vector (lane lv holds channels [lv*EPL, (lv+1)*EPL), EPL = head_dim/4), so a warp
-// works on eight consecutive tokens, each warp by itself: a lane's codes fill a whole store (16 to 128 bits), the stores
+// works on eight consecutive tokens, each warp by itself: a lane's codes fill a whole store (32 to 128 bits), the stores
 // of a warp are contiguous, and nothing is staged in shared memory.  The Walsh-Hadamard butterfly runs its first
 // log2(EPL) stages inside a lane and the remaining two across lanes with shuffles; group minimum/maximum are shuffle
 // reductions over the lanes of a group.  Every add, subtract, multiply and divide is a single IEEE binary32 operation
 // (no contraction), so the stored codes, steps and zero-points are reproducible bit for bit.
 //
-// By its bytes the kernel would be HBM-bound on its BF16 input; in fact it is bound by instruction issue, because the
-// bit-exact contract fixes the operations.  A lane therefore keeps its values as pairs (channel i, channel i + EPL/2) in
+// By its bytes the kernel would be HBM-bound on its BF16 input.  It was bound by instruction issue, because the
+// bit-exact contract fixes the operations; with half the instructions (0.54 issued a cycle) its warps wait for their loads
+// and their own chains.  A lane keeps its values as pairs (channel i, channel i + EPL/2) in
 // the two halves of 64-bit registers and does everything but the last in-lane butterfly stage and the minimum/maximum
 // with the packed instructions (add/mul/fma.rn.f32x2: two IEEE operations each), and adds the zero-point, clamps and packs
 // the codes two at a time as 16-bit integers.  Measured at 24 heads x 4680 tokens, 128 channels, 2 bits, group 64
-// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 22.5 us as here with
-// eight lanes per vector (shorter lanes repeat the per-group work more often), 21.8 us with four (3.0 TB/s); two
+// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 23.6 us as here (2.8 TB/s),
+// 3 % more with eight lanes per vector (shorter lanes repeat the per-group work more often); two
 // tokens in flight per lane and persistent warps with a prefetch: 26.6 us (fewer warps fit).
 #include <math_constants.h>
 
@@ -79,9 +80,9 @@ __device__ __forceinline__ void hadamard(Pairs<EPL>& x, int lv, float c_d) {
   for (int i = 0; i < HP; ++i) x.v[i] = __fmul2_rn(x.v[i], make_float2(c_d, c_d));
 }
 
-// What a lane stores for its vector: its codes (32 to 128 bits, 16 at the least) and its group's step and zero-point.
+// What a lane stores for its vector: its codes (32 to 128 bits) and its group's step and zero-point.
 template <int EPL, int BITS>
-struct Quantized { uint32_t w[EPL * BITS > 32 ? EPL * BITS / 32 : 1]; uint32_t sbyte, zbits; };
+struct Quantized { uint32_t w[EPL * BITS / 32]; uint32_t sbyte, zbits; };
 
 // Quantizes the vector held by kLanes lanes.  The per-group work (range, step, zero-point) is shared by the GROUP/EPL
 // lanes of a group.
@@ -178,8 +179,8 @@ __device__ __forceinline__ Quantized<EPL, BITS> quantize(const Pairs<EPL>& x) {
       acc[k] |= (code(x.v[i].x) | (code(x.v[i].y) << 16)) << pos;
     }
   }
-  if constexpr (F * BITS == 8) out.w[0] = (acc[0] | (acc[0] >> 8)) & 0xFFFFu;
-  else if constexpr (kAcc == 1) out.w[0] = acc[0];
+  static_assert(F * BITS == 16, "full fields");
+  if constexpr (kAcc == 1) out.w[0] = acc[0];
   else {
 #pragma unroll
     for (int k = 0; k < kAcc; k += 2) {            // low fields: the first half of the lane's channels
@@ -264,8 +265,7 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) quantize_append_kerne
     const Quantized<EPL, BITS> q = quantize<EPL, BITS, GROUP>(x);
     if (valid) {
       uint8_t* dst = p.codes[w] + at * CB + lv * (EPL * BITS / 8);
-      if constexpr (EPL * BITS == 16) *reinterpret_cast<uint16_t*>(dst) = (uint16_t)q.w[0];
-      else if constexpr (EPL * BITS == 32) *reinterpret_cast<uint32_t*>(dst) = q.w[0];
+      if constexpr (EPL * BITS == 32) *reinterpret_cast<uint32_t*>(dst) = q.w[0];
       else if constexpr (EPL * BITS == 64) *reinterpret_cast<uint2*>(dst) = make_uint2(q.w[0], q.w[1]);
       else *reinterpret_cast<uint4*>(dst) = make_uint4(q.w[0], q.w[1], q.w[2], q.w[3]);
       if ((lv % lanes_per_group) == 0) {
