@@ -149,7 +149,8 @@ int kvq_quantize_append(const kvq_cache_desc* desc, int64_t cache_len,
                         int64_t n_tokens, kvq_stream_t stream);
 
 /*
- * Bytes of device workspace kvq_attn_corrected needs for this problem (may be 0).  With the tcgen05 kernel
+ * Bytes of device workspace kvq_attn_corrected needs for this problem (may be 0).  For a few query rows
+ * (KVQ_KERNEL_AUTO) it holds the FP32 partial rows of the splits.  With the tcgen05 kernel
  * and a non-empty cache window it holds the rotated query chunk (Section 3.1: q~ = H q in FP16, plus the
  * per-group squared norms nu of Eq. 15, 2 * head_dim + 16 bytes per query row, written by a pre-pass kernel of the same
  * call) and, when the key tiles of a unit are split over several CTAs, their partial results.
@@ -161,7 +162,9 @@ int kvq_attn_workspace_bytes(const kvq_cache_desc* desc, int64_t cache_len,
 /*
  * How many kernels one kvq_attn_corrected call launches for this problem (host-side bookkeeping for
  * benchmarks and launch-bound callers): the attention kernel, the query pre-pass when the cache window
- * is not empty, the merge kernel when units are split over CTAs.  out_count is host memory.  Same
+ * is not empty (not for a few query rows, which have none), the merge kernel when units are split over CTAs.
+ * It counts for a call with the workspace kvq_attn_workspace_bytes asks for and tensors TMA can address: one
+ * that falls back to another kernel for want of either launches that kernel's.  out_count is host memory.  Same
  * argument checks and errors as kvq_attn_workspace_bytes.
  */
 int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len,
@@ -184,8 +187,8 @@ int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len,
  * q: [batch,heads,m_tokens,head_dim] strides q_strides; k_cur, v_cur: [batch,heads,n_cur,head_dim]
  * strides kv_strides; out: strides o_strides.  All device BF16, 16-byte aligned, strides
  * multiples of 8 elements.  A batch or head stride of 0 (a chunk shared by all heads) is accepted: the tcgen05
- * kernel cannot address such a tensor, so KVQ_KERNEL_AUTO runs the warp-level kernel for it and a forced
- * KVQ_KERNEL_TCGEN05 returns KVQ_ERR_UNSUPPORTED.  cache_begin must be a multiple of 16 and
+ * kernel cannot address such a tensor, so KVQ_KERNEL_AUTO runs the warp-level kernel for it (a few query rows: their
+ * own kernel) and a forced KVQ_KERNEL_TCGEN05 returns KVQ_ERR_UNSUPPORTED.  cache_begin must be a multiple of 16 and
  * cache_begin + cache_len <= capacity.  cache_len == 0 is legal (plain attention over the
  * current chunk); n_cur must be >= 1; m_tokens == 0 is a no-op.
  *

@@ -16,8 +16,8 @@
 //
 // What bounds it: instruction issue and latency (37 warp instructions per key and 16 rows at 4 bits, half of them the
 // expansion of the codes; two CTAs of four warps an SM, the ALU pipe half busy), then HBM.  16 rows over 16 384 tokens
-// of 32 heads at 4 bits, group 128: 42 us with the merge, against 87 us in the tcgen05 kernel; three CTAs with spilled
-// registers 47 us, four 76 us; the four score tiles of a step one after the other instead of in turn 45 us.
+// of 32 heads at 4 bits, group 128: 45 us with the merge, against 97 us in the tcgen05 kernel; three CTAs with spilled
+// registers 12 % slower, four 80 %; the four score tiles of a step one after the other instead of in turn 7 %.
 #include <cuda_fp16.h>
 
 #include <type_traits>
