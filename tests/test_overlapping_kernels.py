@@ -35,5 +35,6 @@ def test_both_ctas_of_a_pair_wait_for_the_last_commits():
     with open(os.path.join(CSRC, "attn_sm100.cu")) as f:
         text = re.sub(r"//[^\n]*", "", f.read())
     end = text[text.rindex("++nseg;"):text.index("tmem_dealloc_pair(tmem")]
-    assert re.search(r"rank != 0 && [^;]*cx\.drain\(kDrain \+ warp - 1, 0\);\s*cluster_sync_all\(\);", end)
+    # two warps of the peer's dequantizing role (warps 12 to 15), then the barrier
+    assert re.search(r"rank != 0 && warp < 14\) cx\.drain\(kDrain \+ warp - 12, 0\);.*cluster_sync_all\(\);", end, re.S)
     assert re.search(r"commit\(kDrain \+ qt\);\s*cx\.drain\(kDrain \+ qt, 0\);", text)
