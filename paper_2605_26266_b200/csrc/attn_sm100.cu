@@ -46,7 +46,7 @@
 // The same source also gives the pair kernel (template parameter PAIR): a cluster of two CTAs on 512 query rows
 // whose tensor cores work as one (tcgen05 cta_group::2), described at the kernel; and the kernel for heads of 64
 // channels (D = 64, one CTA per unit): operand tiles one 64-column block wide at the same places, half the MMA steps of a
-// score, 16 heads x 1560 queries over 7 700 keys in 141 us against 650 us in the warp-level kernel.
+// score, 16 heads x 1560 queries over 7 700 keys in 134 us against 650 us in the warp-level kernel.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA records a diagnostic in the caller's status
 // word, all roles leave their loops, in-flight work is drained with a bounded wait, TMEM is freed and the
@@ -248,6 +248,13 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
   q = __ffma2_rn(q, r, make_float2(0.9999280571937561f, 0.9999280571937561f));
   return make_float2(__uint_as_float(__float_as_uint(q.x) + (__float_as_uint(fl.x) << 23)),
                      __uint_as_float(__float_as_uint(q.y) + (__float_as_uint(fl.y) << 23)));
+}
+// A pair of floats as two BF16 pairs: the high parts (cut, not rounded) are returned, `lo` is what they leave, rounded.
+__device__ __forceinline__ uint32_t split_bf16x2(float2 p, uint32_t& lo) {
+  const uint32_t a = __float_as_uint(p.x), b = __float_as_uint(p.y);
+  const float2 rest = __ffma2_rn(make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u)), make_float2(-1.f, -1.f), p);
+  lo = cvt_bf16x2(rest.x, rest.y);
+  return __byte_perm(a, b, 0x7632);
 }
 __device__ __forceinline__ uint32_t hfma2_f16(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
@@ -662,15 +669,13 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   constexpr int G = D / GROUP;
   constexpr int kBlocks = D / 64;                                 // 64-column blocks of an operand tile
   constexpr uint32_t kLoadBytes = kBlocks * kHalfTile;            // bytes of a tile
-  // Heads of 64 channels: the products are 80 columns wide.  Column 64 of every value tile is one (the second 64-column
-  // block of the stages, otherwise unused, holds it for good), so that O carries the row sum of the weights as they were
-  // rounded to BF16, and the output is normalised by it: the rounding of the largest weights then cancels.
-  constexpr bool kOnes = D == 64;
-  constexpr int kNV = kOnes ? 80 : D;                             // columns of O
-  // They also follow the running maximum exactly (the largest weight of a row is then 1, without a rounding): the
-  // warp-level kernel, which served these heads before, does, and with the lazy maximum the outputs were up to 18 %
-  // further from 64-bit results than its.  16 x 1560 queries over 6 144 tokens: 120 us lazy, 141 us exact, 650 us there.
-  constexpr float kGrowth = D == 64 ? 0.f : kRescaleThreshold;
+  // Heads of 64 channels: a weight is handed over as two BF16 parts that together carry 16 bits, and every value product is
+  // done with both (the tensor pipe has room: half the channels).  Rounded to one BF16, weights cost these heads more precision
+  // than the warp-level kernel's, which served them before, unless the running maximum was followed exactly (the largest
+  // weight is then 1, without a rounding), and an exact maximum rescales O in half of the steps.  16 x 1560 queries over 6 144 tokens,
+  // error against 64 bits: 141 us and 1.82e-3 exact with one part, 120 us and 2.01e-3 lazy with one part, 134 us and 1.72e-3
+  // lazy with two (1.66e-3 of it is the rounding of the output).
+  constexpr bool kTwoParts = D == 64;
   static_assert(D == 128 || !PAIR, "a pair's CTAs take one 64-channel block of the values each");
 
   if (tid == 0) {
@@ -705,10 +710,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // bias operand tiles start as zeros (columns beyond the group count stay zero for good)
   for (int i = tid; i < 4 * kXBytes / 16; i += kThreads)
     reinterpret_cast<uint4*>(smem + kOffAx)[i] = make_uint4(0, 0, 0, 0);
-  if constexpr (kOnes) {                         // two 16-byte pieces per row: 1, 0 ... 0
-    const int row = (tid >> 1) & 127, piece = tid & 1;            // 512 threads: two stages x 128 rows x two pieces
-    *reinterpret_cast<uint4*>(smem + kOffV + (tid >> 8) * kTileBytes + sw128_offset(row, 8 + piece)) = make_uint4(piece ? 0u : 0x3F80u, 0, 0, 0);
-  }
   if (warp == 0) {
     if constexpr (PAIR) { tmem_alloc_pair(sbase + kOffMisc, 512); tmem_relinquish_pair(); }
     else { tmem_alloc(sbase + kOffMisc, 512); tmem_relinquish(); }
@@ -865,7 +866,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       constexpr int kM = PAIR ? 256 : 128;
       const uint32_t idesc_bf16 = make_idesc_bf16(kM, 64, 0, 0);
       const uint32_t idesc_f16 = idesc_bf16 & ~((7u << 7) | (7u << 10));     // A, B format 0 = FP16
-      const uint32_t idesc_pv = make_idesc_bf16(kM, kNV, 0, 1);               // B (values) is MN-major
+      const uint32_t idesc_pv = make_idesc_bf16(kM, D, 0, 1);               // B (values) is MN-major
       // commit: one arrival when every MMA issued so far has completed; of a pair, on the barrier of both CTAs
       auto commit = [&](int i) { if constexpr (PAIR) tc_commit_pair(cx.bar(i), (uint16_t)3); else tc_commit(cx.bar(i)); };
       // Descriptors are built once; stepping along K only adds a constant to the 14-bit address field
@@ -923,6 +924,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           mma_ts_off_pair<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
           mma_ts_off_pair<2 * 128>(d_tmem, a_tmem + 16, vd, idesc_pv, 1);
           mma_ts_off_pair<3 * 128>(d_tmem, a_tmem + 24, vd, idesc_pv, 1);
+        } else if constexpr (kTwoParts) {            // keys 0-31: high parts in columns 0-15, low ones in 16-31; keys 32-63: in the next 32
+          mma_ts_off<0 * 128>(d_tmem, a_tmem + 0, vd, idesc_pv, accumulate ? 1u : 0u);
+          mma_ts_off<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
+          mma_ts_off<0 * 128>(d_tmem, a_tmem + 16, vd, idesc_pv, 1);
+          mma_ts_off<1 * 128>(d_tmem, a_tmem + 24, vd, idesc_pv, 1);
+          mma_ts_off<2 * 128>(d_tmem, a_tmem + 32, vd, idesc_pv, 1);
+          mma_ts_off<3 * 128>(d_tmem, a_tmem + 40, vd, idesc_pv, 1);
+          mma_ts_off<2 * 128>(d_tmem, a_tmem + 48, vd, idesc_pv, 1);
+          mma_ts_off<3 * 128>(d_tmem, a_tmem + 56, vd, idesc_pv, 1);
         } else {
           mma_ts_off<0 * 128>(d_tmem, a_tmem + 0, vd, idesc_pv, accumulate ? 1u : 0u);
           mma_ts_off<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
@@ -1049,7 +1059,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             for (int c = 0; c < 4; ++c) mx[c] = max3(mx[c], __uint_as_float(sr[i + 2 * c]), __uint_as_float(sr[i + 2 * c + 1]));
           }
           const float m_new = fmaxf(m_run, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c_row);
-          if (__any_sync(0xFFFFFFFFu, m_new - m_run > kGrowth)) {
+          if (__any_sync(0xFFFFFFFFu, m_new - m_run > kRescaleThreshold)) {
             if (D == 64) odd_max = __any_sync(0xFFFFFFFFu, !(fabsf(m_new) < 0x1p24f));
             if (!fresh) {
               // the product of the previous half (the last one issued on this O) must have retired
@@ -1058,7 +1068,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
               tc_fence_after();
               const float f = ex2(m_run - (D == 64 ? no_key_yet(m_new) : m_new));
 #pragma unroll 1
-              for (int c = 0; c < kNV / 16; ++c) {
+              for (int c = 0; c < D / 16; ++c) {
                 uint32_t r[16];
                 tmem_ld16(o_addr + 16 * c, r);
                 tmem_wait_ld();
@@ -1072,16 +1082,20 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           }
           float2 sum2 = make_float2(0.f, 0.f);
           KVQ_STAMP(3);
+          // 64 channels: the two parts of the weights of keys c .. c + 31 of the half, over those keys' scores
+          auto store_parts = [&](int c, const uint32_t* hi, const uint32_t* lo) {
+            tmem_st16(s_addr + 64 * hf + c, hi);
+            tmem_st16(s_addr + 64 * hf + c + 16, lo);
+          };
           if (D == 64 && odd_max) {
             // Rows whose scores so far are -inf, or so large that an FMA's exact product and the rounded maximum differ by more
             // than an exponential can take (a key masked with the lowest number): product and difference one by one, as in
-            // the warp-level kernel, which served heads of 64 channels before.  The scores are fetched once more, so that
-            // the loop below keeps its registers (16 heads x 1560 rows over 7 700 keys: 137 us without this, 141 as here, 146 with
-            // the scores changed in place).
+            // the warp-level kernel, which served heads of 64 channels before.  Rolled, and the scores are fetched once more,
+            // so that the loop below keeps its registers.
             const float m = no_key_yet(m_run);
 #pragma unroll 1
             for (int c = 0; c < 64; c += 32) {
-              uint32_t r[32];
+              uint32_t r[32], lo[16];
               tmem_ld32(s_addr + 64 * hf + c, r);
               tmem_wait_ld();
 #pragma unroll
@@ -1089,20 +1103,22 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 const float x0 = c + i < nv ? __uint_as_float(r[i]) : -INFINITY, x1 = c + i + 1 < nv ? __uint_as_float(r[i + 1]) : -INFINITY;
                 const float p0 = ex2(__fsub_rn(__fmul_rn(x0, c_row), m)), p1 = ex2(__fsub_rn(__fmul_rn(x1, c_row), m));
                 sum2.x += p0; sum2.y += p1;
-                r[i >> 1] = cvt_bf16x2(p0, p1);
+                r[i >> 1] = split_bf16x2(make_float2(p0, p1), lo[i >> 1]);
               }
-              tmem_st16(s_addr + 64 * hf + c / 2, r);
+              store_parts(c, r, lo);
             }
           } else {
             const float2 c2 = make_float2(c_row, c_row), nm2 = make_float2(-m_run, -m_run);
+            uint32_t lo[16];
 #pragma unroll
             for (int i = 0; i < 64; i += 2) {
               const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2);
               const float2 pr = ((i >> 1) & 3) < (PAIR ? kPolyPairs : 0) ? ex2_poly2(x) : make_float2(ex2(x.x), ex2(x.y));
               sum2 = __fadd2_rn(sum2, pr);
-              sr[i >> 1] = cvt_bf16x2(pr.x, pr.y);
+              sr[i >> 1] = kTwoParts ? split_bf16x2(pr, lo[(i >> 1) & 15]) : cvt_bf16x2(pr.x, pr.y);
+              if (kTwoParts && (i & 31) == 30) store_parts(i & 32, sr + (i & 32) / 2, lo);
             }
-            tmem_st32(s_addr + 64 * hf, sr);
+            if constexpr (!kTwoParts) tmem_st32(s_addr + 64 * hf, sr);
           }
           if (cached) lcac += sum2.x + sum2.y; else lcur += sum2.x + sum2.y;
           tmem_wait_st();
@@ -1124,14 +1140,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // a whole unit writes its rows of the output; a partial segment writes the same normalised rows into its
       // slot, with the statistics the merge kernel weighs them by
       const float l = lcur + lcac;
-      float norm = l;
-      if constexpr (kOnes) {
-        uint32_t r[16];
-        tmem_ld16(o_addr + 64, r);
-        tmem_wait_ld();
-        norm = __uint_as_float(r[0]);
-      }
-      const float inv = D == 64 && !whole && norm == 0.f ? 0.f : 1.0f / norm;      // a range without a weight adds nothing
+      const float inv = D == 64 && !whole && l == 0.f ? 0.f : 1.0f / l;      // a range without a weight adds nothing
       const bool store = !whole || row < p.m_tokens;
       // consecutive 8-column pieces: 16 bytes apart in a row of the output, 4096 bytes apart in a slot
       uint8_t* dst = whole ? reinterpret_cast<uint8_t*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st)
