@@ -86,9 +86,9 @@ extern "C" {
                                             at 2 bits, 1/0.86 at 4), then the one-CTA tcgen05 kernel; head_dim 64 with such
                                             strides and the workspace that kvq_attn_workspace_bytes asks for: the one-CTA
                                             tcgen05 kernel; everything else: the warp-level kernel.  Chunks of up to
-                                            16 query rows (up to 64 over short caches) run, whatever their strides, on a
-                                            kernel of their own for few rows, again if the call brings the
-                                            workspace that kvq_attn_workspace_bytes asks for. */
+                                            16 query rows (up to 64 over short caches) and small problems of more rows run,
+                                            whatever their strides, on a kernel of their own, again if the call brings
+                                            the workspace that kvq_attn_workspace_bytes asks for. */
 #define KVQ_KERNEL_MMA_SYNC   (1u << 8)  /* force the warp-level mma.sync kernel (cross-check / fallback shapes) */
 #define KVQ_KERNEL_TCGEN05    (2u << 8)  /* force the tcgen05/TMEM kernel; KVQ_ERR_UNSUPPORTED unless head_dim is 128 */
 #define KVQ_KERNEL_TCGEN05_PAIR (3u << 8) /* the tcgen05 kernel on pairs of SMs (thread-block clusters of two CTAs that share

@@ -31,6 +31,7 @@ constexpr int kRows = 16;
 constexpr int kWarps = 4;
 constexpr int kStep = 32;            // keys a warp takes at a time
 constexpr int kCtasPerSm = 2;      // up to 255 registers a thread, nothing spilled
+constexpr int kCtasPerSm64 = 3;    // heads of 64 channels
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct SParams {
@@ -158,7 +159,7 @@ __device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p
 // here, 140 us with a branch at each step or an early exit.  Three CTAs an SM for 64 channels (two with the registers of the
 // second form: 237 against 140 us for 32 such rows).
 template <int D, int BITS, int GROUP, bool ANY_ZERO>
-__global__ void __launch_bounds__(kWarps * 32, D == 64 ? 3 : kCtasPerSm) attn_short_kernel(const SParams p) {
+__global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPerSm) attn_short_kernel(const SParams p) {
   constexpr int LD = D + 8;                                        // padded rows of the query tiles
   constexpr int KS = D / 16;                                       // MMA steps over the channels
   constexpr int NT = D / 8;                                        // output tiles of 8 channels
@@ -614,7 +615,20 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   // cost to each tile, stay ahead further: two blocks 69 against 73 at 4 160, 141 against 157 at 10 400 of 160 heads.
   const int64_t blocks = (m_tokens + kRows - 1) / kRows;
   if (blocks == 1) return true;
-  const int64_t bh = (int64_t)d->batch * d->heads, pairs = bh * ((cache_len + 127) / 128 + (n_cur + 127) / 128);
+  // Small problems, whatever the rows: all CTAs run at once and each has few steps, while the other kernel is a chain of three
+  // launches with a prologue of microseconds each.  Counted in steps of 32 keys over all blocks of 16 rows (device time, us, here
+  // against there, 2 bits; 4 bits alike): 64 channels 2 heads x 256 rows over 1 024 keys 8 / 15, at 4 608 steps 14 / 17, at 8 192
+  // 16 / 18, at 8 704 19 / 19, at 10 240 22 / 18; 128 channels at 1 056 steps 11 / 18, at 4 224 17 / 19, at 4 608 19 / 22, at 6 432
+  // 20 / 19, at 8 320 24 / 21.  For 128 channels only up to the 128 rows of one query tile of the other kernel, half of which
+  // idles there.
+  const int64_t bh = (int64_t)d->batch * d->heads;
+  const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
+  if (d->head_dim == 64) {
+    if (bh * blocks <= resident_ctas() / kCtasPerSm * kCtasPerSm64 && bh * blocks * steps <= 8192) return true;
+  } else if (blocks <= 8 && bh * blocks <= resident_ctas() && bh * blocks * steps <= 4608) {
+    return true;
+  }
+  const int64_t pairs = bh * ((cache_len + 127) / 128 + (n_cur + 127) / 128);
   if (d->head_dim == 64) return (blocks == 2 && pairs <= 16384) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 600);
   return bh * blocks <= resident_ctas() && ((blocks == 2 && pairs <= 4200) || (blocks == 3 && pairs <= 1200) || (blocks == 4 && pairs <= 400));
 }
