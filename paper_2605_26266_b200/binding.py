@@ -94,6 +94,20 @@ lib = _load()
 _quantize_append, _attn_workspace_bytes, _attn_corrected = lib.kvq_quantize_append, lib.kvq_attn_workspace_bytes, lib.kvq_attn_corrected
 _BF16 = torch.bfloat16
 
+# The plain calls of the hot path go through a small CPython extension (csrc/py_call.cpp), which reads the tensors without the
+# Python-level accessors: a small append is a few microseconds of Python around a kernel of two (5.7 us a call through ctypes).
+# It answers _NOT_PLAIN to anything else (subclasses, other dtypes or layouts, whatever raises), and where it cannot be loaded
+# (a torch or Python it was not built for) every call takes the ctypes route below it.
+_NOT_PLAIN = -1000
+try:
+    from . import _py_call
+    _py_call.bind(*(C.cast(f, C.c_void_p).value for f in (_quantize_append, _attn_workspace_bytes, _attn_corrected)))
+    _append_call, _attn_call = _py_call.append, _py_call.attn
+except ImportError:
+    def _append_call(*_):
+        return _NOT_PLAIN
+    _attn_call = _append_call
+
 
 class KvqError(RuntimeError):
     def __init__(self, status: int, where: str):
@@ -129,6 +143,9 @@ def _stream() -> int:
     return _raw_stream(_current_device())
 
 
+_capturing = getattr(torch._C, "_cuda_isCurrentStreamCapturing", torch.cuda.is_current_stream_capturing)
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -157,7 +174,7 @@ class Cache:
     def _stream_workspace(self, need, stream, device):
         """Heads of 64 channels had no workspace once, so that calls which only read one cache could run on several streams
         and threads: a buffer for each stream (at most eight are kept), a fresh one for a call that is being captured."""
-        capturing = torch.cuda.is_current_stream_capturing()
+        capturing = _capturing()
         kept = self._stream_workspaces
         ws = None if capturing else kept.get(stream)
         if ws is None or ws.numel() < need:
@@ -186,6 +203,14 @@ class Cache:
         }
 
 
+def _workspace(cache, need, stream, device):
+    """A workspace of `need` bytes where the cache's own does not do."""
+    if cache.desc.head_dim == 64:
+        return cache._stream_workspace(need, stream, device)
+    cache.workspace = torch.empty(need, dtype=torch.uint8, device=device)
+    return cache.workspace
+
+
 def kvq_version() -> int:
     return lib.kvq_version()
 
@@ -199,15 +224,16 @@ def kvq_cache_bytes(desc: kvq_cache_desc):
 def kvq_quantize_append(cache: Cache, k: torch.Tensor, v: torch.Tensor, cache_len: int | None = None) -> int:
     """Appends the chunk k, v ([batch, heads, n, head_dim] BF16, CUDA) at token `cache_len`
     (default: the cache's running length) and returns the new length."""
-    assert k.dtype is _BF16 and v.dtype is _BF16 and k.is_cuda and v.is_cuda
-    shape, st = k.shape, k.stride()
-    assert shape == v.shape and st == v.stride()
     pos = cache.length if cache_len is None else cache_len
-    n = shape[2]
-    status = _quantize_append(C.byref(cache.desc), pos, k.data_ptr(), v.data_ptr(), _strides_of(st), n, _stream())
+    status = _append_call(C.addressof(cache.desc), pos, k, v, _stream()) if k.is_cuda else _NOT_PLAIN
+    if status == _NOT_PLAIN:
+        assert k.dtype is _BF16 and v.dtype is _BF16 and k.is_cuda and v.is_cuda
+        st = k.stride()
+        assert k.shape == v.shape and st == v.stride()
+        status = _quantize_append(C.byref(cache.desc), pos, k.data_ptr(), v.data_ptr(), _strides_of(st), k.shape[2], _stream())
     if status:
         _check(status, "kvq_quantize_append")
-    cache.length = pos + n
+    cache.length = pos + k.shape[2]
     return cache.length
 
 
@@ -230,11 +256,26 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
                        status_word=None):
     """out = corrected attention of q over [cache window ; current chunk].  Tensors are
     [batch, heads, tokens, head_dim] BF16 CUDA; returns `out` (allocated if not given)."""
+    n_cache = cache.length - cache_begin if cache_len is None else cache_len
+    if out is None and type(q) is torch.Tensor:
+        out = torch.empty_like(q, memory_format=torch.contiguous_format)
+    if out is not None and q.is_cuda:
+        stream, ws = _stream(), cache.workspace
+        if ws is None and cache._stream_workspaces and not _capturing():
+            ws = cache._stream_workspaces.get(stream)
+        for _ in range(2):
+            status = _attn_call(C.addressof(cache.desc), cache_begin, n_cache, q, k_cur, v_cur, out, softmax_scale, flags, lse,
+                                cached_mass, status_word, ws, stream)
+            if status <= 0:
+                break
+            ws = _workspace(cache, status, stream, q.device)
+        if status == KVQ_OK:
+            return out
+    # not a plain call, or an error: checked and raised here
     for t in (q, k_cur, v_cur):
         assert t.dtype is _BF16 and t.is_cuda
     kv_shape, kv_st = k_cur.shape, k_cur.stride()
     assert kv_shape == v_cur.shape and kv_st == v_cur.stride()
-    n_cache = cache.length - cache_begin if cache_len is None else cache_len
     if out is None:
         out = torch.empty_like(q, memory_format=torch.contiguous_format)
     m, n_cur, desc, size = q.shape[2], kv_shape[2], C.byref(cache.desc), C.c_size_t(0)
@@ -245,10 +286,7 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
     if need:
         ws = cache.workspace
         if ws is None or ws.numel() < need:
-            if cache.desc.head_dim == 64:
-                ws = cache._stream_workspace(need, stream, q.device)
-            else:
-                ws = cache.workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+            ws = _workspace(cache, need, stream, q.device)
     status = _attn_corrected(
         desc, cache_begin, n_cache, q.data_ptr(), _strides_of(q.stride()), k_cur.data_ptr(), v_cur.data_ptr(),
         _strides_of(kv_st), m, n_cur, out.data_ptr(), _strides_of(out.stride()), float(softmax_scale), flags, _ptr(lse),

@@ -1,4 +1,4 @@
-"""Builds libkvq.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds libkvq.so in-tree with nvcc for sm_100a, and the CPython extension binding.py calls it through (no JIT cache)."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -7,6 +7,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -18,6 +19,9 @@ NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "-Xptxas", "-v", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
 ]
+
+
+PY_CALL = os.path.join(PKG, "_py_call.so")     # the argument marshalling of binding.py
 
 
 def _nvcc() -> str:
@@ -91,7 +95,24 @@ def _build_locked(force: bool, verbose: bool) -> str:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
         _stamp(LIB, lib_digest)
+    _build_py_call(force, verbose)
     return LIB
+
+
+def _build_py_call(force: bool, verbose: bool) -> None:
+    import torch
+
+    src, t = os.path.join(CSRC, "py_call.cpp"), os.path.dirname(torch.__file__)
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(t, "include"),
+           "-I", os.path.join(ROOT, "include"), src, "-o", PY_CALL, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    d = _digest([src, os.path.join(ROOT, "include", "kvq.h")], torch.__version__ + sys.version)
+    if force or not _current(PY_CALL, d):
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or r.returncode != 0:
+            sys.stderr.write(r.stdout + r.stderr)
+        if r.returncode != 0:
+            raise RuntimeError("g++ failed for py_call.cpp")
+        _stamp(PY_CALL, d)
 
 
 if __name__ == "__main__":

@@ -1,0 +1,66 @@
+"""The CPython extension behind the binding: it takes plain calls only, and what it takes gives the bytes of the ctypes route."""
+import pytest
+import torch
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2605_26266_b200 import build
+    build.build_library()
+    from paper_2605_26266_b200 import binding
+    return binding
+
+
+def test_the_extension_is_the_one_that_runs_and_takes_plain_calls_only(B):
+    from paper_2605_26266_b200 import _py_call
+    assert B._append_call is _py_call.append and B._attn_call is _py_call.attn
+    x = torch.zeros(1, 2, 16, 128, dtype=torch.bfloat16)                               # on the CPU
+    for args in [(0, 0, x, x, 0), (0, 0, None, x, 0), ("0", 0, x, x, 0), (0, 0.0, x, x, 0), (0, 0, x, x), (1 << 90, 0, x, x[0], None)]:
+        assert _py_call.append(*args) == B._NOT_PLAIN
+    attn = [0, 0, 0, x, x, x, x, 0.1, 1, None, None, None, None, 0]
+    for i, v in [(0, None), (3, x), (4, "k"), (7, 1), (8, 1.0), (9, 5), (12, b""), (13, None)]:
+        assert _py_call.attn(*(attn[:i] + [v] + attn[i + 1:])) == B._NOT_PLAIN
+    with pytest.raises(TypeError):
+        _py_call.bind(1, 2)
+    cache = B.Cache(1, 2, 128, 2, 64, 128, device="cpu")
+    for k, v in [(x, x), (x.float(), x), (x[:, :, :8], x)]:
+        with pytest.raises(AssertionError):
+            B.kvq_quantize_append(cache, k, v)
+        with pytest.raises(AssertionError):
+            B.kvq_attn_corrected(cache, x, k, v, 0.1, out=x)
+    assert cache.length == 0 and cache.workspace is None
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,m,layout", [(128, 40, "dense"), (128, 300, "interleaved"), (64, 40, "padded"), (64, 700, "dense")])
+def test_both_routes_give_the_same_bytes(B, d, m, layout, monkeypatch):
+    g = torch.Generator(device="cuda").manual_seed(5)
+
+    def tensor(t):
+        x = torch.randn(2, 3, t, d, device="cuda", generator=g).bfloat16()
+        if layout == "interleaved":
+            return x.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+        if layout == "padded":
+            return torch.nn.functional.pad(x, (0, 24))[..., :d]
+        return x
+    pk, pv, q, k, v = tensor(500), tensor(500), tensor(m), tensor(m), tensor(m)
+    results = []
+    for native in (True, False):
+        if not native:
+            monkeypatch.setattr(B, "_append_call", lambda *_: B._NOT_PLAIN)
+            monkeypatch.setattr(B, "_attn_call", lambda *_: B._NOT_PLAIN)
+        cache = B.Cache(2, 3, d, 2, 64, 640)
+        assert B.kvq_quantize_append(cache, pk, pv) == 500 and B.kvq_quantize_append(cache, pk[:, :, :16], pv[:, :, :16]) == 516
+        lse = torch.zeros(2, 3, m, device="cuda")
+        mass, status = torch.zeros_like(lse), torch.zeros(1, dtype=torch.int32, device="cuda")
+        given = torch.empty_like(q)
+        assert B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, out=given, lse=lse, cached_mass=mass, status_word=status) is given
+        made = B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, cache_begin=16, cache_len=400)
+        assert made.is_contiguous()
+        with pytest.raises(B.KvqError) as e:
+            B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, cache_begin=8, out=given)
+        assert e.value.status == B.KVQ_ERR_ALIGNMENT
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        results.append([t.clone() for t in (*cache.buffers, given.view(torch.int16), lse, mass, made.view(torch.int16))])
+    assert all(torch.equal(a, b) for a, b in zip(*results))
