@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
   } sm;
   __shared__ float s_stat[kWarps][3][kRows];                       // m, l_cur, l_cached
 
+  wait_for_previous_grid();                                        // the first kernel of a call: nothing global is touched before
   allow_next_grid();                                               // the merge kernel
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
   const int unit = blockIdx.x / p.splits, split = blockIdx.x - unit * p.splits;
@@ -593,9 +594,9 @@ Plan plan(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t 
 
 template <int D, int BITS, int GROUP>
 int launch(const SParams& p, const Plan& pl, bool any_zero, cudaStream_t st) {
-  if (D == 64 || any_zero) attn_short_kernel<D, BITS, GROUP, true><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
-  else attn_short_kernel<D, BITS, GROUP, D == 64><<<(unsigned)(pl.units * pl.splits), kWarps * 32, 0, st>>>(p);
-  KVQ_CUDA_TRY(cudaGetLastError());
+  const auto kern = D == 64 || any_zero ? attn_short_kernel<D, BITS, GROUP, true> : attn_short_kernel<D, BITS, GROUP, D == 64>;
+  const int r = launch_after(true, 1, dim3((unsigned)(pl.units * pl.splits)), dim3(kWarps * 32), 0, st, kern, p);
+  if (r != KVQ_OK) return r;
   if (pl.splits > 1)
     return launch_after(true, 1, dim3((unsigned)(pl.units * kRows)), dim3(kWarps * 32), 0, st, attn_short_merge_kernel<D>, p);
   return KVQ_OK;

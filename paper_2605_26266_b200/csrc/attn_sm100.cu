@@ -537,6 +537,7 @@ struct RotParams {
 template <int BITS, int GROUP, int D>
 __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
   constexpr int kLanes = D / 8;                      // per row
+  wait_for_previous_grid();                          // whatever wrote the queries, and readers of the workspace
   allow_next_grid();                                 // the attention kernel: its prologue and first tiles need nothing from here
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ln = lane & (kLanes - 1), rsub = lane / kLanes;
@@ -722,6 +723,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
   // TMEM columns: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512); P_q aliases the first 64 columns of S_q.
 
+  if (!p.ax_rows) wait_for_previous_grid();      // no pre-pass: the first kernel of the call, nothing global is touched before
   allow_next_grid();                             // the merge kernel
   if (warp < 4) {
     setmaxnreg_dec<kRegsIssue>();
@@ -1559,13 +1561,14 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk,
   }
   if (rp.qr) {                      // there are cached keys: rotate the query chunk first
     constexpr int kRows = 2048 / D;  // of a block
-    rotate_query_kernel<BITS, GROUP, D><<<dim3((unsigned)((rp.m_tokens + kRows - 1) / kRows), (unsigned)(p.n_units / p.q_blocks)), 256, 0, st>>>(rp);
-    KVQ_CUDA_TRY(cudaGetLastError());
+    const int r = launch_after(true, 1, dim3((unsigned)((rp.m_tokens + kRows - 1) / kRows), (unsigned)(p.n_units / p.q_blocks)), dim3(256), 0, st,
+                               rotate_query_kernel<BITS, GROUP, D>, rp);
+    if (r != KVQ_OK) return r;
   }
   // grid.x counts pairs in the pair kernel: two CTAs each, launched as clusters of two.  Behind the pre-pass the kernel may
   // start early: it has the current chunk's tiles to work on first.
   constexpr int kC = PAIR ? 2 : 1;
-  int r = launch_after(rp.qr != nullptr, kC, dim3(kC * grid.x), dim3(kThreads), kSmemBytes, st, attn_tcgen05_kernel<BITS, GROUP, PAIR, D>, mq, mqr, mk, mv, p);
+  int r = launch_after(true, kC, dim3(kC * grid.x), dim3(kThreads), kSmemBytes, st, attn_tcgen05_kernel<BITS, GROUP, PAIR, D>, mq, mqr, mk, mv, p);
   if (r != KVQ_OK) return r;
   if (p.n_whole != p.n_units)     // units were split over CTAs: combine their partial results
     r = launch_after(true, 1, dim3((unsigned)((p.n_units - p.n_whole) * kC), 16), dim3(256), 0, st, attn_merge_kernel<D>, p, (int)grid.x, PAIR ? 1 : 0);

@@ -115,9 +115,13 @@ int launch_after(bool overlap, int cluster, dim3 grid, dim3 block, size_t smem, 
   return KVQ_OK;
 }
 
-// Kernels of one call overlap where the second does not need the first at once (launch_after): the first allows the next
-// grid's blocks to start when its own have all started, the second waits before it touches what the first writes.  Every
-// block of the second waits, so that work ordered behind it is ordered behind the first too.
+// Kernels overlap (launch_after): one allows the next grid's blocks to start when its own have all started (allow_next_grid), and
+// the next waits before it touches what the one before writes.  Every block of a kernel waits, so that work ordered behind it
+// is ordered behind the ones before too.  The first kernel of a call is launched this way as well: its blocks are placed, and the
+// attention kernel's prologue runs, while the last kernel in the stream, whoever's it is, drains.  It waits before it touches any global
+// memory, and only then allows the next grid, so that the call's later kernels may read the caller's tensors without waiting again.
+// Among other calls (24 heads x 4680 tokens, 16 heads x 1560 rows, 64 heads x 2048 rows, us): append 21.6 -> 19.6, attention
+// 125.4 -> 123.6, 64 channels 134.5 -> 130.5, empty cache 167 -> 163.5.
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

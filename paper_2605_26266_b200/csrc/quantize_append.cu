@@ -14,7 +14,8 @@
 // the two halves of 64-bit registers and does everything but the last in-lane butterfly stage and the minimum/maximum
 // with the packed instructions (add/mul/fma.rn.f32x2: two IEEE operations each), and adds the zero-point, clamps and packs
 // the codes two at a time as 16-bit integers.  Measured at 24 heads x 4680 tokens, 128 channels, 2 bits, group 64
-// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 23.6 us as here (2.8 TB/s),
+// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 23.6 us as here (2.8 TB/s; 19.6 us
+// where launches overlap, see launch_after),
 // 3 % more with eight lanes per vector (shorter lanes repeat the per-group work more often); two
 // tokens in flight per lane and persistent warps with a prefetch: 26.6 us (fewer warps fit).
 #include <math_constants.h>
@@ -237,6 +238,8 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm) quantize_append_kerne
   if (t0 >= p.n_tokens) return;                               // the whole warp
   const int64_t t = t0 + lane / kLanes;
   const bool valid = t < p.n_tokens;
+  wait_for_previous_grid();                                   // whatever wrote the chunk or still reads the cache
+  allow_next_grid();
   RawVec<EPL> raw[2];
   if (valid) {
     const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + t * p.st;
@@ -379,13 +382,14 @@ int launch_quantize_append(const kvq_cache_desc* d, int64_t cache_len, const voi
   const int64_t blocks = (n_tokens + kWarps * kTokPerWarp - 1) / (kWarps * kTokPerWarp);
   if (blocks > 0x7FFFFFFFLL) return KVQ_ERR_UNSUPPORTED;
   const dim3 grid((unsigned)blocks, (unsigned)(d->batch * d->heads)), block(kWarps * 32);
-#define KVQ_QA(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) { quantize_append_kernel<D_, B_, G_><<<grid, block, 0, st>>>(p); launched = true; }
+#define KVQ_QA(D_, B_, G_) if (d->head_dim == D_ && d->bits == B_ && d->group == G_) { err = launch_after(true, 1, grid, block, 0, st, quantize_append_kernel<D_, B_, G_>, p); launched = true; }
   bool launched = false;
+  int err = KVQ_OK;
   KVQ_QA(128, 2, 32) KVQ_QA(128, 2, 64) KVQ_QA(128, 2, 128) KVQ_QA(128, 4, 32) KVQ_QA(128, 4, 64) KVQ_QA(128, 4, 128)
   KVQ_QA(64, 2, 32) KVQ_QA(64, 2, 64) KVQ_QA(64, 4, 32) KVQ_QA(64, 4, 64)
 #undef KVQ_QA
   if (!launched) return KVQ_ERR_UNSUPPORTED;
-  KVQ_CUDA_TRY(cudaGetLastError());
+  if (err != KVQ_OK) return err;
   if (p.skip_k) {                                     // per-channel keys: one CTA per block of `group` tokens
     const int64_t bh = (int64_t)d->batch * d->heads;
     if (bh > 65535) return KVQ_ERR_UNSUPPORTED;
