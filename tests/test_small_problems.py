@@ -44,6 +44,17 @@ def test_where_the_line_lies(B, d, heads, m, n, few):
     assert (workspace(B, d, heads, m, n) == partial_rows(d, heads, m, n)) == few
 
 
+@pytest.mark.parametrize("d,heads,m,n,launches", [
+    (64, 2, 256, 1024, 1), (64, 2, 16, 2032, 1), (64, 1, 16, 2300, 2),                 # 5 and 8 splits; 9
+    (128, 2, 16, 1520, 1), (128, 2, 16, 1800, 2), (128, 3, 16, 100, 1),                # 6 splits; 7; 1
+    (128, 22, 16, 2032, 2), (64, 44, 16, 1000, 1), (64, 45, 16, 1000, 2),              # 176 CTAs of 4 splits, 180
+])
+def test_clusters_merge_without_a_second_launch(B, d, heads, m, n, launches):
+    desc, count = B.kvq_cache_desc(1, heads, d, 2, 64, B.KVQ_ROTATE_K, 65536), C.c_int(0)
+    assert B.lib.kvq_attn_kernel_launches(C.byref(desc), n, m, m, 1, C.byref(count)) == B.KVQ_OK
+    assert count.value == launches and workspace(B, d, heads, m, n) == partial_rows(d, heads, m, n)
+
+
 # d, bits, group, heads, rows, current keys, cached keys
 CASES = [(128, 2, 32, 2, 65, 1, 129), (128, 4, 64, 3, 100, 33, 1000), (128, 2, 128, 2, 128, 128, 31), (128, 4, 128, 1, 127, 64, 4001),
          (64, 2, 64, 3, 1000, 40, 300), (64, 4, 32, 60, 97, 31, 65), (64, 2, 32, 1, 513, 700, 0)]
