@@ -1243,7 +1243,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           for (int i = 0; i < 64; i += 4)
             *reinterpret_cast<float4*>(dst + (i >> 2) * piece) =
                 make_float4(__uint_as_float(sr[i]) * inv, __uint_as_float(sr[i + 1]) * inv, __uint_as_float(sr[i + 2]) * inv, __uint_as_float(sr[i + 3]) * inv);
-        } else if (store) {
+        } else if (PAIR && store && whole && p.out_32) {
           // A lane holds a row, so that the 32 lanes of a store meet 32 lines, and the load/store unit takes these one by one: with
           // 32 bytes a lane there are half as many to take (64 heads x 2048 rows over an empty cache 166 -> 163 us).  In the pair
           // kernel only: the one-CTA kernel's code came out 1 % slower with it, and splits most of its units.
@@ -1252,13 +1252,17 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             uint32_t w[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) w[j] = cvt_bf16x2(__uint_as_float(sr[i + 2 * j]) * inv, __uint_as_float(sr[i + 2 * j + 1]) * inv);
-            uint8_t* at = dst + (8 * hf + (i >> 3)) * piece;
-            if (PAIR && whole && p.out_32) {
-              st_global_32(at, w);
-            } else {
-              *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4*>(at + piece) = make_uint4(w[4], w[5], w[6], w[7]);
-            }
+            st_global_32(dst + 128 * hf + 2 * i, w);
+          }
+        } else if (store) {
+#pragma unroll
+          for (int i = 0; i < 64; i += 8) {
+            uint4 v;
+            v.x = cvt_bf16x2(__uint_as_float(sr[i]) * inv, __uint_as_float(sr[i + 1]) * inv);
+            v.y = cvt_bf16x2(__uint_as_float(sr[i + 2]) * inv, __uint_as_float(sr[i + 3]) * inv);
+            v.z = cvt_bf16x2(__uint_as_float(sr[i + 4]) * inv, __uint_as_float(sr[i + 5]) * inv);
+            v.w = cvt_bf16x2(__uint_as_float(sr[i + 6]) * inv, __uint_as_float(sr[i + 7]) * inv);
+            *reinterpret_cast<uint4*>(dst + (8 * hf + (i >> 3)) * piece) = v;
           }
         }
       }
