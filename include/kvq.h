@@ -162,7 +162,8 @@ int kvq_attn_workspace_bytes(const kvq_cache_desc* desc, int64_t cache_len,
 /*
  * How many kernels one kvq_attn_corrected call launches for this problem (host-side bookkeeping for
  * benchmarks and launch-bound callers): the attention kernel, the query pre-pass when the cache window
- * is not empty (not for a few query rows, which have none), the merge kernel when units are split over CTAs.
+ * is not empty (not for a few query rows or a small problem, which have none), the merge kernel when units are split over
+ * CTAs (small problems: not where a cluster of the CTAs merges them).
  * It counts for a call with the workspace kvq_attn_workspace_bytes asks for and tensors TMA can address: one
  * that falls back to another kernel for want of either launches that kernel's.  out_count is host memory.  Same
  * argument checks and errors as kvq_attn_workspace_bytes.
