@@ -141,11 +141,11 @@ __device__ __forceinline__ void load_keys(Keys<D, BITS>& r, const SParams& p, co
   for (int t = 0; t < 4; ++t) {
     const int64_t tok = st.tok[t >> 1] + g + 8 * (t & 1);
     const uint8_t* src = p.codes[0] + tok * CB + c * (W * 4);
-    if constexpr (W == 1) r.w[t][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
-    else if constexpr (W == 2) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; }
-    else { const uint4 v = __ldg(reinterpret_cast<const uint4*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; r.w[t][2] = v.z; r.w[t][3] = v.w; }
+    if constexpr (W == 1) r.w[t][0] = load_coherent(reinterpret_cast<const uint32_t*>(src));
+    else if constexpr (W == 2) { const uint2 v = load_coherent(reinterpret_cast<const uint2*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; }
+    else { const uint4 v = load_coherent(reinterpret_cast<const uint4*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; r.w[t][2] = v.z; r.w[t][3] = v.w; }
     const int64_t at = tok * G + c * (D / 4) / GROUP;
-    r.step[t] = __ldg(p.scale[0] + at); r.zero[t] = __ldg(p.zero[0] + at);
+    r.step[t] = load_coherent(p.scale[0] + at); r.zero[t] = load_coherent(p.zero[0] + at);
   }
 }
 // Tokens past the window: step and zero-point 0, so that scores are finite (and masked later) and values exact zeros, whatever
@@ -170,11 +170,11 @@ __device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p
   for (int i = 0; i < 8; ++i) {
     const int64_t tok = st.tok[i >> 2] + 2 * c + (i & 1) + 8 * ((i >> 1) & 1);
     const uint8_t* src = p.codes[1] + tok * CB + g * B;
-    if constexpr (B == 2) r.w[i][0] = __ldg(reinterpret_cast<const uint16_t*>(src));
-    else if constexpr (B == 4) r.w[i][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
-    else { const uint2 v = __ldg(reinterpret_cast<const uint2*>(src)); r.w[i][0] = v.x; r.w[i][1] = v.y; }
+    if constexpr (B == 2) r.w[i][0] = load_coherent(reinterpret_cast<const uint16_t*>(src));
+    else if constexpr (B == 4) r.w[i][0] = load_coherent(reinterpret_cast<const uint32_t*>(src));
+    else { const uint2 v = load_coherent(reinterpret_cast<const uint2*>(src)); r.w[i][0] = v.x; r.w[i][1] = v.y; }
     const int64_t at = tok * G + g * (D / 8) / GROUP;
-    r.step[i] = __ldg(p.scale[1] + at); r.zero[i] = __ldg(p.zero[1] + at);
+    r.step[i] = load_coherent(p.scale[1] + at); r.zero[i] = load_coherent(p.zero[1] + at);
   }
 }
 
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
     for (int r = warp * (32 / LPR) + lane / LPR; r < kRows; r += kWarps * 32 / LPR) {
       const int row = row0 + r;
       uint4 raw = make_uint4(0, 0, 0, 0);
-      if (row < p.m_tokens) raw = __ldg(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
+      if (row < p.m_tokens) raw = load_coherent(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
       *reinterpret_cast<uint4*>(sm.in.q + r * LD + ln * 8) = raw;
       const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
       float x[8];
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
       const uint4* src = reinterpret_cast<const uint4*>(p.kc + (int64_t)b * p.kv_sb + (int64_t)h * p.kv_sh + (int64_t)min(k0 + 8 * t + g, p.n_cur - 1) * p.kv_st + c * (D / 4));
 #pragma unroll
       for (int i = 0; i < D / 32; ++i) {
-        const uint4 v = __ldg(src + i);
+        const uint4 v = load_coherent(src + i);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int col = c * (D / 4) + 8 * i + 4 * j;
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int key = 16 * kk + 2 * c + (u & 1) + 8 * (u >> 1);
-          v[u] = key < nv ? __ldg(reinterpret_cast<const uint4*>(vbase + (int64_t)(k0 + key) * p.v_st) + i) : make_uint4(0, 0, 0, 0);
+          v[u] = key < nv ? load_coherent(reinterpret_cast<const uint4*>(vbase + (int64_t)(k0 + key) * p.v_st) + i) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {

@@ -311,7 +311,8 @@ struct Raw {   // packed codes and metadata of one cached token (keys or values)
 };
 
 // Loads NW code words of the token, starting at word `word0` (a multiple of 4), into r.w[0 .. NW), and the token's
-// metadata.  NW is the whole row, or half of it for a CTA of a pair.
+// metadata.  NW is the whole row, or half of it for a CTA of a pair.  The read-only path is sound here: the cache is read behind a pre-pass
+// only, and this kernel's blocks start after every block of the pre-pass has waited for whatever wrote the cache.
 template <int BITS, int G, int D, int NW = Raw<BITS, D>::kWords>
 __device__ __forceinline__ void load_raw(Raw<BITS, D>& r, const uint8_t* codes, const uint8_t* scale, const uint16_t* zero,
                                          int64_t tok, bool valid, int word0 = 0) {
@@ -600,7 +601,7 @@ __global__ void __launch_bounds__(256) rotate_query_kernel(const RotParams p) {
     const int row = (blockIdx.x * 8 + warp) * (32 / kLanes) + rsub;
     const bool valid = row < p.m_tokens;             // no early exit: the shuffles below need every lane
     uint4 raw = make_uint4(0, 0, 0, 0);
-    if (valid) raw = __ldg(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
+    if (valid) raw = load_coherent(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
     float x[8];
     x[0] = bf16_bits_to_f32(raw.x & 0xFFFFu); x[1] = bf16_bits_to_f32(raw.x >> 16);
     x[2] = bf16_bits_to_f32(raw.y & 0xFFFFu); x[3] = bf16_bits_to_f32(raw.y >> 16);

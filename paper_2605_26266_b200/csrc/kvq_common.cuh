@@ -124,6 +124,14 @@ int launch_after(bool overlap, int cluster, dim3 grid, dim3 block, size_t smem, 
 // 125.4 -> 123.6, 64 channels 134.5 -> 130.5, empty cache 167 -> 163.5.
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// How a kernel that waits there reads what a grid before may have written: with an ordinary load.  The read-only path (`__ldg`,
+// ld.global.nc) is defined only for memory that nothing writes during the kernel, and such a kernel has started by then; nor does the
+// wait hold back loads that the compiler takes for invariant.
+template <typename T>
+__device__ __forceinline__ T load_coherent(const T* p) {
+  __builtin_assume(__isGlobal(p));
+  return *p;
+}
 
 // ---- device-side number-format helpers -------------------------------------------------
 

@@ -1,6 +1,7 @@
-"""Kernels of one call overlap (programmatic dependent launch): what an earlier kernel of the call writes into the workspace
-may still be written while a later one runs.  Such memory must not be read through the read-only path (`__ldg`,
-ld.global.nc), which is defined only for memory that nothing writes during the kernel.  Checked in the sources."""
+"""Kernels overlap (programmatic dependent launch): blocks start while the grid before still runs, and wait there.  What that grid, or
+one before it, may write - the workspace, and for a call's first kernel every tensor and the cache - must not be read through the
+read-only path (`__ldg`, ld.global.nc), which is defined only for memory that nothing writes during the kernel.  Checked in
+the sources."""
 import os
 import re
 
@@ -27,6 +28,28 @@ def test_workspace_is_not_read_through_the_read_only_path(name, pointers):
     assert "wait_for_previous_grid()" in text and all(p in text for p in pointers[:1])
     bad = [a for a in ldg_arguments(text) if any(re.search(rf"\b{p}\b", a) for p in pointers)]
     assert not bad, bad
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+@pytest.mark.parametrize("name", sorted(n for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh"))))
+def test_kernels_that_wait_read_with_ordinary_loads(name):
+    text = source(name)
+    assert ".nc." not in text
+    if "wait_for_previous_grid();" not in text:               # ordinary launches only
+        return
+    assert "launch_after(true" in text or name == "kvq_common.cuh"
+    if name != "attn_sm100.cu":
+        assert "__ldg(" not in text
+        return
+    # the cached tiles of the tcgen05 kernel: it starts behind the pre-pass, whose blocks have all waited before they let it start
+    body = text[text.index("void load_raw("):text.index("void load_raw_staged(")]
+    assert text.count("__ldg(") == body.count("__ldg(")
+    pre_pass = text[text.index(" rotate_query_kernel(const RotParams p)"):]
+    assert pre_pass.index("wait_for_previous_grid();") < pre_pass.index("allow_next_grid();") < pre_pass.index("load_coherent(")
 
 
 def test_both_ctas_of_a_pair_wait_for_the_last_commits():
