@@ -46,7 +46,7 @@
 // The same source also gives the pair kernel (template parameter PAIR): a cluster of two CTAs on 512 query rows
 // whose tensor cores work as one (tcgen05 cta_group::2), described at the kernel; and the kernel for heads of 64
 // channels (D = 64, one CTA per unit): operand tiles one 64-column block wide at the same places, half the MMA steps of a
-// score, 16 heads x 1560 queries over 7 700 keys in 126 us against 650 us in the warp-level kernel.
+// score, 16 heads x 1560 queries over 7 700 keys in 129 us against 650 us in the warp-level kernel.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA records a diagnostic in the caller's status
 // word, all roles leave their loops, in-flight work is drained with a bounded wait, TMEM is freed and the
@@ -79,8 +79,7 @@ constexpr int kOffBar = kOffBx + 2 * kXBytes;
 constexpr int kNumBars = 32;                       // mbarriers, 8 bytes each (enum Bar below)
 static_assert(kNumBars * 8 <= 256, "barrier area");
 constexpr int kOffMisc = kOffBar + 256;
-constexpr int kOffForm = kOffMisc + 64;            // 64 channels: format of the cached values, [tile % 4][32 keys of the tile]
-constexpr int kSmemBytes = kOffForm + 64 + 1024;   // + slack to align the base to 1024
+constexpr int kSmemBytes = kOffMisc + 64 + 1024;   // + slack to align the base to 1024
 
 // kSFull, kPFull and kODone have four barriers each: index 2 * (half of the key tile) + (query tile); each of
 // them completes once per key tile, so that a waiter is never more than one phase behind
@@ -233,8 +232,7 @@ __device__ __forceinline__ float ex2(float x) {
 // Of every four pairs of scores, how many take their exponentials on the FMA pipe instead of the MUFU (16 lanes
 // per SM: the two softmax warps of a scheduler share 4).  Measured: one of four is worth 2 to 5 % in the pair
 // kernel, where the MUFU is what the softmax groups wait for; in the one-CTA kernel the extra instructions cost as
-// much as they save, so it keeps the MUFU for all (a quarter of the FP16 weights of 64-channel
-// heads from the FMA pipe: 126 -> 124 us, but the log-sum-exp of a row with one key is then 7e-5 off).
+// much as they save, so it keeps the MUFU for all.
 constexpr int kPolyPairs = 1;
 // 2^x for a pair of arguments without the MUFU: x = n + r with n the nearest integer (taken from the low mantissa
 // bits of x + 1.5 * 2^23) and r in [-0.5, 0.5]; 2^r by a cubic (relative error 7.5e-5, far below the BF16
@@ -258,11 +256,6 @@ __device__ __forceinline__ uint32_t split_bf16x2(float2 p, uint32_t& lo) {
   const float2 rest = __ffma2_rn(make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u)), make_float2(-1.f, -1.f), p);
   lo = cvt_bf16x2(rest.x, rest.y);
   return __byte_perm(a, b, 0x7632);
-}
-__device__ __forceinline__ uint32_t cvt_f16x2(float lo, float hi) {
-  uint32_t d;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-  return d;
 }
 // 32 bytes to a 32-byte boundary.
 __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8]) {
@@ -532,43 +525,6 @@ __device__ __forceinline__ void dequant_values(const Raw<BITS, D>& r, uint8_t* t
   }
 }
 
-// Values in FP16, exactly (value_exact_f16 holds for the token's groups).
-template <int BITS, int GROUP, int D>
-__device__ __forceinline__ void dequant_values_f16(const Raw<BITS, D>& r, uint8_t* tile, int row) {
-  constexpr int G = D / GROUP;
-  constexpr float kOff = (BITS == 2) ? 4.f : 16.f;
-  uint32_t step2[4], c2[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float ds = raw_step<BITS, D>(r, j);
-    step2[j] = pack_f16x2_sat(ds, ds);
-    const float c = -(kOff + raw_zero<BITS, D>(r, j)) * ds;
-    c2[j] = pack_f16x2_sat(c, c);
-  }
-#pragma unroll
-  for (int wi = 0; wi < Raw<BITS, D>::kWords; ++wi) {
-    const int j = (wi * (32 / BITS)) / GROUP;
-    const uint32_t st = pick_group<G>(step2, j), cc = pick_group<G>(c2, j), w = r.w[wi];
-    constexpr uint32_t kEven = BITS == 2 ? 0x33333333u : 0x0F0F0F0Fu;
-    const uint32_t lo = w & kEven, hi = (w >> BITS) & kEven;
-    const uint32_t z[2] = {(lo & 0xFFFFu) | (hi << 16), (lo >> 16) | (hi & 0xFFFF0000u)};    // code 2 i in the low half, 2 i + 1 in the high one
-    constexpr int kPairs = 8 / BITS;                             // of each of the two
-    uint32_t o[2 * kPairs];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int i = 0; i < kPairs; ++i) {
-        constexpr int kTo = BITS == 2 ? 8 : 6;                   // where a code's lowest bit goes
-        const int from = 2 * BITS * i;
-        const uint32_t x = from <= kTo ? z[u] << (kTo - from) : z[u] >> (from - kTo);
-        o[u * kPairs + i] = hfma2_f16(and_or(x, BITS == 2 ? 0x03000300u : 0x03C003C0u, BITS == 2 ? 0x44004400u : 0x4C004C00u), st, cc);
-      }
-#pragma unroll
-    for (int q = 0; q < 2 * kPairs; q += 4)
-      *reinterpret_cast<uint4*>(tile + sw128_offset(row, (wi * 2 * kPairs + q) / 4)) = make_uint4(o[q], o[q + 1], o[q + 2], o[q + 3]);
-  }
-}
-
 // Pre-pass over the query chunk (one launch before the attention kernel): q~ = (1/sqrt d) H (signs . q) in
 // FP32, stored as FP16 with the contraction dimension permuted the way the dequantized keys are laid out,
 // and -(sigma/24) nu_{m,j} (per-group squared norms of q~) as a BF16 high part plus a BF16 low part.  The
@@ -713,13 +669,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   auto expect_tx_lead = [&](int i, uint32_t bytes) {
     if constexpr (PAIR) mbar_arrive_expect_tx_cluster(lead(i), bytes); else mbar_arrive_expect_tx(cx.bar(i), bytes);
   };
-  // 64 channels: whether the values of the two runs of 32 keys of half hf of cached tile number `it` are FP16.  Written by the
-  // dequantizing warps before they hand the tile's keys over; four tiles deep, because they are at most two tiles ahead of a softmax
-  // group (the value stage of the tile before last has to be given back first).
-  auto value_form = [&](int it, int hf) {
-    const volatile int* f = reinterpret_cast<const volatile int*>(smem + kOffForm) + (it & 3) * 4 + 2 * hf;
-    return make_int2(f[0], f[1]);
-  };
   // first query row of this CTA in schedule unit `unit` (a unit is 256 rows, 512 for a pair)
   auto unit_row0 = [&](int unit, int bh) { return (unit - bh * p.q_blocks) * (2 * kC * kBlockM) + (int)rank * 2 * kBlockM; };
   const int n_rt = (p.n_cur + kBlockN - 1) / kBlockN;
@@ -728,14 +677,14 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   constexpr int G = D / GROUP;
   constexpr int kBlocks = D / 64;                                 // 64-column blocks of an operand tile
   constexpr uint32_t kLoadBytes = kBlocks * kHalfTile;            // bytes of a tile
-  // Heads of 64 channels: rounded to one BF16, weights cost these heads more precision than the warp-level kernel's, which served
-  // them before, unless the running maximum was followed exactly (the largest weight is then 1, without a rounding), and an
-  // exact maximum rescales O in half of the steps.  So weights carry more bits: cached values that are exact in FP16 and BF16
-  // alike (groups that reach zero or nearly so; decided per 32 keys) meet FP16 weights; the others, and the current chunk's BF16
-  // values, meet weights in two BF16 parts, 16 bits, and every product is done with both (the tensor pipe has room: half the
-  // channels).  16 x 1560 queries over 6 144 tokens, error against 64 bits: 141 us and 1.82e-3 exact with one BF16 part, 120 us and
-  // 2.01e-3 lazy with one, 130 us and 1.72e-3 lazy with two parts throughout (1.66e-3 of it is the rounding of the output), 126 us
-  // and 1.72e-3 as here.
+  // Heads of 64 channels: a weight is handed over as two BF16 parts that together carry 16 bits, and every value product is
+  // done with both (the tensor pipe has room: half the channels).  Rounded to one BF16, weights cost these heads more precision
+  // than the warp-level kernel's, which served them before, unless the running maximum was followed exactly (the largest
+  // weight is then 1, without a rounding), and an exact maximum rescales O in half of the steps.  16 x 1560 queries over 6 144 tokens,
+  // error against 64 bits: 141 us and 1.82e-3 exact with one part, 120 us and 2.01e-3 lazy with one part, 134 us and 1.72e-3
+  // lazy with two (1.66e-3 of it is the rounding of the output); 129 us since the launches of a call overlap those before it.
+  // FP16 weights, against cached values that are exact in FP16, took 4 % less, but FP16 ends at 2^-24: keys that far below the
+  // largest of their row, which may be all there is where that key's value is zero, were lost or a quarter too large.
   constexpr bool kTwoParts = D == 64;
   static_assert(D == 128 || !PAIR, "a pair's CTAs take one 64-channel block of the values each");
 
@@ -929,7 +878,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const uint32_t idesc_bf16 = make_idesc_bf16(kM, 64, 0, 0);
       const uint32_t idesc_f16 = idesc_bf16 & ~((7u << 7) | (7u << 10));     // A, B format 0 = FP16
       const uint32_t idesc_pv = make_idesc_bf16(kM, D, 0, 1);               // B (values) is MN-major
-      const uint32_t idesc_pv16 = idesc_pv & ~((7u << 7) | (7u << 10));       // both operands FP16
       // commit: one arrival when every MMA issued so far has completed; of a pair, on the barrier of both CTAs
       auto commit = [&](int i) { if constexpr (PAIR) tc_commit_pair(cx.bar(i), (uint16_t)3); else tc_commit(cx.bar(i)); };
       // Descriptors are built once; stepping along K only adds a constant to the 14-bit address field
@@ -978,7 +926,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       };
       // O_qt += P V over keys 64 hf .. 64 hf + 63 of stage s; P (BF16 pairs) sits in the first 32 of that half's
       // score columns
-      auto issue_pv = [&](int s, int hf, bool accumulate, int f16_0, int f16_1) {
+      auto issue_pv = [&](int s, int hf, bool accumulate) {
         if (!leader) return;
         const uint64_t vd = dv0 + (uint64_t)(s * (kTileBytes >> 4) + hf * (4 * 128));
         const uint32_t d_tmem = tmem + 256 + qt * 128, a_tmem = tmem + qt * 128 + hf * 64;
@@ -987,20 +935,15 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           mma_ts_off_pair<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
           mma_ts_off_pair<2 * 128>(d_tmem, a_tmem + 16, vd, idesc_pv, 1);
           mma_ts_off_pair<3 * 128>(d_tmem, a_tmem + 24, vd, idesc_pv, 1);
-        } else if constexpr (kTwoParts) {            // 32 keys: 16 columns of high parts, or of FP16 weights, then 16 of low parts
-          const uint32_t id0 = f16_0 ? idesc_pv16 : idesc_pv, id1 = f16_1 ? idesc_pv16 : idesc_pv;
-          mma_ts_off<0 * 128>(d_tmem, a_tmem + 0, vd, id0, accumulate ? 1u : 0u);
-          mma_ts_off<1 * 128>(d_tmem, a_tmem + 8, vd, id0, 1);
-          if (!f16_0) {
-            mma_ts_off<0 * 128>(d_tmem, a_tmem + 16, vd, id0, 1);
-            mma_ts_off<1 * 128>(d_tmem, a_tmem + 24, vd, id0, 1);
-          }
-          mma_ts_off<2 * 128>(d_tmem, a_tmem + 32, vd, id1, 1);
-          mma_ts_off<3 * 128>(d_tmem, a_tmem + 40, vd, id1, 1);
-          if (!f16_1) {
-            mma_ts_off<2 * 128>(d_tmem, a_tmem + 48, vd, id1, 1);
-            mma_ts_off<3 * 128>(d_tmem, a_tmem + 56, vd, id1, 1);
-          }
+        } else if constexpr (kTwoParts) {            // keys 0-31: high parts in columns 0-15, low ones in 16-31; keys 32-63: in the next 32
+          mma_ts_off<0 * 128>(d_tmem, a_tmem + 0, vd, idesc_pv, accumulate ? 1u : 0u);
+          mma_ts_off<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
+          mma_ts_off<0 * 128>(d_tmem, a_tmem + 16, vd, idesc_pv, 1);
+          mma_ts_off<1 * 128>(d_tmem, a_tmem + 24, vd, idesc_pv, 1);
+          mma_ts_off<2 * 128>(d_tmem, a_tmem + 32, vd, idesc_pv, 1);
+          mma_ts_off<3 * 128>(d_tmem, a_tmem + 40, vd, idesc_pv, 1);
+          mma_ts_off<2 * 128>(d_tmem, a_tmem + 48, vd, idesc_pv, 1);
+          mma_ts_off<3 * 128>(d_tmem, a_tmem + 56, vd, idesc_pv, 1);
         } else {
           mma_ts_off<0 * 128>(d_tmem, a_tmem + 0, vd, idesc_pv, accumulate ? 1u : 0u);
           mma_ts_off<1 * 128>(d_tmem, a_tmem + 8, vd, idesc_pv, 1);
@@ -1047,8 +990,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 if (first && hf == 0 && !(ok = cx.wait(kOFree + qt, sp ^ 1, 209))) break;
                 KVQ_STAMP(34);
                 tc_fence_after();
-                const int2 form = kTwoParts && t >= n_rt ? value_form(it, hf) : make_int2(0, 0);
-                issue_pv(s, hf, !(first && hf == 0), form.x, form.y);
+                issue_pv(s, hf, !(first && hf == 0));
               }
               if (op == 1 && leader) commit(kVEmpty + s);
               KVQ_STAMP(10 + qt);
@@ -1156,40 +1098,26 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             tmem_st16(s_addr + 64 * hf + c, hi);
             tmem_st16(s_addr + 64 * hf + c + 16, lo);
           };
-          const int2 form = kTwoParts && cached ? value_form(it, hf) : make_int2(0, 0);
-          if (kTwoParts && (odd_max || form.x != form.y)) {
+          if (D == 64 && odd_max) {
             // Rows whose scores so far are -inf, or so large that an FMA's exact product and the rounded maximum differ by more
             // than an exponential can take (a key masked with the lowest number): product and difference one by one, as in
-            // the warp-level kernel, which served heads of 64 channels before.  So are halves with values of both formats.
-            // Rolled, and the scores are fetched once more, so that the loops below keep their registers.
+            // the warp-level kernel, which served heads of 64 channels before.  Rolled, and the scores are fetched once more,
+            // so that the loop below keeps its registers.
             const float m = no_key_yet(m_run);
 #pragma unroll 1
             for (int c = 0; c < 64; c += 32) {
               uint32_t r[32], lo[16];
               tmem_ld32(s_addr + 64 * hf + c, r);
               tmem_wait_ld();
-              const bool f16 = c ? form.y : form.x;
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 const float x0 = c + i < nv ? __uint_as_float(r[i]) : -INFINITY, x1 = c + i + 1 < nv ? __uint_as_float(r[i + 1]) : -INFINITY;
                 const float p0 = ex2(__fsub_rn(__fmul_rn(x0, c_row), m)), p1 = ex2(__fsub_rn(__fmul_rn(x1, c_row), m));
                 sum2.x += p0; sum2.y += p1;
-                const uint32_t hi = split_bf16x2(make_float2(p0, p1), lo[i >> 1]);
-                r[i >> 1] = f16 ? cvt_f16x2(p0, p1) : hi;
+                r[i >> 1] = split_bf16x2(make_float2(p0, p1), lo[i >> 1]);
               }
               store_parts(c, r, lo);
             }
-          } else if (kTwoParts && form.x) {
-            const float2 c2 = make_float2(c_row, c_row), nm2 = make_float2(-m_run, -m_run);
-#pragma unroll
-            for (int i = 0; i < 64; i += 2) {
-              const float2 x = __ffma2_rn(make_float2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2);
-              const float2 pr = make_float2(ex2(x.x), ex2(x.y));
-              sum2 = __fadd2_rn(sum2, pr);
-              sr[i >> 1] = cvt_f16x2(pr.x, pr.y);
-            }
-            tmem_st16(s_addr + 64 * hf, sr);
-            tmem_st16(s_addr + 64 * hf + 32, sr + 16);
           } else {
             const float2 c2 = make_float2(c_row, c_row), nm2 = make_float2(-m_run, -m_run);
             uint32_t lo[16];
@@ -1331,14 +1259,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           load_raw_staged<BITS, G, D, kNW>(rk, raw_codes, raw_meta, raw_meta + kRawKZero, k_key,
                                         ct * kBlockN + k_key < p.n_cached, k_word0);
         }
-        bool values_f16 = false;
-        if (kTwoParts && ct >= 0) {              // each warp for its 32 keys; the issuers and the softmax warps follow
-          values_f16 = true;
-#pragma unroll
-          for (int j = 0; j < G; ++j) values_f16 &= value_exact_f16<BITS>(raw_zero<BITS, D>(rv, j));
-          values_f16 = __all_sync(0xFFFFFFFFu, values_f16);
-          if (lane == 0) reinterpret_cast<volatile int*>(smem + kOffForm)[(it & 3) * 4 + warp - 12] = values_f16;
-        }
         if (ct >= 0) {
           dequant_keys<BITS, GROUP, D, kNW>(rk, smem + kOffK + s * kTileBytes, k_row, k_word0);
           if (p.correction && k_word0 == 0) {   // B_extra row: step_j^2, exact in BF16
@@ -1383,8 +1303,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                                         ct * kBlockN + dt < p.n_cached, v_word0);
         }
         if (ct >= 0) {
-          if (kTwoParts && values_f16) dequant_values_f16<BITS, GROUP, D>(rv, smem + kOffV + s * kTileBytes, dt);
-          else dequant_values<BITS, GROUP, D, kNW>(rv, smem + kOffV + s * kTileBytes, dt, v_word0, v_piece0);
+          dequant_values<BITS, GROUP, D, kNW>(rv, smem + kOffV + s * kTileBytes, dt, v_word0, v_piece0);
           fence_proxy_async_smem();
           if (!PAIR && t + 1 < sg.te) load_raw<BITS, G, D, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v1), v1 < p.n_cached, v_word0);
           if constexpr (PAIR) {

@@ -167,9 +167,6 @@ __device__ __forceinline__ float no_key_yet(float m) { return m == __int_as_floa
 // zero and 16 + zero have 8 bits.  False for NaN and infinities.
 template <int BITS>
 __device__ __forceinline__ bool key_constant_exact(float zero) { return fabsf((BITS == 2 ? 4.f : 16.f) + zero) <= 112.f; }
-// Values without any rounding, in FP16 as in BF16: code - zero and a step have four bits each, the product eight, below 2^13.
-template <int BITS>
-__device__ __forceinline__ bool value_exact_f16(float zero) { return BITS == 2 ? fabsf(zero - 1.5f) <= 13.5f : fabsf(zero - 7.5f) <= 7.5f; }
 template <int BITS>
 __device__ __forceinline__ bool value_constant_exact(float zero) {
   return BITS == 2 ? fabsf(4.f + zero) <= 16.f : fabsf(16.f + zero - 15.5f) <= 240.5f;

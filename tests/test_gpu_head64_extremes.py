@@ -1,0 +1,33 @@
+"""Heads of 64 channels on the tcgen05 kernel: weights far below the largest of their row, and values that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1024, 65536])
+@pytest.mark.parametrize("bits_below", [0.0, 9.7, 16.3, 24.3, 25.2, 30.0, 60.4])
+def test_one_strong_key_over_many_weak_ones(n, bits_below):
+    """One current key whose value is zero, and n cached keys that many bits below it: the output is all theirs.  Each weight has
+    eight bits or more whatever its size, and their sum is counted in FP32, so the bound is that of a BF16 output, and twice over
+    for the FP32 score (an error of 2^-24 of 60 bits)."""
+    from paper_2605_26266_b200 import binding as B
+    heads, m = max(1, 16384 // n) * 5, 200                        # beyond the few-row kernel: more than 8 192 steps
+    assert heads * -(-m // 16) * (n // 32 + 1) > 8192
+    cache = B.Cache(1, heads, 64, 2, 64, n, rotate_k=False)
+    k = torch.zeros(1, heads, n, 64, device="cuda", dtype=torch.bfloat16)              # scores 0
+    v = (torch.arange(64, device="cuda") % 4).to(torch.bfloat16).expand(1, heads, n, 64).contiguous()      # step 1, zero-point 0: exact
+    B.kvq_quantize_append(cache, k, v)
+    q, kc, vc = (torch.zeros(1, heads, t, 64, device="cuda", dtype=torch.bfloat16) for t in (m, 1, 1))
+    q[..., 0], kc[..., 0] = 8.0, float(bits_below) * np.log(2.0)
+    lse = torch.zeros(1, heads, m, dtype=torch.float32, device="cuda")
+    mass = torch.zeros_like(lse)
+    out = B.kvq_attn_corrected(cache, q, kc, vc, 0.125, B.KVQ_CORRECTION_OFF, lse=lse, cached_mass=mass)
+    score = kc[0, 0, 0, 0].double().cpu()                                              # q . k / 8
+    weak = n * torch.exp(-score)
+    want = (weak / (1 + weak) * (torch.arange(64) % 4)).expand(1, heads, m, 64)
+    assert torch.equal(out.cpu()[..., ::4], torch.zeros(1, heads, m, 16, dtype=torch.bfloat16))
+    assert ((out.cpu().double() - want).abs() <= 2.0 ** -8 * want).all()
+    assert ((mass.cpu().double() - weak / (1 + weak)).abs() <= 1e-4 * weak).all()
+    assert ((lse.cpu().double() - (score + torch.log1p(weak))).abs() <= 1e-4).all()

@@ -1,9 +1,8 @@
 """The tcgen05 kernel for heads of 64 channels, which KVQ_KERNEL_AUTO takes for problems of more than a few thousand steps: enough
 heads that every shape below runs on it, rows and keys at the edges of its tiles, whole and split units, against the oracle on three
-of the heads.  Weights carry 11 bits (FP16) or 16 (two BF16 parts), so what is left of the error is the rounding of the output, which
-the test takes from the oracle's own result, and the FP16 rounding of the rotated query (a few per cent of it); with weights in
-one BF16 part it is 1.2 times that rounding.  Values far from zero are rounded to BF16 themselves: as much again, at most, where a row
-has one key."""
+of the heads.  Weights travel as two BF16 parts, so what is left of the error is the rounding of the output, which the test takes from the
+oracle's own result, and the FP16 rounding of the rotated query (a few per cent of it); with weights in one BF16 part it is 1.2
+times that rounding.  Values far from zero are rounded to BF16 themselves: as much again, at most, where a row has one key."""
 import numpy as np
 import pytest
 import torch
@@ -14,8 +13,7 @@ from tests import kvq_testlib as T
 
 pytestmark = pytest.mark.gpu
 
-# heads, rows, current keys, cached keys, bits, group, runs of 16 cached tokens, of six, whose values lie far from zero (these and
-# the 32 tokens a run falls into take two BF16 parts, the rest FP16 weights)
+# heads, rows, current keys, cached keys, bits, group, runs of 16 cached tokens, of six, whose values lie far from zero
 CASES = [(150, 65, 1, 129, 2, 64, 0), (150, 128, 64, 127, 4, 32, 0), (90, 129, 65, 300, 2, 32, 0), (90, 256, 128, 64, 4, 64, 0), (60, 257, 63, 0, 2, 64, 0),
          (40, 300, 300, 1500, 2, 64, 0), (150, 65, 1, 129, 2, 64, 1), (90, 129, 65, 300, 4, 32, 1), (40, 300, 300, 1500, 2, 32, 3)]
 
