@@ -250,10 +250,13 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
   return make_float2(__uint_as_float(__float_as_uint(q.x) + (__float_as_uint(fl.x) << 23)),
                      __uint_as_float(__float_as_uint(q.y) + (__float_as_uint(fl.y) << 23)));
 }
-// A pair of floats as two BF16 pairs: the high parts (cut, not rounded) are returned, `lo` is what they leave, rounded.
+// A pair of weights (not negative) as two BF16 pairs: the high parts (cut, not rounded) are returned, `lo` is what they leave, rounded.
+// A 2^-20 of the high part stays in it: the low part of a weight that a BF16 holds, 1 above all, would otherwise be 0, and with an
+// infinite value its product NaN.  So it is positive like the high part, down to weights of 2^-106; 2^-20 is nothing beside its rounding.
 __device__ __forceinline__ uint32_t split_bf16x2(float2 p, uint32_t& lo) {
+  constexpr float kCut = -(1.f - 0x1p-20f);
   const uint32_t a = __float_as_uint(p.x), b = __float_as_uint(p.y);
-  const float2 rest = __ffma2_rn(make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u)), make_float2(-1.f, -1.f), p);
+  const float2 rest = __ffma2_rn(make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u)), make_float2(kCut, kCut), p);
   lo = cvt_bf16x2(rest.x, rest.y);
   return __byte_perm(a, b, 0x7632);
 }

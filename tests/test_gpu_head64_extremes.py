@@ -31,3 +31,27 @@ def test_one_strong_key_over_many_weak_ones(n, bits_below):
     assert ((out.cpu().double() - want).abs() <= 2.0 ** -8 * want).all()
     assert ((mass.cpu().double() - weak / (1 + weak)).abs() <= 1e-4 * weak).all()
     assert ((lse.cpu().double() - (score + torch.log1p(weak))).abs() <= 1e-4).all()
+
+
+@pytest.mark.parametrize("kind", ["equal", "random", "one"])
+def test_infinite_values_stay_infinite(kind):
+    """A weight that is exactly 1, or has no more than eight bits, leaves nothing for its second part, and 0 * inf is NaN."""
+    from paper_2605_26266_b200 import binding as B
+    heads, m, n, n_cur = 75, 200, 200, 1 if kind == "one" else 130
+    g = torch.Generator(device="cuda").manual_seed(3)
+    draw = lambda t: torch.randn(1, heads, t, 64, device="cuda", generator=g).bfloat16()
+    cache = B.Cache(1, heads, 64, 2, 64, 256)
+    B.kvq_quantize_append(cache, draw(n), draw(n))
+    q, k, v = draw(m), draw(n_cur), draw(n_cur)
+    if kind == "equal":
+        q.zero_()                                                                      # every weight is 1
+    at = n_cur // 2
+    v[..., at, 3], v[..., at, 7], v[..., at, 40] = float("inf"), float("-inf"), float("nan")
+    v[..., 0, 50], v[..., n_cur - 1, 51] = float("inf"), float("-inf")
+    want = B.kvq_attn_corrected(cache, q, k, v, 0.125, B.KVQ_CORRECTION_ON | B.KVQ_KERNEL_MMA_SYNC)
+    got = B.kvq_attn_corrected(cache, q, k, v, 0.125, B.KVQ_CORRECTION_ON)
+    assert torch.isposinf(want[..., 3]).all() and torch.isneginf(want[..., 7]).all() and torch.isnan(want[..., 40]).all()
+    for same in (torch.isposinf, torch.isneginf, torch.isnan):
+        assert torch.equal(same(got), same(want))
+    finite = torch.isfinite(want)
+    assert (got[finite].float() - want[finite].float()).norm() < 1e-2 * want[finite].float().norm()
