@@ -271,7 +271,11 @@ def kvq_attn_corrected(cache: Cache, q, k_cur, v_cur, softmax_scale, flags=KVQ_C
             ws = _workspace(cache, status, stream, q.device)
         if status == KVQ_OK:
             return out
-    # not a plain call, or an error: checked and raised here
+        if status != _NOT_PLAIN:      # refused or failed, and not issued again; the size query is host arithmetic and tells which call it was
+            size = C.c_size_t(0)
+            _check(_attn_workspace_bytes(C.byref(cache.desc), n_cache, q.shape[2], k_cur.shape[2], flags, C.byref(size)), "kvq_attn_workspace_bytes")
+            _check(status, "kvq_attn_corrected")
+    # not a plain call: checked and raised here
     for t in (q, k_cur, v_cur):
         assert t.dtype is _BF16 and t.is_cuda
     kv_shape, kv_st = k_cur.shape, k_cur.stride()

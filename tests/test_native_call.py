@@ -31,6 +31,34 @@ def test_the_extension_is_the_one_that_runs_and_takes_plain_calls_only(B):
     assert cache.length == 0 and cache.workspace is None
 
 
+def test_a_call_that_fails_is_not_issued_again(B, monkeypatch):
+    """A status of the native call is raised as it is: some of its kernels may have been launched, and the second call's could
+    succeed."""
+    class OnDevice:                                              # as much of a tensor as the route up to the status looks at
+        is_cuda, dtype, device, shape = True, torch.bfloat16, "cuda:0", (1, 2, 16, 128)
+        stride, data_ptr = (lambda self: (4096, 2048, 128, 1)), (lambda self: 4096)
+    issued = []
+
+    def native(*args):
+        issued.append(args)
+        return B.KVQ_ERR_CUDA
+
+    def through_ctypes(*args):
+        issued.append(args)
+        return B.KVQ_OK
+    monkeypatch.setattr(B, "_attn_call", native)
+    monkeypatch.setattr(B, "_attn_corrected", through_ctypes)
+    monkeypatch.setattr(B, "_stream", lambda: 0)
+    cache, x = B.Cache(1, 2, 128, 2, 64, 128, device="cpu"), OnDevice()
+    cache.workspace = torch.empty(1 << 20, dtype=torch.uint8)
+    with pytest.raises(B.KvqError, match="kvq_attn_corrected") as e:
+        B.kvq_attn_corrected(cache, x, x, x, 0.1, cache_len=64, out=x)
+    assert e.value.status == B.KVQ_ERR_CUDA and len(issued) == 1
+    with pytest.raises(B.KvqError, match="kvq_attn_workspace_bytes"):        # refused before that: named as ever
+        B.kvq_attn_corrected(cache, x, x, x, 0.1, flags=1 << 20, cache_len=64, out=x)
+    assert len(issued) == 2
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("d,m,layout", [(128, 40, "dense"), (128, 300, "interleaved"), (64, 40, "padded"), (64, 700, "dense")])
 def test_both_routes_give_the_same_bytes(B, d, m, layout, monkeypatch):
