@@ -13,6 +13,8 @@ import os
 
 import torch
 
+from .build import py_call_target
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libkvq.so")
 
@@ -96,11 +98,13 @@ _BF16 = torch.bfloat16
 
 # The plain calls of the hot path go through a small CPython extension (csrc/py_call.cpp), which reads the tensors without the
 # Python-level accessors: a small append is a few microseconds of Python around a kernel of two (5.7 us a call through ctypes).
-# It answers _NOT_PLAIN to anything else (subclasses, other dtypes or layouts, whatever raises), and where it cannot be loaded
-# (a torch or Python it was not built for) every call takes the ctypes route below it.
+# It answers _NOT_PLAIN to anything else (subclasses, other dtypes or layouts, whatever raises), and where it cannot be loaded or
+# was built for another torch or Python every call takes the ctypes route below it.
 _NOT_PLAIN = -1000
 try:
     from . import _py_call
+    if getattr(_py_call, "built_for", None) != py_call_target(torch.__version__):
+        raise ImportError("_py_call is of another torch or Python")
     _py_call.bind(*(C.cast(f, C.c_void_p).value for f in (_quantize_append, _attn_workspace_bytes, _attn_corrected)))
     _append_call, _attn_call = _py_call.append, _py_call.attn
 except ImportError:

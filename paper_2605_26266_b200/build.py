@@ -21,7 +21,15 @@ NVCC_FLAGS = [
 ]
 
 
-PY_CALL = os.path.join(PKG, "_py_call.so")     # the argument marshalling of binding.py
+PY_CALL = os.path.join(PKG, "_py_call" + sysconfig.get_config_var("EXT_SUFFIX"))     # the argument marshalling of binding.py
+PY_CALL_FLAGS = ["-O2", "-std=c++17", "-shared", "-fPIC"]
+PY_CALL_LIBS = ["-ltorch_python", "-ltorch_cpu", "-lc10"]
+
+
+def py_call_target(torch_version: str) -> str:
+    """What the extension is compiled for.  It reads torch's and Python's objects by their layout, so binding.py compares this with the
+    string that was compiled in before it uses it."""
+    return f"torch {torch_version} python {sys.hexversion:#x}"
 
 
 def _nvcc() -> str:
@@ -103,9 +111,10 @@ def _build_py_call(force: bool, verbose: bool) -> None:
     import torch
 
     src, t = os.path.join(CSRC, "py_call.cpp"), os.path.dirname(torch.__file__)
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(t, "include"),
-           "-I", os.path.join(ROOT, "include"), src, "-o", PY_CALL, "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
-    d = _digest([src, os.path.join(ROOT, "include", "kvq.h")], torch.__version__ + sys.version)
+    target = py_call_target(torch.__version__)
+    cmd = ["g++"] + PY_CALL_FLAGS + [f'-DKVQ_BUILT_FOR="{target}"', "-I", sysconfig.get_paths()["include"], "-I", os.path.join(t, "include"),
+           "-I", os.path.join(ROOT, "include"), src, "-o", PY_CALL, "-L", os.path.join(t, "lib")] + PY_CALL_LIBS
+    d = _digest([src, os.path.join(ROOT, "include", "kvq.h")], " ".join([target] + PY_CALL_FLAGS + PY_CALL_LIBS))
     if force or not _current(PY_CALL, d):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or r.returncode != 0:

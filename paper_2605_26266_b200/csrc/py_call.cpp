@@ -122,4 +122,10 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_py_call", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__py_call(void) { return PyModule_Create(&module); }
+// Nothing of torch's layout is touched here: binding.py looks at built_for (the torch and the Python of the headers above) before it
+// calls anything else.
+PyMODINIT_FUNC PyInit__py_call(void) {
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "built_for", KVQ_BUILT_FOR) < 0) { Py_DECREF(m); return nullptr; }
+  return m;
+}

@@ -1,4 +1,7 @@
 """The CPython extension behind the binding: it takes plain calls only, and what it takes gives the bytes of the ctypes route."""
+import runpy
+import types
+
 import pytest
 import torch
 
@@ -29,6 +32,22 @@ def test_the_extension_is_the_one_that_runs_and_takes_plain_calls_only(B):
         with pytest.raises(AssertionError):
             B.kvq_attn_corrected(cache, x, k, v, 0.1, out=x)
     assert cache.length == 0 and cache.workspace is None
+
+
+@pytest.mark.parametrize("built_for", [None, "torch 1.0 python 0x30c03f0"])
+def test_an_extension_of_another_torch_or_python_is_not_used(B, monkeypatch, built_for):
+    """It would load and read tensors by the layout it was compiled with."""
+    import paper_2605_26266_b200 as package
+
+    def used(*_):
+        raise AssertionError("used")
+    other = types.ModuleType("_py_call")
+    other.bind = other.append = other.attn = used
+    if built_for:
+        other.built_for = built_for
+    monkeypatch.setattr(package, "_py_call", other, raising=False)
+    again = runpy.run_path(B.__file__, run_name=B.__name__)                    # the module once more, beside the one that is loaded
+    assert again["_append_call"]() == again["_attn_call"]() == B._NOT_PLAIN
 
 
 def test_a_call_that_fails_is_not_issued_again(B, monkeypatch):
