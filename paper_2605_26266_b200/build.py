@@ -8,6 +8,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -103,7 +104,13 @@ def _build_locked(force: bool, verbose: bool) -> str:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
         _stamp(LIB, lib_digest)
-    _build_py_call(force, verbose)
+    try:
+        _build_py_call(force, verbose)
+    except (ImportError, OSError, RuntimeError) as e:      # no torch, no g++, no Python.h
+        for f in (PY_CALL, PY_CALL + ".stamp"):            # of other sources, if there is one
+            if os.path.exists(f):
+                os.remove(f)
+        warnings.warn(f"{os.path.basename(PY_CALL)} was not built ({e}); binding.py calls libkvq.so through ctypes, a few microseconds slower")
     return LIB
 
 

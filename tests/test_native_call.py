@@ -50,6 +50,27 @@ def test_an_extension_of_another_torch_or_python_is_not_used(B, monkeypatch, bui
     assert again["_append_call"]() == again["_attn_call"]() == B._NOT_PLAIN
 
 
+@pytest.mark.parametrize("how", ["no compiler", "no Python.h"])
+def test_the_library_is_built_without_the_extension(B, monkeypatch, tmp_path, how):
+    """The library is complete without it, and the binding has its ctypes route; a file of former sources is not left behind."""
+    from paper_2605_26266_b200 import build
+    run = build.subprocess.run
+
+    def without_gxx(cmd, **kw):
+        if cmd[0] != "g++":
+            return run(cmd, **kw)
+        if how == "no compiler":
+            raise FileNotFoundError("g++")
+        return build.subprocess.CompletedProcess(cmd, 1, "", "Python.h: No such file or directory")
+    former = tmp_path / "_py_call.so"
+    former.write_bytes(b"former")
+    monkeypatch.setattr(build, "PY_CALL", str(former))
+    monkeypatch.setattr(build.subprocess, "run", without_gxx)
+    with pytest.warns(UserWarning, match="ctypes"):
+        assert build.build_library() == build.LIB
+    assert not former.exists()
+
+
 def test_a_call_that_fails_is_not_issued_again(B, monkeypatch):
     """A status of the native call is raised as it is: some of its kernels may have been launched, and the second call's could
     succeed."""
