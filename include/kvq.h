@@ -16,6 +16,15 @@
  *   - The caller owns every buffer.  The library allocates no device memory,
  *     never synchronises and only enqueues work on the given stream.  Calls that
  *     touch one cache must be ordered by the caller (same stream or events).
+ *   - The first kernel of a call is launched programmatically
+ *     (cudaLaunchAttributeProgrammaticStreamSerialization): it is placed while the
+ *     kernel before it in the stream drains, and waits for the end of that kernel
+ *     before it touches any memory.  That orders it behind everything earlier too,
+ *     unless the kernel directly before it is itself launched programmatically and
+ *     ends without any of its blocks having waited (griddepcontrol.wait,
+ *     cudaGridDependencySynchronize): such a kernel may end ahead of the one it
+ *     overlaps.  Put an ordinary launch between it and the call.  The kernels of
+ *     this library always wait.
  *   - Argument errors are detected on the host before anything is launched and
  *     leave all buffers untouched.  A CUDA launch error is returned as
  *     KVQ_ERR_CUDA; kvq_last_cuda_error() gives the cudaError_t value.
