@@ -52,6 +52,44 @@ def test_kernels_that_wait_read_with_ordinary_loads(name):
     assert pre_pass.index("wait_for_previous_grid();") < pre_pass.index("allow_next_grid();") < pre_pass.index("load_coherent(")
 
 
+def kernels(text):
+    """(name, body) of every __global__ function."""
+    for m in re.finditer(r"__global__ void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\(", text):
+        i = text.index("{", text.index(") {", m.end()))
+        depth, j = 1, i + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[j], 0)
+            j += 1
+        yield m.group(1), text[i:j]
+
+
+def without_wait(text):
+    """Kernels that are not launched the ordinary way and touch memory, or let the next grid start, without having waited."""
+    out = []
+    for name, body in kernels(text):
+        if re.search(rf"\b{name}(<[^;{{}}<>]*>)?<<<", text):
+            continue
+        wait = body.find("wait_for_previous_grid();")
+        if wait < 0 or 0 <= body.find("allow_next_grid();") < wait:
+            out.append(name)
+    return out
+
+
+def test_every_kernel_that_may_start_early_waits():
+    found = set()
+    for name in sorted(n for n in os.listdir(CSRC) if n.endswith(".cu")):
+        text = source(name)
+        assert without_wait(text) == []
+        early = {k for k, body in kernels(text) if "wait_for_previous_grid();" in body}
+        for m in [m.start() for m in re.finditer(r"wait_for_previous_grid\(\);", text)]:      # the check sees a missing one
+            cut = text[:m] + text[m + len("wait_for_previous_grid();"):]
+            kernel = next(k for k, body in kernels(text) if text.index(body) <= m < text.index(body) + len(body))
+            assert without_wait(cut) == [kernel] or kernel == "attn_tcgen05_kernel"            # which waits in several roles
+        found |= early
+    assert found == {"attn_short_kernel", "attn_short_merge_kernel", "rotate_query_kernel", "attn_tcgen05_kernel", "attn_merge_kernel",
+                     "quantize_append_kernel"}
+
+
 def test_both_ctas_of_a_pair_wait_for_the_last_commits():
     """Commits of a pair (tc_commit_pair) arrive on the barriers of both CTAs at times of their own.  The leader drains its copy of
     the last ones; the peer has to drain its own before the cluster barrier that lets it leave."""
