@@ -252,7 +252,7 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
 }
 // A pair of weights (not negative) as two BF16 pairs: the high parts (cut, not rounded) are returned, `lo` is what they leave, rounded.
 // A 2^-20 of the high part stays in it: the low part of a weight that a BF16 holds, 1 above all, would otherwise be 0, and with an
-// infinite value its product NaN.  So it is positive like the high part, down to weights of 2^-106 (of at most 1); 2^-20 is nothing beside its rounding.
+// infinite value its product NaN.  So it is positive like the high part, down to weights of 2^-106; 2^-20 is nothing beside its rounding.
 __device__ __forceinline__ uint32_t split_bf16x2(float2 p, uint32_t& lo) {
   constexpr float kCut = -(1.f - 0x1p-20f);
   const uint32_t a = __float_as_uint(p.x), b = __float_as_uint(p.y);
@@ -1042,7 +1042,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     int it = 0, nseg = 0;
     bool ok = qt < p.n_qt;                                    // a tile without rows: nothing to do
     while (ok && sch.next(sg)) {
-      float m_run = -INFINITY, lcur = 0.f, lcac = 0.f;   // running max (log2 units; 64 channels: 8 above it), row sums over current / cached keys
+      float m_run = -INFINITY, lcur = 0.f, lcac = 0.f;   // running max (log2 units), row sums over current / cached keys
       bool fresh = true;                                 // no product has been added to O in this segment yet
       bool odd_max = true;                               // 64 channels: a maximum of the warp is -inf (no key yet) or very large
       for (int t = sg.tb; ok && t < sg.te; ++t, ++it) {
@@ -1072,10 +1072,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
             for (int c = 0; c < 4; ++c) mx[c] = max3(mx[c], __uint_as_float(sr[i + 2 * c]), __uint_as_float(sr[i + 2 * c + 1]));
           }
-          // 64 channels: weights are taken against 2^8 times the lazy maximum, so that none exceeds 1 and the product with the largest
-          // value a BF16 holds is finite, as it was with the exact maximum
-          const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-          const float m_new = fmaxf(m_run, D == 64 ? fmaf(top, c_row, kRescaleThreshold) : top * c_row);
+          const float m_new = fmaxf(m_run, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * c_row);
           if (__any_sync(0xFFFFFFFFu, m_new - m_run > kRescaleThreshold)) {
             if (D == 64) odd_max = __any_sync(0xFFFFFFFFu, !(fabsf(m_new) < 0x1p24f));
             if (!fresh) {
