@@ -46,7 +46,7 @@
 // The same source also gives the pair kernel (template parameter PAIR): a cluster of two CTAs on 512 query rows
 // whose tensor cores work as one (tcgen05 cta_group::2), described at the kernel; and the kernel for heads of 64
 // channels (D = 64, one CTA per unit): operand tiles one 64-column block wide at the same places, half the MMA steps of a
-// score, 16 heads x 1560 queries over 7 700 keys in 129 us against 650 us in the warp-level kernel.
+// score, 16 heads x 1560 queries over 7 700 keys in 130 us against 650 us in the warp-level kernel.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA records a diagnostic in the caller's status
 // word, all roles leave their loops, in-flight work is drained with a bounded wait, TMEM is freed and the
@@ -250,11 +250,15 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
   return make_float2(__uint_as_float(__float_as_uint(q.x) + (__float_as_uint(fl.x) << 23)),
                      __uint_as_float(__float_as_uint(q.y) + (__float_as_uint(fl.y) << 23)));
 }
-// A pair of weights (not negative) as two BF16 pairs: the high parts (cut, not rounded) are returned, `lo` is what they leave, rounded.
-// A 2^-20 of the high part stays in it: the low part of a weight that a BF16 holds, 1 above all, would otherwise be 0, and with an
-// infinite value its product NaN.  So it is positive like the high part, down to weights of 2^-106; 2^-20 is nothing beside its rounding.
-__device__ __forceinline__ uint32_t split_bf16x2(float2 p, uint32_t& lo) {
+// A pair of weights (not negative, at most 2^8), times kPartScale, as two BF16 pairs: the high parts (cut, not rounded) are returned,
+// `lo` is what they leave, rounded.  The scale keeps the product of the largest weight with the largest value a BF16 holds finite, as it
+// was with the exact maximum, whose weights are at most 1; O is scaled back where it is normalised.
+// A 2^-20 of the high part stays in the low one: that of a weight that a BF16 holds, 1 above all, would otherwise be 0, and with an
+// infinite value its product NaN.  So it is positive like the high part, down to weights of 2^-98; 2^-20 is nothing beside its rounding.
+constexpr float kPartScale = 0x1p-8f;
+__device__ __forceinline__ uint32_t split_bf16x2(float2 w, uint32_t& lo) {
   constexpr float kCut = -(1.f - 0x1p-20f);
+  const float2 p = __fmul2_rn(w, make_float2(kPartScale, kPartScale));
   const uint32_t a = __float_as_uint(p.x), b = __float_as_uint(p.y);
   const float2 rest = __ffma2_rn(make_float2(__uint_as_float(a & 0xFFFF0000u), __uint_as_float(b & 0xFFFF0000u)), make_float2(kCut, kCut), p);
   lo = cvt_bf16x2(rest.x, rest.y);
@@ -685,7 +689,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // than the warp-level kernel's, which served them before, unless the running maximum was followed exactly (the largest
   // weight is then 1, without a rounding), and an exact maximum rescales O in half of the steps.  16 x 1560 queries over 6 144 tokens,
   // error against 64 bits: 141 us and 1.82e-3 exact with one part, 120 us and 2.01e-3 lazy with one part, 134 us and 1.72e-3
-  // lazy with two (1.66e-3 of it is the rounding of the output); 129 us since the launches of a call overlap those before it.
+  // lazy with two (1.66e-3 of it is the rounding of the output); 130 us as here, since the launches of a call overlap those before it.
   // FP16 weights, against cached values that are exact in FP16, took 4 % less, but FP16 ends at 2^-24: keys that far below the
   // largest of their row, which may be all there is where that key's value is zero, were lost or a quarter too large.
   constexpr bool kTwoParts = D == 64;
@@ -1154,7 +1158,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // a whole unit writes its rows of the output; a partial segment writes the same normalised rows into its
       // slot, with the statistics the merge kernel weighs them by
       const float l = lcur + lcac;
-      const float inv = D == 64 && !whole && l == 0.f ? 0.f : 1.0f / l;      // a range without a weight adds nothing
+      const float inv = D == 64 && !whole && l == 0.f ? 0.f : (kTwoParts ? 1.0f / kPartScale : 1.0f) / l;      // a range without a weight adds nothing
       const bool store = !whole || row < p.m_tokens;
       // consecutive 8-column pieces: 16 bytes apart in a row of the output, 4096 bytes apart in a slot
       uint8_t* dst = whole ? reinterpret_cast<uint8_t*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)row * p.o_st)

@@ -1,4 +1,5 @@
-"""Heads of 64 channels on the tcgen05 kernel: weights far below the largest of their row, and values that are not finite."""
+"""Heads of 64 channels on the tcgen05 kernel: weights far below the largest of their row, and values that are not finite or
+the largest a BF16 holds."""
 import numpy as np
 import pytest
 import torch
@@ -55,3 +56,21 @@ def test_infinite_values_stay_infinite(kind):
         assert torch.equal(same(got), same(want))
     finite = torch.isfinite(want)
     assert (got[finite].float() - want[finite].float()).norm() < 1e-2 * want[finite].float().norm()
+
+
+@pytest.mark.parametrize("rise", [1.0, 3.5, 7.5, 20.0])
+def test_the_largest_values_stay_finite(rise):
+    """A key some bits above those before it has a weight of at most 1, so that its value may be the largest BF16 number."""
+    from paper_2605_26266_b200 import binding as B
+    heads, m, n_cur, n = 75, 200, 130, 64
+    cache = B.Cache(1, heads, 64, 2, 64, 128)
+    zeros = lambda t: torch.zeros(1, heads, t, 64, device="cuda", dtype=torch.bfloat16)
+    B.kvq_quantize_append(cache, zeros(n), zeros(n))
+    q, k, v = zeros(m), zeros(n_cur), zeros(n_cur)
+    q[..., 0], k[..., 100, 0] = 8.0, rise * np.log(2.0)                               # the other scores are 0
+    largest = torch.finfo(torch.bfloat16).max
+    v[..., 100, 3], v[..., 100, 7] = largest, -largest
+    want = B.kvq_attn_corrected(cache, q, k, v, 0.125, B.KVQ_CORRECTION_OFF | B.KVQ_KERNEL_MMA_SYNC)
+    got = B.kvq_attn_corrected(cache, q, k, v, 0.125, B.KVQ_CORRECTION_OFF)
+    assert torch.isfinite(want).all() and torch.isfinite(got).all()
+    assert ((got - want).double().abs() <= 2.0 ** -7 * want.double().abs()).all()
