@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
       const bool have = has_part(c0 + j);
       const uint8_t* sl = slot_of(have ? c0 + j : c_last);
       const float* st = reinterpret_cast<const float*>(sl + kSlotStats);
-      sm[j] = have ? st[r256] : -INFINITY;                  // weight 2^(-inf) = 0 for the slots that are not there
+      sm[j] = have ? st[r256] : -INFINITY;                  // not a maximum
       sc[j] = st[256 + r256]; sa[j] = st[512 + r256];
       a[j] = *reinterpret_cast<const uint4*>(sl + ((size_t)cg * 256 + r256) * 16);
     }
@@ -1430,6 +1430,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
     if (c0 != c_first) fetch(c0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+      if (!has_part(c0 + j)) continue;                      // the whole block: the last range's rows again, and 0 * inf would be NaN
       const float f = exp2f(sm[j] - m);
       const float lc = f * sc[j], la = f * sa[j];
       l_cur += lc; l_cac += la;

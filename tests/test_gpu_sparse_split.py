@@ -1,5 +1,6 @@
 """A last round with fewer tile steps than CTAs: some of the ranges it is cut into are empty, and the slots of their CTAs must not
-reach the merge.  The workspace is filled with NaN, or with the finite partial rows of another problem, before the call."""
+reach the merge.  The workspace is filled with NaN, or with the finite partial rows of another problem, before the call.  Nor do the
+places beyond the last range."""
 import numpy as np
 import pytest
 import torch
@@ -43,3 +44,23 @@ def test_empty_ranges_of_the_last_round(d, heads, m, n, bits, kernel):
         assert np.abs(lse.cpu().numpy()[0][picked][:, rows] - want["lse"]).max() < 2e-2
         first = out if first is None else first
         assert torch.equal(out.view(torch.int16), first.view(torch.int16))
+
+
+@pytest.mark.parametrize("d,heads,m,n,n_cur", [(64, 8, 300, 0, 4000), (64, 8, 300, 256, 2000), (128, 8, 300, 0, 4000), (128, 8, 300, 0, 2000), (128, 3, 600, 0, 5000)])
+def test_infinite_values_in_the_last_range_of_a_unit(d, heads, m, n, n_cur):
+    """Ranges are merged four at a time, and the places of the last four that are empty repeat the last range with weight zero."""
+    from paper_2605_26266_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(4)
+    draw = lambda t: torch.randn(1, heads, t, d, device="cuda", generator=g).bfloat16()
+    cache = B.Cache(1, heads, d, 2, 64, 256)
+    if n:
+        B.kvq_quantize_append(cache, draw(n), draw(n))
+    q, k, v = draw(m), draw(n_cur), draw(n_cur)
+    v[..., n_cur - 1, 3], v[..., n_cur - 1, d - 2], v[..., 0, 5] = float("inf"), float("-inf"), float("inf")
+    want = B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, B.KVQ_CORRECTION_OFF | B.KVQ_KERNEL_MMA_SYNC)
+    assert torch.isposinf(want[..., 3]).all() and torch.isneginf(want[..., d - 2]).all() and torch.isposinf(want[..., 5]).all()
+    kernels = [0] if d == 64 else [0, B.KVQ_KERNEL_TCGEN05, B.KVQ_KERNEL_TCGEN05_PAIR]
+    for kernel in kernels:
+        got = B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, B.KVQ_CORRECTION_OFF | kernel)
+        for same in (torch.isposinf, torch.isneginf, torch.isnan):
+            assert torch.equal(same(got), same(want))
