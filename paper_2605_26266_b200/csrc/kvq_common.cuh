@@ -111,7 +111,11 @@ int launch_after(bool overlap, int cluster, dim3 grid, dim3 block, size_t smem, 
     ++n;
   }
   cfg.attrs = attr; cfg.numAttrs = n;
-  KVQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess) {
+    cudaGetLastError();                                // or the next call's ordinary launch would report it again
+    return record_cuda_error(e);
+  }
   return KVQ_OK;
 }
 
