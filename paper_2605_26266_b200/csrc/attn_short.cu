@@ -15,10 +15,11 @@
 // part, step^2 is exact in BF16).  Ranges of one (batch, head) leave FP32 partial rows that a second kernel, or in small
 // problems the cluster of their CTAs, merges in a fixed order.
 //
-// What bounds it: instruction issue and latency (37 warp instructions per key and 16 rows at 4 bits, half of them the
+// What bounds it: instruction issue and latency (36 warp instructions per key and 16 rows at 4 bits, half of them the
 // expansion of the codes; two CTAs of four warps an SM, the ALU pipe half busy), then HBM.  16 rows over 16 384 tokens
-// of 32 heads at 4 bits, group 128: 37.5 us with the merge, against 97 us in the tcgen05 kernel; three CTAs with spilled
-// registers 12 % slower (without spills, the query in shared memory, 5 %), four 80 %; the four score tiles of a step one after the other instead of in turn 7 %.
+// of 32 heads at 4 bits, group 128: 41 us with the merge where inputs change from call to call, 39 on the same ones (at 2 bits, group
+// 64, 36 against 58 in the tcgen05 kernel); three CTAs with spilled registers 12 % slower (without spills, the query in shared
+// memory, 5 %), four 80 %; the four score tiles of a step one after the other instead of in turn 7 %.
 #include <cuda_fp16.h>
 
 #include <type_traits>
@@ -681,20 +682,23 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   if ((flags & KVQ_KERNEL_MASK) != KVQ_KERNEL_AUTO || (flags & KVQ_CORRECTION_EXACT) || (d->flags & KVQ_K_PER_CHANNEL) || m_tokens < 1)
     return false;
   // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
-  // prologue and a larger merge.  Measured with both kernels as they are, 2 to 1024 heads (us here against there, 128 channels, 2
-  // bits): one block of rows is 1 to 2 times as fast here.  Two are up to about 4 200 (head, 128-key tile) pairs (48 against 50
-  // at 2 080 of 32 heads, 4 bits 87 against 93 at 4 160 of 64; 149 against 142 at 8 224), three up to 1 200 (47 against 48 at 1 088),
-  // four up to 400 (22 against 28 at 130, 22 against 22 at 320, 34 against 28 at 544), as long as all CTAs run at once: 32 rows
-  // of 160 heads take 18 against 15 at 160 pairs, 242 against 179 at 10 400.  64 channels, where the other kernel has more fixed
-  // cost to each tile, stay ahead further: two blocks 69 against 73 at 4 160, 141 against 157 at 10 400 of 160 heads.
+  // prologue and a larger merge.  Both kernels as they are, device time of a call among others on the same inputs (us here /
+  // there, 128 channels, 2 bits, group 64): one block of rows is faster here (32 heads over 16 384 keys 36 / 58, over none 4.9 / 5.8).
+  // The lines for two blocks (4 200 (head, 128-key tile) pairs), three (1 200) and four (400), as long as all CTAs run at once, were
+  // drawn when launches did not overlap those before them yet, which the other kernel's chain of three gained more from; now
+  // two blocks meet at some 1 100 pairs (32 heads 25 / 25 at 1 056, 40 / 37 at 2 080, 70 / 58 at 4 128), three at 600 (20 / 20 at
+  // 544, 29 / 25 at 1 056), four at 400 (18 / 21 at 288, 14 / 15 at 320, 22 / 21 at 576).  64 channels, where the other kernel has more
+  // fixed cost to each tile, stay ahead further: two blocks 29 / 40 at 2 080, 50 / 62 at 4 128, 123 / 136 at 10 400 of 160 heads.
   const int64_t blocks = (m_tokens + kRows - 1) / kRows;
   if (blocks == 1) return true;
   // Small problems, whatever the rows: all CTAs run at once and each has few steps, while the other kernel is a chain of three
-  // launches with a prologue of microseconds each.  Counted in steps of 32 keys over all blocks of 16 rows (device time, us, here
-  // against there, 2 bits; 4 bits alike): 64 channels 2 heads x 256 rows over 1 024 keys 8 / 15, at 4 608 steps 14 / 17, at 8 192
-  // 16 / 18, at 8 704 19 / 19, at 10 240 22 / 18; 128 channels at 1 056 steps 11 / 18, at 4 224 17 / 19, at 4 608 19 / 22, at 6 432
-  // 20 / 19, at 8 320 24 / 21.  For 128 channels only up to the 128 rows of one query tile of the other kernel, half of which
-  // idles there.
+  // launches with a prologue of microseconds each.  Counted in steps of 32 keys over all blocks of 16 rows (as above; 4 bits
+  // alike): 64 channels 2 heads x 256 rows over 1 024 keys, 1 280 steps, 7.5 / 14.6; at 4 352 steps 12 / 18; at 5 120 13 / 15 to 14 /
+  // 15; at 8 192 the other kernel's units of 256 rows decide, 17 / 27 with one (16 384 keys), 17 / 22 with two, 17 / 16 with sixteen (8
+  // heads x 512 rows over 512 keys; 2 x 1 000 over 1 024 18 / 15, the worst met); at 10 240 21 / 16 and 22 / 17.  128 channels at 1 056
+  // steps 11 / 17, at 4 224 17 / 18, at 4 608 18 / 21, at 6 432 20 / 18; over an empty cache, where the other kernel is one launch as
+  // well, 5.8 / 6.6 for 16 heads x 128 rows and 7.6 / 6.6 for 32.  For 128 channels only up to the 128 rows of one query tile of the
+  // other kernel, half of which idles there.
   const int64_t bh = (int64_t)d->batch * d->heads;
   const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
   if (d->head_dim == 64) {

@@ -689,7 +689,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // than the warp-level kernel's, which served them before, unless the running maximum was followed exactly (the largest
   // weight is then 1, without a rounding), and an exact maximum rescales O in half of the steps.  16 x 1560 queries over 6 144 tokens,
   // error against 64 bits: 141 us and 1.82e-3 exact with one part, 120 us and 2.01e-3 lazy with one part, 134 us and 1.72e-3
-  // lazy with two (1.66e-3 of it is the rounding of the output); 130 us as here, since the launches of a call overlap those before it.
+  // lazy with two (1.66e-3 of it is the rounding of the output), all on the same inputs again and again; 130 us as here, since the
+  // launches of a call overlap those before it.
   // FP16 weights, against cached values that are exact in FP16, took 4 % less, but FP16 ends at 2^-24: keys that far below the
   // largest of their row, which may be all there is where that key's value is zero, were lost or a quarter too large.
   constexpr bool kTwoParts = D == 64;
@@ -1181,8 +1182,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 make_float4(__uint_as_float(sr[i]) * inv, __uint_as_float(sr[i + 1]) * inv, __uint_as_float(sr[i + 2]) * inv, __uint_as_float(sr[i + 3]) * inv);
         } else if (PAIR && store && whole && p.out_32) {
           // A lane holds a row, so that the 32 lanes of a store meet 32 lines, and the load/store unit takes these one by one: with
-          // 32 bytes a lane there are half as many to take (64 heads x 2048 rows over an empty cache 166 -> 163 us).  In the pair
-          // kernel only: the one-CTA kernel's code came out 1 % slower with it, and splits most of its units.
+          // 32 bytes a lane there are half as many to take (64 heads x 2048 rows over an empty cache, the same again and again, 166 ->
+          // 163 us).  In the pair kernel only: the one-CTA kernel's code came out 1 % slower with it, and splits most of its units.
 #pragma unroll
           for (int i = 0; i < 64; i += 16) {
             uint32_t w[8];
@@ -1391,7 +1392,8 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   // Partials are taken four at a time with all of their loads issued before any is used: a thread moves only
   // 16 bytes per partial, so the kernel lives on loads in flight.  The first four, mostly all, are fetched once, rows and
   // statistics together; with the maximum from a pass of its own, FP64 divisions above and the wait in front of them, 16 heads x
-  // 1560 rows took 123.4 us (122.0 as here), of 64 channels 126.6 (124.3).
+  // 1560 rows took 1 to 2 % more on the same inputs again and again (123.4 against 122.0 us; where inputs change, 129 us, the
+  // difference is within what two runs differ by).
   // CTA c of the schedule is CTA kc * c + rank of the grid; every CTA of the grid has two slots
   auto slot_of = [&](int c) { return p.partial + (size_t)(2 * (kc * c + rank) + (c == c_first ? first_slot : 0)) * kSlotBytes; };
   // With fewer tile steps than CTAs (a last round of few units of few tiles) some ranges between the first and the last are

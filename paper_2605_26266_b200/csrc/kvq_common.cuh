@@ -126,8 +126,8 @@ int launch_after(bool overlap, int cluster, dim3 grid, dim3 block, size_t smem, 
 // memory, and only then allows the next grid, so that the call's later kernels may read the caller's tensors without waiting again.
 // The wait is for the grid directly before; that one's end implies the end of what lies before it, as with an ordinary launch, unless it
 // overlaps that and never waited, which kvq.h therefore asks callers not to put right in front of a call.
-// Among other calls (24 heads x 4680 tokens, 16 heads x 1560 rows, 64 heads x 2048 rows, us): append 21.6 -> 19.6, attention
-// 125.4 -> 123.6, 64 channels 134.5 -> 130.5, empty cache 167 -> 163.5.
+// Among other calls on the same inputs (24 heads x 4680 tokens, 16 heads x 1560 rows, 64 heads x 2048 rows, us): append 21.6 ->
+// 19.6, attention 125.4 -> 123.6, 64 channels 134.5 -> 130.5, empty cache 167 -> 163.5.
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // How a kernel that waits there reads what a grid before may have written: with an ordinary load.  The read-only path (`__ldg`,

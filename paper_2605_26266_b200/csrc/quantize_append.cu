@@ -14,8 +14,9 @@
 // the two halves of 64-bit registers and does everything but the last in-lane butterfly stage and the minimum/maximum
 // with the packed instructions (add/mul/fma.rn.f32x2: two IEEE operations each), and adds the zero-point, clamps and packs
 // the codes two at a time as 16-bit integers.  Measured at 24 heads x 4680 tokens, 128 channels, 2 bits, group 64
-// (66 MB): 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile; 23.6 us as here (2.8 TB/s; 19.6 us
-// where launches overlap, see launch_after, 18.0 us with 32 bytes a load),
+// (66 MB), the same inputs again and again: 36.9 us with one IEEE operation per instruction, persistent blocks and a staged tile;
+// 23.6 us without either (19.6 us where launches overlap, see launch_after, and 18.0 us as here, with 32 bytes a load; 20.2 us, 3.27
+// TB/s, where inputs change from call to call),
 // 3 % more with eight lanes per vector (shorter lanes repeat the per-group work more often); two
 // tokens in flight per lane and persistent warps with a prefetch: 26.6 us (fewer warps fit).
 #include <math_constants.h>
@@ -202,7 +203,8 @@ __device__ __forceinline__ void load_raw_vec(RawVec<EPL>& v, const uint16_t* p, 
   for (int i = 0; i < EPL / 8; ++i) v.r[i] = load_coherent(reinterpret_cast<const uint4*>(p) + lv * (EPL / 8) + i);
 }
 // The same with 32 bytes an instruction, from rows on 32-byte boundaries: a lane's channels are 64 bytes (32), so that an instruction of
-// 16 bytes a lane meets every line of eight tokens and takes a quarter of it.  24 heads x 4680 tokens, 128 channels: 19.6 -> 18.0 us.
+// 16 bytes a lane meets every line of eight tokens and takes a quarter of it.  24 heads x 4680 tokens, 128 channels, the same again and
+// again: 19.6 -> 18.0 us.
 template <int EPL>
 __device__ __forceinline__ void load_raw_vec_32(RawVec<EPL>& v, const uint16_t* p, int lv) {
 #pragma unroll
