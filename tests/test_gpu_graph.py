@@ -90,3 +90,64 @@ def test_auto_kernels_replayed_from_a_graph(d, heads, tokens):
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
+@pytest.mark.parametrize("d,heads,m,n", [(64, 2, 256, 1024), (128, 32, 16, 8192), (128, 16, 300, 3072), (128, 24, 1024, 2048), (128, 40, 700, 0), (64, 40, 300, 1024)])
+def test_calls_behind_joins(d, heads, m, n):
+    """Calls whose first kernel follows two nodes (a join of two streams) or a copy: the bytes of the synchronised chain, eager and
+    replayed."""
+    from paper_2605_26266_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(31)
+    draw = lambda t: torch.randn(1, heads, t, d, device="cuda", generator=g).bfloat16()
+    cache = B.Cache(1, heads, d, 2, 64, (max(n, 128) + 127) // 128 * 128 + 1024)
+    past = draw(max(n, 16)), draw(max(n, 16))
+    q0, k0, v0 = draw(m), draw(m), draw(m)
+    q, k, v, q2 = (torch.empty_like(q0) for _ in range(4))
+    outs = [torch.empty_like(q0) for _ in range(4)]
+    big = torch.zeros(1 << 24, device="cuda")
+    side = torch.cuda.Stream()
+
+    def chain(sync):
+        main = torch.cuda.current_stream()
+        for a, b in ((q, q0), (k, k0), (v, v0)):
+            a.copy_(b)
+        if n:
+            B.kvq_quantize_append(cache, *past, cache_len=0)
+        for i in range(4):
+            side.wait_stream(main)
+            big.add_(1.0)
+            q.mul_(1.03125)                                       # main: the queries
+            with torch.cuda.stream(side):                         # side: the chunk, quantized into the window
+                k.neg_()
+                sync()
+                if n:
+                    B.kvq_quantize_append(cache, k, v, cache_len=0)
+                if i == 2:
+                    k.zero_()
+            sync()
+            main.wait_stream(side)
+            B.kvq_attn_corrected(cache, q, k, v, d ** -0.5, cache_len=n, out=outs[i])     # behind both
+            sync()
+            q2.copy_(outs[i])
+            v.copy_(q2)                                           # a copy node right before the next call on this stream
+            sync()
+            k.copy_(k0)
+            B.kvq_attn_corrected(cache, q2, k, v, d ** -0.5, cache_len=n, out=outs[i])
+            sync()
+    chain(torch.cuda.synchronize)
+    torch.cuda.synchronize()
+    want = [o.clone() for o in outs] + [b.clone() for b in cache.buffers]
+    chain(lambda: None)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(outs + cache.buffers, want))
+    graph = torch.cuda.CUDAGraph()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        chain(lambda: None)
+    for _ in range(4):
+        for o in outs:
+            o.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(outs + cache.buffers, want))
