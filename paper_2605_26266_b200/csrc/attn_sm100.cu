@@ -728,6 +728,9 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // bias operand tiles start as zeros (columns beyond the group count stay zero for good)
   for (int i = tid; i < 4 * kXBytes / 16; i += kThreads)
     reinterpret_cast<uint4*>(smem + kOffAx)[i] = make_uint4(0, 0, 0, 0);
+  // A pair's allocation concerns both CTAs' TMEM: the peer has to run by then.  The two are placed together but need not start together
+  // (an SM may have to change its split of L1 and shared memory first).
+  if constexpr (PAIR) { __syncwarp(); cluster_sync_all(); }
   if (warp == 0) {
     if constexpr (PAIR) { tmem_alloc_pair(sbase + kOffMisc, 512); tmem_relinquish_pair(); }
     else { tmem_alloc(sbase + kOffMisc, 512); tmem_relinquish(); }
@@ -1337,17 +1340,18 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
   }
 
+  wait_for_previous_grid();                      // also in a CTA that had no cached tile
   __syncthreads();
   // A pair leaves together: neither CTA's shared memory or TMEM may go while the other still arrives on its
   // barriers or the leader's MMAs still read its operands (every role above has come out through bounded waits).
   if constexpr (PAIR) cluster_sync_all();
-  wait_for_previous_grid();                      // also in a CTA that had no cached tile
   if (warp == 0) {
     tc_fence_after();
     if constexpr (PAIR) tmem_dealloc_pair(tmem, 512); else tmem_dealloc(tmem, 512);
     // a wait that gave up left its diagnostic code in the abort word: report the first one
     if (lane == 0 && misc[1] != 0 && p.status) atomicCAS(p.status, 0, misc[1]);
   }
+  if constexpr (PAIR) { __syncwarp(); cluster_sync_all(); }      // both have given their TMEM back before one's SM takes another CTA
 }
 
 // Combines the partial results of every unit whose key tiles were split over several CTAs.

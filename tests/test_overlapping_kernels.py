@@ -99,3 +99,14 @@ def test_both_ctas_of_a_pair_wait_for_the_last_commits():
     # two warps of the peer's dequantizing role (warps 12 to 15), then the barrier
     assert re.search(r"rank != 0 && warp < 14\) cx\.drain\(kDrain \+ warp - 12, 0\);.*cluster_sync_all\(\);", end, re.S)
     assert re.search(r"commit\(kDrain \+ qt\);\s*cx\.drain\(kDrain \+ qt, 0\);", text)
+
+
+def test_a_pair_is_there_while_its_tensor_memory_is_allocated_and_freed():
+    """tcgen05.alloc and .dealloc with cta_group::2 concern the TMEM of both CTAs of a cluster.  CTAs of a cluster are placed together
+    but do not start or end together, so a barrier of the cluster stands in front of the first and behind the second."""
+    body = dict(kernels(source("attn_sm100.cu")))["attn_tcgen05_kernel"]
+    before, rest = body.split("tmem_alloc_pair(")
+    assert "cluster_sync_all();" in before
+    inside, after = rest.split("tmem_dealloc_pair(")
+    assert inside.count("cluster_sync_all();") == 2 and "wait_for_previous_grid" not in inside[inside.rindex("cluster_sync_all();"):]
+    assert "cluster_sync_all();" in after
