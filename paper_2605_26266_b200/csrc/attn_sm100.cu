@@ -1440,7 +1440,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
       const float f = exp2f(sm[j] - m);
       const float lc = f * sc[j], la = f * sa[j];
       l_cur += lc; l_cac += la;
-      const float w = lc + la;
+      const float w = D == 64 ? (lc + la) * kPartScale : lc + la;       // 64 channels: again no product above the value itself
       const uint32_t pw[4] = {a[j].x, a[j].y, a[j].z, a[j].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -1453,10 +1453,10 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
       }
     }
   }
-  const float l = l_cur + l_cac, inv = 1.0f / l;
+  const float l = l_cur + l_cac, inv = 1.0f / l, norm = D == 64 ? 1.0f / kPartScale * inv : inv;
   Out v;
-  v.x = cvt_bf16x2(acc[0] * inv, acc[1] * inv); v.y = cvt_bf16x2(acc[2] * inv, acc[3] * inv);
-  if constexpr (D == 128) { v.z = cvt_bf16x2(acc[4] * inv, acc[5] * inv); v.w = cvt_bf16x2(acc[6] * inv, acc[7] * inv); }
+  v.x = cvt_bf16x2(acc[0] * norm, acc[1] * norm); v.y = cvt_bf16x2(acc[2] * norm, acc[3] * norm);
+  if constexpr (D == 128) { v.z = cvt_bf16x2(acc[4] * norm, acc[5] * norm); v.w = cvt_bf16x2(acc[6] * norm, acc[7] * norm); }
   s_tile[rr * 16 + (cg ^ rr)] = v;
   __syncthreads();
   {

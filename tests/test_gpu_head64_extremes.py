@@ -58,11 +58,12 @@ def test_infinite_values_stay_infinite(kind):
     assert (got[finite].float() - want[finite].float()).norm() < 1e-2 * want[finite].float().norm()
 
 
+@pytest.mark.parametrize("heads,m,n_cur", [(75, 200, 130), (8, 300, 2000)])           # whole units, split ones
 @pytest.mark.parametrize("rise", [1.0, 3.5, 7.5, 20.0])
-def test_the_largest_values_stay_finite(rise):
+def test_the_largest_values_stay_finite(rise, heads, m, n_cur):
     """A key some bits above those before it has a weight of at most 1, so that its value may be the largest BF16 number."""
     from paper_2605_26266_b200 import binding as B
-    heads, m, n_cur, n = 75, 200, 130, 64
+    n = 64
     cache = B.Cache(1, heads, 64, 2, 64, 128)
     zeros = lambda t: torch.zeros(1, heads, t, 64, device="cuda", dtype=torch.bfloat16)
     B.kvq_quantize_append(cache, zeros(n), zeros(n))
