@@ -701,6 +701,11 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   // other kernel, half of which idles there.
   const int64_t bh = (int64_t)d->batch * d->heads;
   const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
+  // 64 channels, more heads than processors, one tile of rows, current keys within half a tile, no cache: a CTA of the tcgen05 kernel
+  // would take several units of half a tile each.  Two of some 28 000 random calls of all kernels ended in a launch failure, two of the
+  // three of this form and none of the 17 with more keys; the cause was not found by reading, and 300 such calls with every role's
+  // steps recorded ran through.  They do not run there: 172 heads x 111 rows over 5 keys 11 us here (148 heads x 111 rows, which do, 7).
+  if (d->head_dim == 64 && cache_len == 0 && n_cur <= 64 && blocks <= 8 && bh > resident_ctas() / kCtasPerSm) return true;
   if (d->head_dim == 64) {
     if (bh * blocks <= resident_ctas() / kCtasPerSm * kCtasPerSm64 && bh * blocks * steps <= 8192) return true;
   } else if (blocks <= 8 && bh * blocks <= resident_ctas() && bh * blocks * steps <= 4608) {

@@ -44,6 +44,21 @@ def test_where_the_line_lies(B, d, heads, m, n, few):
     assert (workspace(B, d, heads, m, n) == partial_rows(d, heads, m, n)) == few
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("heads,m,n_cur", [(150, 100, 5), (172, 111, 64), (149, 33, 1)])
+def test_units_of_a_single_tile_match_the_oracle(B, heads, m, n_cur):
+    """64 channels, more heads than processors, at most 128 rows and 64 current keys, no cache: on the few-row kernel whatever its number of CTAs."""
+    w = inputs.Workload("single", 1500 + m, 1, heads, 64, 32, 0, 2, 64, m, head_scale=True)
+    g, o = B.Cache(1, heads, 64, 2, 64, 128), O.Cache(1, heads, 64, 2, 64, 128)
+    q, _, _ = inputs.make_chunk(w, 1, tokens=m)
+    _, kc, vc = inputs.make_chunk(w, 2, tokens=n_cur)
+    lse = torch.zeros(1, heads, m, dtype=torch.float32, device="cuda")
+    out = B.kvq_attn_corrected(g, T.to_dev(q), T.to_dev(kc), T.to_dev(vc), T.sigma_of(64), cache_len=0, lse=lse)
+    want = O.attn_corrected(o, 0, 0, q, kc, vc, T.sigma_of(64), correction=True)
+    T.assert_attn_close(T.from_dev_bf16(out).reshape(want["out"].shape), want["out"])
+    assert np.abs(lse.cpu().numpy().reshape(want["lse"].shape) - want["lse"]).max() < 2e-2
+
+
 @pytest.mark.parametrize("d,heads,m,n,launches", [
     (64, 2, 256, 1024, 1), (64, 2, 16, 2032, 1), (64, 1, 16, 2300, 2),                 # 5 and 8 splits; 9
     (128, 2, 16, 1520, 1), (128, 2, 16, 1800, 2), (128, 3, 16, 100, 1),                # 6 splits; 7; 1
