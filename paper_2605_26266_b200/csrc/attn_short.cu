@@ -5,21 +5,24 @@
 // exponentials, and a dequantization into shared memory that 16 rows cannot pay for).  Here a CTA takes 16 rows of one
 // (batch, head) and a range of the keys, each of its four warps takes every fourth step of 32 keys, and the packed codes
 // go from global memory through registers straight into the B operands of mma.sync: the contraction over channels
-// may run in any order, so a lane takes the D/4 consecutive channels whose codes it can load at once, and the output
-// channels may be numbered in any order, so a lane takes D/8 consecutive ones of the values of its four keys.  A lane's
-// channels then lie in one group: one step and one zero-point per key and lane.  Nothing is staged in shared memory but the
-// query rows.
+// may run in any order, so a lane takes the D/4 channels whose codes it can load at once, and the output channels may be
+// numbered in any order, so a lane takes D/8 consecutive ones of the values of its four keys.  Nothing is staged in shared
+// memory but the query rows.
 //
-// Algorithm 1 as in the other kernels: rotated query and dequantized keys in FP16, weights and values in BF16, FP32
-// sums, exact running maximum; the bias -(sigma/24) sum_j nu_j step_j^2 is one more MMA step (nu as a BF16 high and low
-// part, step^2 is exact in BF16).  Ranges of one (batch, head) leave FP32 partial rows that a second kernel, or in small
-// problems the cluster of their CTAs, merges in a fixed order.
+// Algorithm 1 as in the other kernels: rotated query in FP16, weights and values in BF16, FP32 sums, exact running maximum.
+// Keys of at most two groups a head are not dequantized: their operand is the codes, and step, zero-point and the bias
+// -(sigma/24) sum_j nu_j step_j^2 are applied to the sums in FP32 (code_steps).  With four groups that would be as many
+// instructions as it saves: FP16 keys there, and the bias is one more MMA step (nu as a BF16 high and low part, step^2 is exact in
+// BF16).  Ranges of one (batch, head) leave FP32 partial rows that a second kernel, or in small problems the cluster of their CTAs,
+// merges in a fixed order.
 //
-// What bounds it: instruction issue and latency (36 warp instructions per key and 16 rows at 4 bits, half of them the
-// expansion of the codes; two CTAs of four warps an SM, the ALU pipe half busy), then HBM.  16 rows over 16 384 tokens
-// of 32 heads at 4 bits, group 128: 41 us with the merge where inputs change from call to call, 39 on the same ones (at 2 bits, group
-// 64, 36 against 58 in the tcgen05 kernel); three CTAs with spilled registers 12 % slower (without spills, the query in shared
-// memory, 5 %), four 80 %; the four score tiles of a step one after the other instead of in turn 7 %.
+// What bounds it: latency and instruction issue (two CTAs of four warps an SM, as registers allow), then HBM.  32 heads of 128 channels, 16
+// rows, 16 384 tokens at 4 bits, group 128, where inputs change from call to call: 41.0 us with FP16 keys (36 warp instructions a
+// key), 36.4 with products of codes, 35.4 with the rest as it is here (24 instructions): all query rows and the first keys loaded
+// together, addresses from 32-bit slots, a current step's values on their way while its weights are computed, the merge's rows fetched with
+// their maxima.  Two groups, on the same inputs again and again, 36.2 -> 32.1 us at 2 bits and 37.2 -> 34.2 at 4, four 35.9 -> 34.6 and
+// 37.7 -> 36.2.  Three CTAs an SM: with spilled registers 25 % slower, with the query in shared memory and hardly any spills 4 to 9 %.  The four
+// score tiles of a step one after the other instead of in turn: 7 %.
 #include <cuda_fp16.h>
 
 #include <type_traits>
@@ -45,6 +48,7 @@ struct SParams {
   int heads, rotate, correction;
   int m_tokens, n_cached, n_cur;
   int q_blocks, splits;
+  int split_steps, split_rest;         // steps = splits * split_steps + split_rest
   float scale_log2, ax_coef;           // sigma * log2(e), -sigma / 24
   float* lse; float* cached_mass;
   float* partial;                      // splits > 1: one slot per CTA, see slot_floats
@@ -60,6 +64,11 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 __device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// the first product of a chain
+__device__ __forceinline__ void mma_f16_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+               : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -119,8 +128,9 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// What a lane expands in one step: of the keys 8 t + lane / 4 (t = 0 .. 3) the codes of its D/4 channels, of the values
-// 2 (lane % 4) + {0, 1} + 8 t those of its D/8 channels; and of each the step and zero-point of the lane's group.
+// What a lane expands in one step where a head has four groups: of the keys 8 t + lane / 4 (t = 0 .. 3) the codes of its D/4 channels, of
+// the values 2 (lane % 4) + {0, 1} + 8 t those of its D/8 channels; a lane's channels lie in one group, and of each key it has that one's
+// step and zero-point.
 template <int D, int BITS>
 struct Keys {
   static constexpr int W = D / 4 * BITS / 32;
@@ -132,21 +142,46 @@ struct Values {
   static constexpr int W = B < 4 ? 1 : B / 4;
   uint32_t w[8][W], step[8], zero[8];
 };
-// First tokens of the two halves of a step (16 slots each never straddle the end of the slab, 32 may).
-struct Step { int64_t tok[2]; };
-
+// The same for at most two groups a head: products of keys are taken of the codes themselves, one group at a time, so a lane has D/4/G
+// channels of each; steps and zero-points are those of keys 8 t + 2 (lane % 4) + {0, 1}, all in one load.
 template <int D, int BITS, int GROUP>
-__device__ __forceinline__ void load_keys(Keys<D, BITS>& r, const SParams& p, const Step& st, int g, int c) {
-  constexpr int CB = D * BITS / 8, G = D / GROUP, W = Keys<D, BITS>::W;
+struct CodeKeys {
+  static constexpr int G = D / GROUP, C = GROUP / 4, W = C * BITS < 32 ? 1 : C * BITS / 32;      // channels and words of a group
+  static constexpr int N = C * BITS < 32 ? C : 32 / BITS;                                         // codes of a word
+  uint32_t w[4][G][W], step[4], zero[4][G];
+};
+template <int D, int BITS, int GROUP>
+struct CodeValues {
+  static constexpr int G = D / GROUP, B = D / 8 * BITS / 8, W = B < 4 ? 1 : B / 4;
+  uint32_t w[8][W], step[4], zero[4][G];
+};
+// First slots of the two halves of a step (16 slots each never straddle the end of the slab, 32 may), in the slab of the head.
+struct Step { uint32_t slot[2]; };
+// The cache of one head.  32-bit slots (attn_short_supports), so that an address is one multiply-add.
+struct Slab { const uint8_t* codes[2]; const uint8_t* scale[2]; const uint16_t* zero[2]; };
+
+template <int BYTES, int W>
+__device__ __forceinline__ void load_bytes(uint32_t (&w)[W], const void* src) {
+  if constexpr (BYTES == 1) w[0] = load_coherent(static_cast<const uint8_t*>(src));
+  else if constexpr (BYTES == 2) w[0] = load_coherent(static_cast<const uint16_t*>(src));
+  else if constexpr (BYTES == 4) w[0] = load_coherent(static_cast<const uint32_t*>(src));
+  else if constexpr (BYTES == 8) { const uint2 v = load_coherent(static_cast<const uint2*>(src)); w[0] = v.x; w[1] = v.y; }
+  else { const uint4 v = load_coherent(static_cast<const uint4*>(src)); w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w; }
+}
+// Addresses: one per half of a step and array, the other keys at fixed offsets from it.
+template <int D, int BITS, int GROUP>
+__device__ __forceinline__ void load_keys(Keys<D, BITS>& r, const Slab& p, const Step& st, int g, int c) {
+  constexpr int CB = D * BITS / 8, G = D / GROUP;
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int64_t tok = st.tok[t >> 1] + g + 8 * (t & 1);
-    const uint8_t* src = p.codes[0] + tok * CB + c * (W * 4);
-    if constexpr (W == 1) r.w[t][0] = load_coherent(reinterpret_cast<const uint32_t*>(src));
-    else if constexpr (W == 2) { const uint2 v = load_coherent(reinterpret_cast<const uint2*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; }
-    else { const uint4 v = load_coherent(reinterpret_cast<const uint4*>(src)); r.w[t][0] = v.x; r.w[t][1] = v.y; r.w[t][2] = v.z; r.w[t][3] = v.w; }
-    const int64_t at = tok * G + c * (D / 4) / GROUP;
-    r.step[t] = load_coherent(p.scale[0] + at); r.zero[t] = load_coherent(p.zero[0] + at);
+  for (int u = 0; u < 2; ++u) {
+    const uint8_t* src = p.codes[0] + (uint64_t)(st.slot[u] + g) * CB + c * (CB / 4);
+    const uint64_t at = (uint64_t)(st.slot[u] + g) * G + c * (D / 4) / GROUP;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      load_bytes<CB / 4>(r.w[2 * u + t], src + 8 * t * CB);
+      r.step[2 * u + t] = load_coherent(p.scale[0] + at + 8 * t * G);
+      r.zero[2 * u + t] = load_coherent(p.zero[0] + at + 8 * t * G);
+    }
   }
 }
 // Tokens past the window: step and zero-point 0, so that scores are finite (and masked later) and values exact zeros, whatever
@@ -165,20 +200,91 @@ __device__ __forceinline__ void mask_values(Values<D, BITS>& r, int n_valid, int
     if (2 * c + (i & 1) + 8 * (i >> 1) >= n_valid) r.step[i] = r.zero[i] = 0u;
 }
 template <int D, int BITS, int GROUP>
-__device__ __forceinline__ void load_values(Values<D, BITS>& r, const SParams& p, const Step& st, int g, int c) {
-  constexpr int CB = D * BITS / 8, G = D / GROUP, B = Values<D, BITS>::B;
+__device__ __forceinline__ void load_values(Values<D, BITS>& r, const Slab& p, const Step& st, int g, int c) {
+  constexpr int CB = D * BITS / 8, G = D / GROUP;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t tok = st.tok[i >> 2] + 2 * c + (i & 1) + 8 * ((i >> 1) & 1);
-    const uint8_t* src = p.codes[1] + tok * CB + g * B;
-    if constexpr (B == 2) r.w[i][0] = load_coherent(reinterpret_cast<const uint16_t*>(src));
-    else if constexpr (B == 4) r.w[i][0] = load_coherent(reinterpret_cast<const uint32_t*>(src));
-    else { const uint2 v = load_coherent(reinterpret_cast<const uint2*>(src)); r.w[i][0] = v.x; r.w[i][1] = v.y; }
-    const int64_t at = tok * G + g * (D / 8) / GROUP;
-    r.step[i] = load_coherent(p.scale[1] + at); r.zero[i] = load_coherent(p.zero[1] + at);
+  for (int u = 0; u < 2; ++u) {
+    const uint8_t* src = p.codes[1] + (uint64_t)(st.slot[u] + 2 * c) * CB + g * (CB / 8);
+    const uint64_t at = (uint64_t)(st.slot[u] + 2 * c) * G + g * (D / 8) / GROUP;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int key = (i & 1) + 8 * (i >> 1);
+      load_bytes<CB / 8>(r.w[4 * u + i], src + key * CB);
+      r.step[4 * u + i] = load_coherent(p.scale[1] + at + key * G);
+      r.zero[4 * u + i] = load_coherent(p.zero[1] + at + key * G);
+    }
   }
 }
 
+template <int G>
+__device__ __forceinline__ void load_constants(uint32_t& step, uint32_t (&zero)[G], const Slab& p, int which, uint32_t slot) {
+  uint32_t s[1];
+  load_bytes<2 * G>(s, p.scale[which] + (uint64_t)slot * G);
+  step = s[0];
+  load_bytes<4 * G>(zero, p.zero[which] + (uint64_t)slot * G);
+}
+template <int D, int BITS, int GROUP>
+__device__ __forceinline__ void load_keys(CodeKeys<D, BITS, GROUP>& r, const Slab& p, const Step& st, int g, int c) {
+  using K = CodeKeys<D, BITS, GROUP>;
+  constexpr int CB = D * BITS / 8;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const uint8_t* src = p.codes[0] + (uint64_t)(st.slot[u] + g) * CB + c * (K::C * BITS / 8);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+#pragma unroll
+      for (int gr = 0; gr < K::G; ++gr) load_bytes<K::C * BITS / 8>(r.w[2 * u + t][gr], src + 8 * t * CB + gr * (CB / K::G));
+      load_constants<K::G>(r.step[2 * u + t], r.zero[2 * u + t], p, 0, st.slot[u] + 2 * c + 8 * t);
+    }
+  }
+}
+template <int D, int BITS, int GROUP>
+__device__ __forceinline__ void load_values(CodeValues<D, BITS, GROUP>& r, const Slab& p, const Step& st, int g, int c) {
+  using V = CodeValues<D, BITS, GROUP>;
+  constexpr int CB = D * BITS / 8;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const uint8_t* src = p.codes[1] + (uint64_t)(st.slot[u] + 2 * c) * CB + g * V::B;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) load_bytes<V::B>(r.w[4 * u + i], src + ((i & 1) + 8 * (i >> 1)) * CB);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) load_constants<V::G>(r.step[2 * u + t], r.zero[2 * u + t], p, 1, st.slot[u] + 2 * c + 8 * t);
+  }
+}
+// Steps and zero-points of a pair of keys, as they are loaded: key by key, its groups side by side.  Those of one group:
+template <int G>
+__device__ __forceinline__ float2 steps_of(uint32_t step, int gr) {
+  const uint32_t bytes = G == 1 ? step : __byte_perm(step, 0u, gr == 0 ? 0x4420 : 0x4431);   // the group may be known at run time only
+  uint32_t h;
+  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"((uint16_t)bytes));
+  return __half22float2(*reinterpret_cast<__half2*>(&h));
+}
+template <int G>
+__device__ __forceinline__ uint32_t zeros_of(const uint32_t (&zero)[G], int gr) {      // two BF16
+  return G == 1 ? zero[0] : __byte_perm(zero[0], zero[G - 1], gr == 0 ? 0x5410 : 0x7632);
+}
+__device__ __forceinline__ float2 bf16x2_to_f32(uint32_t z) { return make_float2(__uint_as_float(z << 16), __uint_as_float(z & 0xFFFF0000u)); }
+// 0 past the window, so that scores are finite and weights and values zeros whatever the bytes there are.
+template <int G>
+__device__ __forceinline__ void mask_pairs(uint32_t (&step)[4], uint32_t (&zero)[4][G], int n_valid, int c) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int left = n_valid - (8 * t + 2 * c);                    // valid keys of the pair
+    if (left < 2) {
+      step[t] &= left == 1 ? (G == 1 ? 0xFFu : 0xFFFFu) : 0u;
+      zero[t][0] &= left == 1 ? (G == 1 ? 0xFFFFu : ~0u) : 0u;
+      if (G == 2) zero[t][G - 1] = 0u;
+    }
+  }
+}
+// Where code i of a 16-bit half of a key's word is picked up as an FP16: shifted right by `shift` it starts at bit `bit` of the ten lowest,
+// which hold two codes of 4 bits or five of 2, and the FP16's value is code * 2^(bit - 24), a subnormal and exact.
+struct Place { int shift, bit; };
+template <int BITS>
+__host__ __device__ constexpr Place key_place(int i) {
+  return BITS == 4 ? Place{i < 2 ? 0 : 8, 4 * (i & 1)} : Place{i < 5 ? 0 : 10, 2 * (i < 5 ? i : i - 5)};
+}
+template <int BITS> constexpr int kTopKeyBit = BITS == 4 ? 4 : 8;
 // ANY_ZERO: groups whose constants are not exact (key_constant_exact, value_constant_exact) are expanded in FP32, as in the
 // warp-level kernel, which served the calls this is set for before: heads of 64 channels, and chunks TMA cannot address.  A
 // warp works in 16 bits, notes whether it met such a group, and then takes its steps once more in FP32.  Any branch inside a
@@ -193,11 +299,13 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
   constexpr int KS = D / 16;                                       // MMA steps over the channels
   constexpr int NT = D / 8;                                        // output tiles of 8 channels
   constexpr int G = D / GROUP;
-  constexpr int KW = Keys<D, BITS>::W;
+  constexpr bool kCodes = G <= 2;                                  // products of the codes themselves
+  using KeysT = typename std::conditional<kCodes, CodeKeys<D, BITS, GROUP>, Keys<D, BITS>>::type;
+  using ValuesT = typename std::conditional<kCodes, CodeValues<D, BITS, GROUP>, Values<D, BITS>>::type;
   constexpr int kOStride = D + 4;
   // the query tiles are done with when the warps' outputs are exchanged
   __shared__ __align__(16) union {
-    struct { uint16_t q[kRows * LD], qr[kRows * LD]; float nu[kRows * 4]; } in;
+    struct { uint16_t q[kRows * LD], qr[kRows * LD]; float nu[kRows * 4], sum[kRows * 2]; int shift[kRows]; } in;
     struct { float o[kWarps][kRows * kOStride]; } x;
   } sm;
   __shared__ float s_stat[kWarps][3][kRows];                       // m, l_cur, l_cached
@@ -210,14 +318,45 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
   const int bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
   const int row0 = (unit - bh * p.q_blocks) * kRows;
 
+  // ---- this CTA's share of the steps: cached keys first, then the current chunk's; warp w takes every fourth ----
+  const int n_cs = (p.n_cached + kStep - 1) / kStep;
+  const int first = split * p.split_steps + split * p.split_rest / p.splits, last = (split + 1) * p.split_steps + (split + 1) * p.split_rest / p.splits;
+  int st = first + warp;
+  const int last_c = min(last, n_cs);
+  Slab slab;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int64_t at = (int64_t)bh * p.capacity;
+    slab.codes[i] = p.codes[i] + at * (D * BITS / 8); slab.scale[i] = p.scale[i] + at * G; slab.zero[i] = p.zero[i] + at * G;
+  }
+  auto step_of = [&](int i) {
+    Step x;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const uint32_t slot = (uint32_t)p.cache_begin + (uint32_t)i * kStep + 16 * u;
+      x.slot[u] = slot - (slot >= (uint32_t)p.capacity ? (uint32_t)p.capacity : 0u);
+    }
+    return x;
+  };
+  KeysT keys;
+  auto load_keys_of = [&](int i) { load_keys<D, BITS, GROUP>(keys, slab, step_of(i), g, c); };
   // ---- query rows: as they are, and rotated (FP16, in the order the expanded codes come in), per-group norms ----
   {
     constexpr int LPR = D / 8;                                     // lanes per row, 8 channels each
     const int ln = lane % LPR;
-    for (int r = warp * (32 / LPR) + lane / LPR; r < kRows; r += kWarps * 32 / LPR) {
-      const int row = row0 + r;
-      uint4 raw = make_uint4(0, 0, 0, 0);
-      if (row < p.m_tokens) raw = load_coherent(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
+    constexpr int kAtOnce = kWarps * 32 / LPR;                     // rows
+    uint4 raws[kRows / kAtOnce];                                   // all on their way together, and the first keys behind them
+#pragma unroll
+    for (int it = 0; it < kRows / kAtOnce; ++it) {
+      const int row = row0 + it * kAtOnce + warp * (32 / LPR) + lane / LPR;
+      raws[it] = make_uint4(0, 0, 0, 0);
+      if (row < p.m_tokens) raws[it] = load_coherent(reinterpret_cast<const uint4*>(p.q + (int64_t)b * p.q_sb + (int64_t)h * p.q_sh + (int64_t)row * p.q_st) + ln);
+    }
+    if (st < last_c) load_keys_of(st);
+#pragma unroll
+    for (int it = 0; it < kRows / kAtOnce; ++it) {
+      const int r = it * kAtOnce + warp * (32 / LPR) + lane / LPR;
+      const uint4 raw = raws[it];
       *reinterpret_cast<uint4*>(sm.in.q + r * LD + ln * 8) = raw;
       const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
       float x[8];
@@ -249,29 +388,73 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
 #pragma unroll
       for (int off = 1; off < GROUP / 8; off *= 2) nu += __shfl_xor_sync(0xFFFFFFFFu, nu, off);
       if (ln % (GROUP / 8) == 0) sm.in.nu[r * 4 + ln / (GROUP / 8)] = nu;
-      // a word of 32 / BITS codes expands to the pairs (i, i + 16 / BITS): that order, pair by pair
+      // a word of N codes expands to the pairs (i, i + N / 2): that order, pair by pair
+      if constexpr (kCodes) {
+        // by groups, then lanes; times 2^shift, so that the row's largest value is at 2^14 (rows below 2^-10: 2^24), and 2^-bit of where
+        // the channel's code lies
+        constexpr int N = KeysT::N, C = KeysT::C;
+        float top = 0.f, sum = 0.f;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        constexpr int N = 32 / BITS;
-        const int ch = ln * 8 + e, i = ch % N;
-        const float v = fminf(fmaxf(x[e], -65504.f), 65504.f);
-        sm.in.qr[r * LD + ch / N * N + 2 * (i % (N / 2)) + i / (N / 2)] = __half_as_ushort(__float2half_rn(v));
+        for (int e = 0; e < 8; ++e) top = fmaxf(top, fabsf(x[e]));
+#pragma unroll
+        for (int off = 1; off < LPR; off *= 2) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, off));
+        const int shift = max(-100, min(24, 14 + 127 - (int)(__float_as_uint(top) >> 23)));
+        const float scale = __uint_as_float((uint32_t)(127 + shift) << 23);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int ch = ln * 8 + e, i = ch % N;                   // N is 8 or 16, so i % (N / 2) is known at compile time up to where it matters
+          const int bit = key_place<BITS>(N == 16 ? e : e & 3).bit;
+          const float v = fminf(fmaxf(x[e] * scale * (1.0f / (1 << bit)), -65504.f), 65504.f);
+          const __half hv = __float2half_rn(v);
+          sum += __half2float(hv) * (float)(1 << bit);
+          sm.in.qr[r * LD + ch / N * N + 2 * (i % (N / 2)) + i / (N / 2)] = __half_as_ushort(hv);
+        }
+#pragma unroll
+        for (int off = 1; off < GROUP / 8; off *= 2) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+        if (ln % (GROUP / 8) == 0) sm.in.sum[r * 2 + ln / (GROUP / 8)] = sum * 0x1p-24f;
+        if (ln == 0) sm.in.shift[r] = shift;
+        static_assert(N == 8 || N == 16, "eight channels of a lane: whole words, or the same places in each half");
+        static_assert(C % N == 0, "whole words");
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          constexpr int N = 32 / BITS;
+          const int ch = ln * 8 + e, i = ch % N;
+          sm.in.qr[r * LD + ch / N * N + 2 * (i % (N / 2)) + i / (N / 2)] = __half_as_ushort(__float2half_rn(fminf(fmaxf(x[e], -65504.f), 65504.f)));
+        }
       }
     }
   }
   __syncthreads();
   uint32_t qf[KS][4];
-  constexpr int KPW = 8 / BITS;                                    // MMA steps per word of codes
+  constexpr int KW = kCodes ? D / GROUP * CodeKeys<D, BITS, GROUP>::W : Keys<D, BITS>::W;      // words of a lane
+  constexpr int N = kCodes ? CodeKeys<D, BITS, GROUP>::N : 32 / BITS, KPW = N / 4;              // codes and MMA steps of a word
+  constexpr int KWG = kCodes ? KW / G : KW;                                                   // words of a group
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks) {
-    const int col = (c * KW + ks / KPW) * (32 / BITS) + 4 * (ks % KPW);
+    const int w = ks / KPW, col = ((w / KWG * 4 + c) * KWG + w % KWG) * N + 4 * (ks % KPW);
     const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.qr + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.qr + (g + 8) * LD + col);
     qf[ks][0] = lo.x; qf[ks][1] = hi.x; qf[ks][2] = lo.y; qf[ks][3] = hi.y;
+  }
+  // At most two groups: scores are computed in units of 2^(24 - shift) of their row, s = sum over groups of step (sum_c q'_c code_c - zero
+  // sum_c q'_c) + step^2 nu', in FP32 behind the products of q' and the codes themselves, so that expanding a key is an AND for two codes
+  // and its constants are spent once per key.
+  float row_unit[2], row_scale[2], row_sum[2][2], row_nu[2][2];    // of rows g, g + 8; of these by group
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int r = g + 8 * i, shift = kCodes ? sm.in.shift[r] : 24;
+    row_unit[i] = __uint_as_float((uint32_t)(127 + shift - 24) << 23);
+    row_scale[i] = p.scale_log2 * __uint_as_float((uint32_t)(127 + 24 - shift) << 23);
+#pragma unroll
+    for (int gr = 0; gr < 2; ++gr) {
+      row_sum[i][gr] = kCodes && gr < G ? sm.in.sum[r * 2 + gr] : 0.f;
+      row_nu[i][gr] = kCodes && gr < G && p.correction ? p.ax_coef * sm.in.nu[r * 4 + gr] * row_unit[i] : 0.f;
+    }
   }
   // bias operand: columns 2 c, 2 c + 1 are the high and low part of lane c's group, with ANY_ZERO column 2 c + 8 is the rest
   // (the warp-level kernel applies the bias in FP32); one lane per group counts it
   uint32_t ax[4] = {0u, 0u, 0u, 0u};
-  if (p.correction && c % (4 / G) == 0) {
+  if (!kCodes && p.correction && c % (4 / G) == 0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const float a = p.ax_coef * sm.in.nu[(g + 8 * i) * 4 + c / (4 / G)];
@@ -288,7 +471,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
   for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
   float m_run[2] = {-INFINITY, -INFINITY}, l_cur[2] = {0.f, 0.f}, l_cac[2] = {0.f, 0.f};
   uint32_t pf[8];
-  // online softmax over the 32 scores of a step (this lane: rows g, g + 8, keys 8 t + 2 c + {0, 1}); leaves the weights in pf
+  // online softmax over the 32 scores of a step (this lane: rows g, g + 8, keys 8 t + 2 c + {0, 1}); leaves the weights in their place
   // The maximum is kept as a raw score and subtracted before the scale: exact for the largest score however large it is (a key
   // masked with the lowest number), where the exact product of an FMA and a rounded maximum would differ.
   auto softmax_step = [&](float (&s)[4][4], int n_valid, float (&l)[2]) {
@@ -312,7 +495,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
     if (__any_sync(0xFFFFFFFFu, m_new[0] > m_run[0] || m_new[1] > m_run[1])) {
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const float f = ex2((m_run[r] - no_key_yet(m_new[r])) * p.scale_log2);
+        const float f = ex2((m_run[r] - no_key_yet(m_new[r])) * row_scale[r]);
         l_cur[r] *= f; l_cac[r] *= f;
         m_run[r] = m_new[r];
 #pragma unroll
@@ -325,44 +508,36 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const float m = no_key_yet(m_run[r]);
+      float2 sum;
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(s[t][2 * r], s[t][2 * r + 1]), make_float2(-m, -m)), make_float2(p.scale_log2, p.scale_log2));
-        const float w0 = ex2(x.x), w1 = ex2(x.y);
-        l[r] += w0 + w1;
-        pf[2 * t + r] = pack_bf16(w0, w1);
+        const float2 x = __fmul2_rn(__fadd2_rn(make_float2(s[t][2 * r], s[t][2 * r + 1]), make_float2(-m, -m)), make_float2(row_scale[r], row_scale[r]));
+        const float2 e = make_float2(ex2(x.x), ex2(x.y));
+        sum = t == 0 ? e : __fadd2_rn(sum, e);
+        s[t][2 * r] = e.x; s[t][2 * r + 1] = e.y;
       }
+      l[r] += sum.x + sum.y;
     }
   };
 
-  // ---- this CTA's share of the steps: cached keys first, then the current chunk's; warp w takes every fourth ----
-  const int n_cs = (p.n_cached + kStep - 1) / kStep, n_steps = n_cs + (p.n_cur + kStep - 1) / kStep;
-  const int first = (int)((int64_t)n_steps * split / p.splits), last = (int)((int64_t)n_steps * (split + 1) / p.splits);
-  int st = first + warp;
-  const int last_c = min(last, n_cs);
-  auto step_of = [&](int i) {
-    Step x;
+  auto pack_weights = [&](const float (&s)[4][4]) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      int64_t slot = p.cache_begin + (int64_t)i * kStep + 16 * u;
-      if (slot >= p.capacity) slot -= p.capacity;
-      x.tok[u] = (int64_t)bh * p.capacity + slot;
-    }
-    return x;
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) pf[2 * t + r] = pack_bf16(s[t][2 * r], s[t][2 * r + 1]);
   };
+
   // kFp32: (code - zero) * step in FP32, rounded once.  Otherwise in 16 bits; with ANY_ZERO false if some constants were not
   // exact (such steps are in the sums by then).
-  auto cached_steps = [&](auto fp32) {
+  auto cached_steps = [&](auto fp32, auto& keys) {
     constexpr bool kFp32 = decltype(fp32)::value;
     constexpr float kOff = BITS == 2 ? 4.f : 16.f;
     constexpr uint32_t kMask = (1u << BITS) - 1;
-    Keys<D, BITS> keys;
     bool exact = true;
-    if (st < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st), g, c);
 #pragma unroll 1
     for (; st < last_c; st += kWarps) {
       Values<D, BITS> vals;                                        // on their way while the scores are computed
-      load_values<D, BITS, GROUP>(vals, p, step_of(st), g, c);
+      load_values<D, BITS, GROUP>(vals, slab, step_of(st), g, c);
       float s[4][4];
       const int n_valid = p.n_cached - st * kStep;
       if (n_valid < kStep) mask_keys(keys, n_valid, g);
@@ -402,8 +577,9 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
             const uint32_t (&a)[4] = qf[wi * KPW + j];
             mma_f16(s[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
           }
-      if (st + kWarps < last_c) load_keys<D, BITS, GROUP>(keys, p, step_of(st + kWarps), g, c);
+      if (st + kWarps < last_c) load_keys_of(st + kWarps);
       softmax_step(s, n_valid, l_cac);
+      pack_weights(s);
       if (n_valid < kStep) mask_values(vals, n_valid, c);
       // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
 #pragma unroll
@@ -449,52 +625,204 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
     }
     return !ANY_ZERO || kFp32 || __all_sync(0xFFFFFFFFu, exact);
   };
-  if (!cached_steps(std::false_type{})) {                          // the warp's steps once more
+  // The same for at most two groups a head, with products of the keys' codes.  (Weights times the steps of their values, rounded then, and
+  // code - zero as the values' operand, 8 instructions of 10 a register, took 1 to 2 us of 34 less, but weights near 1 lose what they have
+  // from lying at the top of their binade: errors up to 4 % larger.)
+  auto code_steps = [&](auto fp32, auto& keys, auto& vals) {
+    constexpr bool kFp32 = decltype(fp32)::value;
+    constexpr uint32_t kMask = (1u << BITS) - 1;
+    bool exact = true;
+#pragma unroll 1
+    for (; st < last_c; st += kWarps) {
+      const Step here = step_of(st);
+      load_values<D, BITS, GROUP>(vals, slab, here, g, c);         // on their way while the scores are computed
+      float s[4][4];
+      const int n_valid = p.n_cached - st * kStep;
+#pragma unroll
+      for (int gr = 0; gr < G; ++gr) {
+        float key_step[4], key_zero[4];                            // of key 8 t + g, which the FP32 form expands with
+        if constexpr (kFp32) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const uint64_t at = (uint64_t)(here.slot[t >> 1] + g + 8 * (t & 1)) * G + gr;
+            const bool in = 8 * t + g < n_valid;
+            key_step[t] = in ? e4m3_byte_to_f32(load_coherent(slab.scale[0] + at)) : 0.f;
+            key_zero[t] = in ? bf16_bits_to_f32(load_coherent(slab.zero[0] + at)) : 0.f;
+          }
+        }
+        // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
+        float raw[4][4];
+#pragma unroll
+        for (int wi = 0; wi < KWG; ++wi) {
+          uint32_t w[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t)                              // eight codes of 2 bits: four in each half
+            w[t] = N * BITS < 32 ? __byte_perm(keys.w[t][gr][wi], 0u, 0x4140) : keys.w[t][gr][wi];
+#pragma unroll
+          for (int j = 0; j < KPW; ++j)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              uint32_t bf[2];
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                constexpr int kTop = kTopKeyBit<BITS>;
+                const Place at = key_place<BITS>(2 * j + i);
+                if constexpr (kFp32) {                             // rounded to FP16, then times 2^(bit - top): still exact
+                  const uint32_t x = w[t] >> ((2 * j + i) * BITS);
+                  const uint32_t k2 = pack_f16_sat(((float)(x & kMask) - key_zero[t]) * key_step[t], ((float)((x >> 16) & kMask) - key_zero[t]) * key_step[t]);
+                  const uint32_t down = (uint32_t)(15 + at.bit - kTop) << 10;
+                  bf[i] = fma_f16x2(k2, down | (down << 16), 0u);
+                } else {
+                  bf[i] = (w[t] >> at.shift) & ((kMask | (kMask << 16)) << at.bit);
+                }
+              }
+              const uint32_t (&a)[4] = qf[(gr * KWG + wi) * KPW + j];
+              if (wi == 0 && j == 0) mma_f16_first(raw[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
+              else mma_f16(raw[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
+            }
+        }
+        if (gr == 0 && n_valid < kStep) mask_pairs<G>(keys.step, keys.zero, n_valid, c);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float2 step = steps_of<G>(keys.step[t], gr), zero = bf16x2_to_f32(zeros_of<G>(keys.zero[t], gr));
+          const float2 off = __fmul2_rn(step, make_float2(-zero.x, -zero.y)), sq = __fmul2_rn(step, step);
+          if (ANY_ZERO && !kFp32) exact &= key_constant_exact<BITS>(zero.x) && key_constant_exact<BITS>(zero.y);
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            // the bias last: beside the two sums that cancel it would lose bits
+            const float2 x = make_float2(raw[t][2 * r], raw[t][2 * r + 1]);
+            constexpr float kUnit = 1.0f / (1 << (24 - kTopKeyBit<BITS>));
+            const float2 dot = kFp32 ? __fmul2_rn(x, make_float2(kUnit, kUnit))
+                                     : __ffma2_rn(x, step, __fmul2_rn(off, make_float2(row_sum[r][gr], row_sum[r][gr])));
+            float2 v = __ffma2_rn(sq, make_float2(row_nu[r][gr], row_nu[r][gr]), dot);
+            if (gr > 0) v = __fadd2_rn(v, make_float2(s[t][2 * r], s[t][2 * r + 1]));
+            s[t][2 * r] = v.x; s[t][2 * r + 1] = v.y;
+          }
+        }
+      }
+      if (st + kWarps < last_c) load_keys_of(st + kWarps);
+      if (n_valid < kStep) mask_pairs<G>(vals.step, vals.zero, n_valid, c);
+      softmax_step(s, n_valid, l_cac);
+      pack_weights(s);
+      // values, 16 keys at a time: keys 2 c, 2 c + 1 (and 8 more) side by side in the halves of a register, code i of both at once
+      const int gr = g * (D / 8) / GROUP;                          // of this lane's channels
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk) {
+        uint32_t step2[2], off2[2];
+        float2 ds[2], zs[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const uint32_t z = zeros_of<G>(vals.zero[2 * kk + u], gr);
+          ds[u] = steps_of<G>(vals.step[2 * kk + u], gr);
+          zs[u] = bf16x2_to_f32(z);
+          if (ANY_ZERO && !kFp32) exact &= value_constant_exact<BITS>(zs[u].x) && value_constant_exact<BITS>(zs[u].y);
+          step2[u] = pack_bf16(ds[u].x, ds[u].y);
+          // 2 bits: -(4 + zero) * step, 4 bits: 16 + zero
+          const float2 off = __fadd2_rn(zs[u], make_float2(BITS == 2 ? 4.f : 16.f, BITS == 2 ? 4.f : 16.f));
+          off2[u] = BITS == 2 ? pack_bf16(-off.x * ds[u].x, -off.y * ds[u].y) : pack_bf16(off.x, off.y);
+        }
+        constexpr int kPer = 16 / BITS;                            // codes in half a word
+#pragma unroll
+        for (int hw = 0; hw < NT / kPer; ++hw) {
+          uint32_t z[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            z[u] = __byte_perm(vals.w[4 * kk + 2 * u][hw / 2], vals.w[4 * kk + 2 * u + 1][hw / 2], hw & 1 ? 0x7632 : 0x5410);
+#pragma unroll
+          for (int i = 0; i < kPer; ++i) {
+            uint32_t bf[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              if constexpr (kFp32) {
+                const uint32_t x = z[u] >> (i * BITS);
+                bf[u] = pack_bf16(((float)(x & kMask) - zs[u].x) * ds[u].x, ((float)((x >> 16) & kMask) - zs[u].y) * ds[u].y);
+              } else {
+                const uint32_t x = move_bits(z[u], i * BITS, BITS == 2 ? 5 : 3);
+                if constexpr (BITS == 2) bf[u] = fma_bf16x2((x & 0x00600060u) | 0x40804080u, step2[u], off2[u]);
+                else bf[u] = mul_bf16x2(sub_bf16x2((x & 0x00780078u) | 0x41804180u, off2[u]), step2[u]);
+              }
+            }
+            mma_bf16(acc[hw * kPer + i], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3], bf[0], bf[1]);
+          }
+        }
+      }
+    }
+    return !ANY_ZERO || kFp32 || __all_sync(0xFFFFFFFFu, exact);
+  };
+  auto cached = [&](auto fp32) { ValuesT vals; if constexpr (kCodes) return code_steps(fp32, keys, vals); else return cached_steps(fp32, keys); };
+  if (!cached(std::false_type{})) {                                // the warp's steps once more
     st = first + warp;
+    if (st < last_c) load_keys_of(st);
     m_run[0] = m_run[1] = -INFINITY;
     l_cur[0] = l_cur[1] = l_cac[0] = l_cac[1] = 0.f;
 #pragma unroll
     for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    cached_steps(std::true_type{});
+    cached(std::true_type{});
   }
   // ---- current chunk: unrotated query, BF16 keys and values, no bias ----
+  // 64 channels: keys of the next step and values of this one are on their way while scores and weights are computed; 128, which have no
+  // registers for that: values while the weights are.
+  uint4 kx[4][D / 32];
+  auto load_current_keys = [&](int i) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int key = min((i - n_cs) * kStep + 8 * t + g, p.n_cur - 1);
+      const uint4* src = reinterpret_cast<const uint4*>(p.kc + (int64_t)b * p.kv_sb + (int64_t)h * p.kv_sh + (int64_t)key * p.kv_st + c * (D / 4));
+#pragma unroll
+      for (int j = 0; j < D / 32; ++j) kx[t][j] = load_coherent(src + j);
+    }
+  };
+  constexpr bool kAhead = D == 64;
+  if (kAhead && st < last) load_current_keys(st);
 #pragma unroll 1
   for (; st < last; st += kWarps) {
     const int k0 = (st - n_cs) * kStep, nv = p.n_cur - k0;
+    uint4 vx[D / 64][8];                                           // of keys 2 c + {0, 1} + 8 u, 8 of the lane's channels at a time
+    const uint16_t* vbase = p.vc + (int64_t)b * p.v_sb + (int64_t)h * p.v_sh + g * (D / 8);
+    auto load_current_values = [&]() {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int key = 2 * c + (u & 1) + 8 * (u >> 1);
+#pragma unroll
+        for (int i = 0; i < D / 64; ++i)
+          vx[i][u] = key < nv ? load_coherent(reinterpret_cast<const uint4*>(vbase + (int64_t)(k0 + key) * p.v_st) + i) : make_uint4(0, 0, 0, 0);
+      }
+    };
+    if (kAhead) load_current_values();
+    else load_current_keys(st);
     float s[4][4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
-      const uint4* src = reinterpret_cast<const uint4*>(p.kc + (int64_t)b * p.kv_sb + (int64_t)h * p.kv_sh + (int64_t)min(k0 + 8 * t + g, p.n_cur - 1) * p.kv_st + c * (D / 4));
+    for (int t = 0; t < 4; ++t) s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
 #pragma unroll
-      for (int i = 0; i < D / 32; ++i) {
-        const uint4 v = load_coherent(src + i);
+    for (int i = 0; i < D / 32; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int col = c * (D / 4) + 8 * i + 4 * j;
-          const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.q + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.q + (g + 8) * LD + col);
-          mma_bf16(s[t], lo.x, hi.x, lo.y, hi.y, j ? v.z : v.x, j ? v.w : v.y);
-        }
+      for (int j = 0; j < 2; ++j) {
+        const int col = c * (D / 4) + 8 * i + 4 * j;
+        const uint2 lo = *reinterpret_cast<const uint2*>(sm.in.q + g * LD + col), hi = *reinterpret_cast<const uint2*>(sm.in.q + (g + 8) * LD + col);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) mma_bf16(s[t], lo.x, hi.x, lo.y, hi.y, j ? kx[t][i].z : kx[t][i].x, j ? kx[t][i].w : kx[t][i].y);
       }
+    if (!kAhead) load_current_values();
+    else if (st + kWarps < last) load_current_keys(st + kWarps);
+    if constexpr (kCodes) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[t][e] *= row_unit[e >> 1];
     }
     softmax_step(s, nv, l_cur);
-    const uint16_t* vbase = p.vc + (int64_t)b * p.v_sb + (int64_t)h * p.v_sh + g * (D / 8);
+    pack_weights(s);
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-      for (int i = 0; i < D / 64; ++i) {                           // 8 of the lane's channels at a time
-        uint4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int key = 16 * kk + 2 * c + (u & 1) + 8 * (u >> 1);
-          v[u] = key < nv ? load_coherent(reinterpret_cast<const uint4*>(vbase + (int64_t)(k0 + key) * p.v_st) + i) : make_uint4(0, 0, 0, 0);
-        }
+      for (int i = 0; i < D / 64; ++i) {
+        const uint4 (&v)[8] = vx[i];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const uint32_t sel = e & 1 ? 0x7632 : 0x5410;
           auto word = [&](const uint4& x) { return (e >> 1) == 0 ? x.x : (e >> 1) == 1 ? x.y : (e >> 1) == 2 ? x.z : x.w; };
           mma_bf16(acc[8 * i + e], pf[4 * kk], pf[4 * kk + 1], pf[4 * kk + 2], pf[4 * kk + 3],
-                   __byte_perm(word(v[0]), word(v[1]), sel), __byte_perm(word(v[2]), word(v[3]), sel));
+                   __byte_perm(word(v[4 * kk]), word(v[4 * kk + 1]), sel), __byte_perm(word(v[4 * kk + 2]), word(v[4 * kk + 3]), sel));
         }
       }
   }
@@ -506,14 +834,15 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
     l_cur[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cur[r], 2);
     l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 1);
     l_cac[r] += __shfl_xor_sync(0xFFFFFFFFu, l_cac[r], 2);
-    if (c == 0) { s_stat[warp][0][g + 8 * r] = m_run[r] * p.scale_log2; s_stat[warp][1][g + 8 * r] = l_cur[r]; s_stat[warp][2][g + 8 * r] = l_cac[r]; }
+    if (c == 0) { s_stat[warp][0][g + 8 * r] = m_run[r] * row_scale[r]; s_stat[warp][1][g + 8 * r] = l_cur[r]; s_stat[warp][2][g + 8 * r] = l_cac[r]; }
   }
   __syncthreads();                                                 // also: the query tiles are free
 #pragma unroll
-  for (int j = 0; j < NT; ++j)
+  for (int j = 0; j < NT; j += 4)
 #pragma unroll
     for (int e = 0; e < 4; ++e)
-      sm.x.o[warp][(g + 8 * (e >> 1)) * kOStride + (2 * c + (e & 1)) * (D / 8) + j] = acc[j][e];
+      *reinterpret_cast<float4*>(&sm.x.o[warp][(g + 8 * (e >> 1)) * kOStride + (2 * c + (e & 1)) * (D / 8) + j]) =
+          make_float4(acc[j][e], acc[j + 1][e], acc[j + 2][e], acc[j + 3][e]);
   __syncthreads();
   constexpr int kPerRow = kWarps * 32 / kRows;                     // threads per row
   const int r = threadIdx.x / kPerRow, t8 = threadIdx.x % kPerRow, row = row0 + r;
@@ -599,21 +928,45 @@ __global__ void __launch_bounds__(kWarps * 32) attn_short_merge_kernel(const SPa
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ float s_o[kWarps][D], s_l[kWarps][2];
   const float* slots = p.partial + (size_t)unit * p.splits * slot_floats(D);
+  auto load_row = [&](int s, float (&v)[E], float& lc, float& la) {
+    const float* sl = slots + (size_t)s * slot_floats(D);
+    lc = sl[kRows * D + 16 + r]; la = sl[kRows * D + 32 + r];
+    if constexpr (E == 4) { const float4 u = *reinterpret_cast<const float4*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w; }
+    else { const float2 u = *reinterpret_cast<const float2*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; }
+  };
+  auto maximum_of = [&](int s) { return slots[(size_t)s * slot_floats(D) + kRows * D + r]; };
+  // the warp's first splits, mostly all, come in one trip to memory with the maxima
+  constexpr int kFirst = 4;
+  float v[kFirst][E], fm[kFirst], fc[kFirst], fa[kFirst];
+#pragma unroll
+  for (int i = 0; i < kFirst; ++i) {
+    const int s = warp + kWarps * i;
+    fm[i] = -INFINITY; fc[i] = fa[i] = 0.f;
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[i][e] = 0.f;
+    if (s < p.splits) { fm[i] = maximum_of(s); load_row(s, v[i], fc[i], fa[i]); }
+  }
   float m = -INFINITY;
-  for (int s = lane; s < p.splits; s += 32) m = fmaxf(m, slots[(size_t)s * slot_floats(D) + kRows * D + r]);
+  for (int s = lane; s < p.splits; s += 32) m = fmaxf(m, maximum_of(s));
 #pragma unroll
   for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
   float o[E] = {}, lc = 0.f, la = 0.f;
-#pragma unroll 4
-  for (int s = warp; s < p.splits; s += kWarps) {
-    const float* sl = slots + (size_t)s * slot_floats(D);
-    const float f = ex2(sl[kRows * D + r] - m);
-    lc += f * sl[kRows * D + 16 + r]; la += f * sl[kRows * D + 32 + r];
-    float v[E];
-    if constexpr (E == 4) { const float4 u = *reinterpret_cast<const float4*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w; }
-    else { const float2 u = *reinterpret_cast<const float2*>(sl + r * D + lane * E); v[0] = u.x; v[1] = u.y; }
 #pragma unroll
-    for (int e = 0; e < E; ++e) o[e] += f * v[e];
+  for (int i = 0; i < kFirst; ++i) {
+    if (warp + kWarps * i >= p.splits) break;                      // the whole warp
+    const float f = ex2(fm[i] - m);
+    lc += f * fc[i]; la += f * fa[i];
+#pragma unroll
+    for (int e = 0; e < E; ++e) o[e] += f * v[i][e];
+  }
+#pragma unroll 4
+  for (int s = warp + kWarps * kFirst; s < p.splits; s += kWarps) {
+    float w[E], wc, wa;
+    load_row(s, w, wc, wa);
+    const float f = ex2(maximum_of(s) - m);
+    lc += f * wc; la += f * wa;
+#pragma unroll
+    for (int e = 0; e < E; ++e) o[e] += f * w[e];
   }
 #pragma unroll
   for (int e = 0; e < E; ++e) s_o[warp][lane * E + e] = o[e];
@@ -679,7 +1032,7 @@ int launch(const SParams& p, const Plan& pl, bool any_zero, cudaStream_t st) {
 }  // namespace
 
 bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, uint32_t flags) {
-  if ((flags & KVQ_KERNEL_MASK) != KVQ_KERNEL_AUTO || (flags & KVQ_CORRECTION_EXACT) || (d->flags & KVQ_K_PER_CHANNEL) || m_tokens < 1)
+  if ((flags & KVQ_KERNEL_MASK) != KVQ_KERNEL_AUTO || (flags & KVQ_CORRECTION_EXACT) || (d->flags & KVQ_K_PER_CHANNEL) || m_tokens < 1 || d->capacity > INT32_MAX)
     return false;
   // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
   // prologue and a larger merge.  Both kernels as they are, device time of a call among others on the same inputs (us here /
@@ -745,6 +1098,8 @@ int launch_attn_short(const AttnArgs& a) {
   p.correction = (a.flags & KVQ_CORRECTION_ON) ? 1 : 0;
   p.m_tokens = (int)a.m_tokens; p.n_cached = (int)a.cache_len; p.n_cur = (int)a.n_cur;
   p.q_blocks = (int)pl.q_blocks; p.splits = pl.splits;
+  const int steps = (int)((a.cache_len + kStep - 1) / kStep + (a.n_cur + kStep - 1) / kStep);
+  p.split_steps = steps / pl.splits; p.split_rest = steps % pl.splits;
   p.scale_log2 = a.softmax_scale * kLog2e;
   p.ax_coef = -a.softmax_scale / 24.0f;
   p.lse = a.lse; p.cached_mass = a.cached_mass;
