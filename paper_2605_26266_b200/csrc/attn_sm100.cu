@@ -127,9 +127,10 @@ struct TParams {
   int n_whole;             // units [0, n_whole) are computed whole; the rest are split over all CTAs
   uint8_t* partial;        // workspace: 2 slots per CTA, see kSlotBytes
   const uint16_t* ax_rows; // workspace: bias operand rows written by rotate_query_kernel, [batch*heads][m_tokens][8]
+  int wide_parts;          // 128 channels: partial rows are FP32 (Plan::wide)
 };
 
-// One partial result: the segment's own normalised output O / l as BF16 (heads of 128 channels; heads of 64 have
+// One partial result: the segment's own normalised output O / l as BF16 (heads of 128 channels, unless Plan::wide; heads of 64 have
 // room for FP32 in the same slot, pieces of 4 columns), then FP32 m[256], l_cur[256],
 // l_cached[256] (running maximum in log2 units and the row sums over current and cached keys).  The output is
 // stored by 16-byte pieces of 8 columns, piece (column group g, row r) at (g * 256 + r) * 16: the softmax
@@ -137,7 +138,9 @@ struct TParams {
 // would write 32 pieces 256 bytes apart, and the load/store unit takes them one line at a time).
 constexpr int kSlotStats = 256 * kD * 2;
 constexpr int kSlotBytes = kSlotStats + 3 * 256 * 4;
-static_assert(kSlotBytes % 256 == 0, "slots stay 256-byte aligned");
+constexpr int kWideStats = 256 * kD * 4;           // the same with FP32 rows of 128 channels (Plan::wide)
+constexpr int kWideSlotBytes = kWideStats + 3 * 256 * 4;
+static_assert(kSlotBytes % 256 == 0 && kWideSlotBytes % 256 == 0, "slots stay 256-byte aligned");
 
 // A contiguous run of key tiles [tb, te) of one unit; `slot` is the CTA's partial-result slot if the run is
 // not the whole unit.
@@ -1155,7 +1158,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // ---- segment epilogue: read this row of O out of TMEM, release it, write the normalised row ----
       const int bh = sg.unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
       const bool whole = sg.tb == 0 && sg.te == T;
-      uint8_t* slot = p.partial + (size_t)(2 * blockIdx.x + sg.slot) * kSlotBytes;   // partial segments only
+      const bool wide = D == 128 && p.wide_parts;
+      uint8_t* slot = p.partial + (size_t)(2 * blockIdx.x + sg.slot) * (wide ? kWideSlotBytes : kSlotBytes);   // partial segments only
       ok = __all_sync(0xFFFFFFFFu, cx.wait(kODone + 2 + qt, (it - 1) & 1, 303));            // the last product of the segment is a second half
       if (!ok) break;
       tc_fence_after();
@@ -1179,10 +1183,10 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tc_fence_before();
           arrive_lead(kOFree + qt);
         }
-        if (D == 64 && !whole) {                     // partial rows of 64 channels stay FP32, pieces of 4 columns
+        if ((D == 64 || wide) && !whole) {           // partial rows in FP32, pieces of 4 columns
 #pragma unroll
           for (int i = 0; i < 64; i += 4)
-            *reinterpret_cast<float4*>(dst + (i >> 2) * piece) =
+            *reinterpret_cast<float4*>(dst + (16 * hf + (i >> 2)) * piece) =
                 make_float4(__uint_as_float(sr[i]) * inv, __uint_as_float(sr[i + 1]) * inv, __uint_as_float(sr[i + 2]) * inv, __uint_as_float(sr[i + 3]) * inv);
         } else if (PAIR && store && whole && p.out_32) {
           // A lane holds a row, so that the 32 lanes of a store meet 32 lines, and the load/store unit takes these one by one: with
@@ -1213,7 +1217,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if (p.lse) p.lse[idx] = (m_run + log2f(l)) * 0.6931471805599453f;
           if (p.cached_mass) p.cached_mass[idx] = lcac / l;
         } else {
-          float* st = reinterpret_cast<float*>(slot + kSlotStats);
+          float* st = reinterpret_cast<float*>(slot + (wide ? kWideStats : kSlotStats));
           st[r256] = m_run; st[256 + r256] = lcur; st[512 + r256] = lcac;
         }
       }
@@ -1359,9 +1363,11 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 // grid (n_units - n_whole, 16): a block handles 16 rows x D columns; thread = (piece, row).
 // pair = 1: the schedule's units are 512 rows worked on by CTA pairs (n_ctas counts pairs); the grid has two blocks
 // per unit in x, one for each 256-row half, whose partial results are those of the CTAs of that rank.
-template <int D>
+// WIDE: FP32 rows, of 128 channels half a row a block (z).
+template <int D, bool WIDE>
 __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_ctas, int pair) {
-  constexpr int kCols = D / 16;                        // columns of a 16-byte piece: 8 in BF16, 4 in FP32 (64 channels)
+  constexpr int kCols = WIDE ? 4 : 8;                  // columns of a 16-byte piece
+  constexpr int kStats = D == 128 && WIDE ? kWideStats : kSlotStats, kSlot = D == 128 && WIDE ? kWideSlotBytes : kSlotBytes;
   const int su = pair ? blockIdx.x >> 1 : blockIdx.x, rank = pair ? blockIdx.x & 1 : 0, kc = pair ? 2 : 1;
   const int unit = p.n_whole + su;
   const int T = p.tiles;
@@ -1387,7 +1393,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   // A thread combines the piece (cg, row): consecutive lanes take consecutive rows, which are 16 bytes
   // apart in a slot.  The finished pieces change places through shared memory so that the output rows are
   // written 256 contiguous bytes at a time.
-  using Out = typename std::conditional<D == 64, uint2, uint4>::type;
+  using Out = typename std::conditional<WIDE, uint2, uint4>::type;
   __shared__ Out s_tile[16 * 16];
   const int cg = threadIdx.x >> 4, rr = threadIdx.x & 15;
   const int bh = unit / p.q_blocks, b = bh / p.heads, h = bh - b * p.heads;
@@ -1400,7 +1406,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   // 1560 rows took 1 to 2 % more on the same inputs again and again (123.4 against 122.0 us; where inputs change, 129 us, the
   // difference is within what two runs differ by).
   // CTA c of the schedule is CTA kc * c + rank of the grid; every CTA of the grid has two slots
-  auto slot_of = [&](int c) { return p.partial + (size_t)(2 * (kc * c + rank) + (c == c_first ? first_slot : 0)) * kSlotBytes; };
+  auto slot_of = [&](int c) { return p.partial + (size_t)(2 * (kc * c + rank) + (c == c_first ? first_slot : 0)) * kSlot; };
   // With fewer tile steps than CTAs (a last round of few units of few tiles) some ranges between the first and the last are
   // empty: their CTAs left nothing, and whatever their slots hold is not this call's.
   const long long split_steps = (long long)(p.n_units - p.n_whole) * T;
@@ -1415,10 +1421,10 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
     for (int j = 0; j < 4; ++j) {
       const bool have = has_part(c0 + j);
       const uint8_t* sl = slot_of(have ? c0 + j : c_last);
-      const float* st = reinterpret_cast<const float*>(sl + kSlotStats);
+      const float* st = reinterpret_cast<const float*>(sl + kStats);
       sm[j] = have ? st[r256] : -INFINITY;                  // not a maximum
       sc[j] = st[256 + r256]; sa[j] = st[512 + r256];
-      a[j] = *reinterpret_cast<const uint4*>(sl + ((size_t)cg * 256 + r256) * 16);
+      a[j] = *reinterpret_cast<const uint4*>(sl + ((size_t)(16 * blockIdx.z + cg) * 256 + r256) * 16);
     }
   };
   fetch(c_first);                                      // one trip to memory where there are at most four
@@ -1427,7 +1433,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
     float mm[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      mm[j] = has_part(c0 + j) ? reinterpret_cast<const float*>(slot_of(c0 + j) + kSlotStats)[r256] : -INFINITY;
+      mm[j] = has_part(c0 + j) ? reinterpret_cast<const float*>(slot_of(c0 + j) + kStats)[r256] : -INFINITY;
     m = fmaxf(fmaxf(m, fmaxf(mm[0], mm[1])), fmaxf(mm[2], mm[3]));
   }
   float acc[kCols] = {};
@@ -1445,7 +1451,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
       const uint32_t pw[4] = {a[j].x, a[j].y, a[j].z, a[j].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        if constexpr (D == 64) {
+        if constexpr (WIDE) {
           acc[e] += w * __uint_as_float(pw[e]);
         } else {
           acc[2 * e] += w * bf16_bits_to_f32(pw[e] & 0xFFFFu);
@@ -1457,16 +1463,16 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
   const float l = l_cur + l_cac, inv = 1.0f / l, norm = D == 64 ? 1.0f / kPartScale * inv : inv;
   Out v;
   v.x = cvt_bf16x2(acc[0] * norm, acc[1] * norm); v.y = cvt_bf16x2(acc[2] * norm, acc[3] * norm);
-  if constexpr (D == 128) { v.z = cvt_bf16x2(acc[4] * norm, acc[5] * norm); v.w = cvt_bf16x2(acc[6] * norm, acc[7] * norm); }
+  if constexpr (!WIDE) { v.z = cvt_bf16x2(acc[4] * norm, acc[5] * norm); v.w = cvt_bf16x2(acc[6] * norm, acc[7] * norm); }
   s_tile[rr * 16 + (cg ^ rr)] = v;
   __syncthreads();
   {
     const int orr = threadIdx.x >> 4, ocg = threadIdx.x & 15;          // output side: a row per 16 lanes
     const int orow = row - rr + orr;
     if (orow < p.m_tokens)
-      *reinterpret_cast<Out*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)orow * p.o_st + ocg * kCols) = s_tile[orr * 16 + (ocg ^ orr)];
+      *reinterpret_cast<Out*>(p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)orow * p.o_st + 64 * blockIdx.z + ocg * kCols) = s_tile[orr * 16 + (ocg ^ orr)];
   }
-  if (cg == 0 && row < p.m_tokens) {
+  if (cg == 0 && blockIdx.z == 0 && row < p.m_tokens) {
     const int64_t idx = (int64_t)bh * p.m_tokens + row;
     if (p.lse) p.lse[idx] = (m + log2f(l)) * 0.6931471805599453f;
     if (p.cached_mass) p.cached_mass[idx] = l_cac * inv;
@@ -1566,25 +1572,37 @@ int max_resident_pairs() {
   return n;
 }
 
-struct Plan { int ctas; int n_whole; };
-Plan plan_grid(int64_t n_units, int64_t tiles, int head_dim, bool pair = false) {
+// wide: partial rows of 128 channels in FP32, so that an output row that is put together is as precise as one that is not.
+struct Plan { int ctas; int n_whole; bool wide; };
+Plan plan_grid(int64_t n_units, int64_t tiles, int head_dim, bool pair = false, bool may_be_wide = true) {
   const int sms = pair ? max_resident_pairs() : num_sms();      // CTAs, or CTA pairs, that run at once
   // Heads of 64 channels keep their partial rows in FP32, so that splitting costs no precision, and the kernels of a call
   // overlap: there a split pays from four tile steps on, down to two tiles a CTA (2 heads x 256 rows over 1 280 keys,
   // 20 tile steps: 33 us on two CTAs, 18 us on ten).
-  const int64_t split_cost = head_dim == 64 ? 4 : 10, least = head_dim == 64 ? 2 : 4;
+  // 128 channels: a split costs ten steps of every CTA where most of them have units, and there it leaves BF16 rows, half of what is written
+  // and read back; where at most half have, there is less to merge and it costs six steps (seven of a pair) with FP32 rows.  Same inputs again
+  // and again, us without and with, 2 bits: 32 units of 10 tiles 31.0 / 26.0, 48 of 12 35.3 / 27.1, 64 of 16 47.8 / 39.5, pairs 32 of 14 38.9 /
+  // 36.9; on the other side of the lines 32 of 7 24.7 / 26.1, 110 of 26 71.3 / 78.3, pairs 60 of 40 87.6 / 93.6, 40 of 17 43.8 / 44.5.  Where
+  // units were left over by one whole round the same holds (180 of 10 65.4 / 57.7); after several the CTAs are apart anyway and a split
+  // gains less than it costs (pairs, 34 of 256 units of 16 tiles: 165.9 / 168.2).
+  const int64_t units = n_units >= sms ? n_units % sms : n_units;       // that would be split
+  const int64_t split_cost = head_dim == 64 ? 4 : may_be_wide && n_units < 2 * sms && 2 * units <= sms ? (pair ? 7 : 6) : 10, least = head_dim == 64 ? 2 : 4;
+  const int64_t idle = tiles * (n_units >= sms ? sms - n_units % sms : sms - n_units);      // tile steps that idle processors could take
+  const bool wide = head_dim == 128 && idle <= 10 * sms;
   if (n_units >= sms) {
     const int64_t r = n_units % sms;
-    return {sms, (int)((r == 0 || tiles * (sms - r) <= split_cost * sms) ? n_units : n_units - r)};
+    if (r == 0 || idle <= split_cost * sms) return {sms, (int)n_units, false};
+    return {sms, (int)(n_units - r), wide};
   }
-  if (tiles * (sms - n_units) <= split_cost * sms) return {(int)n_units, (int)n_units};
+  if (idle <= split_cost * sms) return {(int)n_units, (int)n_units, false};
   const int64_t W = n_units * tiles;
   int64_t c = W / least;
   if (c < n_units) c = n_units;
   if (c > sms) c = sms;
   if (c > W) c = W;
-  return {(int)(c < 1 ? 1 : c), 0};
+  return {(int)(c < 1 ? 1 : c), 0, wide};
 }
+constexpr size_t slot_bytes(const Plan& pl) { return pl.wide ? kWideSlotBytes : kSlotBytes; }
 
 template <int BITS, int GROUP, bool PAIR, int D = 128>
 int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk, const CUtensorMap& mv, const TParams& p,
@@ -1608,7 +1626,8 @@ int launch(const CUtensorMap& mq, const CUtensorMap& mqr, const CUtensorMap& mk,
   int r = launch_after(true, kC, dim3(kC * grid.x), dim3(kThreads), kSmemBytes, st, attn_tcgen05_kernel<BITS, GROUP, PAIR, D>, mq, mqr, mk, mv, p);
   if (r != KVQ_OK) return r;
   if (p.n_whole != p.n_units)     // units were split over CTAs: combine their partial results
-    r = launch_after(true, 1, dim3((unsigned)((p.n_units - p.n_whole) * kC), 16), dim3(256), 0, st, attn_merge_kernel<D>, p, (int)grid.x, PAIR ? 1 : 0);
+    r = launch_after(true, 1, dim3((unsigned)((p.n_units - p.n_whole) * kC), 16, p.wide_parts ? 2 : 1), dim3(256), 0, st,
+                     D == 64 || p.wide_parts ? attn_merge_kernel<D, true> : attn_merge_kernel<D, D == 64>, p, (int)grid.x, PAIR ? 1 : 0);
   return r;
 }
 
@@ -1647,12 +1666,15 @@ static size_t rot_area_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t
   return (rows * (2 * (size_t)d->head_dim + 16) + 255) / 256 * 256;
 }
 
-size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair) {
+// Chunks of at most 64 rows come here only where the few-row kernel does not take them, or when asked for: as they always were.
+static bool may_be_wide(int64_t m_tokens) { return m_tokens > 64; }
+
+size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair, bool least) {
   if (m_tokens <= 0) return 0;
   int64_t qb, nu, tiles;
   schedule_shape(d, cache_len, m_tokens, n_cur, &qb, &nu, &tiles, pair);
-  const Plan pl = plan_grid(nu, tiles, d->head_dim, pair);
-  const size_t slots = pl.n_whole != nu ? (size_t)pl.ctas * (pair ? 2 : 1) * 2 * kSlotBytes : 0;
+  const Plan pl = plan_grid(nu, tiles, d->head_dim, pair, !least && may_be_wide(m_tokens));
+  const size_t slots = pl.n_whole != nu ? (size_t)pl.ctas * (pair ? 2 : 1) * 2 * slot_bytes(pl) : 0;
   return rot_area_bytes(d, cache_len, m_tokens) + slots;
 }
 
@@ -1660,7 +1682,7 @@ int attn_tcgen05_kernel_launches(const kvq_cache_desc* d, int64_t cache_len, int
   if (m_tokens <= 0) return 0;
   int64_t qb, nu, tiles;
   schedule_shape(d, cache_len, m_tokens, n_cur, &qb, &nu, &tiles, pair);
-  const Plan pl = plan_grid(nu, tiles, d->head_dim, pair);
+  const Plan pl = plan_grid(nu, tiles, d->head_dim, pair, may_be_wide(m_tokens));
   return 1 + (cache_len > 0 ? 1 : 0) + (pl.n_whole != nu ? 1 : 0);   // attention, query pre-pass, merge
 }
 
@@ -1714,6 +1736,7 @@ static int launch_planned(const AttnArgs& a, const Plan& pl, int64_t qb, int64_t
   p.partial = slots;
   p.ax_rows = rp.ax;
   p.n_whole = pl.n_whole;
+  p.wide_parts = pl.wide ? 1 : 0;
   p.n_qt = !pair && a.m_tokens <= kBlockM ? 1 : 2;
   dim3 grid((unsigned)pl.ctas);
 #define KVQ_LAUNCH(B_, G_) (pair ? launch<B_, G_, true>(mq, mqr, mk, mv, p, rp, grid, a.stream) \
@@ -1740,7 +1763,10 @@ int launch_attn_tcgen05(const AttnArgs& a) {
   int64_t qb, nu, tiles;
   schedule_shape(a.desc, a.cache_len, a.m_tokens, a.n_cur, &qb, &nu, &tiles, pair);
   if (nu * tiles > 0x7FFFFFFFLL) return KVQ_ERR_UNSUPPORTED;
-  const Plan pl = plan_grid(nu, tiles, a.desc->head_dim, pair);
+  // a workspace that holds no FP32 partial rows, all that was asked for before there were any, gets the plan without them
+  const bool room = a.workspace && reinterpret_cast<uintptr_t>(a.workspace) % 256 == 0 &&
+                    a.workspace_bytes >= attn_tcgen05_workspace_bytes(a.desc, a.cache_len, a.m_tokens, a.n_cur, pair);
+  const Plan pl = plan_grid(nu, tiles, a.desc->head_dim, pair, room && may_be_wide(a.m_tokens));
   // workspace: [rotated-query area][partial-result slots]; its size was checked by the caller
   const size_t rot = rot_area_bytes(a.desc, a.cache_len, a.m_tokens);
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
@@ -1785,7 +1811,7 @@ int launch_attn_tcgen05_static(const AttnArgs& a) {
   int64_t qb, nu, tiles;
   schedule_shape(d, a.cache_len, a.m_tokens, a.n_cur, &qb, &nu, &tiles);
   if (nu * tiles > 0x7FFFFFFFLL) return KVQ_ERR_UNSUPPORTED;
-  Plan pl = plan_grid(nu, tiles, d->head_dim);
+  Plan pl = plan_grid(nu, tiles, d->head_dim, false, false);
   bool need_slots = false;
   if (pl.n_whole != nu) {
     if (pl.n_whole > 0) {

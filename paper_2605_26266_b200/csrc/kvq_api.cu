@@ -267,7 +267,7 @@ int kvq_attn_corrected(const kvq_cache_desc* desc, int64_t cache_begin, int64_t 
   // of its own: a call that brings none, too little, or one that is not aligned, keeps it.
   if (tc && desc->head_dim == 64 && !holds(rotv + attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, false))) tc = false;
   if (!few) {
-    const size_t need = rotv + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens)) : 0);
+    const size_t need = rotv + (tc ? attn_tcgen05_workspace_bytes(desc, cache_len, m_tokens, n_cur, is_pair(desc, flags, m_tokens), true) : 0);
     if (need > 0) {
       if (!workspace) return KVQ_ERR_WORKSPACE;
       // large enough for the kernel kvq_attn_workspace_bytes plans with, which only its alignment keeps from it

@@ -83,7 +83,8 @@ bool attn_tcgen05_counts(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
 // Can TMA address the call's Q, K_cur, V_cur (no zero stride in a real dimension, byte strides below 2^40)?
 bool attn_tcgen05_addressable(const AttnArgs& a);
 // pair: the CTA-pair form of the kernel (KVQ_KERNEL_TCGEN05_PAIR), which plans 512-row units over SM pairs
-size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair);
+// least: what it can do with, the plan without FP32 partial rows of 128 channels
+size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair, bool least = false);
 int attn_tcgen05_kernel_launches(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair);
 int launch_attn_tcgen05(const AttnArgs& a);
 // Cycle budget of the tcgen05 kernel's device-side waits for later launches (0 = the default of about a second).
