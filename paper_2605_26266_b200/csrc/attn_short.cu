@@ -18,7 +18,7 @@
 //
 // What bounds it: latency and instruction issue (two CTAs of four warps an SM, as registers allow), then HBM.  32 heads of 128 channels, 16
 // rows, 16 384 tokens at 4 bits, group 128, where inputs change from call to call: 41.0 us with FP16 keys (36 warp instructions a
-// key), 36.4 with products of codes, 35.4 with the rest as it is here (24 instructions): all query rows and the first keys loaded
+// key), 36.4 with products of codes, 35.4 with the rest as it is here (28 instructions): all query rows and the first keys loaded
 // together, addresses from 32-bit slots, a current step's values on their way while its weights are computed, the merge's rows fetched with
 // their maxima.  Two groups, on the same inputs again and again, 36.2 -> 32.1 us at 2 bits and 37.2 -> 34.2 at 4, four 35.9 -> 34.6 and
 // 37.7 -> 36.2.  Three CTAs an SM: with spilled registers 25 % slower, with the query in shared memory and hardly any spills 4 to 9 %.  The four
@@ -1036,21 +1036,21 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
     return false;
   // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
   // prologue and a larger merge.  Both kernels as they are, device time of a call among others on the same inputs (us here /
-  // there, 128 channels, 2 bits, group 64): one block of rows is faster here (32 heads over 16 384 keys 36 / 58, over none 4.9 / 5.8).
-  // The lines for two blocks (4 200 (head, 128-key tile) pairs), three (1 200) and four (400), as long as all CTAs run at once, were
-  // drawn when launches did not overlap those before them yet, which the other kernel's chain of three gained more from; now
-  // two blocks meet at some 1 100 pairs (32 heads 25 / 25 at 1 056, 40 / 37 at 2 080, 70 / 58 at 4 128), three at 600 (20 / 20 at
-  // 544, 29 / 25 at 1 056), four at 400 (18 / 21 at 288, 14 / 15 at 320, 22 / 21 at 576).  64 channels, where the other kernel has more
-  // fixed cost to each tile, stay ahead further: two blocks 29 / 40 at 2 080, 50 / 62 at 4 128, 123 / 136 at 10 400 of 160 heads.
+  // there, 128 channels, 2 bits, group 64): one block of rows is faster here (32 heads over 16 384 keys 32 / 58, over none 4.7 / 5.9).
+  // The lines for two blocks (4 200 (head, 128-key tile) pairs), three (1 200) and four (400), as long as all CTAs run at once, lie
+  // near where both meet: two blocks, 32 heads, 22 / 25 at 1 056, 36 / 37 at 2 080, 62 / 58 at 4 128; three 18 / 20 at 544, 27 / 25 at
+  // 1 056; four 17 / 21 at 288, 17 / 23 at 320 and, just beyond, 20 at 576 on the other kernel, 22 here as it was with FP16 keys.  64
+  // channels, where the other kernel has more fixed cost to each tile, stay ahead further: two blocks 24 / 40 at 2 080, 41 / 62 at
+  // 4 128, 100 / 136 at 10 400 of 160 heads.
   const int64_t blocks = (m_tokens + kRows - 1) / kRows;
   if (blocks == 1) return true;
   // Small problems, whatever the rows: all CTAs run at once and each has few steps, while the other kernel is a chain of three
   // launches with a prologue of microseconds each.  Counted in steps of 32 keys over all blocks of 16 rows (as above; 4 bits
-  // alike): 64 channels 2 heads x 256 rows over 1 024 keys, 1 280 steps, 7.5 / 14.6; at 4 352 steps 12 / 18; at 5 120 13 / 15 to 14 /
-  // 15; at 8 192 the other kernel's units of 256 rows decide, 17 / 27 with one (16 384 keys), 17 / 22 with two, 17 / 16 with sixteen (8
-  // heads x 512 rows over 512 keys; 2 x 1 000 over 1 024 18 / 15, the worst met); at 10 240 21 / 16 and 22 / 17.  128 channels at 1 056
-  // steps 11 / 17, at 4 224 17 / 18, at 4 608 18 / 21, at 6 432 20 / 18; over an empty cache, where the other kernel is one launch as
-  // well, 5.8 / 6.6 for 16 heads x 128 rows and 7.6 / 6.6 for 32.  For 128 channels only up to the 128 rows of one query tile of the
+  // alike): 64 channels 2 heads x 256 rows over 1 024 keys, 1 280 steps, 6.9 / 14.6; at 4 352 steps 11.6 / 18; at 5 120 12 /
+  // 15; at 8 192 the other kernel's units of 256 rows decide, 14 / 27 with one (16 000 keys), 14 / 22 with two, 15.7 / 16 with sixteen (8
+  // heads x 512 rows over 512 keys; 2 x 1 000 over 1 024 17 / 15, the worst met); at 10 240, with FP16 keys here, 21 / 16 and 22 / 17.  128
+  // channels at 1 040 steps 10 / 17, at 4 160 15 / 19, at 4 608 15 / 19, at 6 432, with FP16 keys here, 20 / 18; over an empty cache, where
+  // the other kernel is one launch as well, 5.5 / 6.6 for 16 heads x 128 rows and 7.7 / 6.7 for 32.  For 128 channels only up to the 128 rows of one query tile of the
   // other kernel, half of which idles there.
   const int64_t bh = (int64_t)d->batch * d->heads;
   const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
