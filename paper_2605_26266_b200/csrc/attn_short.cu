@@ -105,6 +105,12 @@ __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
+// A zero-point within 2^96, so that its product with a step and a row's sum is a number also where it is none.
+__device__ __forceinline__ uint32_t finite_bf16x2(uint32_t a) {
+  uint32_t d;
+  asm("{\n\t.reg .b32 t;\n\tmin.bf16x2 t, %1, %2;\n\tmax.bf16x2 %0, t, %3;\n\t}" : "=r"(d) : "r"(a), "r"(0x6F806F80u), "r"(0xEF80EF80u));
+  return d;
+}
 // x shifted so that bit `from` lands on bit `to` (both known at compile time once unrolled)
 __device__ __forceinline__ uint32_t move_bits(uint32_t x, int from, int to) { return from <= to ? x << (to - from) : x >> (from - to); }
 
@@ -684,7 +690,10 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
         if (gr == 0 && n_valid < kStep) mask_pairs<G>(keys.step, keys.zero, n_valid, c);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          const float2 step = steps_of<G>(keys.step[t], gr), zero = bf16x2_to_f32(zeros_of<G>(keys.zero[t], gr));
+          const uint32_t zeros = zeros_of<G>(keys.zero[t], gr);
+          // 128 channels: a key that was appended with an infinite channel takes all of the weight or none, as where FP16 keys saturate; 64
+          // channels: its scores are not numbers, as in the FP32 form
+          const float2 step = steps_of<G>(keys.step[t], gr), zero = bf16x2_to_f32(D == 128 && !ANY_ZERO ? finite_bf16x2(zeros) : zeros);
           const float2 off = __fmul2_rn(step, make_float2(-zero.x, -zero.y)), sq = __fmul2_rn(step, step);
           if (ANY_ZERO && !kFp32) exact &= key_constant_exact<BITS>(zero.x) && key_constant_exact<BITS>(zero.y);
 #pragma unroll

@@ -58,3 +58,23 @@ def test_queries_of_any_size(d, bits, group):
         assert torch.equal(got[0].view(torch.int16), want[0].view(torch.int16)) and torch.equal(got[1], want[1]), e
     got = run(-30)
     assert torch.isfinite(got[0].float()).all() and (got[1] - want[1]).abs().max() <= 2.0 ** -5 * want[1].abs().max()
+
+
+@pytest.mark.parametrize("bits,group", [(2, 64), (2, 128), (4, 64), (4, 128)])
+def test_zero_points_that_are_no_numbers(bits, group):
+    """A key appended with an infinite channel has an infinite zero-point; with 128 channels its scores stay finite (as where FP16 keys
+    saturate) and it takes all of a row's weight or none, exactly as a zero-point of 2^96."""
+    from paper_2605_26266_b200 import binding as B
+    heads, m, n = 3, 16, 200
+    w = inputs.Workload("zeros", 1900 + bits + group, 1, heads, 128, 32, 0, bits, group, bits)
+    _, k, v = inputs.make_chunk(w, 0, tokens=n)
+    q, kc, vc = (T.to_dev(x) for x in inputs.make_chunk(w, 1, tokens=m))
+    outs = []
+    for bad in ((float("inf"), -float("inf"), float("nan")), (2.0 ** 96, -2.0 ** 96, 2.0 ** 96)):
+        g = B.Cache(1, heads, 128, bits, group, 256)
+        B.kvq_quantize_append(g, T.to_dev(k), T.to_dev(v))
+        bits16 = torch.tensor(bad, device="cuda").bfloat16().view(torch.int16)
+        for h in range(heads):
+            g.views()["k_zero"][0, h, 40 + 60 * h, 0] = bits16[h]
+        outs.append(B.kvq_attn_corrected(g, q, kc, vc, T.sigma_of(128), B.KVQ_CORRECTION_ON))
+    assert torch.isfinite(outs[0].float()).all() and torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
