@@ -1258,6 +1258,14 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         load_raw<BITS, G, D, kNW>(rk, p.k_codes, p.k_scale, p.k_zero, tok_of(k0), k0 < p.n_cached, k_word0);
         load_raw<BITS, G, D, kNW>(rv, p.v_codes, p.v_scale, p.v_zero, tok_of(v0), v0 < p.n_cached, v_word0);
       }
+      if (sg.te <= n_rt) {
+        // No rotation in this segment: keep the phase count in step.  Only once every score product of the previous segment has retired,
+        // or the arrival would stand for one of a warp that has not written its rows of A_extra yet (after a segment of one cached
+        // tile this warp may be that far ahead); and before this segment's own products can be, which wait for the arrivals below.
+        ok = __all_sync(0xFFFFFFFFu, cx.wait(kQEmpty, (nseg & 1) ^ 1, 402));
+        if (!ok) break;
+        arrive_lead(kQRotFull);
+      }
       for (int t = sg.tb; t < sg.te; ++t, ++it) {
         const int s = it & 1;
         const uint32_t ph = (it >> 1) & 1;
@@ -1334,7 +1342,6 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         KVQ_STAMP(21);
       }
       if (!ok) break;
-      if (sg.te <= n_rt) arrive_lead(kQRotFull);   // no rotation in this segment: keep the phase count in step
       ++nseg;
     }
     // The leader's commits arrive on the peer's barriers too, asynchronously: the peer waits for its copy of the last ones, or

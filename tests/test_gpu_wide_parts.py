@@ -78,3 +78,27 @@ def test_a_workspace_without_room_for_them():
     torch.cuda.synchronize()
     assert (room[rotated:] == 0xAB).all()
     T.assert_attn_close(T.from_dev_bf16(out), T.from_dev_bf16(want))
+
+
+@pytest.mark.parametrize("kernel,heads,m,n_cur,n", [
+    ("KVQ_KERNEL_TCGEN05", 180, 100, 100, 1020),           # ranges of one and two tiles: a unit's last cached tile, then the next one's only current one
+    ("KVQ_KERNEL_TCGEN05", 181, 200, 60, 1100),
+    ("KVQ_KERNEL_TCGEN05_PAIR", 100, 300, 100, 1200),
+])
+def test_short_ranges_again_and_again(kernel, heads, m, n_cur, n):
+    """A range may end one unit and begin another with a tile each: the bias rows of the one are all there before its scores are computed,
+    whichever of the expanding warps is ahead."""
+    from paper_2605_26266_b200 import binding as B
+    w = inputs.Workload("again", 1960 + heads + m, 1, heads, 128, 32, 0, 2, 64, 1, head_scale=True)
+    g = B.Cache(1, heads, 128, 2, 64, 1280)
+    _, k, v = (T.to_dev(x) for x in inputs.make_chunk(w, 0, tokens=n))
+    B.kvq_quantize_append(g, k, v)
+    q = T.to_dev(inputs.make_chunk(w, 1, tokens=m)[0])
+    kc, vc = (T.to_dev(x) for x in inputs.make_chunk(w, 2, tokens=n_cur)[1:])
+    flags = B.KVQ_CORRECTION_ON | getattr(B, kernel)
+    want, out = B.kvq_attn_corrected(g, q, kc, vc, T.sigma_of(128), flags), torch.empty_like(q)
+    differ = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(1000):
+        B.kvq_attn_corrected(g, q, kc, vc, T.sigma_of(128), flags, out=out)
+        differ += (out.view(torch.int16) != want.view(torch.int16)).any()
+    assert differ.item() == 0
