@@ -1350,6 +1350,17 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if constexpr (PAIR) {
       if (rank != 0 && warp < 14) cx.drain(kDrain + warp - 12, 0);
     }
+    // Nor need separate commits arrive in order, so that one that has been seen says nothing of those before it: the last of every
+    // barrier that no role waits for any more is waited for too (the softmax groups see the last ones of scores and second halves).
+    if (ok) {
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {
+        if (warp == 12 && it > i) cx.drain(kKEmpty + i, ((it - 1 - i) >> 1) & 1);
+        if (warp == 13 && it > i) cx.drain(kVEmpty + i, ((it - 1 - i) >> 1) & 1);
+        if (warp == 14 && it > 0 && i < p.n_qt) cx.drain(kODone + i, (it - 1) & 1);
+        if (warp == 15 && nseg > 0) cx.drain(i == 0 ? kQEmpty : kQCurDone, (nseg - 1) & 1);
+      }
+    }
   }
 
   wait_for_previous_grid();                      // also in a CTA that had no cached tile

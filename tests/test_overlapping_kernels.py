@@ -110,3 +110,30 @@ def test_a_pair_is_there_while_its_tensor_memory_is_allocated_and_freed():
     inside, after = rest.split("tmem_dealloc_pair(")
     assert inside.count("cluster_sync_all();") == 2 and "wait_for_previous_grid" not in inside[inside.rindex("cluster_sync_all();"):]
     assert "cluster_sync_all();" in after
+
+
+def test_every_barrier_that_is_committed_on_is_waited_for_before_the_exit():
+    """Commits arrive on their barriers in no promised order, and where nobody waits for one it may arrive in the shared memory of the CTA
+    that comes next.  Of the barriers the issuers commit on, the softmax groups wait for every phase of kSFull and for the last one of a
+    segment on kODone + 2; the issuers drain kDrain; the last phases of all others are drained by the dequantizing warps.  Their parities, from the
+    number of tiles and segments, against a count of the commits."""
+    body = dict(kernels(source("attn_sm100.cu")))["attn_tcgen05_kernel"]
+    committed = {re.match(r"k\w+", a).group(0) for a in re.findall(r"\bcommit\(([^()]+)\);", body)}
+    assert committed == {"kSFull", "kODone", "kKEmpty", "kVEmpty", "kQEmpty", "kQCurDone", "kDrain"}
+    tail = body[body.rindex("++nseg;"):body.rindex("wait_for_previous_grid();")]
+    drained = dict(re.findall(r"cx\.drain\((k\w+) \+ i, ([^;]+)\);", tail))
+    assert set(drained) == {"kKEmpty", "kVEmpty", "kODone"}
+    assert "cx.drain(i == 0 ? kQEmpty : kQCurDone, (nseg - 1) & 1);" in tail
+    assert "cx.wait(kSFull + 2 * hf + qt, it & 1, 301)" in body and "cx.wait(kODone + 2 + qt, (it - 1) & 1, 303)" in body
+    parity = {k: eval("lambda it, i: " + v.replace("kODone", "")) for k, v in drained.items()}
+    for tiles in range(1, 9):
+        phases = {(k, i): 0 for k in drained for i in range(2)}
+        for t in range(tiles):                            # tile t uses stage t % 2; a tile's first half of O is committed once
+            phases["kKEmpty", t & 1] += 1
+            phases["kVEmpty", t & 1] += 1
+            phases["kODone", 0] += 1
+            phases["kODone", 1] += 1
+        for (k, i), n in phases.items():
+            assert (n == 0) == (k != "kODone" and tiles <= i)
+            if n:
+                assert parity[k](tiles, i) == (n - 1) & 1, (k, i, tiles)
