@@ -734,7 +734,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     reinterpret_cast<uint4*>(smem + kOffAx)[i] = make_uint4(0, 0, 0, 0);
   // A pair's allocation concerns both CTAs' TMEM: the peer has to run by then.  The two are placed together but need not start together
   // (an SM may have to change its split of L1 and shared memory first).
-  if constexpr (PAIR) { __syncwarp(); cluster_sync_all(); }
+  __syncwarp();                                  // lane 0 comes from the barriers; the allocation wants the whole warp at once
+  if constexpr (PAIR) cluster_sync_all();
   if (warp == 0) {
     if constexpr (PAIR) { tmem_alloc_pair(sbase + kOffMisc, 512); tmem_relinquish_pair(); }
     else { tmem_alloc(sbase + kOffMisc, 512); tmem_relinquish(); }
@@ -1369,6 +1370,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // barriers or the leader's MMAs still read its operands (every role above has come out through bounded waits).
   if constexpr (PAIR) cluster_sync_all();
   if (warp == 0) {
+    __syncwarp();                                // as for the allocation: lane 0 comes from the TMA role
     tc_fence_after();
     if constexpr (PAIR) tmem_dealloc_pair(tmem, 512); else tmem_dealloc(tmem, 512);
     // a wait that gave up left its diagnostic code in the abort word: report the first one

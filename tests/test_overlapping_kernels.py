@@ -137,3 +137,14 @@ def test_every_barrier_that_is_committed_on_is_waited_for_before_the_exit():
             assert (n == 0) == (k != "kODone" and tiles <= i)
             if n:
                 assert parity[k](tiles, i) == (n - 1) & 1, (k, i, tiles)
+
+
+def test_a_warp_is_whole_where_it_allocates_and_frees_tensor_memory():
+    """tcgen05.alloc, .relinquish_alloc_permit and .dealloc are .sync.aligned: all lanes of the warp execute them together.  Lane 0 has run code
+    of its own before both, and nothing promises that the lanes have met again without a __syncwarp()."""
+    body = dict(kernels(source("attn_sm100.cu")))["attn_tcgen05_kernel"]
+    one_lane = body.index("if (tid == 0) {")
+    before = body[one_lane:body.index("tmem_alloc(")]
+    assert re.search(r"\n  __syncwarp\(\);\s*if constexpr \(PAIR\) cluster_sync_all\(\);\s*if \(warp == 0\) \{\s*if constexpr \(PAIR\) \{ tmem_alloc_pair", before)
+    role = body.index("if (lane == 0) {", body.index("tmem_alloc("))
+    assert re.search(r"if \(warp == 0\) \{\s*__syncwarp\(\);[^{}]*tmem_dealloc_pair\(tmem, 512\); else tmem_dealloc\(tmem, 512\);", body[role:])
