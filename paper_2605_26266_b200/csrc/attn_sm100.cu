@@ -106,6 +106,14 @@ constexpr float kLog2e = 1.4426950408889634f;
 // registers per thread after reallocation: 128 * 96 + 256 * 144 + 128 * 112 = 63488 <= 65536
 constexpr int kRegsIssue = 96, kRegsSoftmax = 144, kRegsDequant = 112;
 constexpr float kRescaleThreshold = 8.0f;          // lazy rescale of O: only when the max grows by > 2^8
+// 128 channels: where the running maximum of a part of a unit starts.  A part may begin with keys that the caller has masked through a
+// channel, or hold no others: scores of -inf, or of some -4e37, where the FMA's exact product and the rounded maximum are further
+// apart than an exponential can take.  Below this number, where they are up to 2^6 apart, a part's keys have no weight.  A whole unit starts at
+// -inf, and as it always did takes its maximum from whatever its first keys are.  (The way of 64 channels, product and difference one
+// by one while a maximum is that low, gives such rows even then; as code beside the loop of exponentials it cost 128 channels 3 to 9 %: 16
+// heads x 1560 rows over 6240 tokens 131.7 -> 143.8 us, 32 x 256 over 65 536 300.0 -> 312.1; this way 123.5 -> 123.9 and 283.8 -> 284.6 on the
+// same inputs again and again.)
+constexpr float kNoScore = -0x1p31f;
 
 struct TParams {
   uint16_t* out; int64_t o_sb, o_sh, o_st;
@@ -1055,7 +1063,8 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     int it = 0, nseg = 0;
     bool ok = qt < p.n_qt;                                    // a tile without rows: nothing to do
     while (ok && sch.next(sg)) {
-      float m_run = -INFINITY, lcur = 0.f, lcac = 0.f;   // running max (log2 units), row sums over current / cached keys
+      // running max (log2 units), row sums over current / cached keys
+      float m_run = D == 128 && sg.unit >= p.n_whole ? kNoScore : -INFINITY, lcur = 0.f, lcac = 0.f;
       bool fresh = true;                                 // no product has been added to O in this segment yet
       bool odd_max = true;                               // 64 channels: a maximum of the warp is -inf (no key yet) or very large
       for (int t = sg.tb; ok && t < sg.te; ++t, ++it) {
@@ -1464,6 +1473,8 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const TParams p, int n_
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (!has_part(c0 + j)) continue;                      // the whole block: the last range's rows again, and 0 * inf would be NaN
+      // A part without a score: its sums are 0 and its rows NaN, or with ex2_poly2 what is left of masked keys.  All parts: 0 / 0, as computed whole.
+      if (D == 128 && sm[j] == kNoScore) continue;
       const float f = exp2f(sm[j] - m);
       const float lc = f * sc[j], la = f * sa[j];
       l_cur += lc; l_cac += la;
