@@ -25,6 +25,7 @@
 // score tiles of a step one after the other instead of in turn: 7 %.
 #include <cuda_fp16.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "kvq_common.cuh"
@@ -50,6 +51,7 @@ struct SParams {
   int q_blocks, splits;
   int split_steps, split_rest;         // steps = splits * split_steps + split_rest
   float scale_log2, ax_coef;           // sigma * log2(e), -sigma / 24
+  float q_limit;                       // products of codes: rotated query channels count as at most this, see launch_attn_short
   float* lse; float* cached_mass;
   float* partial;                      // splits > 1: one slot per CTA, see slot_floats
 };
@@ -401,17 +403,16 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
         constexpr int N = KeysT::N, C = KeysT::C;
         float top = 0.f, sum = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) top = fmaxf(top, fabsf(x[e]));
+        for (int e = 0; e < 8; ++e) { x[e] = fminf(fmaxf(x[e], -p.q_limit), p.q_limit); top = fmaxf(top, fabsf(x[e])); }
 #pragma unroll
         for (int off = 1; off < LPR; off *= 2) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, off));
-        const int shift = max(-100, min(24, 14 + 127 - (int)(__float_as_uint(top) >> 23)));
+        const int shift = min(24, 14 + 127 - (int)(__float_as_uint(top) >> 23));      // -100 at least, by q_limit
         const float scale = __uint_as_float((uint32_t)(127 + shift) << 23);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int ch = ln * 8 + e, i = ch % N;                   // N is 8 or 16, so i % (N / 2) is known at compile time up to where it matters
           const int bit = key_place<BITS>(N == 16 ? e : e & 3).bit;
-          const float v = fminf(fmaxf(x[e] * scale * (1.0f / (1 << bit)), -65504.f), 65504.f);
-          const __half hv = __float2half_rn(v);
+          const __half hv = __float2half_rn(x[e] * scale * (1.0f / (1 << bit)));
           sum += __half2float(hv) * (float)(1 << bit);
           sm.in.qr[r * LD + ch / N * N + 2 * (i % (N / 2)) + i / (N / 2)] = __half_as_ushort(hv);
         }
@@ -1111,6 +1112,10 @@ int launch_attn_short(const AttnArgs& a) {
   p.split_steps = steps / pl.splits; p.split_rest = steps % pl.splits;
   p.scale_log2 = a.softmax_scale * kLog2e;
   p.ax_coef = -a.softmax_scale / 24.0f;
+  // Scores in log2 units have to stay below 2^128, and a row's scale with them, or the parts of a row cannot be merged.  With keys in FP16's
+  // range they are below 2^23 times scale_log2 and this limit.  Ordinary scales leave queries room up to some 2^106; from scales of 2^87 on
+  // channels are held where FP16 keys and queries held them.  (2^115 at most: the unit of a row, 2^(shift - 24), is a normal number.)
+  p.q_limit = ldexpf(65504.f, min(99, max(0, 87 - ilogbf(p.scale_log2))));
   p.lse = a.lse; p.cached_mass = a.cached_mass;
   p.partial = static_cast<float*>(a.workspace);
   const bool any_zero = !attn_tcgen05_addressable(a);

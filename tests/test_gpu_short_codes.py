@@ -78,3 +78,23 @@ def test_zero_points_that_are_no_numbers(bits, group):
             g.views()["k_zero"][0, h, 40 + 60 * h, 0] = bits16[h]
         outs.append(B.kvq_attn_corrected(g, q, kc, vc, T.sigma_of(128), B.KVQ_CORRECTION_ON))
     assert torch.isfinite(outs[0].float()).all() and torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
+
+
+@pytest.mark.parametrize("d,bits,group", FORMATS)
+def test_large_queries_under_the_largest_scales(d, bits, group):
+    """Where a scale near 1e30 leaves no room above them, channels beyond FP16's largest number count as that number, as with FP16 keys: scores
+    stay below 2^127 and the row is the same bits as that of the clamped query."""
+    from paper_2605_26266_b200 import binding as B
+    heads, m, n = 3, 16, 500
+    w = inputs.Workload("extreme", 1850 + d + group, 1, heads, d, 32, 0, bits, group, bits)
+    g = B.Cache(1, heads, d, bits, group, 512, rotate_k=False)
+    _, k, v = (T.to_dev(x) for x in inputs.make_chunk(w, 0, tokens=n))
+    B.kvq_quantize_append(g, k, v)
+    q = T.to_dev(inputs.make_chunk(w, 1, tokens=m)[0]) * 2.0 ** 19
+    kc, vc = torch.zeros(2, 1, heads, 1, d, dtype=torch.bfloat16, device="cuda")
+    got = []
+    for rows in (q, q.clamp(-65536, 65536)):
+        lse = torch.empty(1, heads, m, dtype=torch.float32, device="cuda")
+        got.append((B.kvq_attn_corrected(g, rows, kc, vc, 9e29, B.KVQ_CORRECTION_OFF, lse=lse), lse))
+    assert torch.isfinite(got[0][0].float()).all() and torch.isfinite(got[0][1]).all()
+    assert torch.equal(got[0][0].view(torch.int16), got[1][0].view(torch.int16)) and torch.equal(got[0][1], got[1][1])
