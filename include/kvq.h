@@ -307,7 +307,8 @@ int kvq_unpack_codes(const kvq_cache_desc* desc, int which, int64_t begin, int64
  * unrotated score product done), 104 (stage of the packed-tile ring free); MMA issuer 201 (query tile), 203 (value tile), 204 (probabilities), 205 (key
  * tile), 207 (rotated query), 209 (output accumulator read out); softmax warps 301 (scores), 302 (product
  * retired before a rescale), 303 (last product before the epilogue); dequantization warps 401 (key stage free),
- * 402 (query tile, for the bias rows), 404 (value stage free), 406 (packed tile in the ring).
+ * 402 (query tile, for the bias rows), 403 (query buffer free, in a part of a unit without cached tiles), 404 (value stage
+ * free), 406 (packed tile in the ring).
  *
  * kvq_status_word_result maps a status word read back by the caller (host value) to KVQ_OK (0) or
  * KVQ_ERR_TIMEOUT (anything else).

@@ -1272,7 +1272,7 @@ attn_tcgen05_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // No rotation in this segment: keep the phase count in step.  Only once every score product of the previous segment has retired,
         // or the arrival would stand for one of a warp that has not written its rows of A_extra yet (after a segment of one cached
         // tile this warp may be that far ahead); and before this segment's own products can be, which wait for the arrivals below.
-        ok = __all_sync(0xFFFFFFFFu, cx.wait(kQEmpty, (nseg & 1) ^ 1, 402));
+        ok = __all_sync(0xFFFFFFFFu, cx.wait(kQEmpty, (nseg & 1) ^ 1, 403));
         if (!ok) break;
         arrive_lead(kQRotFull);
       }

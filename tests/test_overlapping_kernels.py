@@ -148,3 +148,18 @@ def test_a_warp_is_whole_where_it_allocates_and_frees_tensor_memory():
     assert re.search(r"\n  __syncwarp\(\);\s*if constexpr \(PAIR\) cluster_sync_all\(\);\s*if \(warp == 0\) \{\s*if constexpr \(PAIR\) \{ tmem_alloc_pair", before)
     role = body.index("if (lane == 0) {", body.index("tmem_alloc("))
     assert re.search(r"if \(warp == 0\) \{\s*__syncwarp\(\);[^{}]*tmem_dealloc_pair\(tmem, 512\); else tmem_dealloc\(tmem, 512\);", body[role:])
+
+
+def test_a_site_code_names_one_wait():
+    """The code that an expired wait leaves in the status word tells which one it was; kvq.h lists them."""
+    text = source("attn_sm100.cu")
+    at = {}
+    for m in re.finditer(r"cx\.wait\([^;]*?, (\d{3})\)", text):
+        at.setdefault(int(m.group(1)), []).append(m.start())
+    assert {c for c, places in at.items() if len(places) > 1} == {402}
+    a, b = at[402]                                            # the two forms of one wait, a pair's and a CTA's
+    assert text[a:b].count(";") == 1 and "else ok = " in text[a:b]
+    with open(os.path.join(CSRC, "..", "..", "include", "kvq.h")) as f:
+        header = f.read()
+    listed = header[header.index("Site codes:"):header.index("kvq_status_word_result maps")]
+    assert set(at) == {int(c) for c in re.findall(r"\b(\d{3}) \(", listed)}
