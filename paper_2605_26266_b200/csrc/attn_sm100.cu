@@ -1613,7 +1613,7 @@ Plan plan_grid(int64_t n_units, int64_t tiles, int head_dim, bool pair = false, 
   // 128 channels: a split costs ten steps of every CTA where most of them have units, and there it leaves BF16 rows, half of what is written
   // and read back; where at most half have, there is less to merge and it costs six steps (seven of a pair) with FP32 rows.  Same inputs again
   // and again, us without and with, 2 bits: 32 units of 10 tiles 31.0 / 26.0, 48 of 12 35.3 / 27.1, 64 of 16 47.8 / 39.5, pairs 32 of 14 38.9 /
-  // 36.9; on the other side of the lines 32 of 7 24.7 / 26.1, 110 of 26 71.3 / 78.3, pairs 60 of 40 87.6 / 93.6, 40 of 17 43.8 / 44.5.  Where
+  // 36.9, one query tile in use (64 rows) 40 of 12 25.8 / 18.5, 50 of 10 23.0 / 21.3; on the other side of the lines 32 of 7 24.7 / 26.1, 110 of 26 71.3 / 78.3, pairs 60 of 40 87.6 / 93.6, 40 of 17 43.8 / 44.5.  Where
   // units were left over by one whole round the same holds (180 of 10 65.4 / 57.7); after several the CTAs are apart anyway and a split
   // gains less than it costs (pairs, 34 of 256 units of 16 tiles: 165.9 / 168.2).
   const int64_t units = n_units >= sms ? n_units % sms : n_units;       // that would be split
@@ -1697,8 +1697,10 @@ static size_t rot_area_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t
   return (rows * (2 * (size_t)d->head_dim + 16) + 255) / 256 * 256;
 }
 
-// Chunks of at most 64 rows come here only where the few-row kernel does not take them, or when asked for: as they always were.
-static bool may_be_wide(int64_t m_tokens) { return m_tokens > 64; }
+// A block of 16 rows is the few-row kernel's whatever its keys, and comes here only when this kernel is asked for or the workspace suits
+// nothing else.  Callers find that size by asking for this kernel's, which for such a chunk therefore stays below the few-row
+// kernel's: the rotated queries' room.  From 17 rows on a split pays as for any chunk (plan_grid).
+static bool may_be_wide(int64_t m_tokens) { return m_tokens > 16; }
 
 size_t attn_tcgen05_workspace_bytes(const kvq_cache_desc* d, int64_t cache_len, int64_t m_tokens, int64_t n_cur, bool pair, bool least) {
   if (m_tokens <= 0) return 0;

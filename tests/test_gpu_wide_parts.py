@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     ("KVQ_KERNEL_TCGEN05", 16, 700, 700, 700, 144),        # 48 units of 12 tiles, four tiles a CTA
     ("KVQ_KERNEL_TCGEN05", 30, 256, 129, 1000, 75),        # 30 of 10
     ("KVQ_KERNEL_TCGEN05", 180, 100, 100, 1020, 148),      # 32 of 9 behind a round of 148, one query tile
+    ("KVQ_KERNEL_TCGEN05", 40, 64, 64, 1400, 120),         # 40 of 12: a chunk of few rows like any other
     ("KVQ_KERNEL_TCGEN05_PAIR", 32, 300, 512, 1279, 148),  # 32 of 14 on 74 pairs
     ("KVQ_KERNEL_TCGEN05_PAIR", 100, 513, 300, 600, 148),  # 52 of 8 behind two rounds: not split, the pair's line is higher
     ("KVQ_KERNEL_TCGEN05_PAIR", 100, 200, 300, 900, 148),  # 26 of 11 behind a round of 74
