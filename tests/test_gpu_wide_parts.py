@@ -1,6 +1,8 @@
 """128 channels, few units of few tiles: split with FP32 partial rows, by both tcgen05 kernels, all units and a last round of them; against the
-oracle and no further from it than output rounding and weights in BF16 put a unit that is not split, from workspaces full of NaN and of
+oracle and no further from it than the same call without room for them, whose units are not split, from workspaces full of NaN and of
 another call's rows."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -23,7 +25,7 @@ pytestmark = pytest.mark.gpu
 ])
 def test_fp32_parts(kernel, heads, m, n_cur, n, ctas):
     from paper_2605_26266_b200 import binding as B
-    picked = sorted({0, heads - 1, heads // 2, heads - 7})
+    picked = [heads - 16, heads - 13, heads - 7, heads - 1]      # of units that are split
     w = inputs.Workload("wide", 1950 + heads + m, 1, heads, 128, 32, 0, 2, 64, 1, head_scale=True)
     g, o = B.Cache(1, heads, 128, 2, 64, 1408), O.Cache(1, len(picked), 128, 2, 64, 1408)
     _, k, v = inputs.make_chunk(w, 0, tokens=n)
@@ -36,22 +38,27 @@ def test_fp32_parts(kernel, heads, m, n_cur, n, ctas):
     rotated = -(-heads * m * 272 // 256) * 256
     if torch.cuda.get_device_properties(0).multi_processor_count == 148 and m != 513:
         assert need - rotated == ctas * 2 * (256 * 128 * 4 + 3 * 256 * 4)
-    rows = np.unique(np.r_[0, 31, 127 % m, 128 % m, 255 % m, 256 % m, m - 1])
-    want = O.attn_corrected(o, 0, n, q[:, picked], kc[:, picked], vc[:, picked], sigma, correction=True, rows=rows)
+    want = O.attn_corrected(o, 0, n, q[:, picked], kc[:, picked], vc[:, picked], sigma, correction=True)
     args = (g, T.to_dev(q), T.to_dev(kc), T.to_dev(vc), sigma, flags)
     g.workspace = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda")
+    dq, dk, dv, st = *args[1:4], B._strides
+    whole = torch.empty_like(dq)
+    assert B.lib.kvq_attn_corrected(C.byref(g.desc), 0, n, dq.data_ptr(), st(dq), dk.data_ptr(), dv.data_ptr(), st(dk), m, n_cur, whole.data_ptr(), st(whole),
+                                    sigma, flags, None, None, g.workspace.data_ptr(), rotated, None, B._stream()) == B.KVQ_OK
+    error = lambda x: np.linalg.norm(T.from_dev_bf16(x)[0][picked] - want["out"]) / np.linalg.norm(want["out"])
     first = None
     for fill in (0xFF, 0x3F):
         g.workspace.fill_(fill)
         lse = torch.empty(1, heads, m, dtype=torch.float32, device="cuda")
         mass = torch.empty_like(lse)
         out = B.kvq_attn_corrected(*args, lse=lse, cached_mass=mass)
-        got = T.from_dev_bf16(out)[0][picked][:, rows]
+        got = T.from_dev_bf16(out)[0][picked]
         T.assert_attn_close(got, want["out"], f"fill {fill:#x}")
-        # output and weights in BF16 (2^-9 of a value at most, 2^-9 / sqrt(3) in the mean, each) and FP16 queries: below 3e-3
-        assert np.linalg.norm(got.reshape(-1) - want["out"].reshape(-1)) <= 3e-3 * np.linalg.norm(want["out"])
-        assert np.abs(lse.cpu().numpy()[0][picked][:, rows] - want["lse"].reshape(len(picked), -1)).max() < 2e-2
-        assert np.abs(mass.cpu().numpy()[0][picked][:, rows] - want["cached_mass"].reshape(len(picked), -1)).max() < 1e-2
+        # A split by itself lowers the error by 1 to 4 % (each part's largest weight is exact).  Rows rounded to BF16, 2^-9 / sqrt(3) of a value at most,
+        # would add some 1e-3 in quadrature to 2.3e-3
+        assert error(out) <= 1.01 * error(whole)
+        assert np.abs(lse.cpu().numpy()[0][picked] - want["lse"].reshape(len(picked), -1)).max() < 2e-2
+        assert np.abs(mass.cpu().numpy()[0][picked] - want["cached_mass"].reshape(len(picked), -1)).max() < 1e-2
         first = out if first is None else first
         assert torch.equal(out.view(torch.int16), first.view(torch.int16))
 
@@ -59,8 +66,6 @@ def test_fp32_parts(kernel, heads, m, n_cur, n, ctas):
 def test_a_workspace_without_room_for_them():
     """A call may bring what was asked for before there were FP32 partial rows, the rotated queries' room: the units are not split then, and
     nothing behind the workspace is touched."""
-    import ctypes as C
-
     from paper_2605_26266_b200 import binding as B
     heads, m, n = 16, 700, 700
     w = inputs.Workload("room", 1990, 1, heads, 128, 32, 0, 2, 64, 1)
