@@ -207,9 +207,12 @@ int kvq_attn_kernel_launches(const kvq_cache_desc* desc, int64_t cache_len,
  * cached_mass_out  optional device float [batch,heads,m_tokens]: P_S of Eq. (4), the softmax mass on
  *                  cached keys; NULL to skip.
  * workspace        device scratch of at least kvq_attn_workspace_bytes() bytes, 256-byte aligned;
- *                  may be NULL when that size is 0.  Contents need not be initialised.  Of that size, FP32 partial rows (128
- *                  channels, few units of few tiles: at least 134 144 bytes for each of two slots a CTA) may be left out: the
- *                  units are then not split.  KVQ_KERNEL_AUTO has a
+ *                  may be NULL when that size is 0.  Contents need not be initialised.  Of the size of a call of 128 channels with
+ *                  few query blocks and few key tiles, whose tiles are split, FP32 partial rows may be left out: it is accepted with batch *
+ *                  heads * m_tokens * (2 * head_dim + 16) bytes, rounded up to a multiple of 256 (none when cache_len is 0), and with
+ *                  KVQ_ROTATE_V and cache_len > 0 another 2 * batch * heads * n_cur * head_dim, rounded up likewise.  Its tiles are then not
+ *                  split: one launch fewer than kvq_attn_kernel_launches() counts, and the last bits of the output may be others than with the
+ *                  whole size.  Calls whose partial rows may not be left out refuse that size.  KVQ_KERNEL_AUTO has a
  *                  slower kernel for a call whose workspace is missing, too small or not aligned where that kernel
  *                  served such calls without one (heads of 64 channels, tensors TMA cannot address; unless KVQ_ROTATE_V),
  *                  and for a few query rows the tcgen05 kernel if the workspace suits only that; otherwise it is refused

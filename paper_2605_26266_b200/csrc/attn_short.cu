@@ -674,7 +674,8 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
               for (int i = 0; i < 2; ++i) {
                 constexpr int kTop = kTopKeyBit<BITS>;
                 const Place at = key_place<BITS>(2 * j + i);
-                if constexpr (kFp32) {                             // rounded to FP16, then times 2^(bit - top): still exact
+                // rounded to FP16, then times 2^(bit - top): exact, as such keys, whole numbers times an E4M3, are multiples of 2^-9
+                if constexpr (kFp32) {
                   const uint32_t x = w[t] >> ((2 * j + i) * BITS);
                   const uint32_t k2 = pack_f16_sat(((float)(x & kMask) - key_zero[t]) * key_step[t], ((float)((x >> 16) & kMask) - key_zero[t]) * key_step[t]);
                   const uint32_t down = (uint32_t)(15 + at.bit - kTop) << 10;
@@ -692,8 +693,8 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const uint32_t zeros = zeros_of<G>(keys.zero[t], gr);
-          // 128 channels: a key that was appended with an infinite channel takes all of the weight or none, as where FP16 keys saturate; 64
-          // channels: its scores are not numbers, as in the FP32 form
+          // 128 channels: a key that was appended with an infinite channel takes all of the weight or none, as where FP16 keys saturate.  With
+          // ANY_ZERO its scores are not numbers here, but such a zero-point is not exact either: the FP32 form follows, whose keys saturate
           const float2 step = steps_of<G>(keys.step[t], gr), zero = bf16x2_to_f32(D == 128 && !ANY_ZERO ? finite_bf16x2(zeros) : zeros);
           const float2 off = __fmul2_rn(step, make_float2(-zero.x, -zero.y)), sq = __fmul2_rn(step, step);
           if (ANY_ZERO && !kFp32) exact &= key_constant_exact<BITS>(zero.x) && key_constant_exact<BITS>(zero.y);
