@@ -1048,27 +1048,29 @@ bool attn_short_supports(const kvq_cache_desc* d, int64_t cache_len, int64_t m_t
   // Every 16 rows expand the codes again, 256 rows of the tcgen05 kernel once; but that kernel has a pre-pass, a larger
   // prologue and a larger merge.  Both kernels as they are, device time of a call among others on the same inputs (us here /
   // there, 128 channels, 2 bits, group 64): one block of rows is faster here (32 heads over 16 384 keys 32 / 58, over none 4.7 / 5.9).
-  // The lines for two blocks (4 200 (head, 128-key tile) pairs), three (1 200) and four (400), as long as all CTAs run at once, lie
-  // near where both meet: two blocks, 32 heads, 22 / 25 at 1 056, 36 / 37 at 2 080, 62 / 58 at 4 128; three 18 / 20 at 544, 27 / 25 at
-  // 1 056; four 17 / 21 at 288, 17 / 23 at 320 and, just beyond, 20 at 576 on the other kernel, 22 here as it was with FP16 keys.  64
-  // channels, where the other kernel has more fixed cost to each tile, stay ahead further: two blocks 24 / 40 at 2 080, 41 / 62 at
+  // The lines for two blocks (4 200 (head, 128-key tile) pairs), three (1 200) and four (400), as long as all CTAs run at once, were
+  // drawn for FP16 keys and launches that did not overlap.  With both kernels as they are they meet near 2 500, 900 and 480: two blocks, 32
+  // heads, 23 / 25 at 1 056, 36 / 38 at 2 112, 50 / 47 at 3 104, 63 / 58 at 4 128; three 19 / 20 at 544, 22 / 24 at 800, 27 / 25 at 1 056; four
+  // 17 / 20 at 320, 21 / 20 at 480, 24 / 20 at 576.  Between there and the lines a call takes up to a tenth longer here.  64 channels, where the other kernel has more fixed cost to each tile, stay ahead further: two blocks 24 / 40 at 2 080, 41 / 62 at
   // 4 128, 100 / 136 at 10 400 of 160 heads.
   const int64_t blocks = (m_tokens + kRows - 1) / kRows;
   if (blocks == 1) return true;
   // Small problems, whatever the rows: all CTAs run at once and each has few steps, while the other kernel is a chain of three
   // launches with a prologue of microseconds each.  Counted in steps of 32 keys over all blocks of 16 rows (as above; 4 bits
   // alike): 64 channels 2 heads x 256 rows over 1 024 keys, 1 280 steps, 6.9 / 14.6; at 4 352 steps 11.6 / 18; at 5 120 12 /
-  // 15; at 8 192 the other kernel's units of 256 rows decide, 14 / 27 with one (16 000 keys), 14 / 22 with two, 15.7 / 16 with sixteen (8
-  // heads x 512 rows over 512 keys; 2 x 1 000 over 1 024 17 / 15, the worst met); at 10 240, with FP16 keys here, 21 / 16 and 22 / 17.  128
-  // channels at 1 040 steps 10 / 17, at 4 160 15 / 19, at 4 608 15 / 19, at 6 432, with FP16 keys here, 20 / 18; over an empty cache, where
-  // the other kernel is one launch as well, 5.5 / 6.6 for 16 heads x 128 rows and 7.7 / 6.7 for 32.  For 128 channels only up to the 128 rows of one query tile of the
-  // other kernel, half of which idles there.
+  // 15; at 8 192 the other kernel's units of 256 rows decide, 14 / 27 with one (16 000 keys), 14 / 22 with two, 15.6 / 15.8 with sixteen (8
+  // heads x 512 rows over 512 keys; 2 x 1 000 over 1 024 17 / 15, the worst met); at 10 240 18.6 / 17.1 (8 x 512 over 768), 18.3 / 17.0 (4 x 1 024
+  // over 256), 15.8 / 20.1 (16 x 320 over 700).  128 channels at 1 040 steps 10 / 17, at 4 160 15 / 19, at 4 608 15 / 19 to 17.4 / 17.8, at 6 400 20.5 / 18.2
+  // (16 heads x 128 rows) and 18.6 / 18.4 (16 x 96); over an empty cache, where the other kernel is one launch as well, 5.5 / 6.6 for 16 heads x
+  // 128 rows and 7.7 / 6.7 for 32.  For 128 channels only up to the 128 rows of one query tile of the other kernel, half of which idles there.
   const int64_t bh = (int64_t)d->batch * d->heads;
   const int64_t steps = (cache_len + kStep - 1) / kStep + (n_cur + kStep - 1) / kStep;
   // 64 channels, more heads than processors, one tile of rows, current keys within half a tile, no cache: a CTA of the tcgen05 kernel
   // would take several units of half a tile each.  Two of some 28 000 random calls of all kernels ended in a launch failure, two of the
   // three of this form and none of the 17 with more keys; the cause was not found by reading, and 300 such calls with every role's
-  // steps recorded ran through.  They do not run there: 172 heads x 111 rows over 5 keys 11 us here (148 heads x 111 rows, which do, 7).
+  // steps recorded ran through.  Two gaps found since, one-CTA exits that left commits unwaited for and allocations by a warp that might not be
+  // whole, are closed; that they were the cause is not known.  Such calls do not run there: 172 heads x 111 rows over 5 keys 11 us here (148
+  // heads x 111 rows, which do, 7).
   if (d->head_dim == 64 && cache_len == 0 && n_cur <= 64 && blocks <= 8 && bh > resident_ctas() / kCtasPerSm) return true;
   if (d->head_dim == 64) {
     if (bh * blocks <= resident_ctas() / kCtasPerSm * kCtasPerSm64 && bh * blocks * steps <= 8192) return true;
