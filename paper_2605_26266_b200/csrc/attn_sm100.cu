@@ -1613,17 +1613,23 @@ Plan plan_grid(int64_t n_units, int64_t tiles, int head_dim, bool pair = false, 
   // 128 channels: a split costs ten steps of every CTA where most of them have units, and there it leaves BF16 rows, half of what is written
   // and read back; where at most half have, there is less to merge and it costs six steps (seven of a pair) with FP32 rows.  Same inputs again
   // and again, us without and with, 2 bits: 32 units of 10 tiles 31.0 / 26.0, 48 of 12 35.3 / 27.1, 64 of 16 47.8 / 39.5, pairs 32 of 14 38.9 /
-  // 36.9, one query tile in use (64 rows) 40 of 12 25.8 / 18.5, 50 of 10 23.0 / 21.3; on the other side of the lines 32 of 7 24.7 / 26.1, 110 of 26 71.3 / 78.3, pairs 60 of 40 87.6 / 93.6, 40 of 17 43.8 / 44.5.  Where
-  // units were left over by one whole round the same holds (180 of 10 65.4 / 57.7); after several the CTAs are apart anyway and a split
-  // gains less than it costs (pairs, 34 of 256 units of 16 tiles: 165.9 / 168.2).
-  const int64_t units = n_units >= sms ? n_units % sms : n_units;       // that would be split
-  const int64_t split_cost = head_dim == 64 ? 4 : may_be_wide && n_units < 2 * sms && 2 * units <= sms ? (pair ? 7 : 6) : 10, least = head_dim == 64 ? 2 : 4;
-  const int64_t idle = tiles * (n_units >= sms ? sms - n_units % sms : sms - n_units);      // tile steps that idle processors could take
+  // 36.9, one query tile in use (64 rows) 40 of 12 25.8 / 18.5, 50 of 10 23.0 / 21.3; on the other side of the lines 32 of 7 24.7 / 26.1, 110 of
+  // 26 71.3 / 78.3, pairs 60 of 40 87.6 / 93.6, 40 of 17 43.8 / 44.5; seven tiles are no two ranges of four (20 of 7 18.6 / 19.5).
+  // Where units were left over by one whole round the same holds (180 of 10 65.4 / 57.7), with more than three eighths of the CTAs a step
+  // later (pairs 32 of 13 67.2 / 68.8, of 17 83.0 / 80.2; 57 of 10 63.5 / 65.3, 74 of 13 57.2 / 60.2, of 16 103 / 94.5).  But such units are cut
+  // for all CTAs however few their tiles are, and with less than one a CTA the merge looks for its parts among empty ranges: left over 2 of 8 tiles
+  // 36.6 / 119, 11 of 9 41.6 / 50.4, 16 of 9 42.0 / 46.7, pairs 6 of 10 54.0 / 58.1; from one on 14 of 11 48.0 / 41.0, 18 of 9 42.7 / 35.9, pairs
+  // 8 of 10 53.9 / 47.1.  After several rounds the CTAs are apart anyway and a split gains less than it costs (pairs, 34 of 256 units of 16
+  // tiles: 165.9 / 168.2).
+  const bool behind = n_units >= sms;
+  const int64_t units = behind ? n_units % sms : n_units;       // that would be split
+  const bool cheap = may_be_wide && n_units < 2 * sms && 2 * units <= sms && (behind ? units * tiles >= sms : tiles >= 2 * 4);
+  const int64_t split_cost = head_dim == 64 ? 4 : !cheap ? 10 : (pair ? 7 : 6) + (behind && 8 * units > 3 * sms ? 1 : 0), least = head_dim == 64 ? 2 : 4;
+  const int64_t idle = tiles * (sms - units);      // tile steps that idle processors could take
   const bool wide = head_dim == 128 && idle <= 10 * sms;
-  if (n_units >= sms) {
-    const int64_t r = n_units % sms;
-    if (r == 0 || idle <= split_cost * sms) return {sms, (int)n_units, false};
-    return {sms, (int)(n_units - r), wide};
+  if (behind) {
+    if (units == 0 || idle <= split_cost * sms) return {sms, (int)n_units, false};
+    return {sms, (int)(n_units - units), wide};
   }
   if (idle <= split_cost * sms) return {(int)n_units, (int)n_units, false};
   const int64_t W = n_units * tiles;

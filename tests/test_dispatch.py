@@ -60,3 +60,25 @@ def test_64_channels_beyond_the_counts_of_the_tcgen05_kernel(B):
     desc, size = B.kvq_cache_desc(1, 64, 64, 2, 64, B.KVQ_ROTATE_K, 65536), C.c_size_t(0)
     for m in (1 << 18, 1 << 20):
         assert B.lib.kvq_attn_workspace_bytes(C.byref(desc), 65536, m, m, B.KVQ_KERNEL_TCGEN05, C.byref(size)) == B.KVQ_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("kernel,heads,m,tiles,split", [
+    # 148 CTAs, 74 pairs; tiles: the chunk's and the cache's.  Few units: from six idle tile steps a CTA on, seven a pair, and two ranges of four
+    ("TCGEN05", 32, 256, 7, False), ("TCGEN05", 32, 256, 8, True), ("TCGEN05", 14, 256, 7, False), ("TCGEN05", 74, 256, 12, False), ("TCGEN05", 74, 256, 13, True),
+    ("TCGEN05_PAIR", 37, 512, 14, False), ("TCGEN05_PAIR", 37, 512, 15, True),
+    # left over by a whole round: only with a tile step for every CTA, and a step later with many units
+    ("TCGEN05", 150, 256, 8, False), ("TCGEN05", 150, 120, 10, False), ("TCGEN05", 158, 256, 10, False), ("TCGEN05", 164, 256, 9, False),
+    ("TCGEN05", 162, 256, 10, False), ("TCGEN05", 162, 256, 11, True), ("TCGEN05", 166, 256, 9, True), ("TCGEN05", 180, 100, 9, True),
+    ("TCGEN05", 205, 256, 10, False), ("TCGEN05", 190, 256, 9, True), ("TCGEN05", 222, 256, 13, False), ("TCGEN05", 222, 256, 15, True),
+    ("TCGEN05_PAIR", 76, 512, 10, False), ("TCGEN05_PAIR", 82, 512, 9, False), ("TCGEN05_PAIR", 82, 512, 10, True),
+    ("TCGEN05_PAIR", 106, 512, 13, False), ("TCGEN05_PAIR", 106, 512, 15, True),
+    ("TCGEN05", 300, 256, 9, False),                                                                                     # by several
+])
+def test_few_units_of_few_tiles_are_split_where_that_is_faster(B, kernel, heads, m, tiles, split):
+    flags = B.KVQ_CORRECTION_ON | getattr(B, "KVQ_KERNEL_" + kernel)
+    cached = 128 * (tiles - -(-m // 128)) - 5
+    size, launches = plan(B, 128, 1, heads, m, m, cached, flags)
+    rotated = -(-heads * m * 272 // 256) * 256
+    assert (launches == 3) == split == (size > rotated)                      # pre-pass, attention, and a merge where units are split
+    if split:
+        assert (size - rotated) % (2 * 134144) == 0                          # FP32 rows
