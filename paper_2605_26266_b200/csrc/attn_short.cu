@@ -292,7 +292,6 @@ template <int BITS>
 __host__ __device__ constexpr Place key_place(int i) {
   return BITS == 4 ? Place{i < 2 ? 0 : 8, 4 * (i & 1)} : Place{i < 5 ? 0 : 10, 2 * (i < 5 ? i : i - 5)};
 }
-template <int BITS> constexpr int kTopKeyBit = BITS == 4 ? 4 : 8;
 // ANY_ZERO: groups whose constants are not exact (key_constant_exact, value_constant_exact) are expanded in FP32, as in the
 // warp-level kernel, which served the calls this is set for before: heads of 64 channels, and chunks TMA cannot address.  A
 // warp works in 16 bits, notes whether it met such a group, and then takes its steps once more in FP32.  Any branch inside a
@@ -643,22 +642,25 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
     for (; st < last_c; st += kWarps) {
       const Step here = step_of(st);
       load_values<D, BITS, GROUP>(vals, slab, here, g, c);         // on their way while the scores are computed
-      float s[4][4];
+      float s[4][4], raw[4][4];                                    // FP32 form: keys themselves, one chain of products over both groups
       const int n_valid = p.n_cached - st * kStep;
 #pragma unroll
       for (int gr = 0; gr < G; ++gr) {
-        float key_step[4], key_zero[4];                            // of key 8 t + g, which the FP32 form expands with
+        float key_step[4], key_zero[4];                            // of key 8 t + g, which the FP32 form expands with: the lane with c = g / 2 has it
         if constexpr (kFp32) {
+          if (gr == 0 && n_valid < kStep) mask_pairs<G>(keys.step, keys.zero, n_valid, c);
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
-            const uint64_t at = (uint64_t)(here.slot[t >> 1] + g + 8 * (t & 1)) * G + gr;
-            const bool in = 8 * t + g < n_valid;
-            key_step[t] = in ? e4m3_byte_to_f32(load_coherent(slab.scale[0] + at)) : 0.f;
-            key_zero[t] = in ? bf16_bits_to_f32(load_coherent(slab.zero[0] + at)) : 0.f;
+            const uint32_t both = zeros_of<G>(keys.zero[t], gr);
+            const float2 steps = steps_of<G>(keys.step[t], gr);
+            const int from = (lane & ~3) | (g >> 1);
+            const uint32_t zero = __shfl_sync(0xFFFFFFFFu, both, from);
+            const float s0 = __shfl_sync(0xFFFFFFFFu, steps.x, from), s1 = __shfl_sync(0xFFFFFFFFu, steps.y, from);
+            key_step[t] = g & 1 ? s1 : s0;
+            key_zero[t] = __uint_as_float(g & 1 ? zero & 0xFFFF0000u : zero << 16);
           }
         }
         // the four tiles in turn: a tile's products are one chain, and four chains hide each other's latency
-        float raw[4][4];
 #pragma unroll
         for (int wi = 0; wi < KWG; ++wi) {
           uint32_t w[4];
@@ -672,24 +674,20 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
               uint32_t bf[2];
 #pragma unroll
               for (int i = 0; i < 2; ++i) {
-                constexpr int kTop = kTopKeyBit<BITS>;
                 const Place at = key_place<BITS>(2 * j + i);
-                // rounded to FP16, then times 2^(bit - top): exact, as such keys, whole numbers times an E4M3, are multiples of 2^-9
-                if constexpr (kFp32) {
+                if constexpr (kFp32) {                             // rounded to FP16
                   const uint32_t x = w[t] >> ((2 * j + i) * BITS);
-                  const uint32_t k2 = pack_f16_sat(((float)(x & kMask) - key_zero[t]) * key_step[t], ((float)((x >> 16) & kMask) - key_zero[t]) * key_step[t]);
-                  const uint32_t down = (uint32_t)(15 + at.bit - kTop) << 10;
-                  bf[i] = fma_f16x2(k2, down | (down << 16), 0u);
+                  bf[i] = pack_f16_sat(((float)(x & kMask) - key_zero[t]) * key_step[t], ((float)((x >> 16) & kMask) - key_zero[t]) * key_step[t]);
                 } else {
                   bf[i] = (w[t] >> at.shift) & ((kMask | (kMask << 16)) << at.bit);
                 }
               }
               const uint32_t (&a)[4] = qf[(gr * KWG + wi) * KPW + j];
-              if (wi == 0 && j == 0) mma_f16_first(raw[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
+              if (wi == 0 && j == 0 && (!kFp32 || gr == 0)) mma_f16_first(raw[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
               else mma_f16(raw[t], a[0], a[1], a[2], a[3], bf[0], bf[1]);
             }
         }
-        if (gr == 0 && n_valid < kStep) mask_pairs<G>(keys.step, keys.zero, n_valid, c);
+        if (!kFp32 && gr == 0 && n_valid < kStep) mask_pairs<G>(keys.step, keys.zero, n_valid, c);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const uint32_t zeros = zeros_of<G>(keys.zero[t], gr);
@@ -702,11 +700,15 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
           for (int r = 0; r < 2; ++r) {
             // the bias last: beside the two sums that cancel it would lose bits
             const float2 x = make_float2(raw[t][2 * r], raw[t][2 * r + 1]);
-            constexpr float kUnit = 1.0f / (1 << (24 - kTopKeyBit<BITS>));
-            const float2 dot = kFp32 ? __fmul2_rn(x, make_float2(kUnit, kUnit))
-                                     : __ffma2_rn(x, step, __fmul2_rn(off, make_float2(row_sum[r][gr], row_sum[r][gr])));
-            float2 v = __ffma2_rn(sq, make_float2(row_nu[r][gr], row_nu[r][gr]), dot);
-            if (gr > 0) v = __fadd2_rn(v, make_float2(s[t][2 * r], s[t][2 * r + 1]));
+            const float2 sum = make_float2(s[t][2 * r], s[t][2 * r + 1]), nu = make_float2(row_nu[r][gr], row_nu[r][gr]);
+            float2 v;
+            if constexpr (kFp32) {
+              v = gr == 0 ? __fmul2_rn(sq, nu) : __ffma2_rn(sq, nu, sum);
+              if (gr == G - 1) v = __ffma2_rn(x, make_float2(0x1p-24f, 0x1p-24f), v);
+            } else {
+              v = __ffma2_rn(sq, nu, __ffma2_rn(x, step, __fmul2_rn(off, make_float2(row_sum[r][gr], row_sum[r][gr]))));
+              if (gr > 0) v = __fadd2_rn(v, sum);
+            }
             s[t][2 * r] = v.x; s[t][2 * r + 1] = v.y;
           }
         }
@@ -764,6 +766,15 @@ __global__ void __launch_bounds__(kWarps * 32, D == 64 ? kCtasPerSm64 : kCtasPer
   if (!cached(std::false_type{})) {                                // the warp's steps once more
     st = first + warp;
     if (st < last_c) load_keys_of(st);
+    if constexpr (kCodes) {                                        // with keys themselves: the query without the powers of two of the codes' places
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t up = (uint32_t)(15 + key_place<BITS>(2 * (ks % KPW) + (i >> 1)).bit) << 10;
+          qf[ks][i] = fma_f16x2(qf[ks][i], up | (up << 16), 0u);
+        }
+    }
     m_run[0] = m_run[1] = -INFINITY;
     l_cur[0] = l_cur[1] = l_cac[0] = l_cac[1] = 0.f;
 #pragma unroll
